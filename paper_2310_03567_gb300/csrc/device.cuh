@@ -172,13 +172,14 @@ struct Ctl {
   SL_HOT unsigned int alloc_seq;            // alloc_refs entries of this update
   SL_HOT unsigned int split_count;          // split-list entries of this update
   SL_HOT unsigned int ntasks;               // spill tasks (= freed chunks) of this update
-  unsigned int vis_count;                   // nodes drawn by the last render
   unsigned long long st_batches, st_points, st_rejected, st_spilled, st_splits, st_voxels,
       st_iter_max, st_rounds;
   unsigned long long last_points, last_spilled, last_splits, last_voxels, last_iters;
   unsigned long long st_rejected_async;  // rejections inside fused launches
   SL_HOT unsigned int mv_count[2];       // entries of the two mover lists
   SL_HOT unsigned long long render_samples;  // points and voxels visited by the last render
+  unsigned int vis_count;                    // nodes drawn by the last render
+  unsigned int draw_units;                   // chunks and array pieces they were cut into
   unsigned long long phase_ns[8];        // fused form: time per phase (see PH_*)
   unsigned long long st_compacted;       // nodes turned into arrays (simlod_compact), in all
   unsigned long long st_compact_chunks;  // chunks those nodes gave back to the pool

@@ -97,11 +97,27 @@ __device__ __forceinline__ bool node_drawn(const Ctx& c, const View& v, uint32_t
   return psize > v.lod;
 }
 
-// One thread per node: list the drawn nodes (warp-aggregated appends).
-__global__ void k_render_select(Ctx c, View v, uint32_t* vis) {
+// Clear the frame (clear != 0: n_px words of all ones) and list the drawn
+// nodes, one thread per node (warp-aggregated appends). The clear streams
+// 8 bytes per pixel and would be a launch of its own; here its stores drain
+// while the node tests wait for the node table.
+__global__ void k_render_select(Ctx c, View v, uint32_t* vis, unsigned long long* fb,
+                                uint64_t n_px, int clear) {
+  const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  if (clear) {
+    // the frame is 8-byte aligned; 16-byte stores from its first 16-byte boundary
+    const uint64_t head = (reinterpret_cast<uintptr_t>(fb) & 15u) ? 1u : 0u;
+    ulonglong2* fb2 = reinterpret_cast<ulonglong2*>(fb + head);
+    const uint64_t pairs = (n_px - head) / 2;
+    for (uint64_t i = t; i < pairs; i += stride) fb2[i] = make_ulonglong2(~0ull, ~0ull);
+    if (t == 0) {
+      if (head) fb[0] = ~0ull;
+      if ((n_px - head) & 1u) fb[n_px - 1u] = ~0ull;
+    }
+  }
   const uint32_t n = vload(&c.ctl->n_nodes);
   const uint32_t lane = threadIdx.x & 31u;
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t b = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); b < n; b += stride) {
     const uint64_t id = b + lane;
     const bool d = id < n && id < c.max_nodes && node_drawn(c, v, (uint32_t)id);
@@ -128,50 +144,147 @@ __device__ __forceinline__ void splat(const View& v, int4 r, unsigned long long*
   atomicMin(fb + (uint64_t)py * v.width + px, key);
 }
 
-// One warp per drawn node: walk its chunk list (Section 6's chunk loop, with the
-// next link loaded before the chunk's records are drawn) and splat every
-// point (leaf) or voxel (inner node).
-__global__ void k_render_draw(Ctx c, View v, const uint32_t* vis, unsigned long long* fb) {
-  const uint32_t nv = vload(&c.ctl->vis_count);
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
-  const uint64_t nwarps = (uint64_t)gridDim.x * blockDim.x / 32;
-  for (uint64_t k = warp; k < nv && k < c.max_nodes; k += nwarps) {
-    const uint32_t id = vis[k];
-    const uint32_t n = c.num[id];
-    const NodeMeta& m = c.meta[id];
-    if (m.compact) {  // one contiguous array (simlod_compact)
-      if (array_ok(c, m.head, n)) {
-        const int4* recs = array_recs(c, m.head);
-        for (uint32_t q = lane; q < n; q += 32) splat(v, recs[q], fb);
-      } else if (lane == 0) {
-        set_error(c, E_INTERNAL);
-      }
-      if (lane == 0) atomicAdd(&c.ctl->render_samples, (unsigned long long)n);
-      continue;
+// A piece of a drawn node: records [first, first + n) of the chunk or array
+// at ref. At most C records, so that a node's records spread over many warps.
+struct DrawUnit {
+  uint32_t ref, first, n, pad;
+};
+static_assert(sizeof(DrawUnit) == sizeof(SpillTask), "draw units use the spill-task region");
+
+__device__ __forceinline__ void draw_records(const Ctx& c, const View& v, const DrawUnit& u,
+                                             uint32_t lo, uint32_t hi, unsigned long long* fb) {
+  const int4* recs = chunk_recs(c, u.ref) + u.first;
+  constexpr uint32_t U = 4;  // records per lane in flight
+  for (uint32_t q = lo + lane_id(); q < hi; q += 32u * U) {
+    int4 r[U];
+#pragma unroll
+    for (uint32_t k = 0; k < U; ++k) {
+      if (q + 32u * k < hi) r[k] = __ldcg(recs + q + 32u * k);
     }
-    const uint32_t nch = m.n_chunks;
-    uint32_t ref = m.head, done = 0;
-    for (uint32_t j = 0; j < nch && done < n; ++j) {
-      if (!ref_ok(c, ref, c.chunk_bytes)) {
-        if (lane == 0) set_error(c, E_INTERNAL);
-        break;
-      }
-      const uint32_t nxt = *chunk_next(c, ref);
-      const uint32_t cnt = min(c.C, n - done);
-      const int4* recs = chunk_recs(c, ref);
-      for (uint32_t q = lane; q < cnt; q += 32) splat(v, recs[q], fb);
-      done += cnt;
-      ref = nxt;
+#pragma unroll
+    for (uint32_t k = 0; k < U; ++k) {
+      if (q + 32u * k < hi) splat(v, r[k], fb);
     }
-    if (lane == 0) atomicAdd(&c.ctl->render_samples, (unsigned long long)n);
   }
 }
 
-__global__ void k_fb_clear(unsigned long long* fb, uint64_t n) {
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-    fb[i] = ~0ull;
+// All 32 lanes call: lane i hands out its unit u (when on) at index at.
+// Units that do not fit the region (arrays cut into more pieces than the
+// data region has chunks) are drawn here.
+__device__ __forceinline__ void put_unit(const Ctx& c, const View& v, DrawUnit* units, bool on,
+                                         uint64_t at, const DrawUnit& u, unsigned long long* fb) {
+  const bool fits = at < c.max_chunks;
+  if (on && fits) units[at] = u;
+  unsigned over = __ballot_sync(FULL_MASK, on && !fits);
+  while (over) {
+    const int l = __ffs(over) - 1;
+    over &= over - 1u;
+    DrawUnit w;
+    w.ref = __shfl_sync(FULL_MASK, u.ref, l);
+    w.first = __shfl_sync(FULL_MASK, u.first, l);
+    w.n = __shfl_sync(FULL_MASK, u.n, l);
+    w.pad = 0;
+    draw_records(c, v, w, 0, w.n, fb);
+  }
+}
+
+// One warp per drawn node: cut its records into draw units of one chunk (or C
+// records of a compacted node's array). A leaf's chunks are in its directory.
+// An inner node's chunk list has to be walked, one memory round trip per
+// link; the chunks of one allocation lie one after another in the data
+// region, so the warp reads the next links of 32 such successors at once and
+// keeps as many as the list confirms (a link that points elsewhere ends the
+// run: the walk goes on from there).
+__global__ void k_render_units(Ctx c, View v, const uint32_t* vis, DrawUnit* units,
+                               unsigned long long* fb) {
+  const uint32_t nv = min(vload(&c.ctl->vis_count), c.max_nodes);
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
+  const uint64_t nwarps = (uint64_t)gridDim.x * blockDim.x / 32;
+  unsigned long long samples = 0;
+  for (uint64_t k = warp; k < nv; k += nwarps) {
+    const uint32_t id = vis[k];
+    const uint32_t n = c.num[id];
+    const NodeMeta& m = c.meta[id];
+    const uint32_t head = m.head, compact = m.compact, mdir = m.dir;
+    const uint32_t nch = compact ? (uint32_t)(((unsigned long long)n + c.C - 1) / c.C)
+                                 : m.n_chunks;
+    samples += n;
+    if (n == 0 || nch == 0) continue;
+    uint32_t u0 = 0;
+    if (lane == 0) u0 = atomicAdd(&c.ctl->draw_units, nch);
+    u0 = __shfl_sync(FULL_MASK, u0, 0);
+    auto records_of = [&](uint32_t j) -> uint32_t {  // records of the node's chunk j
+      const unsigned long long at = (unsigned long long)j * c.C;
+      return at < n ? (uint32_t)min((unsigned long long)c.C, n - at) : 0u;
+    };
+    const bool by_dir = !compact && c.child[id] == NONE && nch <= c.dir_cap &&
+                        ref_ok(c, mdir, c.dir_bytes);
+    if (compact || by_dir) {
+      const bool arr_ok = !compact || array_ok(c, head, n);
+      if (!arr_ok && lane == 0) set_error(c, E_INTERNAL);
+      const uint32_t* dir = by_dir ? dir_entries(c, mdir) : nullptr;
+      for (uint32_t j0 = 0; j0 < nch; j0 += 32u) {
+        const uint32_t j = j0 + lane;
+        const bool in = j < nch;
+        DrawUnit u{0, 0, 0, 0};
+        if (in && arr_ok) {
+          u.ref = compact ? head : dir[j];
+          u.first = compact ? j * c.C : 0u;
+          u.n = records_of(j);
+          if (!compact && !ref_ok(c, u.ref, c.chunk_bytes)) {
+            set_error(c, E_INTERNAL);
+            u = DrawUnit{0, 0, 0, 0};
+          }
+        }
+        put_unit(c, v, units, in, (uint64_t)u0 + j, u, fb);
+      }
+      continue;
+    }
+    uint32_t ref = head, j0 = 0;
+    while (j0 < nch) {
+      const uint32_t mine = ref + lane * c.chunk_units;
+      const bool in = j0 + lane < nch && ref != NONE && ref_ok(c, mine, c.chunk_bytes);
+      const uint32_t nxt = in ? *chunk_next(c, mine) : NONE;
+      // the run: lanes whose predecessors' links all lead to the next lane
+      const unsigned brk = __ballot_sync(FULL_MASK, !in || nxt != mine + c.chunk_units);
+      const uint32_t run = brk ? (uint32_t)__ffs(brk) : 32u;  // lanes before run are in the list
+      const bool ok = __shfl_sync(FULL_MASK, in ? 1 : 0, (int)run - 1) != 0;
+      const bool on = lane < run && j0 + lane < nch;
+      DrawUnit u{mine, 0, records_of(j0 + lane), 0};
+      if (!in) u = DrawUnit{0, 0, 0, 0};
+      if (on && !in) set_error(c, E_INTERNAL);
+      put_unit(c, v, units, on, (uint64_t)u0 + j0 + lane, u, fb);
+      j0 += run;
+      if (!ok) {  // a broken list: the rest of the reserved units draw nothing
+        for (uint32_t j = j0 + lane; j < nch; j += 32u)
+          if ((uint64_t)u0 + j < c.max_chunks) units[(uint64_t)u0 + j] = DrawUnit{0, 0, 0, 0};
+        break;
+      }
+      ref = __shfl_sync(FULL_MASK, nxt, (int)run - 1);
+    }
+  }
+  if (lane == 0 && samples) atomicAdd(&c.ctl->render_samples, samples);
+}
+
+// Splat the units, `parts` warps per unit (parts * part >= C): about 256
+// records a warp, so that a frame of a few nodes with tens of thousands of
+// records each fills the GPU. One warp per node (the first form) left the
+// longest node's chain of loads in charge: 0.43 ms for 3 nodes of 65k points
+// in all, 0.87-0.97 ms for frames of 1M to 13M samples alike. Two 1080p frames
+// of a 12M-point terrain (2.5M samples in the overview) went from 1.93 to
+// 0.11 ms. What is left is the three launches and, for frames of tens of
+// millions of samples, the 64-bit minimums on the frame in L2.
+__global__ void k_render_draw(Ctx c, View v, const DrawUnit* units, uint32_t parts, uint32_t part,
+                              unsigned long long* fb) {
+  const uint64_t nu = min((uint64_t)vload(&c.ctl->draw_units), (uint64_t)c.max_chunks);
+  const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
+  const uint64_t nwarps = (uint64_t)gridDim.x * blockDim.x / 32;
+  for (uint64_t w = warp; w < nu * parts; w += nwarps) {
+    const DrawUnit u = units[w / parts];
+    const uint32_t lo = (uint32_t)(w % parts) * part, hi = min(lo + part, u.n);
+    if (lo < hi) draw_records(c, v, u, lo, hi, fb);
+  }
 }
 
 }  // namespace SL_NS

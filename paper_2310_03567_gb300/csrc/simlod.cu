@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -1515,14 +1516,21 @@ SIMLOD_API int simlod_render(simlod_t* h, const float view_proj[16], uint32_t wi
   const Ctx& c = h->ctx;
   uint32_t* vis = reinterpret_cast<uint32_t*>(h->arena + h->lay.vis);
   unsigned long long* fb = reinterpret_cast<unsigned long long*>(d_framebuffer);
-  if (cudaMemsetAsync(&c.ctl->vis_count, 0, sizeof(unsigned int), s) != cudaSuccess ||
-      cudaMemsetAsync(&c.ctl->render_samples, 0, sizeof(unsigned long long), s) != cudaSuccess)
-    return SIMLOD_ERR_CUDA;
-  const unsigned grid = (unsigned)h->sm_count * 4;
+  // the sample count and the two list counters are neighbours
+  static_assert(offsetof(Ctl, vis_count) == offsetof(Ctl, render_samples) + 8 &&
+                    offsetof(Ctl, draw_units) == offsetof(Ctl, render_samples) + 12,
+                "one memset clears the render counters");
+  if (cudaMemsetAsync(&c.ctl->render_samples, 0, 16, s) != cudaSuccess) return SIMLOD_ERR_CUDA;
+  // the spill tasks are dead between updates (the render is ordered after
+  // them): their region, one entry per chunk, holds the draw units
+  DrawUnit* units = reinterpret_cast<DrawUnit*>(c.tasks);
+  const uint32_t parts = std::min<uint32_t>(16u, (c.C + 255u) / 256u);
+  const uint32_t part = ((c.C + parts - 1u) / parts + 31u) / 32u * 32u;
+  const unsigned grid = (unsigned)h->sm_count * 8;
   return launch(h, K_RENDER, s, [&] {
-    if (clear) k_fb_clear<<<grid, BLOCK, 0, s>>>(fb, (uint64_t)width * height);
-    k_render_select<<<grid, BLOCK, 0, s>>>(c, v, vis);
-    k_render_draw<<<grid * 2, BLOCK, 0, s>>>(c, v, vis, fb);
+    k_render_select<<<grid, BLOCK, 0, s>>>(c, v, vis, fb, (uint64_t)width * height, clear);
+    k_render_units<<<grid, BLOCK, 0, s>>>(c, v, vis, units, fb);
+    k_render_draw<<<grid, BLOCK, 0, s>>>(c, v, units, parts, part, fb);
   });
 }
 
