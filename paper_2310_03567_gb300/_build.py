@@ -91,7 +91,7 @@ def variant_flags(k: int) -> list[str]:
             f"-DSL_VARIANT_LAUNCH=sl_fused_variant_launch_{k}",
             f"-DSL_PHASE_BLOCK={block}", f"-DSL_PHASE_MIN_BLOCKS={per_sm}",
             f"-DSL_NODE_CACHE={cache}", f"-DSL_STORE_UNROLL={store_u}",
-            f"-DSL_DESCENT_GROUP={group}"]
+            f"-DSL_COUNT_UNROLL={group}"]
 
 
 def compile_commands(extra: list[str] | None = None, obj_dir: str = OBJ_DIR):

@@ -3,26 +3,32 @@
 // The update of one batch follows Section 5 of the paper, re-planned for a
 // GPU that can keep the per-update working set in L2:
 //
-//  count1  every batch point walks from the root to its leaf. At every inner
-//          node on the way it tests the node's occupancy bit (Section 3.3);
-//          an empty cell makes the point a contender for a new voxel. At the
-//          leaf it is counted (Section 5.1, "Counting"); the leaf is kept per
-//          point (its cursor).
-//  decide  per candidate node: a leaf whose stored + counted points exceed T
+//  count   every batch point walks from the root to its leaf and is counted
+//          there (Section 5.1, "Counting"); the leaf is kept per point (its
+//          cursor).
+//  decide  per candidate leaf: one whose stored + counted points exceed T
 //          splits (Section 5.1, "Splitting"): 8 children, a grid, and one
-//          spill task per chunk of its stored points. Any other counted node
+//          spill task per chunk of its stored points. Any other counted leaf
 //          is final and gets its chunks now (Section 5.3).
 //  advance points whose cursor node split in the previous round (batch
 //          points, and the stored points of split leaves, copied out of their
-//          old chunks at their first move) sample that node's grid and move
-//          one level down, counting into the child; the grids of the previous
-//          round's splits are zeroed alongside. Repeated with decide until
-//          nothing splits: the paper's iterative deepening, but each round
-//          touches only the points that have to move (mover lists).
-//  store   every point goes to its cursor leaf at the next free slot; every
-//          new voxel goes to its node (Section 5.4); occupancy bits are set
-//          here, after all claims of the update; the chunks of split leaves
-//          return to the pool (Section 3.4).
+//          old chunks at their first move) move one level down, counting into
+//          the child; the grids of the previous round's splits are zeroed
+//          alongside. Repeated with decide until nothing splits: the paper's
+//          iterative deepening, but each round touches only the points that
+//          have to move (mover lists).
+//  claim   with every point at its final leaf, the points sample the grids
+//          (Section 3.3) from the leaf's parent upwards. Cells nest: a cell of
+//          a node lies inside one cell of the node's parent. So a point whose
+//          cell is occupied already is done with every coarser level too, and
+//          so is a point that meets a lower arrival index in its cell: that
+//          point has the lower index in the coarser cells as well. Most points
+//          stop at their first claim, where a walk from the root claimed at
+//          every level (4.8 claims a point on a shuffled building scan).
+//  store   every point goes to its cursor leaf at the next free slot, and the
+//          inner nodes get the chunks of their new voxels; then every new
+//          voxel goes to its node (Section 5.4), occupancy bits are set, and
+//          the chunks of split leaves return to the pool (Section 3.4).
 //
 // Voxel claims: the paper lets the first point that finds an empty cell win.
 // Here all contenders of an update for a (node, cell) meet in an open-
@@ -30,8 +36,7 @@
 // lowest arrival index wins regardless of thread timing. The table entries of
 // an update are listed (the backlog of Section 5.2) and cleared by store.
 //
-// Descents read the node table (first child, grid reference) from a copy in
-// shared memory of the first NODE_CACHE nodes (the node ids of the upper
+// Descents read the node table (first child) from a copy in shared memory of the first NODE_CACHE nodes (the node ids of the upper
 // levels are the smallest): the plain form's count / advance kernels load it,
 // the persistent kernel loads it once and patches it after every decide
 // round with the nodes that split or were created.
@@ -63,23 +68,14 @@ constexpr uint32_t CHUNK_HEADER = 16;
 #ifndef SL_NODE_CACHE
 #define SL_NODE_CACHE 4096
 #endif
-#ifndef SL_DESCENT_GROUP
-#define SL_DESCENT_GROUP 2
-#endif
 #ifndef SL_PHASE_BLOCK
 #define SL_PHASE_BLOCK 512
 #endif
 #ifndef SL_PHASE_MIN_BLOCKS
 #define SL_PHASE_MIN_BLOCKS 2
 #endif
-#ifndef SL_HASH_BUCKET
-#define SL_HASH_BUCKET 0
-#endif
 #ifndef SL_ADVANCE_UNROLL
 #define SL_ADVANCE_UNROLL 1
-#endif
-#ifndef SL_ADVANCE_RUNS
-#define SL_ADVANCE_RUNS 0  // 1: the advance phase merges lanes with equal keys first
 #endif
 #ifndef SL_CTL_VIEW
 #define SL_CTL_VIEW 1
@@ -95,6 +91,9 @@ constexpr uint32_t CHUNK_HEADER = 16;
 #endif
 #ifndef SL_COUNT_UNROLL
 #define SL_COUNT_UNROLL 1
+#endif
+#ifndef SL_CLAIM_UNROLL
+#define SL_CLAIM_UNROLL 1
 #endif
 #ifndef SL_STORE_UNROLL
 #define SL_STORE_UNROLL 2
@@ -112,9 +111,7 @@ constexpr uint32_t CHUNK_HEADER = 16;
 #define SL_COUNT_CHUNK_DIV 8  // a chunk size keeps at least this many chunks per warp
 #endif
 constexpr uint32_t NODE_CACHE = SL_NODE_CACHE;         // nodes mirrored in shared memory
-constexpr uint32_t NODE_CACHE_BYTES = NODE_CACHE * 8;  // child + grid reference
 constexpr uint32_t ZERO_UNIT = 4096;                   // bytes of grid zeroed per warp unit
-constexpr int DESCENT_GROUP = SL_DESCENT_GROUP;        // levels whose grid words load together
 constexpr int ADVANCE_U = SL_ADVANCE_UNROLL;           // advance units a warp carries at a time
 constexpr int COUNT_U = SL_COUNT_UNROLL;               // count units a warp carries at a time
 #ifndef SL_WBUF
@@ -125,14 +122,14 @@ constexpr int PHASE_BLOCK = SL_PHASE_BLOCK;            // threads of count / adv
 constexpr int PHASE_MIN_BLOCKS = SL_PHASE_MIN_BLOCKS;  // resident blocks per SM they aim for
 // dynamic shared memory of the count / advance / fused blocks
 #ifndef SL_MVBUF
-#define SL_MVBUF 256
+#define SL_MVBUF 288
 #endif
 constexpr uint32_t MVBUF = SL_MVBUF;                    // mover-list entries staged per warp
 constexpr uint32_t TALLY_LOG2 = 9;                      // block tally cache: 512 nodes
 constexpr uint32_t TALLY_SLOTS = 1u << TALLY_LOG2;
 // dynamic shared memory of the count / advance / fused blocks: node cache,
 // new-cell staging, mover staging, block tally cache
-constexpr uint32_t SMEM_WBUF = 2 * NODE_CACHE;                        // in u32 words
+constexpr uint32_t SMEM_WBUF = NODE_CACHE;                            // in u32 words
 constexpr uint32_t SMEM_MVBUF = SMEM_WBUF + (PHASE_BLOCK / 32) * WBUF;
 constexpr uint32_t SMEM_TALLY = SMEM_MVBUF + (PHASE_BLOCK / 32) * MVBUF * 2;
 constexpr uint32_t PHASE_SMEM_BYTES = 4 * (SMEM_TALLY + 2 * TALLY_SLOTS);
@@ -165,6 +162,10 @@ struct Ctl {
   unsigned long long chunks_bumped;         // chunks taken from the data region
   SL_HOT unsigned int n_nodes;
   SL_HOT int pool_top;                      // chunk refs in the pool
+  unsigned long long bump0;                 // bump at the end of the last update: the grids of
+                                            //   nodes that split in this one lie above it
+  unsigned int key_rate;                    // expected voxel keys per 1,024 points of an update
+  unsigned int open;                        // 1: restored voxels do not nest (see k_check_nested)
   unsigned int error;                       // sticky E_* bits
   unsigned int reject;                      // out-of-cube point seen in this update
   SL_HOT unsigned int spill_count;          // re-inserted points of this update
@@ -192,7 +193,7 @@ struct Ctl {
 static_assert(sizeof(Ctl) % 16 == 0, "Ctl size");
 
 // Phases of the fused form, for its phase clock.
-enum : int { PH_COUNT = 0, PH_DECIDE, PH_ADVANCE, PH_STORE, PH_END, PH_ROLLBACK, PH_LAUNCH, PH_OTHER };
+enum : int { PH_COUNT = 0, PH_DECIDE, PH_ADVANCE, PH_STORE, PH_END, PH_CLAIM, PH_LAUNCH, PH_OTHER };
 
 // Per-node metadata that the count/advance hot loops do not touch.
 struct NodeMeta {
@@ -207,11 +208,17 @@ struct NodeMeta {
   uint32_t st_base;     //   and the records stored before this update
   uint32_t touched;     // updates applied when the node last received records (1 = the first)
   uint32_t compact;     // 1: the records are one contiguous array (head), not a chunk list
-  uint32_t pad[2];
+  uint32_t up;          // parent | parent's level << MV_NODE_BITS, NONE at the root
+  uint32_t up_grid;     // the parent's occupancy grid
 };
 static_assert(sizeof(NodeMeta) == 64, "NodeMeta size");
 static_assert(offsetof(NodeMeta, st_nch) == 32 && offsetof(NodeMeta, st_base) == 44,
               "the store map is one aligned 16-byte load");
+static_assert(offsetof(NodeMeta, up) == 56, "up and up_grid are one aligned 8-byte load");
+
+constexpr uint32_t MV_SPILL = 1u << 31;
+constexpr uint32_t MV_NODE_BITS = 27;  // node ids below 2^27 (the node table limit)
+constexpr uint32_t MV_NODE_MASK = (1u << MV_NODE_BITS) - 1u;
 
 struct __align__(16) HSlot {
   unsigned long long key;  // (node << 3G) | cell, HASH_EMPTY when free
@@ -342,16 +349,14 @@ __device__ __forceinline__ uint32_t* dir_entries(const Ctx& c, uint32_t ref) {
 }
 
 // Coordinates relative to the root minimum; false when outside the root cube.
+// The cube lies in the int32 range and its side is at most 2^31, so the
+// wrapped 32-bit difference is below the side exactly for the points inside.
 __device__ __forceinline__ bool rel_coords(const Ctx& c, int4 p, uint32_t& rx, uint32_t& ry,
                                            uint32_t& rz) {
-  long long dx = (long long)p.x - c.rmin[0];
-  long long dy = (long long)p.y - c.rmin[1];
-  long long dz = (long long)p.z - c.rmin[2];
-  long long side = 1ll << c.rlog2;
-  rx = (uint32_t)dx;
-  ry = (uint32_t)dy;
-  rz = (uint32_t)dz;
-  return dx >= 0 && dy >= 0 && dz >= 0 && dx < side && dy < side && dz < side;
+  rx = (uint32_t)p.x - (uint32_t)c.rmin[0];
+  ry = (uint32_t)p.y - (uint32_t)c.rmin[1];
+  rz = (uint32_t)p.z - (uint32_t)c.rmin[2];
+  return ((rx | ry | rz) >> c.rlog2) == 0u;
 }
 
 // Octant of a point inside a node of side 2^L (L >= 1): bit L-1 per axis.
@@ -375,10 +380,9 @@ __device__ __forceinline__ uint32_t cell_index(uint32_t rx, uint32_t ry, uint32_
 
 // ------------------------------------------------------- node-table cache
 
-// Shared-memory copy of child[] and gridref[] for nodes [0, NODE_CACHE).
+// Shared-memory copy of child[] for nodes [0, NODE_CACHE).
 struct NodeCache {
   uint32_t* child;
-  uint32_t* grid;
   uint32_t n;  // cached nodes
 };
 
@@ -386,7 +390,6 @@ struct NodeCache {
 __device__ __forceinline__ NodeCache node_cache_at(uint32_t* smem, uint32_t n_nodes) {
   NodeCache nc;
   nc.child = smem;
-  nc.grid = smem + NODE_CACHE;
   nc.n = n_nodes < NODE_CACHE ? n_nodes : NODE_CACHE;
   return nc;
 }
@@ -396,24 +399,18 @@ __device__ __forceinline__ NodeCache node_cache_at(uint32_t* smem, uint32_t n_no
 __device__ __forceinline__ void node_cache_load(const Ctx& c, uint32_t* smem, uint32_t lo,
                                                 uint32_t hi) {
   hi = hi < NODE_CACHE ? hi : NODE_CACHE;
-  for (uint32_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-    smem[i] = c.child[i];
-    smem[NODE_CACHE + i] = c.gridref[i];
-  }
+  for (uint32_t i = lo + threadIdx.x; i < hi; i += blockDim.x) smem[i] = c.child[i];
 }
 
 // The whole block brings the cache up to date after a decide round: the
-// nodes of the split entries [s_lo, s_hi) became inner (child and grid set),
-// the nodes [n_lo, n_hi) were created (leaves without a grid). Nothing else
-// in the node table changes during an update. The caller synchronises.
+// nodes of the split entries [s_lo, s_hi) became inner, the nodes
+// [n_lo, n_hi) were created. Nothing else in the node table changes during an
+// update. The caller synchronises.
 __device__ __forceinline__ void node_cache_patch(const Ctx& c, uint32_t* smem, uint32_t s_lo,
                                                  uint32_t s_hi, uint32_t n_lo, uint32_t n_hi) {
   for (uint32_t e = s_lo + threadIdx.x; e < s_hi; e += blockDim.x) {
     const uint32_t id = c.splits[e].node;
-    if (id < NODE_CACHE) {
-      smem[id] = c.child[id];
-      smem[NODE_CACHE + id] = c.gridref[id];
-    }
+    if (id < NODE_CACHE) smem[id] = c.child[id];
   }
   node_cache_load(c, smem, n_lo, n_hi);
 }
@@ -467,10 +464,6 @@ __device__ __forceinline__ uint32_t node_child(const Ctx& c, NodeCache nc, uint3
   return id < nc.n ? nc.child[id] : c.child[id];
 }
 
-__device__ __forceinline__ uint32_t node_grid(const Ctx& c, NodeCache nc, uint32_t id) {
-  return id < nc.n ? nc.grid[id] : c.gridref[id];
-}
-
 // -------------------------------------------------------- voxel claims
 
 template <typename T>
@@ -491,56 +484,81 @@ __device__ __forceinline__ ulonglong2 slot_load(const HSlot* s) {
   return kv;
 }
 
-// First claim-table slot of a key (node << 3G | cell). By default it is the
-// top log2(slots) bits of key * 2^64 / phi (multiplicative hashing: one
-// 64-bit multiply instead of the two of a 64-bit finalizer; where a key sits
-// does not change which point wins). With SL_HASH_FIB=0 a 64-bit finalizer
-// places every key at random, or, with SL_HASH_BUCKET, runs of
-// 2^SL_HASH_BUCKET cells along x share one randomly placed bucket of slots,
-// so that the neighbouring cells a warp claims fall on a few cache lines.
-#ifndef SL_HASH_FIB
-#define SL_HASH_FIB 1
-#endif
-__device__ __forceinline__ uint32_t claim_slot(const Ctx& c, unsigned long long key) {
-#if SL_HASH_FIB
-  const uint32_t bits = (uint32_t)__popc(c.hash_mask);  // the table has at least 2 slots
-  return (uint32_t)((key * 0x9E3779B97F4A7C15ull) >> (64u - bits)) & c.hash_mask;
-#elif SL_HASH_BUCKET
-  constexpr uint32_t B = SL_HASH_BUCKET;
-  return (((uint32_t)fmix64(key >> B) << B) | ((uint32_t)key & ((1u << B) - 1u))) & c.hash_mask;
-#else
-  return (uint32_t)fmix64(key) & c.hash_mask;
-#endif
+// The claim table of one update. A key (node << 3G | cell) is looked for along
+// a fixed sequence of slots: CLAIM_NEAR of them in the table's first near + 1
+// slots, as many as the update's expected keys call for, then in the whole
+// table (two slots per backlog entry, whatever the data). So the updates
+// of a stream use the same lines again, which stay in L2, where a table sized
+// for the largest update took new lines from DRAM every time: claims of a
+// uniform stream of 500k batches 0.90 against 1.27 ms a pass, of a shuffled
+// building scan 1.20 against 1.40 ms.
+// Cells that differ in the low CLAIM_BUCKET bits of their x sit in one bucket
+// of 8 neighbouring slots (128 bytes), because the cells that a warp claims
+// are neighbours (a 16M-point terrain: 0.69 against 0.94 ms). The bucket is
+// the top bits of (key without those bits) * 2^64 / phi. The near step is odd,
+// so that a sequence reaches every slot, and one more than a bucket, so that
+// keys that meet do not fill each other's buckets (0.69 against 0.82 ms with
+// the next slot); the far step is an odd part of the hash, which leaves the
+// full near part at once. Where a key sits does not change which point wins.
+constexpr uint32_t CLAIM_BUCKET = 3;
+constexpr uint32_t CLAIM_LOW = (1u << CLAIM_BUCKET) - 1u;
+constexpr uint32_t CLAIM_STEP = (1u << CLAIM_BUCKET) + 1u;
+constexpr int CLAIM_NEAR = 16;
+
+__device__ __forceinline__ uint32_t claim_slot(unsigned long long key, uint32_t mask) {
+  const uint32_t top =
+      (uint32_t)(((key >> CLAIM_BUCKET) * 0x9E3779B97F4A7C15ull) >> 32) >> __clz(mask);
+  return ((top & ~CLAIM_LOW) | ((uint32_t)key & CLAIM_LOW)) & mask;  // (mask > 0)
 }
 
-// Probes after the first for `key` (slot h held another key): returns true,
-// with the slot in h, when this call put the key into the table (the cell is
-// new in this update); a slot already holding the key is lowered to val if
-// val is smaller.
-__device__ bool hash_claim_rest(const Ctx& c, unsigned long long key, unsigned long long val,
-                                uint32_t& h) {
+// The near mask of an update of n points, batch and re-inserted, that is
+// expected to make `rate` / 1024 keys per point (Ctl::key_rate): 6 to 12
+// slots per expected key. (Fewer lengthen the probes, more leave L2: 0.5, 1,
+// 2 and 4 slots per point took 1.26, 1.20, 1.31 and 1.34 ms on the building
+// scan with 0.11 keys per point, 2 and 4 took 1.80 and 1.09 ms on the uniform
+// stream with 1.4.)
+__device__ __forceinline__ uint32_t claim_near_mask(const Ctx& c, uint64_t n, uint32_t rate) {
+  const uint64_t want = n * rate * 6u / 1024u;
+  if (want > c.hash_mask) return c.hash_mask;
+  return want <= 1024u ? (c.hash_mask < 1023u ? c.hash_mask : 1023u)
+                       : FULL_MASK >> __clz((uint32_t)want - 1u);
+}
+
+// Probes after the first for `key` (slot h held another key). CLAIM_NEW, with
+// the slot in h: this call put the key into the table (the cell is new in this
+// update); CLAIM_LOWERED: the slot held the key with a larger value (or
+// another call is putting it in); CLAIM_BEATEN: it holds a lower value.
+enum : int { CLAIM_NEW = 0, CLAIM_LOWERED, CLAIM_BEATEN };
+
+__device__ int hash_claim_rest(const Ctx& c, unsigned long long key, unsigned long long val,
+                               uint32_t near, uint32_t& h) {
+  uint32_t mask = near, step = CLAIM_STEP;
   for (int probe = 1; probe < MAX_PROBES; ++probe) {
-    h = (h + 1u) & c.hash_mask;
+    h = (h + step) & mask;
+    if (probe == CLAIM_NEAR) {
+      mask = c.hash_mask;
+      h = claim_slot(key, mask);
+      step = (uint32_t)(key * 0x9E3779B97F4A7C15ull >> 16) | 1u;
+    }
     HSlot* s = c.hash + h;
     const ulonglong2 kv = slot_load(s);
-    unsigned long long k = kv.x;
+    unsigned long long k = kv.x, v = kv.y;
     if (k == HASH_EMPTY) {
       k = atomicCAS(&s->key, HASH_EMPTY, key);
+      v = HASH_EMPTY;
       if (k == HASH_EMPTY) {
         atomicMin(&s->val, val);
-        return true;
+        return CLAIM_NEW;
       }
-      if (k == key) atomicMin(&s->val, val);
-      else continue;
-      return false;
     }
     if (k == key) {
-      if (kv.y > val) atomicMin(&s->val, val);
-      return false;
+      if (v < val) return CLAIM_BEATEN;
+      atomicMin(&s->val, val);
+      return CLAIM_LOWERED;
     }
   }
   set_error(c, E_BACKLOG);
-  return false;
+  return CLAIM_BEATEN;
 }
 
 // ------------------------------------------------ lane runs (warp groups)
@@ -577,18 +595,6 @@ __device__ __forceinline__ LaneRun lane_run(bool on, T v) {
   const unsigned breaks = (heads | ~onm) & ~lanes_upto(r.first);
   r.end = breaks ? (uint32_t)__ffs(breaks) - 1u : 32u;
   return r;
-}
-
-// All 32 lanes call: the minimum of v over this lane and the lanes after it
-// in its run (at the run's first lane: the run's minimum).
-__device__ __forceinline__ unsigned long long run_min(unsigned long long v, const LaneRun& r) {
-  const uint32_t lane = lane_id();
-#pragma unroll
-  for (uint32_t d = 1; d < 32u; d <<= 1) {
-    const unsigned long long o = __shfl_down_sync(FULL_MASK, v, d);
-    if (lane + d < r.end && o < v) v = o;
-  }
-  return v;
 }
 
 // Per-warp staging of the table slots of new cells (shared memory), flushed
@@ -665,24 +671,25 @@ __device__ __forceinline__ void mover_add(const Ctx& c, MoverBuf& mb, int list, 
   mb.n += k;
 }
 
-// All 32 lanes call. Lanes with lead[j] offer val[j] for cell key[j] of node
-// node[j] to the update's claim table; the lowest value wins. The first
-// probes of all N items are issued together (their key loads, then their
+// All 32 lanes call. Lanes with lead[j] offer val[j] for key[j] (a cell of
+// node[j]) to the update's claim table, where the lowest value wins. The
+// first probes of all N items are issued together (their loads, then their
 // compare-and-swaps), so the items pay about two L2 round trips together. A
 // key new in this update is staged for the backlog and counted towards its
-// node's new voxels.
+// node's new voxels. on[j] becomes true in lanes that met no lower value.
 template <int N>
-__device__ __forceinline__ void warp_claim_global(const Ctx& c, WarpBuf& wb, const bool (&lead)[N],
-                                                  const unsigned long long (&key)[N],
-                                                  const unsigned long long (&val)[N],
-                                                  const uint32_t (&node)[N]) {
+__device__ __forceinline__ void warp_claim(const Ctx& c, WarpBuf& wb, const bool (&lead)[N],
+                                           const unsigned long long (&key)[N],
+                                           const unsigned long long (&val)[N],
+                                           const uint32_t (&node)[N], uint32_t near,
+                                           bool (&on)[N]) {
   const uint32_t lane = lane_id();
   bool cas[N], inst[N];
   uint32_t h[N];
   unsigned long long k0[N], v0[N];
 #pragma unroll
   for (int j = 0; j < N; ++j) {
-    h[j] = claim_slot(c, key[j]);
+    h[j] = claim_slot(key[j], near);
     k0[j] = v0[j] = 0ull;
     if (lead[j]) {
       const ulonglong2 kv = slot_load(c.hash + h[j]);
@@ -703,12 +710,17 @@ __device__ __forceinline__ void warp_claim_global(const Ctx& c, WarpBuf& wb, con
     inst[j] = false;
     if (lead[j]) {
       if (cas[j] && k0[j] == HASH_EMPTY) {
-        inst[j] = true;
+        inst[j] = on[j] = true;
         atomicMin(&c.hash[h[j]].val, val[j]);
       } else if (k0[j] == key[j]) {
-        if (v0[j] > val[j]) atomicMin(&c.hash[h[j]].val, val[j]);
+        if (v0[j] > val[j]) {
+          on[j] = true;
+          atomicMin(&c.hash[h[j]].val, val[j]);
+        }
       } else {
-        inst[j] = hash_claim_rest(c, key[j], val[j], h[j]);
+        const int got = hash_claim_rest(c, key[j], val[j], near, h[j]);
+        inst[j] = got == CLAIM_NEW;
+        if (got != CLAIM_BEATEN) on[j] = true;
       }
     }
   }
@@ -725,32 +737,6 @@ __device__ __forceinline__ void warp_claim_global(const Ctx& c, WarpBuf& wb, con
     }
     wb.n += ni;
   }
-}
-
-// All 32 lanes call. For each of N items j, lanes with want[j] contend for
-// the cell key[j] = (node[j], cell) with val = (gidx << 32 | rgba); the lowest
-// gidx wins. Lanes with equal keys in a run are merged first and only the
-// run's lowest gidx goes to the global table. SORTED: gidx grows with the
-// lane, so a run's first lane holds its lowest gidx.
-template <int N, bool SORTED>
-__device__ __forceinline__ void warp_claim(const Ctx& c, WarpBuf& wb, const bool (&want)[N],
-                                           const unsigned long long (&key)[N],
-                                           const uint32_t (&gidx)[N], const uint32_t (&rgba)[N],
-                                           const uint32_t (&node)[N]) {
-  bool any = false;
-#pragma unroll
-  for (int j = 0; j < N; ++j) any = any || want[j];
-  if (__ballot_sync(FULL_MASK, any) == 0u) return;
-  bool lead[N];
-  unsigned long long val[N];
-#pragma unroll
-  for (int j = 0; j < N; ++j) {
-    val[j] = ((unsigned long long)gidx[j] << 32) | rgba[j];
-    const LaneRun r = lane_run(want[j], key[j]);
-    if (!SORTED) val[j] = run_min(want[j] ? val[j] : ~0ull, r);
-    lead[j] = want[j] && r.head;
-  }
-  warp_claim_global<N>(c, wb, lead, key, val, node);
 }
 
 // All 32 lanes call. Lanes with `valid` count one point into `leaf` (one
@@ -784,183 +770,84 @@ __device__ __forceinline__ uint32_t count_chunk_log2(uint64_t units, uint64_t nw
 
 // ------------------------------------------------------------ phase: count1
 
-// Iteration 1 for the batch points [0, n): descend, claim, count. `smem`
-// holds PHASE_SMEM_BYTES of dynamic shared memory; n_nodes is the node count.
+// Iteration 1 for the batch points [0, n): descend and count. `smem` holds
+// PHASE_SMEM_BYTES of dynamic shared memory.
 __device__ void phase_count1(const Ctx& c, uint32_t* smem, const NodeCache nc, const int4* pts,
-                             uint64_t n, unsigned long long base, uint64_t warp0,
-                             uint64_t nwarps) {
-  constexpr int U = COUNT_U, D = DESCENT_GROUP;
+                             uint64_t n, uint64_t warp0, uint64_t nwarps) {
+  constexpr int U = COUNT_U;
   tally_init(smem);
   __syncthreads();  // also publishes the caller's node-cache writes
-  WarpBuf wb = warp_buf(smem);
   const uint32_t lane = lane_id();
   // each warp carries U units of 32 points (warp_unit k, k + 1, ...) at a
-  // time so that their L2 round trips overlap; the next units' points are
-  // loaded while the current ones descend
+  // time so that their descents overlap; the next units' points are loaded
+  // while the current ones descend
   const uint32_t chl = count_chunk_log2((n + 31) / 32, nwarps);
-#if SL_COUNT_PREFETCH
   int4 pn[U];
 #pragma unroll
   for (int j = 0; j < U; ++j) {
     const uint64_t i = warp_unit(warp0, nwarps, j, chl) * 32 + lane;
     pn[j] = i < n ? __ldcg(pts + i) : make_int4(0, 0, 0, 0);
   }
-#endif
   for (uint64_t k0 = 0; warp_unit(warp0, nwarps, k0, chl) * 32 < n; k0 += U) {
     bool valid[U], walking[U];
-    int4 p[U];
-    uint32_t rx[U], ry[U], rz[U], node[U], L[U], gidx[U];
+    uint32_t rx[U], ry[U], rz[U], node[U], L[U];
     uint64_t iu[U];
+    bool any = false;
 #pragma unroll
     for (int j = 0; j < U; ++j) {
       const uint64_t i = warp_unit(warp0, nwarps, k0 + j, chl) * 32 + lane;
       iu[j] = i;
       valid[j] = i < n;
-#if SL_COUNT_PREFETCH
-      p[j] = pn[j];
+      const int4 p = pn[j];
       const uint64_t inext = warp_unit(warp0, nwarps, k0 + j + U, chl) * 32 + lane;
       pn[j] = inext < n ? __ldcg(pts + inext) : make_int4(0, 0, 0, 0);
-#else
-      p[j] = valid[j] ? __ldcg(pts + i) : make_int4(0, 0, 0, 0);
-#endif
-      gidx[j] = (uint32_t)(base + i);
-    }
-#pragma unroll
-    for (int j = 0; j < U; ++j) {
-      rx[j] = ry[j] = rz[j] = 0;
-      if (valid[j] && !rel_coords(c, p[j], rx[j], ry[j], rz[j])) {
+      if (!rel_coords(c, p, rx[j], ry[j], rz[j]) && valid[j]) {
         atomicOr(&c.ctl->reject, 1u);
         valid[j] = false;
       }
       node[j] = 0;
       L[j] = c.rlog2;
       walking[j] = valid[j];
+      any = any || walking[j];
     }
-    for (;;) {
-      bool any = false;
-#pragma unroll
-      for (int j = 0; j < U; ++j) any = any || walking[j];
-      if (!__any_sync(FULL_MASK, any)) break;
-      // Walk up to D levels through the node table first and issue their
-      // grid-word loads together (their addresses do not depend on each
-      // other), then test the bits and claim all of them at once.
-      uint32_t gnode[U * D], gcell[U * D], gword[U * D];
-      bool ginner[U * D];
+    while (any) {
+      any = false;
 #pragma unroll
       for (int j = 0; j < U; ++j) {
-#pragma unroll
-        for (int k = 0; k < D; ++k) {
-          const int s = j * D + k;
-          ginner[s] = false;
-          gnode[s] = node[j];
-          gcell[s] = 0;
-          gword[s] = 0;
-          if (walking[j]) {
-            const uint32_t ch = node_child(c, nc, node[j]);
-            if (ch == NONE) {
-              walking[j] = false;
-            } else {
-              const uint32_t gref = node_grid(c, nc, node[j]);
-              const uint32_t cell = cell_index(rx[j], ry[j], rz[j], L[j], c.G);
-              const uint32_t nxt = ch + octant(rx[j], ry[j], rz[j], L[j]);
-              if (!ref_ok(c, gref, c.grid_bytes) || nxt >= c.max_nodes) {
-                set_error(c, E_INTERNAL);
-                walking[j] = false;
-              } else {
-                ginner[s] = true;
-                gcell[s] = cell;
-                gword[s] = grid_words(c, gref)[cell >> 5];
-                node[j] = nxt;
-                --L[j];
-              }
-            }
-          }
+        if (!walking[j]) continue;
+        const uint32_t ch = node_child(c, nc, node[j]);
+        if (ch == NONE) {
+          walking[j] = false;
+        } else if (ch + 8u > c.max_nodes || L[j] == 0u) {
+          set_error(c, E_INTERNAL);
+          walking[j] = false;
+        } else {
+          node[j] = ch + octant(rx[j], ry[j], rz[j], L[j]);
+          --L[j];
+          any = true;
         }
       }
-      bool want[U * D];
-      unsigned long long key[U * D];
-      uint32_t gg[U * D], gc[U * D];
-#pragma unroll
-      for (int s = 0; s < U * D; ++s) {
-        want[s] = ginner[s] && ((gword[s] >> (gcell[s] & 31u)) & 1u) == 0u;
-        key[s] = ((unsigned long long)gnode[s] << (3u * c.G)) | gcell[s];
-        gg[s] = gidx[s / D];
-        gc[s] = (uint32_t)p[s / D].w;
-      }
-      warp_claim<U * D, true>(c, wb, want, key, gg, gc, gnode);
     }
+    __syncwarp();
 #pragma unroll
     for (int j = 0; j < U; ++j) {
       warp_tally(c, smem, valid[j], node[j]);
       if (valid[j]) c.b_cur[iu[j]] = node[j];
     }
   }
-  warp_flush(c, wb);
   tally_flush(c, smem);
 }
 
 // ----------------------------------------------------------- phase: advance
 
-// U items per lane whose cursor node split in the previous round (moving[j]:
-// the cursor cur[j], at level lvl[j], has children ch[j]) sample that node's
-// grid (empty until store, so every point contends) and move one level down,
-// counting into the child. cur[j] then holds the new cursor.
-template <int U>
-__device__ __forceinline__ void advance_items(const Ctx& c, WarpBuf& wb, const bool (&moving)[U],
-                                              const int4 (&p)[U], const uint32_t (&gidx)[U],
-                                              const uint32_t (&lvl)[U], const uint32_t (&ch)[U],
-                                              uint32_t (&cur)[U]) {
-  uint32_t nxt[U], rgba[U];
-  unsigned long long key[U];
-#pragma unroll
-  for (int j = 0; j < U; ++j) {
-    uint32_t rx = 0, ry = 0, rz = 0, cell = 0;
-    nxt[j] = cur[j];
-    if (moving[j]) {
-      rel_coords(c, p[j], rx, ry, rz);
-      const uint32_t L = c.rlog2 - lvl[j];
-      cell = cell_index(rx, ry, rz, L, c.G);
-      nxt[j] = ch[j] + octant(rx, ry, rz, L);
-    }
-    key[j] = ((unsigned long long)cur[j] << (3u * c.G)) | cell;
-    rgba[j] = (uint32_t)p[j].w;
-  }
-#if SL_ADVANCE_RUNS
-  warp_claim<U, false>(c, wb, moving, key, gidx, rgba, cur);
-#else
-  // Every moving lane offers its own value: the movers of one warp rarely
-  // share a cell (lane runs merged 1.4 % of these claims), so the run and
-  // its 64-bit segmented minimum would cost more than they save. Lanes with
-  // the same key meet in the table, where one compare-and-swap puts the key
-  // in and every lower value lowers the slot.
-  bool any = false;
-#pragma unroll
-  for (int j = 0; j < U; ++j) any = any || moving[j];
-  if (__ballot_sync(FULL_MASK, any) != 0u) {
-    unsigned long long val[U];
-#pragma unroll
-    for (int j = 0; j < U; ++j) val[j] = ((unsigned long long)gidx[j] << 32) | rgba[j];
-    warp_claim_global<U>(c, wb, moving, key, val, cur);
-  }
-#endif
-#pragma unroll
-  for (int j = 0; j < U; ++j) {
-    warp_tally(c, wb.smem, moving[j], nxt[j]);
-    cur[j] = nxt[j];
-  }
-}
-
 // A mover-list entry (8 bytes) is a point whose cursor moved in the last
 // advance round: x = MV_SPILL | spill entry, or a batch point index; y = its
 // cursor node (MV_NODE_BITS bits) | that node's level << MV_NODE_BITS.
-constexpr uint32_t MV_SPILL = 1u << 31;
-constexpr uint32_t MV_NODE_BITS = 27;  // node ids below 2^27 (the node table limit)
-constexpr uint32_t MV_NODE_MASK = (1u << MV_NODE_BITS) - 1u;
 
 // Advance round r of the expansion (r >= 2 counts decide rounds): zero the
 // grids of the splits [s_lo, s_hi) of the previous decide, then move every
-// point whose cursor node split there one level down (advance_items), and
-// list the points that moved in mover list out_list.
+// point whose cursor node split there one level down, counting it into the
+// child, and list the points that moved in mover list out_list.
 //
 // Only nodes created in the previous round can split in a later one (every
 // leaf that existed before the update was decided in the first round), so
@@ -972,12 +859,11 @@ constexpr uint32_t MV_NODE_MASK = (1u << MV_NODE_BITS) - 1u;
 // level. Points are cut into 32-item warp units (a unit of a task never
 // crosses into the next task).
 __device__ void phase_advance(const Ctx& c, uint32_t* smem, const NodeCache nc, const int4* pts,
-                              uint64_t n, unsigned long long base, uint32_t t_hi, uint32_t s_lo,
-                              uint32_t s_hi, int in_list, uint32_t n_in, int out_list,
-                              uint64_t warp0, uint64_t nwarps) {
+                              uint64_t n, uint32_t t_hi, uint32_t s_lo, uint32_t s_hi,
+                              int in_list, uint32_t n_in, int out_list, uint64_t warp0,
+                              uint64_t nwarps) {
   tally_init(smem);
   __syncthreads();  // also publishes the caller's node-cache writes
-  WarpBuf wb = warp_buf(smem);
   MoverBuf mb = mover_buf(smem);
   const uint32_t lane = lane_id();
   const uint32_t zpg = (c.grid_bytes + ZERO_UNIT - 1) / ZERO_UNIT;  // zero units per grid
@@ -1005,13 +891,13 @@ __device__ void phase_advance(const Ctx& c, uint32_t* smem, const NodeCache nc, 
   // here: the movers of dense regions then load few warps)
   for (uint64_t k0 = 0; warp_unit(warp0, nwarps, k0, 0) < units; k0 += AU) {
     bool valid[AU], spill[AU], have_p[AU], mv[AU];
-    uint32_t idx[AU], cur[AU], lvl[AU], g[AU], ch[AU];  // idx: batch point index or spill entry
+    uint32_t idx[AU], cur[AU], lvl[AU], ch[AU];  // idx: batch point index or spill entry
     int4 p[AU];
 #pragma unroll
     for (int j = 0; j < AU; ++j) {
       const uint64_t w = warp_unit(warp0, nwarps, k0 + j, 0);
       valid[j] = spill[j] = have_p[j] = false;
-      idx[j] = cur[j] = lvl[j] = g[j] = 0;
+      idx[j] = cur[j] = lvl[j] = 0;
       p[j] = make_int4(0, 0, 0, 0);
       if (w >= units) {
         // past the end: nothing
@@ -1034,9 +920,8 @@ __device__ void phase_advance(const Ctx& c, uint32_t* smem, const NodeCache nc, 
         if (valid[j]) {
           // the point leaves its chunk (which returns to the pool at store)
           p[j] = chunk_recs(c, tk.ref)[q];
-          g[j] = chunk_aux(c, tk.ref)[q];
           c.sp_rec[idx[j]] = p[j];
-          c.sp_gidx[idx[j]] = g[j];
+          c.sp_gidx[idx[j]] = chunk_aux(c, tk.ref)[q];
           have_p[j] = true;
         }
       } else {
@@ -1067,19 +952,18 @@ __device__ void phase_advance(const Ctx& c, uint32_t* smem, const NodeCache nc, 
       if (mv[j]) {
         if (first) lvl[j] = c.meta[cur[j]].level;
         if (!have_p[j]) {
-          if (spill[j]) {
-            p[j] = c.sp_rec[idx[j]];
-            g[j] = c.sp_gidx[idx[j]];
-          } else {
-            p[j] = __ldcg(pts + idx[j]);
-            g[j] = (uint32_t)(base + idx[j]);
-          }
+          p[j] = spill[j] ? c.sp_rec[idx[j]] : __ldcg(pts + idx[j]);
         }
       }
     }
-    advance_items<AU>(c, wb, mv, p, g, lvl, ch, cur);
 #pragma unroll
     for (int j = 0; j < AU; ++j) {
+      if (mv[j]) {
+        uint32_t rx, ry, rz;
+        rel_coords(c, p[j], rx, ry, rz);
+        cur[j] = ch[j] + octant(rx, ry, rz, c.rlog2 - lvl[j]);
+      }
+      warp_tally(c, smem, mv[j], cur[j]);
       if (mv[j]) {
         if (spill[j]) c.sp_cur[idx[j]] = cur[j];
         else c.b_cur[idx[j]] = cur[j];
@@ -1089,8 +973,186 @@ __device__ void phase_advance(const Ctx& c, uint32_t* smem, const NodeCache nc, 
                            cur[j] | ((lvl[j] + 1u) << MV_NODE_BITS)));
     }
   }
-  warp_flush(c, wb);
   mover_flush(c, mb, out_list);
+  tally_flush(c, smem);
+}
+
+// ------------------------------------------------------------- phase: claim
+
+// Points of a warp that go on to the next coarser level wait in shared memory
+// (in the mover staging, which the claim phase does not use) until 32 of them
+// make a full warp: about one point in ten survives its first claim, so
+// walking on at once would leave most lanes idle for every further level.
+constexpr int CLAIM_U = SL_CLAIM_UNROLL;  // units of 32 points a warp claims for at once
+constexpr uint32_t CLAIM_QUEUE = 32 * (CLAIM_U + 1);
+static_assert(6 * CLAIM_QUEUE <= 2 * MVBUF, "the claim queue fits the mover staging");
+struct ClaimQueue {
+  uint32_t* q;  // node | spill flag, rx, ry, rz, rgba, gidx: CLAIM_QUEUE words each
+  uint32_t n;   // the same value in every lane
+};
+
+// One claim of one point: the parent of `node`.
+struct ClaimItem {
+  uint32_t node;  // MV_SPILL: a re-inserted point
+  uint32_t rx, ry, rz, rgba, gidx;
+};
+
+// What the claim phase needs to know about the update: nodes0 = nodes before
+// it, grid0 = first grid reference of its own splits, open = Ctl::open, near =
+// claim_near_mask.
+struct ClaimArgs {
+  uint32_t nodes0, grid0, open, near;
+};
+
+// All 32 lanes call: lanes with on[j] sample the grid of their node's parent.
+// SORTED: the items are units of consecutive batch points or of re-inserted
+// ones. gidx grows with the lane in the former, so that of a run of lanes in
+// one cell only the first has to claim, and the others are done (unless the
+// voxels do not nest). Points that have to go on join the queue, naming the
+// parent.
+template <int N, bool SORTED>
+__device__ __forceinline__ void claim_level(const Ctx& c, WarpBuf& wb, ClaimQueue& cq,
+                                            const ClaimArgs& a, const bool (&on)[N],
+                                            const ClaimItem (&it)[N]) {
+  const uint32_t lane = lane_id();
+  uint32_t par[N], word[N], cell[N];
+  bool want[N], more[N];
+  unsigned long long key[N], val[N];
+  uint2 up[N];
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    up[j] = on[j] ? *reinterpret_cast<const uint2*>(&c.meta[it[j].node & MV_NODE_MASK].up)
+                  : make_uint2(NONE, 0u);
+  }
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    par[j] = up[j].x & MV_NODE_MASK;
+    word[j] = cell[j] = 0;
+    want[j] = false;
+    if (up[j].x != NONE) {
+      cell[j] = cell_index(it[j].rx, it[j].ry, it[j].rz, c.rlog2 - (up[j].x >> MV_NODE_BITS), c.G);
+      if (!ref_ok(c, up[j].y, c.grid_bytes) || par[j] >= c.max_nodes) {
+        set_error(c, E_INTERNAL);
+      } else {
+        want[j] = true;
+        // a grid of this update's own splits is empty until the store
+        if (up[j].y < a.grid0) word[j] = grid_words(c, up[j].y)[cell[j] >> 5];
+      }
+    }
+  }
+  bool lead[N];
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    more[j] = want[j] && a.open != 0u;
+    want[j] = want[j] && ((word[j] >> (cell[j] & 31u)) & 1u) == 0u;
+    key[j] = ((unsigned long long)par[j] << (3u * c.G)) | cell[j];
+    val[j] = ((unsigned long long)it[j].gidx << 32) | it[j].rgba;
+    lead[j] = want[j];
+    if (SORTED) {
+      const LaneRun r = lane_run(want[j], key[j]);  // all lanes take part
+      // (a head wants its claim)
+      lead[j] = (it[j].node & MV_SPILL) || a.open ? want[j] : r.head;
+    }
+  }
+  warp_claim<N>(c, wb, lead, key, val, par, a.near, more);
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    // a re-inserted point sampled the grids above its old leaf when it came
+    if ((it[j].node & MV_SPILL) && par[j] < a.nodes0) more[j] = false;
+    const unsigned mm = __ballot_sync(FULL_MASK, more[j]);
+    if (mm == 0u) continue;
+    if (more[j]) {
+      uint32_t* q = cq.q + cq.n + __popc(mm & ((1u << lane) - 1u));
+      q[0] = par[j] | (it[j].node & MV_SPILL);
+      q[CLAIM_QUEUE] = it[j].rx;
+      q[2 * CLAIM_QUEUE] = it[j].ry;
+      q[3 * CLAIM_QUEUE] = it[j].rz;
+      q[4 * CLAIM_QUEUE] = it[j].rgba;
+      q[5 * CLAIM_QUEUE] = it[j].gidx;
+    }
+    cq.n += (uint32_t)__popc(mm);
+  }
+  __syncwarp();
+}
+
+// All 32 lanes call: take 32 points (the last time: what is left) from the
+// queue and claim for them, while more than `keep` wait.
+__device__ __forceinline__ void claim_drain(const Ctx& c, WarpBuf& wb, ClaimQueue& cq,
+                                            const ClaimArgs& a, uint32_t keep) {
+  while (cq.n > keep) {
+    const uint32_t k = cq.n < 32u ? cq.n : 32u;
+    cq.n -= k;
+    const bool on[1] = {lane_id() < k};
+    ClaimItem it[1] = {{0, 0, 0, 0, 0, 0}};
+    if (on[0]) {
+      const uint32_t* q = cq.q + cq.n + lane_id();
+      it[0] = ClaimItem{q[0], q[CLAIM_QUEUE], q[2 * CLAIM_QUEUE], q[3 * CLAIM_QUEUE],
+                        q[4 * CLAIM_QUEUE], q[5 * CLAIM_QUEUE]};
+    }
+    __syncwarp();
+    claim_level<1, false>(c, wb, cq, a, on, it);
+  }
+}
+
+// The re-inserted points (spill records [0, n_spill)) and the batch points
+// [0, n), each from its final leaf's parent upwards. The re-inserted points
+// come first: they have the lowest indices, so batch points stop at them.
+// Each warp carries CLAIM_U units at a time, so that their round trips
+// overlap, and loads the next ones' points and cursors meanwhile.
+__device__ void phase_claim(const Ctx& c, uint32_t* smem, const int4* pts, uint64_t n,
+                            unsigned long long base, uint32_t n_spill, const ClaimArgs& a,
+                            uint64_t warp0, uint64_t nwarps) {
+  constexpr int U = CLAIM_U;
+  tally_init(smem);
+  __syncthreads();
+  WarpBuf wb = warp_buf(smem);
+  ClaimQueue cq;
+  cq.q = smem + SMEM_MVBUF + (threadIdx.x / 32) * MVBUF * 2;
+  cq.n = 0;
+  const uint32_t lane = lane_id();
+  // units [0, us) are re-inserted points, the rest batch points
+  const uint64_t us = ((uint64_t)n_spill + 31) / 32, units = us + (n + 31) / 32;
+  const uint32_t chl = count_chunk_log2(units, nwarps);
+  int4 pn[U];
+  uint32_t curn[U];
+  auto load = [&](uint64_t w, int4& p, uint32_t& cur) {  // cur = NONE: no point
+    p = make_int4(0, 0, 0, 0);
+    cur = NONE;
+    if (w < us) {
+      const uint64_t e = w * 32 + lane;
+      if (e < n_spill) {
+        p = c.sp_rec[e];
+        cur = c.sp_cur[e] | MV_SPILL;
+      }
+    } else {
+      const uint64_t i = (w - us) * 32 + lane;
+      if (i < n) {
+        p = __ldcg(pts + i);
+        cur = c.b_cur[i];
+      }
+    }
+  };
+#pragma unroll
+  for (int j = 0; j < U; ++j) load(warp_unit(warp0, nwarps, j, chl), pn[j], curn[j]);
+  for (uint64_t k = 0; warp_unit(warp0, nwarps, k, chl) < units; k += U) {
+    bool on[U];
+    ClaimItem it[U];
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const uint64_t w = warp_unit(warp0, nwarps, k + j, chl);
+      on[j] = curn[j] != NONE;
+      rel_coords(c, pn[j], it[j].rx, it[j].ry, it[j].rz);
+      it[j].node = curn[j];
+      it[j].rgba = (uint32_t)pn[j].w;
+      it[j].gidx = w >= us ? (uint32_t)(base + (w - us) * 32 + lane)
+                           : (on[j] ? c.sp_gidx[w * 32 + lane] : 0u);
+      load(warp_unit(warp0, nwarps, k + j + U, chl), pn[j], curn[j]);
+    }
+    claim_level<U, true>(c, wb, cq, a, on, it);
+    claim_drain(c, wb, cq, a, 31u);
+  }
+  claim_drain(c, wb, cq, a, 0u);
+  warp_flush(c, wb);
   tally_flush(c, smem);
 }
 
@@ -1230,7 +1292,8 @@ __device__ void split_leaf(const Ctx& c, uint32_t id) {
     cm.st_base = 0;
     cm.touched = 0;
     cm.compact = 0;
-    cm.pad[0] = cm.pad[1] = 0;
+    cm.up = id | (m.level << MV_NODE_BITS);
+    cm.up_grid = (uint32_t)(g / REF_BYTES);
     c.meta[c0 + k] = cm;
     c.child[c0 + k] = NONE;
     c.gridref[c0 + k] = NONE;
@@ -1298,54 +1361,44 @@ __device__ void restore_chunks(const Ctx& c, uint32_t id, bool leaf) {
   __syncwarp();
 }
 
-// All 32 lanes of a warp call for one candidate node.
+// All 32 lanes of a warp call for one candidate node (a leaf: inner nodes have
+// no counts before the claim phase).
 __device__ __forceinline__ void decide_node(const Ctx& c, uint32_t id) {
   const uint32_t k = c.cnt[id];
   if (k == 0) return;
-  if (c.meta[id].compact) restore_chunks(c, id, c.child[id] == NONE);
-  const uint32_t num = c.num[id];
-  if (c.child[id] == NONE) {
-    const uint32_t total = num + k;
+  const bool leaf = c.child[id] == NONE;
+  if (c.meta[id].compact) restore_chunks(c, id, leaf);
+  const uint32_t total = c.num[id] + k;
+  if (leaf) {
     const uint32_t L = c.rlog2 - c.meta[id].level;
     if (total > c.T && L > 0) {
       split_leaf(c, id);
       return;
     }
-    alloc_chunks(c, id, total, true);
-    __syncwarp();
-    if (lane_id() == 0) c.num[id] = total;
-  } else {
-    alloc_chunks(c, id, num + k, false);
-    __syncwarp();
-    if (lane_id() == 0) c.num[id] = num + k;
   }
-  if (lane_id() == 0) c.cnt[id] = 0;
+  alloc_chunks(c, id, total, leaf);
+  __syncwarp();
+  if (lane_id() == 0) {
+    c.num[id] = total;
+    c.cnt[id] = 0;
+  }
 }
 
-// Candidates, one warp each: the nodes split in the previous round (their
-// voxels are now all claimed) and the node id range [n_lo, n_hi).
+// Candidates, one warp each: the node id range [n_lo, n_hi). In the expansion
+// rounds these are leaves; after the claim phase the counts left are the inner
+// nodes' new voxels, which get their chunks here.
 // zero_list >= 0: also empty that mover list (the next advance round fills
 // it; the round before last was its reader).
-__device__ void phase_decide(const Ctx& c, uint32_t s_lo, uint32_t s_hi, uint32_t n_lo,
-                             uint32_t n_hi, int zero_list, uint64_t warp0, uint64_t nwarps) {
-  const uint64_t ns = s_hi - s_lo, nn = n_hi - n_lo;
+__device__ void phase_decide(const Ctx& c, uint32_t n_lo, uint32_t n_hi, int zero_list,
+                             uint64_t warp0, uint64_t nwarps) {
   if (zero_list >= 0 && warp0 == 0 && lane_id() == 0) c.ctl->mv_count[zero_list] = 0;
-  for (uint64_t w = warp0; w < ns + nn; w += nwarps) {
-    const uint32_t id = w < ns ? c.splits[s_lo + w].node : (uint32_t)(n_lo + (w - ns));
-    decide_node(c, id);
-  }
+  for (uint64_t w = n_lo + warp0; w < n_hi; w += nwarps) decide_node(c, (uint32_t)w);
 }
 
-// The batch was rejected (a point outside the root cube): undo the counts
-// and claims of its count round, nodes [0, n_nodes), so nothing changed.
+// The batch was rejected (a point outside the root cube): undo the counts of
+// its count round, nodes [0, n_nodes), so nothing changed.
 __device__ void phase_rollback(const Ctx& c, uint32_t n_nodes, uint64_t t0, uint64_t nthreads) {
   for (uint64_t t = t0; t < n_nodes; t += nthreads) c.cnt[t] = 0;
-  const uint32_t nk = min(*reinterpret_cast<volatile unsigned int*>(&c.ctl->nkeys), c.backlog_cap);
-  for (uint64_t t = t0; t < nk; t += nthreads) {
-    HSlot* s = c.hash + c.keys[t];
-    s->key = HASH_EMPTY;
-    s->val = HASH_EMPTY;
-  }
 }
 
 // -------------------------------------------------------------- phase: store
@@ -1512,30 +1565,32 @@ __device__ __forceinline__ void put_rec(const Ctx& c, uint32_t ref, uint32_t q, 
 constexpr int STORE_U = SL_STORE_UNROLL;
 static_assert(3 * 256 <= 2 * TALLY_SLOTS, "the block placement table fits the tally region");
 
-// Store the batch points, the n_spill re-inserted points (from the spill
-// records) and the n_keys new voxels, each at the next free slot of its node;
-// hand the n_tasks chunks of split leaves (one per task) to the pool above
-// pool_top (the caller then raises pool_top). Loops are warp-uniform so that the
-// lanes of a warp share one slot reservation per node; each lane carries
+// Slots for U items per lane: per block in the persistent kernel (smem), per
+// warp in the plain form's kernels (smem == nullptr).
+template <int U>
+__device__ __forceinline__ void place_items(const Ctx& c, uint32_t* smem, const bool (&valid)[U],
+                                            const uint32_t (&node)[U], uint32_t (&ref)[U],
+                                            uint32_t (&q)[U]) {
+#if SL_STORE_BLOCK
+  if (smem) {
+    block_place<U>(c, smem, valid, node, ref, q);
+    return;
+  }
+#endif
+  warp_place<U>(c, valid, node, ref, q);
+}
+
+// Store the batch points and the n_spill re-inserted points (from the spill
+// records), each at the next free slot of its leaf. Loops are block-uniform so
+// that a block's items share their slot reservations; each lane carries
 // STORE_U items at a time so that their L2 round trips overlap.
 __device__ void phase_store(const Ctx& c, uint32_t* smem, const int4* pts, uint64_t n,
-                            unsigned long long base, uint32_t n_spill, uint32_t n_tasks,
-                            uint32_t n_keys, int pool_top, uint64_t t0, uint64_t nthreads) {
+                            unsigned long long base, uint32_t n_spill, uint64_t t0,
+                            uint64_t nthreads) {
   constexpr int U = STORE_U;
-  const uint32_t lane = lane_id();
   // block-uniform loops: item j of thread t in round b is b + j * nthreads + t
   const uint64_t blk = t0 - threadIdx.x, stride = nthreads;
   const uint64_t me = threadIdx.x;
-  auto place = [&](const bool (&valid)[U], const uint32_t (&node)[U], uint32_t (&ref)[U],
-                   uint32_t (&q)[U]) {
-#if SL_STORE_BLOCK
-    if (smem) {
-      block_place<U>(c, smem, valid, node, ref, q);
-      return;
-    }
-#endif
-    warp_place<U>(c, valid, node, ref, q);
-  };
 #if SL_STORE_BLOCK
   if (smem) block_place_init(smem);
 #endif
@@ -1573,7 +1628,7 @@ __device__ void phase_store(const Ctx& c, uint32_t* smem, const int4* pts, uint6
         valid[j] = false;
       }
     }
-    place(valid, node, ref, q);
+    place_items<U>(c, smem, valid, node, ref, q);
 #pragma unroll
     for (int j = 0; j < U; ++j) put_rec(c, ref[j], q[j], p[j], (uint32_t)(base + b0 + j * stride + me));
   }
@@ -1593,10 +1648,24 @@ __device__ void phase_store(const Ctx& c, uint32_t* smem, const int4* pts, uint6
         valid[j] = false;
       }
     }
-    place(valid, node, ref, q);
+    place_items<U>(c, smem, valid, node, ref, q);
 #pragma unroll
     for (int j = 0; j < U; ++j) put_rec(c, ref[j], q[j], r[j], g[j]);
   }
+}
+
+// Store the n_keys new voxels, each at the next free slot of its node, set
+// their occupancy bits and clear their table slots; hand the n_tasks chunks of
+// split leaves (one per task) to the pool above pool_top (phase_end then
+// raises it).
+__device__ void phase_store_voxels(const Ctx& c, uint32_t* smem, uint32_t n_tasks, uint32_t n_keys,
+                                   int pool_top, uint64_t t0, uint64_t nthreads) {
+  constexpr int U = STORE_U;
+  const uint64_t blk = t0 - threadIdx.x, stride = nthreads;
+  const uint64_t me = threadIdx.x;
+#if SL_STORE_BLOCK
+  if (smem) block_place_init(smem);
+#endif
   const uint32_t G = c.G, cmask = (1u << (3u * G)) - 1u, amask = (1u << G) - 1u;
   for (uint64_t b0 = blk; b0 < n_keys; b0 += U * stride) {
     bool valid[U];
@@ -1626,7 +1695,7 @@ __device__ void phase_store(const Ctx& c, uint32_t* smem, const int4* pts, uint6
       if (valid[j] && !ok) set_error(c, E_INTERNAL);
       valid[j] = ok;
     }
-    place(valid, node, ref, q);
+    place_items<U>(c, smem, valid, node, ref, q);
 #pragma unroll
     for (int j = 0; j < U; ++j) {
       if (!valid[j]) continue;
@@ -1644,13 +1713,23 @@ __device__ void phase_store(const Ctx& c, uint32_t* smem, const int4* pts, uint6
       sl[j]->val = HASH_EMPTY;
     }
   }
-  (void)lane;
   const int top = pool_top > 0 ? pool_top : 0;
   if ((unsigned long long)top + n_tasks > c.max_chunks) {
     if (t0 == 0) set_error(c, E_POOL);
     return;
   }
   for (uint64_t q = t0; q < n_tasks; q += nthreads) c.pool[top + q] = c.pending[q];
+}
+
+// Expected new voxels per 1,024 points of the next update: those of the
+// octree so far (`voxels` made by `points`, re-insertions counted), as if half
+// an update of `last` points had come before it and made a voxel for every
+// second point.
+__device__ __forceinline__ uint32_t key_rate_of(unsigned long long voxels,
+                                                unsigned long long points,
+                                                unsigned long long last) {
+  const unsigned long long r = (voxels + last / 4u) * 1024u / (points + last / 2u + 1u);
+  return r < 16u ? 16u : r > 16384u ? 16384u : (uint32_t)r;
 }
 
 // One thread: close an applied update (advance gidx, return the freed
@@ -1682,13 +1761,15 @@ __device__ void phase_end(const Ctx& c, uint64_t n, uint32_t iters) {
   t->ntasks = 0;
   t->mv_count[0] = 0;
   t->mv_count[1] = 0;
+  t->bump0 = t->bump;
+  t->key_rate = key_rate_of(t->st_voxels, t->st_points + t->st_spilled,
+                            n + t->last_spilled);
 }
 
-// One thread: close a rejected update (the rollback undid its counters).
+// One thread: close a rejected update (the rollback undid its counts).
 __device__ void phase_end_rejected(const Ctx& c) {
   Ctl* t = c.ctl;
   t->reject = 0;
-  t->nkeys = 0;
   t->st_rejected += 1;
 }
 

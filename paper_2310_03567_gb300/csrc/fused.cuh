@@ -69,8 +69,8 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
 // next one) into the block's shared copy, so that one load per block, not
 // one per warp, reaches the control block's L2 lines.
 struct CtlView {
-  unsigned long long base;
-  uint32_t n_nodes, reject, split_count, ntasks, spill_count, nkeys, stop;
+  unsigned long long base, bump0;
+  uint32_t n_nodes, key_rate, open, reject, split_count, ntasks, spill_count, nkeys, stop;
   int pool_top;
   uint32_t mv_count[2];
 };
@@ -111,6 +111,9 @@ __device__ __forceinline__ bool grid_barrier(const Ctx& c, FusedCtl* f, CtlView*
 #if SL_CTL_VIEW
     if (ok && view) {
       view->base = vload(&c.ctl->base);
+      view->bump0 = vload(&c.ctl->bump0);
+      view->key_rate = vload(&c.ctl->key_rate);
+      view->open = vload(&c.ctl->open);
       view->n_nodes = vload(&c.ctl->n_nodes);
       view->reject = vload(&c.ctl->reject);
       view->split_count = vload(&c.ctl->split_count);
@@ -237,14 +240,14 @@ __global__ void __launch_bounds__(FUSED_BLOCK, PHASE_MIN_BLOCKS) k_fused(Ctx c, 
       bd.pts = c.staging;
     }
     if (bd.n) {
-      phase_count1(c, smem, node_cache_at(smem, nodes0), bd.pts, bd.n, base, warp0, nwarps);
+      phase_count1(c, smem, node_cache_at(smem, nodes0), bd.pts, bd.n, warp0, nwarps);
       if (!grid_barrier(c, f, vw)) return;
       clk.tick(c, PH_COUNT);
       rejected = SL_CV(reject, &c.ctl->reject) != 0u;  // set only by the count round
       if (rejected) {
         phase_rollback(c, nodes0, tid, nthreads);
         if (!grid_barrier(c, f)) return;  // all have read the flag before it is cleared
-        clk.tick(c, PH_ROLLBACK);
+        clk.tick(c, PH_OTHER);
         if (tid == 0) {
           phase_end_rejected(c);
           c.ctl->st_rejected_async += 1;
@@ -255,8 +258,7 @@ __global__ void __launch_bounds__(FUSED_BLOCK, PHASE_MIN_BLOCKS) k_fused(Ctx c, 
         // t_hi: spill tasks (all made by the first decide round)
         uint32_t s_lo = 0, s_hi = 0, n_lo = 0, n_hi = nodes0, t_hi = 0, iters = 1;
         for (;;) {
-          phase_decide(c, s_lo, s_hi, n_lo, n_hi, iters >= 3 ? (int)((iters - 1) & 1u) : -1,
-                       warp0, nwarps);
+          phase_decide(c, n_lo, n_hi, iters >= 3 ? (int)((iters - 1) & 1u) : -1, warp0, nwarps);
           if (!grid_barrier(c, f, vw)) return;
           clk.tick(c, PH_DECIDE);
           const uint32_t sc = SL_CV(split_count, &c.ctl->split_count);
@@ -277,19 +279,29 @@ __global__ void __launch_bounds__(FUSED_BLOCK, PHASE_MIN_BLOCKS) k_fused(Ctx c, 
           const int in_list = iters >= 2 ? (int)((iters - 2) & 1u) : -1;
           const uint32_t n_in =
               in_list >= 0 ? SL_CV(mv_count[in_list], &c.ctl->mv_count[in_list]) : 0u;
-          phase_advance(c, smem, node_cache_at(smem, nn), bd.pts, bd.n, base, t_hi, s_lo, s_hi,
-                        in_list, n_in, (int)((iters - 1) & 1u), warp0, nwarps);
+          phase_advance(c, smem, node_cache_at(smem, nn), bd.pts, bd.n, t_hi, s_lo, s_hi, in_list,
+                        n_in, (int)((iters - 1) & 1u), warp0, nwarps);
           ++iters;
           if (!grid_barrier(c, f)) return;
           clk.tick(c, PH_ADVANCE);
         }
         // (the last decide round's barrier filled the view)
-        const uint32_t n_tasks = SL_CV(ntasks, &c.ctl->ntasks);
         const uint32_t n_spill = min(SL_CV(spill_count, &c.ctl->spill_count), c.spill_cap);
+        const uint32_t nodes1 = SL_CV(n_nodes, &c.ctl->n_nodes);
+        const ClaimArgs ca{nodes0, (uint32_t)(SL_CV(bump0, &c.ctl->bump0) / REF_BYTES),
+                           SL_CV(open, &c.ctl->open), 
+                           claim_near_mask(c, bd.n + n_spill, SL_CV(key_rate, &c.ctl->key_rate))};
+        phase_claim(c, smem, bd.pts, bd.n, base, n_spill, ca, warp0, nwarps);
+        if (!grid_barrier(c, f)) return;
+        clk.tick(c, PH_CLAIM);
+        phase_decide(c, 0, nodes1, -1, warp0, nwarps);  // chunks for the new voxels
+        phase_store(c, smem, bd.pts, bd.n, base, n_spill, tid, nthreads);
+        if (!grid_barrier(c, f, vw)) return;
+        clk.tick(c, PH_STORE);
+        const uint32_t n_tasks = SL_CV(ntasks, &c.ctl->ntasks);
         const uint32_t n_keys = min(SL_CV(nkeys, &c.ctl->nkeys), c.backlog_cap);
         const int pool_top = SL_CV(pool_top, &c.ctl->pool_top);
-        phase_store(c, smem, bd.pts, bd.n, base, n_spill, n_tasks, n_keys, pool_top, tid,
-                    nthreads);
+        phase_store_voxels(c, smem, n_tasks, n_keys, pool_top, tid, nthreads);
         if (!grid_barrier(c, f)) return;
         clk.tick(c, PH_STORE);
         if (tid == 0) phase_end(c, bd.n, iters);

@@ -25,7 +25,7 @@ extern "C" int SL_VARIANT_INFO(sl_variant_info* out) {
   out->min_blocks = PHASE_MIN_BLOCKS;
   out->node_cache = NODE_CACHE;
   out->store_unroll = STORE_U;
-  out->descent_group = DESCENT_GROUP;
+  out->descent_group = COUNT_U;
   out->smem_bytes = PHASE_SMEM_BYTES;
   out->max_per_sm = 0;
   if (cudaFuncSetAttribute(k_fused, cudaFuncAttributeMaxDynamicSharedMemorySize,

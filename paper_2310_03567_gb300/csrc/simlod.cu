@@ -35,6 +35,8 @@ __global__ void k_init(Ctx c) {
     for (int k = 0; k < 8; ++k) t->phase_ns[k] = phase_ns[k];
     t->n_nodes = 1;
     t->bump = c.dir_bytes;  // the root's chunk directory is the first data ref
+    t->bump0 = t->bump;
+    t->key_rate = key_rate_of(0, 0, 1024);
     NodeMeta m;
     memset(&m, 0, sizeof(m));
     m.min[0] = c.rmin[0];
@@ -44,6 +46,7 @@ __global__ void k_init(Ctx c) {
     m.head = m.tail = NONE;
     m.dir = 0;
     m.st_tail = NONE;
+    m.up = m.up_grid = NONE;
     c.meta[0] = m;
     c.child[0] = NONE;
     c.gridref[0] = NONE;
@@ -60,47 +63,96 @@ __global__ void k_fill_hash(HSlot* h, uint64_t n) {
   }
 }
 
-__global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_count1(Ctx c, const int4* pts, uint64_t n,
-                                                    unsigned long long base, uint32_t n_nodes) {
+__global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_count1(Ctx c, const int4* pts,
+                                                                    uint64_t n, uint32_t n_nodes) {
   extern __shared__ uint32_t smem[];
   const uint64_t warps_per_block = blockDim.x / 32;
   node_cache_load(c, smem, 0, n_nodes);
-  phase_count1(c, smem, node_cache_at(smem, n_nodes), pts, n, base,
+  phase_count1(c, smem, node_cache_at(smem, n_nodes), pts, n,
                blockIdx.x * warps_per_block + threadIdx.x / 32,
                (uint64_t)gridDim.x * warps_per_block);
 }
 
 // Decide / allocate; after the first count round of a rejected batch (no
 // thread changes the reject flag during this kernel) undo that round instead.
-__global__ void __launch_bounds__(BLOCK) k_decide(Ctx c, uint32_t s_lo, uint32_t s_hi,
-                                                   uint32_t n_lo, uint32_t n_hi, int zero_list) {
+__global__ void __launch_bounds__(BLOCK) k_decide(Ctx c, uint32_t n_lo, uint32_t n_hi,
+                                                   int zero_list) {
   const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   const uint64_t nt = (uint64_t)gridDim.x * blockDim.x;
   if (*reinterpret_cast<volatile unsigned int*>(&c.ctl->reject)) {
     phase_rollback(c, n_hi, t0, nt);
     return;
   }
-  phase_decide(c, s_lo, s_hi, n_lo, n_hi, zero_list, t0 / 32, nt / 32);
+  phase_decide(c, n_lo, n_hi, zero_list, t0 / 32, nt / 32);
 }
 
 __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_advance(Ctx c, const int4* pts, uint64_t n,
-                                                     unsigned long long base, uint32_t n_nodes,
-                                                     uint32_t t_hi, uint32_t s_lo, uint32_t s_hi,
-                                                     int in_list, uint32_t n_in, int out_list) {
+                                                     uint32_t n_nodes, uint32_t t_hi, uint32_t s_lo,
+                                                     uint32_t s_hi, int in_list, uint32_t n_in,
+                                                     int out_list) {
   extern __shared__ uint32_t smem[];
   const uint64_t warps_per_block = blockDim.x / 32;
   node_cache_load(c, smem, 0, n_nodes);
-  phase_advance(c, smem, node_cache_at(smem, n_nodes), pts, n, base, t_hi, s_lo, s_hi, in_list,
-                n_in, out_list,
-                blockIdx.x * warps_per_block + threadIdx.x / 32,
+  phase_advance(c, smem, node_cache_at(smem, n_nodes), pts, n, t_hi, s_lo, s_hi, in_list, n_in,
+                out_list, blockIdx.x * warps_per_block + threadIdx.x / 32,
                 (uint64_t)gridDim.x * warps_per_block);
 }
 
+__global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_claim(Ctx c, const int4* pts, uint64_t n,
+                                                     unsigned long long base, uint32_t n_spill,
+                                                     uint32_t nodes0) {
+  extern __shared__ uint32_t smem[];
+  const uint64_t warps_per_block = blockDim.x / 32;
+  const ClaimArgs a{nodes0, (uint32_t)(vload(&c.ctl->bump0) / REF_BYTES), vload(&c.ctl->open),
+                    claim_near_mask(c, n + n_spill, vload(&c.ctl->key_rate))};
+  phase_claim(c, smem, pts, n, base, n_spill, a, blockIdx.x * warps_per_block + threadIdx.x / 32,
+              (uint64_t)gridDim.x * warps_per_block);
+}
+
+// The points and, their nodes' chunks being there too, the voxels.
 __global__ void __launch_bounds__(BLOCK) k_store(Ctx c, const int4* pts, uint64_t n,
                                                   unsigned long long base, uint32_t n_spill,
                                                   uint32_t n_tasks, uint32_t n_keys, int pool_top) {
-  phase_store(c, nullptr, pts, n, base, n_spill, n_tasks, n_keys, pool_top,
-              blockIdx.x * (uint64_t)blockDim.x + threadIdx.x, (uint64_t)gridDim.x * blockDim.x);
+  const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+  const uint64_t nt = (uint64_t)gridDim.x * blockDim.x;
+  phase_store(c, nullptr, pts, n, base, n_spill, t0, nt);
+  phase_store_voxels(c, nullptr, n_tasks, n_keys, pool_top, t0, nt);
+}
+
+// Whether a restored octree's voxels nest, as those of every octree built by
+// inserts do: each voxel's cell, and each point, lies in an occupied cell of
+// the parent node. The claim phase stops at the first occupied cell of a walk
+// upwards only then (Ctl::open). One block per node; a restored node's chunks
+// lie one after another in the data region.
+__global__ void k_check_nested(Ctx c) {
+  const uint32_t n = min(vload(&c.ctl->n_nodes), c.max_nodes);
+  const uint32_t lim = (1u << c.G) - 1u;
+  for (uint32_t id = blockIdx.x; id < n; id += gridDim.x) {
+    const NodeMeta& m = c.meta[id];
+    if (m.up == NONE || !ref_ok(c, m.up_grid, c.grid_bytes)) continue;
+    const uint32_t cnt = c.num[id], head = m.head, par = m.up & MV_NODE_MASK;
+    const uint32_t L = c.rlog2 - (m.up >> MV_NODE_BITS);  // the parent's log2 size
+    const bool inner = c.child[id] != NONE;
+    const uint32_t oct = id - c.child[par];
+    const uint32_t* words = grid_words(c, m.up_grid);
+    for (uint32_t i = threadIdx.x; i < cnt; i += blockDim.x) {
+      const uint32_t ref = head + i / c.C * c.chunk_units, q = i % c.C;
+      if (!ref_ok(c, ref, c.chunk_bytes)) break;
+      uint32_t cell;
+      if (inner) {
+        const uint32_t v = chunk_aux(c, ref)[q];
+        uint32_t ax[3];
+        for (uint32_t a = 0; a < 3; ++a)
+          ax[a] = ((((oct >> a) & 1u) << c.G) + ((v >> (a * c.G)) & lim)) >> 1;
+        cell = ax[0] | (ax[1] << c.G) | (ax[2] << (2u * c.G));
+      } else {
+        uint32_t rx, ry, rz;
+        rel_coords(c, chunk_recs(c, ref)[q], rx, ry, rz);
+        cell = cell_index(rx, ry, rz, L, c.G);
+      }
+      if (((words[cell >> 5] >> (cell & 31u)) & 1u) == 0u) c.ctl->open = 1u;
+    }
+  }
 }
 
 // Compaction of cold nodes (the paper's closing direction: nodes that are no
@@ -189,7 +241,7 @@ int fused_info_0(sl_variant_info* out) {
   out->min_blocks = PHASE_MIN_BLOCKS;
   out->node_cache = NODE_CACHE;
   out->store_unroll = STORE_U;
-  out->descent_group = DESCENT_GROUP;
+  out->descent_group = COUNT_U;
   out->smem_bytes = PHASE_SMEM_BYTES;
   out->max_per_sm = 0;
   if (cudaFuncSetAttribute(k_fused, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -251,9 +303,9 @@ const VariantFns kVariants[SL_N_VARIANTS] = {
 
 // ================================================================ host side
 
-enum KernelId { K_COUNT = 0, K_DECIDE, K_ADVANCE, K_STORE, K_END, K_FUSED, K_INIT, K_RENDER };
+enum KernelId { K_COUNT = 0, K_DECIDE, K_ADVANCE, K_STORE, K_END, K_FUSED, K_CLAIM, K_RENDER };
 static const char* const kKernelNames[SIMLOD_N_KERNELS] = {
-    "count1", "decide", "advance", "store", "end", "fused_update", "init", "render"};
+    "count1", "decide", "advance", "store", "end", "fused_update", "claim", "render"};
 
 struct Layout {
   size_t ctl, fctl, batches, child, gridref, cnt, num, meta, pool, pending, alloc_refs, splits,
@@ -550,11 +602,11 @@ int insert_device(simlod_t* h, const int4* pts, uint64_t n, cudaStream_t s) {
   const unsigned gp = std::max(1u, std::min<unsigned>(grid_for(h, n, PBLOCK), (unsigned)PHASE_MIN_BLOCKS * h->sm_count));
   int rc;
   rc = launch(h, K_COUNT, s, [&] {
-    k_count1<<<gp, PBLOCK, PHASE_SMEM_BYTES, s>>>(c, pts, n, base, nodes0);
+    k_count1<<<gp, PBLOCK, PHASE_SMEM_BYTES, s>>>(c, pts, n, nodes0);
   });
   if (rc) return poison(h, rc);
   rc = launch(h, K_DECIDE, s, [&] {
-    k_decide<<<grid_for(h, 32ull * nodes0, BLOCK), BLOCK, 0, s>>>(c, 0, 0, 0, nodes0, -1);
+    k_decide<<<grid_for(h, 32ull * nodes0, BLOCK), BLOCK, 0, s>>>(c, 0, nodes0, -1);
   });
   if (rc) return poison(h, rc);
   if ((rc = read_ctl(h, s))) return poison(h, rc);
@@ -583,16 +635,15 @@ int insert_device(simlod_t* h, const int4* pts, uint64_t n, cudaStream_t s) {
         std::max(1u, std::min<unsigned>(grid_for(h, units * 32, PBLOCK), (unsigned)PHASE_MIN_BLOCKS * h->sm_count));
     const uint32_t nn = n_hi;
     rc = launch(h, K_ADVANCE, s, [&] {
-      k_advance<<<ga, PBLOCK, PHASE_SMEM_BYTES, s>>>(c, pts, n, base, nn, t_hi, s_lo, s_hi,
-                                                     in_list, n_in, out_list);
+      k_advance<<<ga, PBLOCK, PHASE_SMEM_BYTES, s>>>(c, pts, n, nn, t_hi, s_lo, s_hi, in_list,
+                                                     n_in, out_list);
     });
     if (rc) return poison(h, rc);
     ++iters;
-    const uint64_t cand = (uint64_t)(s_hi - s_lo) + (n_hi - n_lo);
+    const uint64_t cand = n_hi - n_lo;
     const int zero_list = iters >= 3 ? (int)((iters - 1) & 1u) : -1;
     rc = launch(h, K_DECIDE, s, [&] {
-      k_decide<<<grid_for(h, 32 * cand, BLOCK), BLOCK, 0, s>>>(c, s_lo, s_hi, n_lo, n_hi,
-                                                              zero_list);
+      k_decide<<<grid_for(h, 32 * cand, BLOCK), BLOCK, 0, s>>>(c, n_lo, n_hi, zero_list);
     });
     if (rc) return poison(h, rc);
     if ((rc = read_ctl(h, s))) return poison(h, rc);
@@ -603,8 +654,20 @@ int insert_device(simlod_t* h, const int4* pts, uint64_t n, cudaStream_t s) {
     n_lo = n_hi;
     n_hi = h->ctl_host->n_nodes;
   }
-  const uint32_t n_tasks = h->ctl_host->ntasks;
   const uint32_t n_spill = std::min<uint32_t>(h->ctl_host->spill_count, c.spill_cap);
+  const uint32_t nodes1 = h->ctl_host->n_nodes;
+  rc = launch(h, K_CLAIM, s, [&] {
+    k_claim<<<gp, PBLOCK, PHASE_SMEM_BYTES, s>>>(c, pts, n, base, n_spill, nodes0);
+  });
+  if (rc) return poison(h, rc);
+  // chunks for the new voxels of the inner nodes
+  rc = launch(h, K_DECIDE, s, [&] {
+    k_decide<<<grid_for(h, 32ull * nodes1, BLOCK), BLOCK, 0, s>>>(c, 0, nodes1, -1);
+  });
+  if (rc) return poison(h, rc);
+  if ((rc = read_ctl(h, s))) return poison(h, rc);
+  if (h->ctl_host->error) return poison(h, error_from_bits(h->ctl_host->error));
+  const uint32_t n_tasks = h->ctl_host->ntasks;
   const uint32_t n_keys = std::min<uint32_t>(h->ctl_host->nkeys, c.backlog_cap);
   const int pool_top = h->ctl_host->pool_top;
   const uint64_t work =
@@ -757,6 +820,8 @@ SIMLOD_API int simlod_create(const simlod_config* cfg, void* d_arena, size_t are
   if (cudaFuncSetAttribute(k_count1, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            PHASE_SMEM_BYTES) != cudaSuccess ||
       cudaFuncSetAttribute(k_advance, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           PHASE_SMEM_BYTES) != cudaSuccess ||
+      cudaFuncSetAttribute(k_claim, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            PHASE_SMEM_BYTES) != cudaSuccess ||
       cudaFuncSetAttribute(k_fused, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            PHASE_SMEM_BYTES) != cudaSuccess) {
@@ -1297,7 +1362,7 @@ SIMLOD_API int simlod_restore(simlod_t* h, const simlod_snapshot_t* snap, void* 
   };
   // node ids: the children of a node are 8 consecutive ids in octant order
   std::vector<uint32_t> rec_of;
-  std::vector<uint32_t> first_child(n, NONE);
+  std::vector<uint32_t> first_child(n, NONE), up(n, NONE);  // up: as NodeMeta::up
   rec_of.reserve(n);
   rec_of.push_back(0);
   for (size_t q = 0; q < rec_of.size(); ++q) {
@@ -1309,6 +1374,7 @@ SIMLOD_API int simlod_restore(simlod_t* h, const simlod_snapshot_t* snap, void* 
       const int64_t c = find(Key{pk.level + 1, 2 * pk.ix + (o & 1), 2 * pk.iy + ((o >> 1) & 1),
                                  2 * pk.iz + ((o >> 2) & 1)});
       if (c < 0 || rec_of.size() >= n) return SIMLOD_ERR_INVALID_ARG;
+      up[rec_of.size()] = (uint32_t)q | ((uint32_t)pk.level << MV_NODE_BITS);
       rec_of.push_back((uint32_t)c);
     }
   }
@@ -1343,6 +1409,8 @@ SIMLOD_API int simlod_restore(simlod_t* h, const simlod_snapshot_t* snap, void* 
     const simlod_node_rec& rec = nodes[r];
     NodeMeta m;
     memset(&m, 0, sizeof(m));
+    m.up = up[id];
+    m.up_grid = id ? gridref[up[id] & MV_NODE_MASK] : NONE;
     for (int a = 0; a < 3; ++a) m.min[a] = rec.min[a];
     m.level = rec.level;
     m.st_tail = NONE;
@@ -1410,7 +1478,9 @@ SIMLOD_API int simlod_restore(simlod_t* h, const simlod_snapshot_t* snap, void* 
     return poison(h, SIMLOD_ERR_CUDA);
   t.base = snap->n_points;
   t.n_nodes = (unsigned int)n;
-  t.bump = bump;
+  t.bump = t.bump0 = bump;
+  // (the key rate stays an empty octree's: a snapshot does not say how often
+  // its points were re-inserted)
   t.chunks_bumped = chunks;
   t.pool_top = 0;
   t.st_points = snap->n_points;
@@ -1425,6 +1495,9 @@ SIMLOD_API int simlod_restore(simlod_t* h, const simlod_snapshot_t* snap, void* 
           cudaSuccess ||
       (bump && cudaMemcpy(c.data, data.data(), bump, cudaMemcpyHostToDevice) != cudaSuccess) ||
       cudaMemcpy(c.ctl, &t, sizeof(Ctl), cudaMemcpyHostToDevice) != cudaSuccess)
+    return poison(h, SIMLOD_ERR_CUDA);
+  k_check_nested<<<(unsigned)std::min<uint64_t>(n, (uint64_t)h->sm_count * 8), BLOCK, 0, s>>>(c);
+  if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
     return poison(h, SIMLOD_ERR_CUDA);
   h->base = snap->n_points;
   h->n_nodes = (uint32_t)n;
@@ -1678,7 +1751,7 @@ SIMLOD_API int simlod_get_timing(simlod_t* h, simlod_timing* out) {
     out->ms[k] = h->ms[k];
   }
   static const char* const kPhaseNames[SIMLOD_N_PHASES] = {
-      "count", "decide", "advance", "store", "end", "rollback", "launch", "other"};
+      "count", "decide", "advance", "store", "end", "claim", "launch", "other"};
   int rc = read_ctl(h, h->last_stream);
   if (rc) return rc;
   for (int k = 0; k < SIMLOD_N_PHASES; ++k) {
