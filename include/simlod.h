@@ -108,7 +108,7 @@ typedef struct {
 typedef struct {
   uint64_t batches, points, rejected_batches;
   uint64_t spilled, splits, voxels, iterations_max;
-  uint64_t rounds; /* expansion rounds summed over updates (one control-block read each) */
+  uint64_t rounds; /* expansion rounds (tree levels decided one after another) summed over updates */
   uint64_t nodes;
   uint64_t chunks_bumped, chunks_pool;
   uint64_t arena_bytes, data_bytes, data_used;
@@ -180,9 +180,10 @@ SIMLOD_API int simlod_create(const simlod_config* cfg, void* d_arena, size_t are
  * point ever accepted gets gidx k. n = 0 is a no-op.
  *
  * The work runs on `stream`, in stream order after earlier work there. The
- * expansion rounds are steered from the host: the call waits for the stream
- * once per round (a read of the control block), then enqueues the final
- * store and returns without waiting for it. d_pts must therefore stay valid
+ * call enqueues the update up to the allocation of its chunks, waits for the
+ * stream once (a read of the control block; once more for every further
+ * histogram round of an unusually deep split), then enqueues the final store
+ * and returns without waiting for it. d_pts must therefore stay valid
  * and unchanged until `stream` has passed the insert (record an event or
  * synchronise). Returns SIMLOD_ERR_OUT_OF_BOUNDS, with the octree and the
  * gidx counter unchanged, when any point lies outside the root cube. Calls on

@@ -7,16 +7,18 @@
 //          there (Section 5.1, "Counting"); the leaf is kept per point (its
 //          cursor).
 //  decide  per candidate leaf: one whose stored + counted points exceed T
-//          splits (Section 5.1, "Splitting"): 8 children, a grid, and one
-//          spill task per chunk of its stored points. Any other counted leaf
-//          is final and gets its chunks now (Section 5.3).
-//  advance points whose cursor node split in the previous round (batch
-//          points, and the stored points of split leaves, copied out of their
-//          old chunks at their first move) move one level down, counting into
-//          the child; the grids of the previous round's splits are zeroed
-//          alongside. Repeated with decide until nothing splits: the paper's
-//          iterative deepening, but each round touches only the points that
-//          have to move (mover lists).
+//          splits (Section 5.1, "Splitting"): one spill task per chunk of its
+//          stored points. Any other counted leaf is final and gets its chunks
+//          now (Section 5.3).
+//  hist    the points of the leaves that split (batch points, and the stored
+//          points in the old chunks) are counted into the cubes up to 5 levels
+//          below their leaf (HIST_DEPTH).
+//  build   one block per split leaf sums the counts upwards and creates the
+//          whole subtree at once: an inner node wherever a cube holds more
+//          than T points. decide then gives its leaves their chunks; a leaf of
+//          the lowest level that still holds too many goes round again. The
+//          paper deepens the tree one level per counting round, which read
+//          every moving point 2.3 times over on a shuffled building scan.
 //  claim   with every point at its final leaf, the points sample the grids
 //          (Section 3.3) from the leaf's parent upwards. Cells nest: a cell of
 //          a node lies inside one cell of the node's parent. So a point whose
@@ -74,9 +76,6 @@ constexpr uint32_t CHUNK_HEADER = 16;
 #ifndef SL_PHASE_MIN_BLOCKS
 #define SL_PHASE_MIN_BLOCKS 2
 #endif
-#ifndef SL_ADVANCE_UNROLL
-#define SL_ADVANCE_UNROLL 1
-#endif
 #ifndef SL_CTL_VIEW
 #define SL_CTL_VIEW 1
 #endif
@@ -112,7 +111,6 @@ constexpr uint32_t CHUNK_HEADER = 16;
 #endif
 constexpr uint32_t NODE_CACHE = SL_NODE_CACHE;         // nodes mirrored in shared memory
 constexpr uint32_t ZERO_UNIT = 4096;                   // bytes of grid zeroed per warp unit
-constexpr int ADVANCE_U = SL_ADVANCE_UNROLL;           // advance units a warp carries at a time
 constexpr int COUNT_U = SL_COUNT_UNROLL;               // count units a warp carries at a time
 #ifndef SL_WBUF
 #define SL_WBUF 128
@@ -120,18 +118,15 @@ constexpr int COUNT_U = SL_COUNT_UNROLL;               // count units a warp car
 constexpr uint32_t WBUF = SL_WBUF;                      // new-cell slots staged per warp
 constexpr int PHASE_BLOCK = SL_PHASE_BLOCK;            // threads of count / advance / fused blocks
 constexpr int PHASE_MIN_BLOCKS = SL_PHASE_MIN_BLOCKS;  // resident blocks per SM they aim for
-// dynamic shared memory of the count / advance / fused blocks
-#ifndef SL_MVBUF
-#define SL_MVBUF 288
-#endif
-constexpr uint32_t MVBUF = SL_MVBUF;                    // mover-list entries staged per warp
 constexpr uint32_t TALLY_LOG2 = 9;                      // block tally cache: 512 nodes
 constexpr uint32_t TALLY_SLOTS = 1u << TALLY_LOG2;
-// dynamic shared memory of the count / advance / fused blocks: node cache,
-// new-cell staging, mover staging, block tally cache
-constexpr uint32_t SMEM_WBUF = NODE_CACHE;                            // in u32 words
-constexpr uint32_t SMEM_MVBUF = SMEM_WBUF + (PHASE_BLOCK / 32) * WBUF;
-constexpr uint32_t SMEM_TALLY = SMEM_MVBUF + (PHASE_BLOCK / 32) * MVBUF * 2;
+// dynamic shared memory of the phase blocks: node cache, new-cell staging,
+// claim queues, block tally cache
+constexpr int CLAIM_U = SL_CLAIM_UNROLL;  // units of 32 points a warp claims for at once
+constexpr uint32_t CLAIM_QUEUE = 32 * (CLAIM_U + 1);  // points that wait for their next claim
+constexpr uint32_t SMEM_WBUF = NODE_CACHE;            // in u32 words
+constexpr uint32_t SMEM_QUEUE = SMEM_WBUF + (PHASE_BLOCK / 32) * WBUF;
+constexpr uint32_t SMEM_TALLY = SMEM_QUEUE + (PHASE_BLOCK / 32) * CLAIM_QUEUE * 6;
 constexpr uint32_t PHASE_SMEM_BYTES = 4 * (SMEM_TALLY + 2 * TALLY_SLOTS);
 
 // Sticky device error bits.
@@ -156,6 +151,15 @@ enum : uint32_t {
 #else
 #define SL_HOT
 #endif
+// An expansion round of the plain form, whose kernels find here what the ones
+// before them left: split entries [s_lo, s_lo + K) are built d levels deep
+// below lvl0 levels of earlier rounds, which made `inner` inner nodes; the
+// nodes of this round begin at n_lo.
+struct PlainRound {
+  uint32_t s_lo, K, inner, d, lvl0, n_lo;
+};
+constexpr uint32_t MAX_ROUNDS = 32;  // a round builds at least one of 31 levels
+
 struct Ctl {
   unsigned long long base;                  // gidx of the next accepted point
   SL_HOT unsigned long long bump;           // bytes taken from the data region
@@ -172,12 +176,15 @@ struct Ctl {
   SL_HOT unsigned int nkeys;                // new voxels (backlog entries) of this update
   SL_HOT unsigned int alloc_seq;            // alloc_refs entries of this update
   SL_HOT unsigned int split_count;          // split-list entries of this update
+  unsigned int split_inner;                 //   those made by the builds (inner nodes below the
+                                            //   split leaves): decide does not change it
   SL_HOT unsigned int ntasks;               // spill tasks (= freed chunks) of this update
+  unsigned int split_most;                  // points of the fullest leaf that splits this round
+  unsigned int iters;                       // expansion rounds of this update (0: no split)
   unsigned long long st_batches, st_points, st_rejected, st_spilled, st_splits, st_voxels,
       st_iter_max, st_rounds;
   unsigned long long last_points, last_spilled, last_splits, last_voxels, last_iters;
   unsigned long long st_rejected_async;  // rejections inside fused launches
-  SL_HOT unsigned int mv_count[2];       // entries of the two mover lists
   SL_HOT unsigned long long render_samples;  // points and voxels visited by the last render
   unsigned int vis_count;                    // nodes drawn by the last render
   unsigned int draw_units;                   // chunks and array pieces they were cut into
@@ -187,7 +194,8 @@ struct Ctl {
   unsigned long long st_decompacted;     // arrays turned back into chunk lists by an insert
   unsigned long long compact_now;        // nodes that are arrays now
   unsigned long long compact_chunks_now; // chunks those arrays stand in for
-  unsigned long long pad_ctl;
+  unsigned int store_blocks;             // plain form: blocks that finished the store
+  PlainRound round[MAX_ROUNDS];
 };
 #undef SL_HOT
 static_assert(sizeof(Ctl) % 16 == 0, "Ctl size");
@@ -208,7 +216,7 @@ struct NodeMeta {
   uint32_t st_base;     //   and the records stored before this update
   uint32_t touched;     // updates applied when the node last received records (1 = the first)
   uint32_t compact;     // 1: the records are one contiguous array (head), not a chunk list
-  uint32_t up;          // parent | parent's level << MV_NODE_BITS, NONE at the root
+  uint32_t up;          // parent | parent's level << NODE_BITS, NONE at the root
   uint32_t up_grid;     // the parent's occupancy grid
 };
 static_assert(sizeof(NodeMeta) == 64, "NodeMeta size");
@@ -216,19 +224,19 @@ static_assert(offsetof(NodeMeta, st_nch) == 32 && offsetof(NodeMeta, st_base) ==
               "the store map is one aligned 16-byte load");
 static_assert(offsetof(NodeMeta, up) == 56, "up and up_grid are one aligned 8-byte load");
 
-constexpr uint32_t MV_SPILL = 1u << 31;
-constexpr uint32_t MV_NODE_BITS = 27;  // node ids below 2^27 (the node table limit)
-constexpr uint32_t MV_NODE_MASK = (1u << MV_NODE_BITS) - 1u;
+constexpr uint32_t NODE_BITS = 27;  // node ids below 2^27 (the node table limit)
+constexpr uint32_t NODE_MASK = (1u << NODE_BITS) - 1u;
 
 struct __align__(16) HSlot {
   unsigned long long key;  // (node << 3G) | cell, HASH_EMPTY when free
   unsigned long long val;  // (gidx << 32) | rgba of the best contender so far
 };
 
-struct SplitEntry {
-  uint32_t node;
-  uint32_t spill_off;
-};
+// A leaf to split is marked in its store cursor (scur, unused until the store
+// phase): SPLIT_MARK | its log2 size << SPLIT_BITS | its split-list entry.
+constexpr uint32_t SPLIT_MARK = 1u << 31;
+constexpr uint32_t SPLIT_BITS = 26;  // split-list entries: at most max_nodes / 8 + 1
+
 
 // The stored points of one chunk of a split leaf, re-inserted this update:
 // point q of the chunk is spill entry dst + q.
@@ -250,14 +258,13 @@ struct Ctx {
   uint32_t* pool;
   uint32_t* pending;  // chunk refs freed by this update's splits (one per task)
   uint32_t* alloc_refs;
-  SplitEntry* splits;
+  uint32_t* splits;   // nodes that split in this update
   SpillTask* tasks;
-  uint32_t* sp_cur;   // per spill entry: cursor node (after its first move)
-  int4* sp_rec;       // per spill entry: the point, copied at its first move
-  uint32_t* sp_gidx;  //   and its gidx
-  uint32_t* b_cur;    // per batch point: cursor node
+  uint32_t* sp_cur;   // per re-inserted point: final leaf
+  uint32_t* b_cur;    // per batch point: leaf of the descent, then final leaf
   uint32_t* scur;     // per node: store cursor of the current update
-  uint2* mv[2];       // mover lists: points that moved in the last advance round
+  uint32_t* hist;     // counts of the cubes below split leaves; zero between updates
+  uint32_t* hist_up;  //   their sums per inner level, and the list of inner nodes
   HSlot* hash;
   uint32_t* keys;     // backlog: table slots of this update's new cells
   uint8_t* data;
@@ -269,7 +276,7 @@ struct Ctx {
   uint32_t hash_mask;
   uint32_t max_nodes, max_chunks, spill_cap, backlog_cap, max_splits;
   uint64_t max_batch;
-  uint64_t mv_cap;  // entries of each mover list (batch + spill capacity)
+  uint64_t hist_words;
   unsigned long long* launch_bar;  // barrier word of the persistent launch (abort bit)
   unsigned long long bar_ns;       // persistent launch: time limit of one grid-barrier wait
   unsigned long long ready_ns;     //   and of one wait for a batch's ready flag
@@ -402,14 +409,14 @@ __device__ __forceinline__ void node_cache_load(const Ctx& c, uint32_t* smem, ui
   for (uint32_t i = lo + threadIdx.x; i < hi; i += blockDim.x) smem[i] = c.child[i];
 }
 
-// The whole block brings the cache up to date after a decide round: the
-// nodes of the split entries [s_lo, s_hi) became inner, the nodes
-// [n_lo, n_hi) were created. Nothing else in the node table changes during an
-// update. The caller synchronises.
+// The whole block brings the cache up to date after a build: the nodes of the
+// split entries [s_lo, s_hi) became inner, the nodes [n_lo, n_hi) were
+// created. Nothing else in the node table changes during an update. The caller
+// synchronises.
 __device__ __forceinline__ void node_cache_patch(const Ctx& c, uint32_t* smem, uint32_t s_lo,
                                                  uint32_t s_hi, uint32_t n_lo, uint32_t n_hi) {
   for (uint32_t e = s_lo + threadIdx.x; e < s_hi; e += blockDim.x) {
-    const uint32_t id = c.splits[e].node;
+    const uint32_t id = c.splits[e];
     if (id < NODE_CACHE) smem[id] = c.child[id];
   }
   node_cache_load(c, smem, n_lo, n_hi);
@@ -426,36 +433,37 @@ __device__ __forceinline__ void tally_init(uint32_t* smem) {
 
 // ------------------------------------------------------ block tally cache
 //
-// Per-update node counters (points counted into a leaf, new voxels of an
-// inner node) are summed per block in shared memory first: a direct-mapped
-// table of TALLY_SLOTS (node, count) pairs. A node whose slot holds another
-// node goes to the global counter at once. Dense regions send thousands of
-// warps to the same few counters; the cache turns their global atomics,
-// which serialise at one L2 slice, into one per block and node.
+// Per-update counters (points counted into a leaf or a cube below a split
+// leaf, new voxels of an inner node) are summed per block in shared memory
+// first: a direct-mapped table of TALLY_SLOTS (index, count) pairs. An index
+// whose slot holds another one goes to the global counter at once. Dense
+// regions send thousands of warps to the same few counters; the cache turns
+// their global atomics, which serialise at one L2 slice, into one per block
+// and counter.
 
-__device__ __forceinline__ void tally_add(const Ctx& c, uint32_t* smem, uint32_t node,
+__device__ __forceinline__ void tally_add(uint32_t* counters, uint32_t* smem, uint32_t i,
                                           uint32_t k) {
 #if SL_BLOCK_TALLY
-  const uint32_t slot = (node * 0x9E3779B1u) >> (32u - TALLY_LOG2);
+  const uint32_t slot = (i * 0x9E3779B1u) >> (32u - TALLY_LOG2);
   uint32_t* tn = smem + SMEM_TALLY;
-  const uint32_t old = tn[slot] == node ? node : atomicCAS(tn + slot, NONE, node);
-  if (old == NONE || old == node) {
+  const uint32_t old = tn[slot] == i ? i : atomicCAS(tn + slot, NONE, i);
+  if (old == NONE || old == i) {
     atomicAdd(tn + TALLY_SLOTS + slot, k);
     return;
   }
 #endif
-  atomicAdd(&c.cnt[node], k);
+  atomicAdd(counters + i, k);
 }
 
 // The whole block calls at the end of a phase: add the cached counts to the
 // global counters.
-__device__ __forceinline__ void tally_flush(const Ctx& c, uint32_t* smem) {
+__device__ __forceinline__ void tally_flush(uint32_t* counters, uint32_t* smem) {
 #if SL_BLOCK_TALLY
   __syncthreads();
   const uint32_t* tn = smem + SMEM_TALLY;
   for (uint32_t i = threadIdx.x; i < TALLY_SLOTS; i += blockDim.x) {
-    const uint32_t node = tn[i], k = tn[TALLY_SLOTS + i];
-    if (node != NONE && k) atomicAdd(&c.cnt[node], k);
+    const uint32_t at = tn[i], k = tn[TALLY_SLOTS + i];
+    if (at != NONE && k) atomicAdd(counters + at, k);
   }
 #endif
 }
@@ -482,6 +490,26 @@ __device__ __forceinline__ ulonglong2 slot_load(const HSlot* s) {
                : "l"(s)
                : "memory");
   return kv;
+}
+
+// Put (key, val) into an empty slot with one 16-byte compare-and-swap; returns
+// what the slot held. (An 8-byte one on the key and a minimum on the value are
+// one more atomic on a scattered line, and leave a moment in which the key is
+// there without its value: claims 0.78 against 0.82 ms on a 16M-point terrain,
+// 1.37 against 1.45 ms on a 40M-point building scan.)
+__device__ __forceinline__ ulonglong2 slot_cas(HSlot* s, unsigned long long key,
+                                               unsigned long long val) {
+  ulonglong2 o;
+  asm volatile(
+      "{\n\t.reg .b128 cmp, swp, old;\n\t"
+      "mov.b128 cmp, {%2, %2};\n\t"
+      "mov.b128 swp, {%3, %4};\n\t"
+      "atom.relaxed.gpu.global.cas.b128 old, [%5], cmp, swp;\n\t"
+      "mov.b128 {%0, %1}, old;\n\t}"
+      : "=l"(o.x), "=l"(o.y)
+      : "l"(HASH_EMPTY), "l"(key), "l"(val), "l"(s)
+      : "memory");
+  return o;
 }
 
 // The claim table of one update. A key (node << 3G | cell) is looked for along
@@ -526,8 +554,8 @@ __device__ __forceinline__ uint32_t claim_near_mask(const Ctx& c, uint64_t n, ui
 
 // Probes after the first for `key` (slot h held another key). CLAIM_NEW, with
 // the slot in h: this call put the key into the table (the cell is new in this
-// update); CLAIM_LOWERED: the slot held the key with a larger value (or
-// another call is putting it in); CLAIM_BEATEN: it holds a lower value.
+// update); CLAIM_LOWERED: the slot held the key with a larger value;
+// CLAIM_BEATEN: it holds a lower one.
 enum : int { CLAIM_NEW = 0, CLAIM_LOWERED, CLAIM_BEATEN };
 
 __device__ int hash_claim_rest(const Ctx& c, unsigned long long key, unsigned long long val,
@@ -544,12 +572,10 @@ __device__ int hash_claim_rest(const Ctx& c, unsigned long long key, unsigned lo
     const ulonglong2 kv = slot_load(s);
     unsigned long long k = kv.x, v = kv.y;
     if (k == HASH_EMPTY) {
-      k = atomicCAS(&s->key, HASH_EMPTY, key);
-      v = HASH_EMPTY;
-      if (k == HASH_EMPTY) {
-        atomicMin(&s->val, val);
-        return CLAIM_NEW;
-      }
+      const ulonglong2 o = slot_cas(s, key, val);
+      k = o.x;
+      v = o.y;
+      if (k == HASH_EMPTY) return CLAIM_NEW;
     }
     if (k == key) {
       if (v < val) return CLAIM_BEATEN;
@@ -629,48 +655,6 @@ __device__ __forceinline__ void warp_flush(const Ctx& c, WarpBuf& wb) {
   __syncwarp();
 }
 
-// Per-warp staging of mover-list entries (shared memory, after the node cache
-// and the new-cell staging), appended to the list with one atomicAdd per
-// flush: one reservation per MVBUF movers instead of one per warp unit.
-struct MoverBuf {
-  uint2* buf;
-  uint32_t n;  // staged entries (the same value in every lane)
-};
-
-__device__ __forceinline__ MoverBuf mover_buf(uint32_t* smem) {
-  MoverBuf mb;
-  mb.buf = reinterpret_cast<uint2*>(smem + SMEM_MVBUF) + (threadIdx.x / 32) * MVBUF;
-  mb.n = 0;
-  return mb;
-}
-
-// All 32 lanes call.
-__device__ __forceinline__ void mover_flush(const Ctx& c, MoverBuf& mb, int list) {
-  if (mb.n == 0u) return;
-  __syncwarp();
-  uint32_t o0 = 0;
-  if (lane_id() == 0) o0 = atomicAdd(&c.ctl->mv_count[list], mb.n);
-  o0 = __shfl_sync(FULL_MASK, o0, 0);
-  for (uint32_t k = lane_id(); k < mb.n; k += 32) {
-    const uint64_t o = (uint64_t)o0 + k;
-    if (o < c.mv_cap) c.mv[list][o] = mb.buf[k];
-    else set_error(c, E_INTERNAL);
-  }
-  mb.n = 0;
-  __syncwarp();
-}
-
-// All 32 lanes call: lanes with `moved` stage entry `ent`.
-__device__ __forceinline__ void mover_add(const Ctx& c, MoverBuf& mb, int list, bool moved,
-                                          uint2 ent) {
-  const unsigned mm = __ballot_sync(FULL_MASK, moved);
-  if (mm == 0u) return;
-  const uint32_t k = (uint32_t)__popc(mm);
-  if (mb.n + k > MVBUF) mover_flush(c, mb, list);
-  if (moved) mb.buf[mb.n + __popc(mm & ((1u << lane_id()) - 1u))] = ent;
-  mb.n += k;
-}
-
 // All 32 lanes call. Lanes with lead[j] offer val[j] for key[j] (a cell of
 // node[j]) to the update's claim table, where the lowest value wins. The
 // first probes of all N items are issued together (their loads, then their
@@ -701,8 +685,9 @@ __device__ __forceinline__ void warp_claim(const Ctx& c, WarpBuf& wb, const bool
   for (int j = 0; j < N; ++j) {
     cas[j] = lead[j] && k0[j] == HASH_EMPTY;
     if (cas[j]) {
-      k0[j] = atomicCAS(&c.hash[h[j]].key, HASH_EMPTY, key[j]);
-      v0[j] = HASH_EMPTY;
+      const ulonglong2 kv = slot_cas(c.hash + h[j], key[j], val[j]);
+      k0[j] = kv.x;
+      v0[j] = kv.y;
     }
   }
 #pragma unroll
@@ -711,7 +696,6 @@ __device__ __forceinline__ void warp_claim(const Ctx& c, WarpBuf& wb, const bool
     if (lead[j]) {
       if (cas[j] && k0[j] == HASH_EMPTY) {
         inst[j] = on[j] = true;
-        atomicMin(&c.hash[h[j]].val, val[j]);
       } else if (k0[j] == key[j]) {
         if (v0[j] > val[j]) {
           on[j] = true;
@@ -733,18 +717,18 @@ __device__ __forceinline__ void warp_claim(const Ctx& c, WarpBuf& wb, const bool
     const LaneRun r = lane_run(inst[j], node[j]);
     if (inst[j]) {
       wb.buf[wb.n + __popc(mi & ((1u << lane) - 1u))] = h[j];
-      if (r.head) tally_add(c, wb.smem, node[j], r.end - lane);
+      if (r.head) tally_add(c.cnt, wb.smem, node[j], r.end - lane);
     }
     wb.n += ni;
   }
 }
 
-// All 32 lanes call. Lanes with `valid` count one point into `leaf` (one
-// addition per run of equal leaves; the slot is given at store).
-__device__ __forceinline__ void warp_tally(const Ctx& c, uint32_t* smem, bool valid,
-                                           uint32_t leaf) {
-  const LaneRun r = lane_run(valid, leaf);
-  if (valid && r.head) tally_add(c, smem, leaf, r.end - lane_id());
+// All 32 lanes call. Lanes with `valid` add one to counters[i] (one addition
+// per run of equal counters).
+__device__ __forceinline__ void warp_tally(uint32_t* counters, uint32_t* smem, bool valid,
+                                           uint32_t i) {
+  const LaneRun r = lane_run(valid, i);
+  if (valid && r.head) tally_add(counters, smem, i, r.end - lane_id());
 }
 
 // The k-th 32-item unit of a phase that a warp handles: chunks of 2^chl
@@ -831,45 +815,280 @@ __device__ void phase_count1(const Ctx& c, uint32_t* smem, const NodeCache nc, c
     __syncwarp();
 #pragma unroll
     for (int j = 0; j < U; ++j) {
-      warp_tally(c, smem, valid[j], node[j]);
+      warp_tally(c.cnt, smem, valid[j], node[j]);
       if (valid[j]) c.b_cur[iu[j]] = node[j];
     }
   }
-  tally_flush(c, smem);
+  tally_flush(c.cnt, smem);
 }
 
-// ----------------------------------------------------------- phase: advance
+// -------------------------------------------------------- phase: histogram
 
-// A mover-list entry (8 bytes) is a point whose cursor moved in the last
-// advance round: x = MV_SPILL | spill entry, or a batch point index; y = its
-// cursor node (MV_NODE_BITS bits) | that node's level << MV_NODE_BITS.
+// The spill tasks as units of 32 re-inserted points (a unit never crosses into
+// the next task).
+__device__ __forceinline__ uint32_t task_units(const Ctx& c) { return (c.C + 31u) / 32u; }
 
-// Advance round r of the expansion (r >= 2 counts decide rounds): zero the
-// grids of the splits [s_lo, s_hi) of the previous decide, then move every
-// point whose cursor node split there one level down, counting it into the
-// child, and list the points that moved in mover list out_list.
-//
-// Only nodes created in the previous round can split in a later one (every
-// leaf that existed before the update was decided in the first round), so
-// only points that moved in the previous round can move again: the first
-// round (in_list < 0) scans every batch cursor and every point of the spill
-// tasks [0, t_hi) (all created by the first decide; their points still sit
-// in the split leaf's chunks and are copied to the spill records here), later
-// rounds only the n_in entries of mover list in_list, which carry cursor and
-// level. Points are cut into 32-item warp units (a unit of a task never
-// crosses into the next task).
-__device__ void phase_advance(const Ctx& c, uint32_t* smem, const NodeCache nc, const int4* pts,
-                              uint64_t n, uint32_t t_hi, uint32_t s_lo, uint32_t s_hi,
-                              int in_list, uint32_t n_in, int out_list, uint64_t warp0,
-                              uint64_t nwarps) {
+// Lane's re-inserted point of unit u of the tasks [0, t_hi): its task, its
+// place in the task's chunk; false past the end of the task.
+__device__ __forceinline__ bool task_point(const Ctx& c, uint32_t u, uint32_t parts, SpillTask& tk,
+                                           uint32_t& q) {
+  const uint32_t t = u / parts;
+  q = (u - t * parts) * 32u + lane_id();
+  tk = c.tasks[t];
+  if (!ref_ok(c, tk.ref, c.chunk_bytes) || tk.n > c.C || tk.node >= c.max_nodes ||
+      (unsigned long long)tk.dst + tk.n > c.spill_cap) {
+    if (lane_id() == 0) set_error(c, E_INTERNAL);
+    return false;
+  }
+  return q < tk.n;
+}
+
+// From `node` down to the leaf that holds the point now.
+__device__ __forceinline__ uint32_t walk_down(const Ctx& c, NodeCache nc, uint32_t node,
+                                              uint32_t rx, uint32_t ry, uint32_t rz) {
+  uint32_t ch = node_child(c, nc, node);
+  if (ch == NONE) return node;
+  uint32_t L = c.rlog2 - c.meta[node].level;
+  while (ch != NONE) {
+    if (ch + 8u > c.max_nodes || L == 0u) {
+      set_error(c, E_INTERNAL);
+      break;
+    }
+    node = ch + octant(rx, ry, rz, L);
+    --L;
+    ch = node_child(c, nc, node);
+  }
+  return node;
+}
+
+// Bits of a 5-bit number, two zeros between them.
+__device__ __forceinline__ uint32_t spread5(uint32_t x) {
+  x = (x | (x << 8)) & 0x100Fu;
+  x = (x | (x << 4)) & 0x10C3u;
+  return (x | (x << 2)) & 0x1249u;
+}
+
+// Levels below a split leaf that one histogram covers, for K leaves of `most`
+// points at most, of an update of n points: 3, one more for every factor of 4
+// that the fullest leaf is over T (points lie on surfaces: four children out
+// of eight), at most HIST_DEPTH and a count per moving point. A leaf that is
+// not deep enough yet goes round again, which reads the points once more; 5
+// levels for every leaf cost more counts than that saves (terrain: build 0.30
+// against 0.11 ms a pass; mixed batches: histogram 0.68 against 0.51 ms), 1 and
+// 2 levels more than the factors took a second round too often (clustered
+// scan: 1.72 and 1.57 against 1.50 ms). hist_words has room for one level.
+constexpr uint32_t HIST_DEPTH = 5;
+__host__ __device__ __forceinline__ uint32_t hist_depth(const Ctx& c, uint32_t K, uint64_t n,
+                                                        uint32_t most) {
+  const uint64_t want = n < 32768u ? 32768u : n;
+  const uint64_t lim = want < c.hist_words ? want : c.hist_words;
+  uint32_t aim = 3, d = 1;
+  while (aim < HIST_DEPTH && ((unsigned long long)c.T << (2u * (aim - 2u))) < most) ++aim;
+  while (d < aim && ((uint64_t)K << (3u * (d + 1u))) <= lim) ++d;
+  return d;
+}
+
+// Count the points of the leaves in the split entries [s_lo, s_lo + K) into
+// the cubes d levels below (hist[entry][Morton index]). In the first round a
+// point's cursor is its leaf; later the leaf is looked up (only leaves of the
+// lowest level of the round before split again, which is rare).
+__device__ void phase_hist(const Ctx& c, uint32_t* smem, const NodeCache nc, const int4* pts,
+                           uint64_t n, uint32_t t_hi, uint32_t s_lo, uint32_t K, uint32_t d,
+                           bool first) {
   tally_init(smem);
   __syncthreads();  // also publishes the caller's node-cache writes
-  MoverBuf mb = mover_buf(smem);
+  if (((uint64_t)K << (3u * d)) > c.hist_words) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) set_error(c, E_INTERNAL);
+    return;  // (the same in every thread)
+  }
+  const uint32_t lane = lane_id(), parts = task_units(c);
+  const uint64_t us = (uint64_t)t_hi * parts, units = us + (n + 31) / 32;
+  // every block takes one range of neighbouring units: its points fall into
+  // few cubes, whose counts its tally cache adds up (a shuffled building scan
+  // of 40M points: 1.03 against 1.47 ms a pass with the units dealt out)
+  const uint64_t per = (units + gridDim.x - 1) / gridDim.x;
+  const uint64_t last = (blockIdx.x + 1ull) * per, end = last < units ? last : units;
+  for (uint64_t w = blockIdx.x * per + threadIdx.x / 32; w < end; w += blockDim.x / 32) {
+    bool on = false, have = false;
+    uint32_t cur = 0;
+    uint64_t i = 0;
+    int4 p = make_int4(0, 0, 0, 0);
+    if (w < us) {
+      SpillTask tk;
+      uint32_t q;
+      on = have = task_point(c, (uint32_t)w, parts, tk, q);
+      if (on) {
+        p = chunk_recs(c, tk.ref)[q];
+        cur = tk.node;
+      }
+    } else {
+      i = (w - us) * 32 + lane;
+      on = i < n;
+      cur = on ? c.b_cur[i] : 0u;
+    }
+    uint32_t rx = 0, ry = 0, rz = 0;
+    if (on && !first) {
+      if (!have) p = __ldcg(pts + i);
+      have = true;
+      rel_coords(c, p, rx, ry, rz);
+      cur = walk_down(c, nc, cur, rx, ry, rz);
+    }
+    const uint32_t mark = on ? c.scur[cur] : 0u;
+    const uint32_t e = (mark & ((1u << SPLIT_BITS) - 1u)) - s_lo;
+    on = (mark & SPLIT_MARK) && e < K;  // e: wraps for entries of earlier rounds
+    uint32_t at = 0;
+    if (on) {
+      if (!have) p = __ldcg(pts + i);
+      rel_coords(c, p, rx, ry, rz);
+      const uint32_t L = (mark >> SPLIT_BITS) & 31u;
+      const uint32_t de = d < L ? d : L, sh = L - de, m = (1u << de) - 1u;
+      const uint32_t cube = spread5((rx >> sh) & m) | (spread5((ry >> sh) & m) << 1) |
+                            (spread5((rz >> sh) & m) << 2);
+      at = (e << (3u * d)) | (cube << (3u * (d - de)));
+    }
+    warp_tally(c.hist, smem, on, at);
+  }
+  tally_flush(c.hist, smem);
+}
+
+// ------------------------------------------------------------ phase: build
+
+// Index of the first cube of level j below a split leaf among its cubes of all
+// levels (8^0 + ... + 8^(j-1)). hist_up holds, per leaf, the sums of levels
+// 0 .. d-1 in this order, then the list of the inner nodes among them.
+__device__ __forceinline__ uint32_t level_first(uint32_t j) { return ((1u << (3u * j)) - 1u) / 7u; }
+
+// One block per split leaf (entries [s_lo, s_lo + K)): sum its cube counts
+// level by level, make every cube with more than T points an inner node (8
+// children with chunk directories, and a grid each, zeroed in the claim
+// phase), leave the leaves' counts in cnt for decide, and clear the histogram.
+// lvl0: levels that earlier rounds of this update built above. A round here
+// stands for d of the paper's: iters counts the paper's, and max_iters bounds
+// them as if they had been made one by one.
+// The subtree of a leaf is a few dozen nodes; the sums read 8^d counts
+// (128 KB at d = 5) from L2, which the other blocks do at the same time.
+__device__ void phase_build(const Ctx& c, uint32_t s_lo, uint32_t K, uint32_t d, uint32_t lvl0,
+                            uint32_t max_iters) {
+  __shared__ uint32_t s_n, s_deep, s_node, s_entry, s_ok;
+  __shared__ unsigned long long s_data;
+  const uint32_t U = level_first(d), bins = 1u << (3u * d);
+  for (uint32_t k = blockIdx.x; k < K; k += gridDim.x) {
+    uint32_t* hist = c.hist + ((uint64_t)k << (3u * d));
+    uint32_t* up = c.hist_up + (uint64_t)k * 2u * U;
+    uint32_t* list = up + U;
+    const uint32_t root = c.splits[s_lo + k];
+    const NodeMeta& m = c.meta[root];
+    const uint32_t L = c.rlog2 - m.level, level = m.level;
+    const int32_t rm[3] = {m.min[0], m.min[1], m.min[2]};
+    if (threadIdx.x == 0) s_n = s_deep = 0;
+    for (uint32_t j = d; j-- > 0;) {
+      const uint32_t* below = j + 1u == d ? hist : up + level_first(j + 1u);
+      for (uint32_t q = threadIdx.x; q < (1u << (3u * j)); q += blockDim.x) {
+        uint32_t t = 0;
+#pragma unroll
+        for (uint32_t o = 0; o < 8; ++o) t += below[8u * q + o];
+        up[level_first(j) + q] = t;
+      }
+      __syncthreads();
+    }
+    // number the inner nodes; an inner node's sum becomes SPLIT_MARK | number
+    for (uint32_t i = threadIdx.x; i < U; i += blockDim.x) {
+      uint32_t j = 0;
+      while (level_first(j + 1u) <= i) ++j;
+      if (i == 0 || (up[i] > c.T && L > j)) {
+        const uint32_t e = atomicAdd(&s_n, 1u);
+        atomicMax(&s_deep, j);
+        list[e] = i;
+        up[i] = SPLIT_MARK | e;
+      }
+    }
+    __syncthreads();
+    const uint32_t ns = s_n;
+    if (threadIdx.x == 0) {
+      const unsigned long long bytes = (unsigned long long)ns * (8u * c.dir_bytes + c.grid_bytes);
+      const uint32_t rounds = lvl0 + s_deep + 1u;
+      s_node = atomicAdd(&c.ctl->n_nodes, 8u * ns);
+      s_data = atomicAdd(&c.ctl->bump, bytes);
+      s_entry = ns > 1u ? atomicAdd(&c.ctl->split_count, ns - 1u) : 0u;
+      if (ns > 1u) atomicAdd(&c.ctl->split_inner, ns - 1u);
+      atomicMax(&c.ctl->iters, rounds + 1u);
+      s_ok = 0;
+      if (rounds >= max_iters) set_error(c, E_ITER_CAP);
+      else if ((unsigned long long)s_node + 8ull * ns > c.max_nodes ||
+               (unsigned long long)s_entry + ns > c.max_splits)
+        set_error(c, E_NODES);
+      else if (s_data + bytes > c.data_bytes) set_error(c, E_ARENA);
+      else s_ok = 1;
+    }
+    __syncthreads();
+    if (s_ok) {
+      const uint32_t node0 = s_node;
+      const unsigned long long grid0 = s_data + (unsigned long long)ns * 8u * c.dir_bytes;
+      auto grid_of = [&](uint32_t e) -> uint32_t {
+        return (uint32_t)((grid0 + (unsigned long long)e * c.grid_bytes) / REF_BYTES);
+      };
+      for (uint32_t t = threadIdx.x; t < 8u * ns; t += blockDim.x) {
+        const uint32_t e = t >> 3, o = t & 7u, i = list[e];
+        uint32_t j = 0;
+        while (level_first(j + 1u) <= i) ++j;
+        const uint32_t q = i - level_first(j);
+        const uint32_t id =
+            j == 0 ? root : node0 + 8u * (up[level_first(j - 1u) + (q >> 3)] & ~SPLIT_MARK) + (q & 7u);
+        const uint32_t path = 8u * q + o, kid = node0 + t;
+        const uint32_t w = j + 1u == d ? hist[path] : up[level_first(j + 1u) + path];
+        const bool inner = j + 1u < d && (w & SPLIT_MARK);
+        NodeMeta cm;
+        for (uint32_t a = 0; a < 3; ++a) {
+          cm.min[a] = rm[a];
+          for (uint32_t l = 0; l <= j; ++l)  // octant digits, the topmost first
+            cm.min[a] += (int32_t)(((path >> (3u * (j - l) + a)) & 1u) << (L - 1u - l));
+        }
+        cm.level = level + j + 1u;
+        cm.n_chunks = 0;
+        cm.head = cm.tail = NONE;
+        cm.dir = inner ? NONE
+                       : (uint32_t)((s_data + (unsigned long long)t * c.dir_bytes) / REF_BYTES);
+        cm.st_nch = 0;
+        cm.st_tail = NONE;
+        cm.st_seq = 0;
+        cm.st_base = 0;
+        cm.touched = 0;
+        cm.compact = 0;
+        cm.up = id | ((level + j) << NODE_BITS);
+        cm.up_grid = grid_of(e);
+        c.meta[kid] = cm;
+        c.child[kid] = inner ? node0 + 8u * (w & ~SPLIT_MARK) : NONE;
+        c.gridref[kid] = inner ? grid_of(w & ~SPLIT_MARK) : NONE;
+        c.cnt[kid] = inner ? 0u : w;
+        c.num[kid] = 0;
+        if (o == 0) {
+          if (j == 0) {
+            c.child[root] = node0 + 8u * e;
+            c.gridref[root] = grid_of(e);
+          } else {
+            // entry numbers without the root's
+            const uint32_t re = up[0] & ~SPLIT_MARK;
+            c.splits[s_entry + (e < re ? e : e - 1u)] = id;
+          }
+        }
+      }
+    }
+    __syncthreads();
+    uint4* h4 = reinterpret_cast<uint4*>(hist);
+    for (uint32_t i = threadIdx.x; i < bins / 4u; i += blockDim.x) h4[i] = make_uint4(0, 0, 0, 0);
+    __syncthreads();  // before s_n is used again
+  }
+}
+
+// Zero the grids of this update's splits (entries [0, s_hi)); the claim phase
+// does so while it claims (nothing reads them before the voxels are stored).
+__device__ __forceinline__ void zero_grids(const Ctx& c, uint32_t s_hi, uint64_t warp0,
+                                           uint64_t nwarps) {
   const uint32_t lane = lane_id();
   const uint32_t zpg = (c.grid_bytes + ZERO_UNIT - 1) / ZERO_UNIT;  // zero units per grid
-  const uint64_t uz = (uint64_t)(s_hi - s_lo) * zpg;
+  const uint64_t uz = (uint64_t)s_hi * zpg;
   for (uint64_t w = warp0; w < uz; w += nwarps) {
-    const uint32_t id = c.splits[s_lo + (uint32_t)(w / zpg)].node;
+    const uint32_t id = c.splits[(uint32_t)(w / zpg)];
     const uint32_t gref = id < c.max_nodes ? c.gridref[id] : NONE;
     if (!ref_ok(c, gref, c.grid_bytes)) {
       if (lane == 0) set_error(c, E_INTERNAL);
@@ -880,112 +1099,15 @@ __device__ void phase_advance(const Ctx& c, uint32_t* smem, const NodeCache nc, 
     int4* g = reinterpret_cast<int4*>(grid_words(c, gref));
     for (uint32_t b = lo / 16 + lane; b < hi / 16; b += 32) g[b] = make_int4(0, 0, 0, 0);
   }
-  const uint32_t parts = (c.C + 31) / 32;  // units per task
-  const bool first = in_list < 0;
-  const uint64_t ub = first ? (n + 31) / 32 : 0;
-  const uint64_t units = first ? ub + (uint64_t)t_hi * parts : ((uint64_t)n_in + 31) / 32;
-  const uint2* in = first ? nullptr : c.mv[in_list];
-  constexpr int AU = ADVANCE_U;
-  // each warp carries AU units (w, w + nwarps, ...) at a time so that their
-  // L2 round trips overlap (chunks of neighbouring units measured slower
-  // here: the movers of dense regions then load few warps)
-  for (uint64_t k0 = 0; warp_unit(warp0, nwarps, k0, 0) < units; k0 += AU) {
-    bool valid[AU], spill[AU], have_p[AU], mv[AU];
-    uint32_t idx[AU], cur[AU], lvl[AU], ch[AU];  // idx: batch point index or spill entry
-    int4 p[AU];
-#pragma unroll
-    for (int j = 0; j < AU; ++j) {
-      const uint64_t w = warp_unit(warp0, nwarps, k0 + j, 0);
-      valid[j] = spill[j] = have_p[j] = false;
-      idx[j] = cur[j] = lvl[j] = 0;
-      p[j] = make_int4(0, 0, 0, 0);
-      if (w >= units) {
-        // past the end: nothing
-      } else if (first && w < ub) {
-        const uint64_t i = w * 32 + lane;
-        valid[j] = i < n;
-        idx[j] = (uint32_t)i;
-        cur[j] = valid[j] ? c.b_cur[i] : 0u;
-      } else if (first) {
-        const uint64_t u = w - ub;
-        const uint32_t t = (uint32_t)(u / parts), q = (uint32_t)(u % parts) * 32u + lane;
-        const SpillTask tk = c.tasks[t];
-        const bool task_ok = ref_ok(c, tk.ref, c.chunk_bytes) && tk.n <= c.C &&
-                             (unsigned long long)tk.dst + tk.n <= c.spill_cap;
-        if (!task_ok && lane == 0) set_error(c, E_INTERNAL);
-        valid[j] = task_ok && q < tk.n;
-        spill[j] = true;
-        idx[j] = tk.dst + q;
-        cur[j] = tk.node;
-        if (valid[j]) {
-          // the point leaves its chunk (which returns to the pool at store)
-          p[j] = chunk_recs(c, tk.ref)[q];
-          c.sp_rec[idx[j]] = p[j];
-          c.sp_gidx[idx[j]] = chunk_aux(c, tk.ref)[q];
-          have_p[j] = true;
-        }
-      } else {
-        const uint64_t k = w * 32 + lane;
-        if (k < n_in) {
-          const uint2 ent = in[k];
-          valid[j] = true;
-          spill[j] = (ent.x & MV_SPILL) != 0u;
-          idx[j] = ent.x & ~MV_SPILL;
-          cur[j] = ent.y & MV_NODE_MASK;
-          lvl[j] = ent.y >> MV_NODE_BITS;
-          if (spill[j] ? idx[j] >= c.spill_cap : idx[j] >= n) {
-            set_error(c, E_INTERNAL);
-            valid[j] = false;
-          }
-        }
-      }
-      if (valid[j] && cur[j] >= c.max_nodes) {
-        set_error(c, E_INTERNAL);
-        valid[j] = false;
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < AU; ++j) {
-      // read a point only when its cursor node split (it moves)
-      ch[j] = valid[j] ? node_child(c, nc, cur[j]) : NONE;
-      mv[j] = ch[j] != NONE && ch[j] + 8u <= c.max_nodes;
-      if (mv[j]) {
-        if (first) lvl[j] = c.meta[cur[j]].level;
-        if (!have_p[j]) {
-          p[j] = spill[j] ? c.sp_rec[idx[j]] : __ldcg(pts + idx[j]);
-        }
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < AU; ++j) {
-      if (mv[j]) {
-        uint32_t rx, ry, rz;
-        rel_coords(c, p[j], rx, ry, rz);
-        cur[j] = ch[j] + octant(rx, ry, rz, c.rlog2 - lvl[j]);
-      }
-      warp_tally(c, smem, mv[j], cur[j]);
-      if (mv[j]) {
-        if (spill[j]) c.sp_cur[idx[j]] = cur[j];
-        else c.b_cur[idx[j]] = cur[j];
-      }
-      mover_add(c, mb, out_list, mv[j],
-                make_uint2(spill[j] ? (idx[j] | MV_SPILL) : idx[j],
-                           cur[j] | ((lvl[j] + 1u) << MV_NODE_BITS)));
-    }
-  }
-  mover_flush(c, mb, out_list);
-  tally_flush(c, smem);
 }
 
 // ------------------------------------------------------------- phase: claim
 
 // Points of a warp that go on to the next coarser level wait in shared memory
-// (in the mover staging, which the claim phase does not use) until 32 of them
-// make a full warp: about one point in ten survives its first claim, so
-// walking on at once would leave most lanes idle for every further level.
-constexpr int CLAIM_U = SL_CLAIM_UNROLL;  // units of 32 points a warp claims for at once
-constexpr uint32_t CLAIM_QUEUE = 32 * (CLAIM_U + 1);
-static_assert(6 * CLAIM_QUEUE <= 2 * MVBUF, "the claim queue fits the mover staging");
+// until 32 of them make a full warp: about one point in ten survives its first
+// claim, so walking on at once would leave most lanes idle for every further
+// level.
+constexpr uint32_t RESPILL = 1u << 31;
 struct ClaimQueue {
   uint32_t* q;  // node | spill flag, rx, ry, rz, rgba, gidx: CLAIM_QUEUE words each
   uint32_t n;   // the same value in every lane
@@ -993,7 +1115,7 @@ struct ClaimQueue {
 
 // One claim of one point: the parent of `node`.
 struct ClaimItem {
-  uint32_t node;  // MV_SPILL: a re-inserted point
+  uint32_t node;  // | RESPILL: a re-inserted point
   uint32_t rx, ry, rz, rgba, gidx;
 };
 
@@ -1021,16 +1143,16 @@ __device__ __forceinline__ void claim_level(const Ctx& c, WarpBuf& wb, ClaimQueu
   uint2 up[N];
 #pragma unroll
   for (int j = 0; j < N; ++j) {
-    up[j] = on[j] ? *reinterpret_cast<const uint2*>(&c.meta[it[j].node & MV_NODE_MASK].up)
+    up[j] = on[j] ? *reinterpret_cast<const uint2*>(&c.meta[it[j].node & NODE_MASK].up)
                   : make_uint2(NONE, 0u);
   }
 #pragma unroll
   for (int j = 0; j < N; ++j) {
-    par[j] = up[j].x & MV_NODE_MASK;
+    par[j] = up[j].x & NODE_MASK;
     word[j] = cell[j] = 0;
     want[j] = false;
     if (up[j].x != NONE) {
-      cell[j] = cell_index(it[j].rx, it[j].ry, it[j].rz, c.rlog2 - (up[j].x >> MV_NODE_BITS), c.G);
+      cell[j] = cell_index(it[j].rx, it[j].ry, it[j].rz, c.rlog2 - (up[j].x >> NODE_BITS), c.G);
       if (!ref_ok(c, up[j].y, c.grid_bytes) || par[j] >= c.max_nodes) {
         set_error(c, E_INTERNAL);
       } else {
@@ -1051,19 +1173,19 @@ __device__ __forceinline__ void claim_level(const Ctx& c, WarpBuf& wb, ClaimQueu
     if (SORTED) {
       const LaneRun r = lane_run(want[j], key[j]);  // all lanes take part
       // (a head wants its claim)
-      lead[j] = (it[j].node & MV_SPILL) || a.open ? want[j] : r.head;
+      lead[j] = (it[j].node & RESPILL) || a.open ? want[j] : r.head;
     }
   }
   warp_claim<N>(c, wb, lead, key, val, par, a.near, more);
 #pragma unroll
   for (int j = 0; j < N; ++j) {
     // a re-inserted point sampled the grids above its old leaf when it came
-    if ((it[j].node & MV_SPILL) && par[j] < a.nodes0) more[j] = false;
+    if ((it[j].node & RESPILL) && par[j] < a.nodes0) more[j] = false;
     const unsigned mm = __ballot_sync(FULL_MASK, more[j]);
     if (mm == 0u) continue;
     if (more[j]) {
       uint32_t* q = cq.q + cq.n + __popc(mm & ((1u << lane) - 1u));
-      q[0] = par[j] | (it[j].node & MV_SPILL);
+      q[0] = par[j] | (it[j].node & RESPILL);
       q[CLAIM_QUEUE] = it[j].rx;
       q[2 * CLAIM_QUEUE] = it[j].ry;
       q[3 * CLAIM_QUEUE] = it[j].rz;
@@ -1094,46 +1216,51 @@ __device__ __forceinline__ void claim_drain(const Ctx& c, WarpBuf& wb, ClaimQueu
   }
 }
 
-// The re-inserted points (spill records [0, n_spill)) and the batch points
-// [0, n), each from its final leaf's parent upwards. The re-inserted points
-// come first: they have the lowest indices, so batch points stop at them.
-// Each warp carries CLAIM_U units at a time, so that their round trips
-// overlap, and loads the next ones' points and cursors meanwhile.
-__device__ void phase_claim(const Ctx& c, uint32_t* smem, const int4* pts, uint64_t n,
-                            unsigned long long base, uint32_t n_spill, const ClaimArgs& a,
-                            uint64_t warp0, uint64_t nwarps) {
+// The re-inserted points (of the spill tasks [0, t_hi)) and the batch points
+// [0, n): each is followed to its final leaf (noted in sp_cur, b_cur for the
+// store phase) and claims from the leaf's parent upwards. The re-inserted
+// points come first: they have the lowest indices, so batch points stop at
+// them. Each warp loads the next unit's points and cursors while it claims.
+__device__ void phase_claim(const Ctx& c, uint32_t* smem, const NodeCache nc, const int4* pts,
+                            uint64_t n, unsigned long long base, uint32_t t_hi, uint32_t s_hi,
+                            const ClaimArgs& a, uint64_t warp0, uint64_t nwarps) {
   constexpr int U = CLAIM_U;
   tally_init(smem);
-  __syncthreads();
+  __syncthreads();  // also publishes the caller's node-cache writes
+  zero_grids(c, s_hi, warp0, nwarps);
   WarpBuf wb = warp_buf(smem);
   ClaimQueue cq;
-  cq.q = smem + SMEM_MVBUF + (threadIdx.x / 32) * MVBUF * 2;
+  cq.q = smem + SMEM_QUEUE + (threadIdx.x / 32) * CLAIM_QUEUE * 6;
   cq.n = 0;
-  const uint32_t lane = lane_id();
+  const uint32_t lane = lane_id(), parts = task_units(c);
   // units [0, us) are re-inserted points, the rest batch points
-  const uint64_t us = ((uint64_t)n_spill + 31) / 32, units = us + (n + 31) / 32;
+  const uint64_t us = (uint64_t)t_hi * parts, units = us + (n + 31) / 32;
   const uint32_t chl = count_chunk_log2(units, nwarps);
   int4 pn[U];
-  uint32_t curn[U];
-  auto load = [&](uint64_t w, int4& p, uint32_t& cur) {  // cur = NONE: no point
+  uint32_t curn[U], gn[U];
+  auto load = [&](uint64_t w, int4& p, uint32_t& cur, uint32_t& g) {  // cur = NONE: no point
     p = make_int4(0, 0, 0, 0);
     cur = NONE;
+    g = 0;
     if (w < us) {
-      const uint64_t e = w * 32 + lane;
-      if (e < n_spill) {
-        p = c.sp_rec[e];
-        cur = c.sp_cur[e] | MV_SPILL;
+      SpillTask tk;
+      uint32_t q;
+      if (task_point(c, (uint32_t)w, parts, tk, q)) {
+        p = chunk_recs(c, tk.ref)[q];
+        g = chunk_aux(c, tk.ref)[q];
+        cur = tk.node | RESPILL;
       }
     } else {
       const uint64_t i = (w - us) * 32 + lane;
       if (i < n) {
         p = __ldcg(pts + i);
+        g = (uint32_t)(base + i);
         cur = c.b_cur[i];
       }
     }
   };
 #pragma unroll
-  for (int j = 0; j < U; ++j) load(warp_unit(warp0, nwarps, j, chl), pn[j], curn[j]);
+  for (int j = 0; j < U; ++j) load(warp_unit(warp0, nwarps, j, chl), pn[j], curn[j], gn[j]);
   for (uint64_t k = 0; warp_unit(warp0, nwarps, k, chl) < units; k += U) {
     bool on[U];
     ClaimItem it[U];
@@ -1141,19 +1268,27 @@ __device__ void phase_claim(const Ctx& c, uint32_t* smem, const int4* pts, uint6
     for (int j = 0; j < U; ++j) {
       const uint64_t w = warp_unit(warp0, nwarps, k + j, chl);
       on[j] = curn[j] != NONE;
+      it[j] = ClaimItem{curn[j], 0, 0, 0, (uint32_t)pn[j].w, gn[j]};
       rel_coords(c, pn[j], it[j].rx, it[j].ry, it[j].rz);
-      it[j].node = curn[j];
-      it[j].rgba = (uint32_t)pn[j].w;
-      it[j].gidx = w >= us ? (uint32_t)(base + (w - us) * 32 + lane)
-                           : (on[j] ? c.sp_gidx[w * 32 + lane] : 0u);
-      load(warp_unit(warp0, nwarps, k + j + U, chl), pn[j], curn[j]);
+      load(warp_unit(warp0, nwarps, k + j + U, chl), pn[j], curn[j], gn[j]);
+      if (on[j]) {
+        const uint32_t cur = it[j].node & ~RESPILL;
+        const uint32_t leaf = walk_down(c, nc, cur, it[j].rx, it[j].ry, it[j].rz);
+        if (w < us) {
+          const uint32_t t = (uint32_t)w / parts;
+          c.sp_cur[c.tasks[t].dst + ((uint32_t)w - t * parts) * 32u + lane] = leaf;
+        } else if (leaf != cur) {
+          c.b_cur[(w - us) * 32 + lane] = leaf;
+        }
+        it[j].node = leaf | (it[j].node & RESPILL);
+      }
     }
     claim_level<U, true>(c, wb, cq, a, on, it);
     claim_drain(c, wb, cq, a, 31u);
   }
   claim_drain(c, wb, cq, a, 0u);
   warp_flush(c, wb);
-  tally_flush(c, smem);
+  tally_flush(c.cnt, smem);
 }
 
 // ------------------------------------------------------------ phase: decide
@@ -1236,28 +1371,21 @@ __device__ void alloc_chunks(const Ctx& c, uint32_t id, uint32_t total, bool lea
   if (lane == 0) m.n_chunks = need;
 }
 
-// Section 5.1, all 32 lanes of a warp call: split leaf `id` whose count
-// exceeds T: 8 children (with chunk directories), a grid for the node (zeroed
-// in the next round), and one spill task per chunk of its stored points;
+// Section 5.1, all 32 lanes of a warp call: list leaf `id`, whose count exceeds
+// T, for the build phase, with one spill task per chunk of its stored points;
 // those chunks return to the pool at the end of the update.
-__device__ void split_leaf(const Ctx& c, uint32_t id) {
+__device__ void split_leaf(const Ctx& c, uint32_t id, uint32_t total) {
   const uint32_t lane = lane_id();
   NodeMeta& m = c.meta[id];
   const uint32_t stored = c.num[id], nch = m.n_chunks, mdir = m.dir;
-  uint32_t c0 = 0, s0 = 0, t0 = 0, e = 0, ok = 1;
-  unsigned long long dbase = 0, g = 0;
+  uint32_t s0 = 0, t0 = 0, e = 0, ok = 1;
   if (lane == 0) {
-    c0 = atomicAdd(&c.ctl->n_nodes, 8u);
-    dbase = atomicAdd(&c.ctl->bump, 8ull * c.dir_bytes + c.grid_bytes);
-    g = dbase + 8ull * c.dir_bytes;
     s0 = atomicAdd(&c.ctl->spill_count, stored);
     t0 = atomicAdd(&c.ctl->ntasks, nch);
     e = atomicAdd(&c.ctl->split_count, 1u);
-    if ((unsigned long long)c0 + 8 > c.max_nodes || e >= c.max_splits) {
+    atomicMax(&c.ctl->split_most, total);
+    if (e >= c.max_splits) {
       set_error(c, E_NODES);
-      ok = 0;
-    } else if (g + c.grid_bytes > c.data_bytes) {
-      set_error(c, E_ARENA);
       ok = 0;
     } else if ((unsigned long long)s0 + stored > c.spill_cap) {
       set_error(c, E_SPILL);
@@ -1269,37 +1397,9 @@ __device__ void split_leaf(const Ctx& c, uint32_t id) {
     }
   }
   if (!__shfl_sync(FULL_MASK, ok, 0)) return;
-  c0 = __shfl_sync(FULL_MASK, c0, 0);
   s0 = __shfl_sync(FULL_MASK, s0, 0);
   t0 = __shfl_sync(FULL_MASK, t0, 0);
   e = __shfl_sync(FULL_MASK, e, 0);
-  dbase = __shfl_sync(FULL_MASK, dbase, 0);
-  g = __shfl_sync(FULL_MASK, g, 0);
-  if (lane < 8) {
-    const uint32_t k = lane;
-    const uint32_t Lc = c.rlog2 - m.level - 1u;  // children's log2 size
-    NodeMeta cm;
-    cm.min[0] = m.min[0] + (int32_t)((k & 1u) << Lc);
-    cm.min[1] = m.min[1] + (int32_t)(((k >> 1) & 1u) << Lc);
-    cm.min[2] = m.min[2] + (int32_t)(((k >> 2) & 1u) << Lc);
-    cm.level = m.level + 1u;
-    cm.n_chunks = 0;
-    cm.head = cm.tail = NONE;
-    cm.dir = (uint32_t)((dbase + (unsigned long long)k * c.dir_bytes) / REF_BYTES);
-    cm.st_nch = 0;
-    cm.st_tail = NONE;
-    cm.st_seq = 0;
-    cm.st_base = 0;
-    cm.touched = 0;
-    cm.compact = 0;
-    cm.up = id | (m.level << MV_NODE_BITS);
-    cm.up_grid = (uint32_t)(g / REF_BYTES);
-    c.meta[c0 + k] = cm;
-    c.child[c0 + k] = NONE;
-    c.gridref[c0 + k] = NONE;
-    c.cnt[c0 + k] = 0;
-    c.num[c0 + k] = 0;
-  }
   const uint32_t* dir = nch ? dir_entries(c, mdir) : nullptr;
   for (uint32_t j = lane; j < nch; j += 32) {
     const uint32_t ref = dir[j];
@@ -1309,14 +1409,13 @@ __device__ void split_leaf(const Ctx& c, uint32_t id) {
   }
   __syncwarp();  // every lane has read m before lane 0 rewrites it
   if (lane == 0) {
-    c.splits[e] = SplitEntry{id, s0};
-    c.gridref[id] = (uint32_t)(g / REF_BYTES);
+    c.splits[e] = id;
+    c.scur[id] = SPLIT_MARK | ((c.rlog2 - m.level) << SPLIT_BITS) | e;
     m.n_chunks = 0;
     m.head = m.tail = NONE;
     m.dir = NONE;
     c.num[id] = 0;
     c.cnt[id] = 0;
-    c.child[id] = c0;
   }
 }
 
@@ -1372,7 +1471,7 @@ __device__ __forceinline__ void decide_node(const Ctx& c, uint32_t id) {
   if (leaf) {
     const uint32_t L = c.rlog2 - c.meta[id].level;
     if (total > c.T && L > 0) {
-      split_leaf(c, id);
+      split_leaf(c, id, total);
       return;
     }
   }
@@ -1387,11 +1486,8 @@ __device__ __forceinline__ void decide_node(const Ctx& c, uint32_t id) {
 // Candidates, one warp each: the node id range [n_lo, n_hi). In the expansion
 // rounds these are leaves; after the claim phase the counts left are the inner
 // nodes' new voxels, which get their chunks here.
-// zero_list >= 0: also empty that mover list (the next advance round fills
-// it; the round before last was its reader).
-__device__ void phase_decide(const Ctx& c, uint32_t n_lo, uint32_t n_hi, int zero_list,
-                             uint64_t warp0, uint64_t nwarps) {
-  if (zero_list >= 0 && warp0 == 0 && lane_id() == 0) c.ctl->mv_count[zero_list] = 0;
+__device__ void phase_decide(const Ctx& c, uint32_t n_lo, uint32_t n_hi, uint64_t warp0,
+                             uint64_t nwarps) {
   for (uint64_t w = n_lo + warp0; w < n_hi; w += nwarps) decide_node(c, (uint32_t)w);
 }
 
@@ -1580,12 +1676,12 @@ __device__ __forceinline__ void place_items(const Ctx& c, uint32_t* smem, const 
   warp_place<U>(c, valid, node, ref, q);
 }
 
-// Store the batch points and the n_spill re-inserted points (from the spill
-// records), each at the next free slot of its leaf. Loops are block-uniform so
+// Store the batch points and the re-inserted points (of the spill tasks
+// [0, t_hi), still in their old chunks), each at the next free slot of its leaf. Loops are block-uniform so
 // that a block's items share their slot reservations; each lane carries
 // STORE_U items at a time so that their L2 round trips overlap.
 __device__ void phase_store(const Ctx& c, uint32_t* smem, const int4* pts, uint64_t n,
-                            unsigned long long base, uint32_t n_spill, uint64_t t0,
+                            unsigned long long base, uint32_t t_hi, uint64_t t0,
                             uint64_t nthreads) {
   constexpr int U = STORE_U;
   // block-uniform loops: item j of thread t in round b is b + j * nthreads + t
@@ -1632,17 +1728,28 @@ __device__ void phase_store(const Ctx& c, uint32_t* smem, const int4* pts, uint6
 #pragma unroll
     for (int j = 0; j < U; ++j) put_rec(c, ref[j], q[j], p[j], (uint32_t)(base + b0 + j * stride + me));
   }
-  for (uint64_t b0 = blk; b0 < n_spill; b0 += U * stride) {
+  const uint32_t parts = task_units(c);
+  const uint64_t n_re = (uint64_t)t_hi * parts * 32u;  // (lanes past a task's end idle)
+  for (uint64_t b0 = blk; b0 < n_re; b0 += U * stride) {
     bool valid[U];
     uint32_t node[U], ref[U], q[U], g[U];
     int4 r[U];
 #pragma unroll
     for (int j = 0; j < U; ++j) {
       const uint64_t e = b0 + j * stride + me;
-      valid[j] = e < n_spill;
-      node[j] = valid[j] ? c.sp_cur[e] : 0u;
-      r[j] = valid[j] ? c.sp_rec[e] : make_int4(0, 0, 0, 0);
-      g[j] = valid[j] ? c.sp_gidx[e] : 0u;
+      valid[j] = false;
+      node[j] = g[j] = 0u;
+      r[j] = make_int4(0, 0, 0, 0);
+      if (e < n_re) {
+        SpillTask tk;
+        uint32_t at;
+        valid[j] = task_point(c, (uint32_t)(e / 32u), parts, tk, at);
+        if (valid[j]) {
+          node[j] = c.sp_cur[tk.dst + at];
+          r[j] = chunk_recs(c, tk.ref)[at];
+          g[j] = chunk_aux(c, tk.ref)[at];
+        }
+      }
       if (valid[j] && node[j] >= c.max_nodes) {
         set_error(c, E_INTERNAL);
         valid[j] = false;
@@ -1709,8 +1816,7 @@ __device__ void phase_store_voxels(const Ctx& c, uint32_t* smem, uint32_t n_task
       v.w = (int32_t)rgba[j];
       put_rec(c, ref[j], q[j], v, cell[j]);
       atomicOr(grid_words(c, gref[j]) + (cell[j] >> 5), 1u << (cell[j] & 31u));
-      sl[j]->key = HASH_EMPTY;
-      sl[j]->val = HASH_EMPTY;
+      *reinterpret_cast<ulonglong2*>(sl[j]) = make_ulonglong2(HASH_EMPTY, HASH_EMPTY);
     }
   }
   const int top = pool_top > 0 ? pool_top : 0;
@@ -1735,8 +1841,9 @@ __device__ __forceinline__ uint32_t key_rate_of(unsigned long long voxels,
 // One thread: close an applied update (advance gidx, return the freed
 // chunks to the pool, fold the update into the stats, clear the per-update
 // counters).
-__device__ void phase_end(const Ctx& c, uint64_t n, uint32_t iters) {
+__device__ void phase_end(const Ctx& c, uint64_t n) {
   Ctl* t = c.ctl;
+  const uint32_t iters = t->iters ? t->iters : 1u;
   const unsigned long long nk =
       min((unsigned long long)t->nkeys, (unsigned long long)c.backlog_cap);
   t->base += n;
@@ -1758,9 +1865,10 @@ __device__ void phase_end(const Ctx& c, uint64_t n, uint32_t iters) {
   t->nkeys = 0;
   t->alloc_seq = 0;
   t->split_count = 0;
+  t->split_inner = 0;
   t->ntasks = 0;
-  t->mv_count[0] = 0;
-  t->mv_count[1] = 0;
+  t->iters = 0;
+  t->split_most = 0;
   t->bump0 = t->bump;
   t->key_rate = key_rate_of(t->st_voxels, t->st_points + t->st_spilled,
                             n + t->last_spilled);

@@ -70,9 +70,8 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
 // one per warp, reaches the control block's L2 lines.
 struct CtlView {
   unsigned long long base, bump0;
-  uint32_t n_nodes, key_rate, open, reject, split_count, ntasks, spill_count, nkeys, stop;
+  uint32_t n_nodes, key_rate, open, reject, split_count, split_inner, split_most, ntasks, spill_count, nkeys, stop;
   int pool_top;
-  uint32_t mv_count[2];
 };
 
 __device__ __forceinline__ bool grid_barrier(const Ctx& c, FusedCtl* f, CtlView* view = nullptr) {
@@ -117,12 +116,12 @@ __device__ __forceinline__ bool grid_barrier(const Ctx& c, FusedCtl* f, CtlView*
       view->n_nodes = vload(&c.ctl->n_nodes);
       view->reject = vload(&c.ctl->reject);
       view->split_count = vload(&c.ctl->split_count);
+      view->split_inner = vload(&c.ctl->split_inner);
+      view->split_most = vload(&c.ctl->split_most);
       view->ntasks = vload(&c.ctl->ntasks);
       view->spill_count = vload(&c.ctl->spill_count);
       view->nkeys = vload(&c.ctl->nkeys);
       view->pool_top = vload(&c.ctl->pool_top);
-      view->mv_count[0] = vload(&c.ctl->mv_count[0]);
-      view->mv_count[1] = vload(&c.ctl->mv_count[1]);
       view->stop = vload(&f->stop);
     }
 #endif
@@ -254,57 +253,57 @@ __global__ void __launch_bounds__(FUSED_BLOCK, PHASE_MIN_BLOCKS) k_fused(Ctx c, 
           f->rejected += 1;
         }
       } else {
-        // s: split-list range of the previous round, n: nodes it created,
-        // t_hi: spill tasks (all made by the first decide round)
-        uint32_t s_lo = 0, s_hi = 0, n_lo = 0, n_hi = nodes0, t_hi = 0, iters = 1;
+        // s_hi: splits so far, [n_lo, n_hi): nodes the last build created, t_hi:
+        // spill tasks (all made by the first decide round), lvl0: levels built
+        uint32_t s_hi = 0, n_lo = 0, n_hi = nodes0, t_hi = 0, lvl0 = 0, inner0 = 0;
         for (;;) {
-          phase_decide(c, n_lo, n_hi, iters >= 3 ? (int)((iters - 1) & 1u) : -1, warp0, nwarps);
+          phase_decide(c, n_lo, n_hi, warp0, nwarps);
           if (!grid_barrier(c, f, vw)) return;
           clk.tick(c, PH_DECIDE);
-          const uint32_t sc = SL_CV(split_count, &c.ctl->split_count);
-          const uint32_t nn = SL_CV(n_nodes, &c.ctl->n_nodes);
+          const uint32_t K = SL_CV(split_count, &c.ctl->split_count) - s_hi;
           const uint32_t nt = SL_CV(ntasks, &c.ctl->ntasks);
-          node_cache_patch(c, smem, s_hi, sc, n_hi, nn);  // this round's splits and new nodes
-          if (iters == 1) t_hi = nt;
+          const bool first = n_lo == 0u;
+          if (first) t_hi = nt;
           else if (nt != t_hi && tid == 0) set_error(c, E_INTERNAL);
-          if (sc == s_hi) break;
-          if (iters >= max_iters) {
-            if (tid == 0) set_error(c, E_ITER_CAP);
-            return;
-          }
-          s_lo = s_hi;
+          if (K == 0u) break;
+          const uint32_t d = hist_depth(c, K, bd.n + SL_CV(spill_count, &c.ctl->spill_count),
+                                        SL_CV(split_most, &c.ctl->split_most));
+          phase_hist(c, smem, node_cache_at(smem, n_hi), bd.pts, bd.n, t_hi, s_hi, K, d, first);
+          if (!grid_barrier(c, f)) return;
+          phase_build(c, s_hi, K, d, lvl0, max_iters);
+          if (!grid_barrier(c, f, vw)) return;
+          clk.tick(c, PH_ADVANCE);
+          // the entries so far: not split_count, which the next decide raises
+          // while a late block still reads its view
+          const uint32_t inner = SL_CV(split_inner, &c.ctl->split_inner);
+          const uint32_t sc = s_hi + K + (inner - inner0);
+          inner0 = inner;
+          const uint32_t nn = SL_CV(n_nodes, &c.ctl->n_nodes);
+          node_cache_patch(c, smem, s_hi, sc, n_hi, nn);
           s_hi = sc;
           n_lo = n_hi;
           n_hi = nn;
-          const int in_list = iters >= 2 ? (int)((iters - 2) & 1u) : -1;
-          const uint32_t n_in =
-              in_list >= 0 ? SL_CV(mv_count[in_list], &c.ctl->mv_count[in_list]) : 0u;
-          phase_advance(c, smem, node_cache_at(smem, nn), bd.pts, bd.n, t_hi, s_lo, s_hi, in_list,
-                        n_in, (int)((iters - 1) & 1u), warp0, nwarps);
-          ++iters;
-          if (!grid_barrier(c, f)) return;
-          clk.tick(c, PH_ADVANCE);
+          lvl0 += d;
         }
         // (the last decide round's barrier filled the view)
         const uint32_t n_spill = min(SL_CV(spill_count, &c.ctl->spill_count), c.spill_cap);
-        const uint32_t nodes1 = SL_CV(n_nodes, &c.ctl->n_nodes);
         const ClaimArgs ca{nodes0, (uint32_t)(SL_CV(bump0, &c.ctl->bump0) / REF_BYTES),
-                           SL_CV(open, &c.ctl->open), 
+                           SL_CV(open, &c.ctl->open),
                            claim_near_mask(c, bd.n + n_spill, SL_CV(key_rate, &c.ctl->key_rate))};
-        phase_claim(c, smem, bd.pts, bd.n, base, n_spill, ca, warp0, nwarps);
+        phase_claim(c, smem, node_cache_at(smem, n_hi), bd.pts, bd.n, base, t_hi, s_hi, ca, warp0,
+                    nwarps);
         if (!grid_barrier(c, f)) return;
         clk.tick(c, PH_CLAIM);
-        phase_decide(c, 0, nodes1, -1, warp0, nwarps);  // chunks for the new voxels
-        phase_store(c, smem, bd.pts, bd.n, base, n_spill, tid, nthreads);
+        phase_decide(c, 0, n_hi, warp0, nwarps);  // chunks for the new voxels
+        phase_store(c, smem, bd.pts, bd.n, base, t_hi, tid, nthreads);
         if (!grid_barrier(c, f, vw)) return;
         clk.tick(c, PH_STORE);
-        const uint32_t n_tasks = SL_CV(ntasks, &c.ctl->ntasks);
         const uint32_t n_keys = min(SL_CV(nkeys, &c.ctl->nkeys), c.backlog_cap);
-        const int pool_top = SL_CV(pool_top, &c.ctl->pool_top);
-        phase_store_voxels(c, smem, n_tasks, n_keys, pool_top, tid, nthreads);
+        phase_store_voxels(c, smem, t_hi, n_keys, SL_CV(pool_top, &c.ctl->pool_top), tid,
+                           nthreads);
         if (!grid_barrier(c, f)) return;
         clk.tick(c, PH_STORE);
-        if (tid == 0) phase_end(c, bd.n, iters);
+        if (tid == 0) phase_end(c, bd.n);
       }
     }
     if (tid == 0) {

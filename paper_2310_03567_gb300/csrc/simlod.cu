@@ -55,12 +55,18 @@ __global__ void k_init(Ctx c) {
   }
 }
 
-__global__ void k_fill_hash(HSlot* h, uint64_t n) {
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    h[i].key = HASH_EMPTY;
-    h[i].val = HASH_EMPTY;
+// Empty the claim table and the histograms: always, or when an update failed
+// half way since they were last empty (a handle that is reset without having
+// been asked for its status does not know).
+__global__ void k_clear_tables(Ctx c, int always) {
+  if (!always && vload(&c.ctl->error) == 0u) return;
+  const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+  const uint64_t nt = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t i = t0; i <= c.hash_mask; i += nt) {
+    c.hash[i].key = HASH_EMPTY;
+    c.hash[i].val = HASH_EMPTY;
   }
+  for (uint64_t i = t0; i < c.hist_words; i += nt) c.hist[i] = 0;
 }
 
 __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_count1(Ctx c, const int4* pts,
@@ -75,48 +81,109 @@ __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_count1(Ctx c, cons
 
 // Decide / allocate; after the first count round of a rejected batch (no
 // thread changes the reject flag during this kernel) undo that round instead.
-__global__ void __launch_bounds__(BLOCK) k_decide(Ctx c, uint32_t n_lo, uint32_t n_hi,
-                                                   int zero_list) {
+__global__ void __launch_bounds__(BLOCK) k_decide(Ctx c, uint32_t n_lo, uint32_t n_hi) {
   const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   const uint64_t nt = (uint64_t)gridDim.x * blockDim.x;
   if (*reinterpret_cast<volatile unsigned int*>(&c.ctl->reject)) {
     phase_rollback(c, n_hi, t0, nt);
     return;
   }
-  phase_decide(c, n_lo, n_hi, zero_list, t0 / 32, nt / 32);
+  phase_decide(c, n_lo, n_hi, t0 / 32, nt / 32);
 }
 
-__global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_advance(Ctx c, const int4* pts, uint64_t n,
-                                                     uint32_t n_nodes, uint32_t t_hi, uint32_t s_lo,
-                                                     uint32_t s_hi, int in_list, uint32_t n_in,
-                                                     int out_list) {
+// The plain form's kernels after the first decide. All are enqueued before the
+// host has seen anything of the update: what they need is in the control
+// block, and they leave at once when the batch was rejected, an error came up
+// or (hist, build, decide_new) no leaf splits. One round of them covers most
+// updates; k_claim and k_alloc_voxels also leave when a leaf still has to
+// split, and the host, which reads the control block then, enqueues another
+// round and them again. A wait for the host per round (7 per update of a
+// clustered scan) took longer than the kernels between.
+// (All threads of the block call and get one answer: another block of the
+// same kernel may set the error meanwhile.)
+__device__ __forceinline__ bool plain_stop(const Ctx& c) {
+  return __syncthreads_or(threadIdx.x == 0 &&
+                          (vload(&c.ctl->reject) != 0u || vload(&c.ctl->error) != 0u)) != 0;
+}
+
+// First split entry after round r and the inner nodes it built (after its
+// build; split_inner stays until the next one).
+__host__ __device__ __forceinline__ uint32_t round_end(const Ctl* t, uint32_t r) {
+  const volatile PlainRound& p = t->round[r];
+  return p.s_lo + p.K + (*static_cast<const volatile unsigned int*>(&t->split_inner) - p.inner);
+}
+
+__global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_hist(Ctx c, const int4* pts,
+                                                                  uint64_t n, uint32_t r) {
   extern __shared__ uint32_t smem[];
-  const uint64_t warps_per_block = blockDim.x / 32;
+  if (plain_stop(c)) return;
+  const uint32_t s_lo = r ? round_end(c.ctl, r - 1u) : 0u;
+  const uint32_t K = vload(&c.ctl->split_count) - s_lo, n_nodes = vload(&c.ctl->n_nodes);
+  const uint32_t d = hist_depth(c, K, n + vload(&c.ctl->spill_count), vload(&c.ctl->split_most));
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    const uint32_t lvl0 = r ? c.ctl->round[r - 1u].lvl0 + c.ctl->round[r - 1u].d : 0u;
+    c.ctl->round[r] = PlainRound{s_lo, K, vload(&c.ctl->split_inner), d, lvl0, n_nodes};
+  }
+  if (K == 0u) return;
   node_cache_load(c, smem, 0, n_nodes);
-  phase_advance(c, smem, node_cache_at(smem, n_nodes), pts, n, t_hi, s_lo, s_hi, in_list, n_in,
-                out_list, blockIdx.x * warps_per_block + threadIdx.x / 32,
-                (uint64_t)gridDim.x * warps_per_block);
+  phase_hist(c, smem, node_cache_at(smem, n_nodes), pts, n, vload(&c.ctl->ntasks), s_lo, K, d,
+             r == 0u);
+}
+
+__global__ void __launch_bounds__(PBLOCK) k_build(Ctx c, uint32_t r, uint32_t max_iters) {
+  if (plain_stop(c)) return;
+  const PlainRound* p = &c.ctl->round[r];
+  if (vload(&p->K)) phase_build(c, vload(&p->s_lo), vload(&p->K), vload(&p->d), vload(&p->lvl0),
+                                max_iters);
+}
+
+__global__ void __launch_bounds__(BLOCK) k_decide_new(Ctx c, uint32_t r) {
+  if (plain_stop(c) || vload(&c.ctl->round[r].K) == 0u) return;
+  phase_decide(c, vload(&c.ctl->round[r].n_lo), vload(&c.ctl->n_nodes),
+               (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) / 32,
+               (uint64_t)gridDim.x * blockDim.x / 32);
 }
 
 __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_claim(Ctx c, const int4* pts, uint64_t n,
-                                                     unsigned long long base, uint32_t n_spill,
-                                                     uint32_t nodes0) {
+                                                     unsigned long long base, uint32_t nodes0,
+                                                     uint32_t r) {
   extern __shared__ uint32_t smem[];
-  const uint64_t warps_per_block = blockDim.x / 32;
+  if (plain_stop(c) || vload(&c.ctl->split_count) != round_end(c.ctl, r)) return;
+  const uint32_t s_hi = vload(&c.ctl->split_count), t_hi = vload(&c.ctl->ntasks);
+  const uint64_t wpb = blockDim.x / 32;
+  if (s_hi == 0u && blockIdx.x * wpb * 32u >= n) return;  // nothing for this block
+  const uint32_t n_nodes = vload(&c.ctl->n_nodes);
   const ClaimArgs a{nodes0, (uint32_t)(vload(&c.ctl->bump0) / REF_BYTES), vload(&c.ctl->open),
-                    claim_near_mask(c, n + n_spill, vload(&c.ctl->key_rate))};
-  phase_claim(c, smem, pts, n, base, n_spill, a, blockIdx.x * warps_per_block + threadIdx.x / 32,
-              (uint64_t)gridDim.x * warps_per_block);
+                    claim_near_mask(c, n + vload(&c.ctl->spill_count), vload(&c.ctl->key_rate))};
+  node_cache_load(c, smem, 0, n_nodes);
+  phase_claim(c, smem, node_cache_at(smem, n_nodes), pts, n, base, t_hi, s_hi, a,
+              blockIdx.x * wpb + threadIdx.x / 32, (uint64_t)gridDim.x * wpb);
 }
 
-// The points and, their nodes' chunks being there too, the voxels.
+// Chunks for the new voxels of the inner nodes.
+__global__ void __launch_bounds__(BLOCK) k_alloc_voxels(Ctx c, uint32_t r) {
+  if (plain_stop(c) || vload(&c.ctl->split_count) != round_end(c.ctl, r)) return;
+  phase_decide(c, 0, vload(&c.ctl->n_nodes),
+               (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) / 32,
+               (uint64_t)gridDim.x * blockDim.x / 32);
+}
+
+// The points and, their nodes' chunks being there too, the voxels; the last
+// block closes the update (a launch of its own took 5 us).
 __global__ void __launch_bounds__(BLOCK) k_store(Ctx c, const int4* pts, uint64_t n,
-                                                  unsigned long long base, uint32_t n_spill,
-                                                  uint32_t n_tasks, uint32_t n_keys, int pool_top) {
+                                                  unsigned long long base, uint32_t t_hi,
+                                                  uint32_t n_keys, int pool_top) {
   const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   const uint64_t nt = (uint64_t)gridDim.x * blockDim.x;
-  phase_store(c, nullptr, pts, n, base, n_spill, t0, nt);
-  phase_store_voxels(c, nullptr, n_tasks, n_keys, pool_top, t0, nt);
+  phase_store(c, nullptr, pts, n, base, t_hi, t0, nt);
+  phase_store_voxels(c, nullptr, t_hi, n_keys, pool_top, t0, nt);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0 && atomicAdd(&c.ctl->store_blocks, 1u) + 1u == gridDim.x) {
+    __threadfence();
+    c.ctl->store_blocks = 0;
+    phase_end(c, n);
+  }
 }
 
 // Whether a restored octree's voxels nest, as those of every octree built by
@@ -130,8 +197,8 @@ __global__ void k_check_nested(Ctx c) {
   for (uint32_t id = blockIdx.x; id < n; id += gridDim.x) {
     const NodeMeta& m = c.meta[id];
     if (m.up == NONE || !ref_ok(c, m.up_grid, c.grid_bytes)) continue;
-    const uint32_t cnt = c.num[id], head = m.head, par = m.up & MV_NODE_MASK;
-    const uint32_t L = c.rlog2 - (m.up >> MV_NODE_BITS);  // the parent's log2 size
+    const uint32_t cnt = c.num[id], head = m.head, par = m.up & NODE_MASK;
+    const uint32_t L = c.rlog2 - (m.up >> NODE_BITS);  // the parent's log2 size
     const bool inner = c.child[id] != NONE;
     const uint32_t oct = id - c.child[par];
     const uint32_t* words = grid_words(c, m.up_grid);
@@ -231,8 +298,6 @@ __global__ void k_compact(Ctx c, uint32_t idle) {
   }
 }
 
-__global__ void k_end(Ctx c, uint64_t n, uint32_t iters) { phase_end(c, n, iters); }
-
 __global__ void k_end_rejected(Ctx c) { phase_end_rejected(c); }
 
 // Kernel instance 0: the k_fused of this file (the header's knobs).
@@ -309,8 +374,8 @@ static const char* const kKernelNames[SIMLOD_N_KERNELS] = {
 
 struct Layout {
   size_t ctl, fctl, batches, child, gridref, cnt, num, meta, pool, pending, alloc_refs, splits,
-      tasks, sp_cur, sp_rec, sp_gidx, b_cur, mv0, mv1, scur, vis, hash, keys, staging, data, end;
-  uint64_t hash_slots, max_chunks, max_splits, data_bytes;
+      tasks, sp_cur, b_cur, hist, hist_up, scur, vis, hash, keys, staging, data, end;
+  uint64_t hash_slots, hist_words, max_chunks, max_splits, data_bytes;
 };
 
 struct simlod {
@@ -369,12 +434,12 @@ bool valid_config(const simlod_config* c) {
   if (c->root_log2 < 1 || c->root_log2 > 31) return false;
   if (c->leaf_capacity < 1 || c->chunk_points < 1 || c->chunk_points > 65536) return false;
   if (c->grid_log2 < 1 || c->grid_log2 > 7) return false;
-  // mover-list entries name a batch point or a spill entry in 31 bits
+  // (31 bits: points of a batch and re-inserted points, told apart by the top bit)
   if (c->max_batch_points < 1 || c->max_batch_points >= (1ull << 31)) return false;
   if (c->spill_capacity >= (1ull << 31) || c->backlog_capacity < 1 ||
       c->backlog_capacity > (1ull << 31))
     return false;
-  if (c->max_nodes < 9 || c->max_nodes > (1ull << MV_NODE_BITS)) return false;
+  if (c->max_nodes < 9 || c->max_nodes > (1ull << NODE_BITS)) return false;
   if ((c->leaf_capacity + (uint64_t)c->chunk_points - 1) / c->chunk_points > (1u << 18))
     return false;  // chunk directories of at most 1 MiB
   for (int a = 0; a < 3; ++a) {
@@ -423,13 +488,17 @@ bool plan_layout(const simlod_config* c, size_t arena_bytes, Layout* L) {
   L->cnt = take(4 * N);
   L->num = take(4 * N);
   L->meta = take(sizeof(NodeMeta) * N);
-  L->splits = take(sizeof(SplitEntry) * L->max_splits);
+  L->splits = take(4 * L->max_splits);
   L->sp_cur = take(4 * S);
   L->b_cur = take(4 * B);
-  L->mv0 = take(8 * (B + S));
-  L->mv1 = take(8 * (B + S));
-  L->sp_rec = take(16 * S);
-  L->sp_gidx = take(4 * S);
+  // an update splits at most (B + S) / (T + 1) leaves, each with the 8 counts
+  // of one level; more levels where there is room for a count per moving point
+  const uint64_t leaves = std::min<uint64_t>(L->max_splits, (B + S) / (c->leaf_capacity + 1ull) + 1);
+  L->hist_words = std::max<uint64_t>(8 * leaves, std::min<uint64_t>(std::max<uint64_t>(B + S, 32768), 32u << 20));
+  L->hist_words = align_up(L->hist_words, 64);
+  L->hist = take(4 * L->hist_words);
+  // sums and list: 2 (8^d - 1) / 7 words for 8^d counts
+  L->hist_up = take(8 * (L->hist_words / 7 + leaves));
   L->scur = take(4 * N);
   L->vis = take(4 * N);
   L->hash = take(sizeof(HSlot) * L->hash_slots);
@@ -470,14 +539,13 @@ void make_ctx(simlod_t* h) {
   c.pool = reinterpret_cast<uint32_t*>(a + L.pool);
   c.pending = reinterpret_cast<uint32_t*>(a + L.pending);
   c.alloc_refs = reinterpret_cast<uint32_t*>(a + L.alloc_refs);
-  c.splits = reinterpret_cast<SplitEntry*>(a + L.splits);
+  c.splits = reinterpret_cast<uint32_t*>(a + L.splits);
   c.tasks = reinterpret_cast<SpillTask*>(a + L.tasks);
   c.sp_cur = reinterpret_cast<uint32_t*>(a + L.sp_cur);
   c.b_cur = reinterpret_cast<uint32_t*>(a + L.b_cur);
-  c.mv[0] = reinterpret_cast<uint2*>(a + L.mv0);
-  c.mv[1] = reinterpret_cast<uint2*>(a + L.mv1);
-  c.sp_rec = reinterpret_cast<int4*>(a + L.sp_rec);
-  c.sp_gidx = reinterpret_cast<uint32_t*>(a + L.sp_gidx);
+  c.hist = reinterpret_cast<uint32_t*>(a + L.hist);
+  c.hist_up = reinterpret_cast<uint32_t*>(a + L.hist_up);
+  c.hist_words = L.hist_words;
   c.scur = reinterpret_cast<uint32_t*>(a + L.scur);
   c.hash = reinterpret_cast<HSlot*>(a + L.hash);
   c.keys = reinterpret_cast<uint32_t*>(a + L.keys);
@@ -502,7 +570,6 @@ void make_ctx(simlod_t* h) {
   c.backlog_cap = (uint32_t)g.backlog_capacity;
   c.max_splits = (uint32_t)L.max_splits;
   c.max_batch = g.max_batch_points;
-  c.mv_cap = g.max_batch_points + g.spill_capacity;
   c.bar_ns = FUSED_BARRIER_NS;
   c.ready_ns = FUSED_READY_NS;
   c.progress = nullptr;  // set per persistent launch (launch_fused)
@@ -600,84 +667,52 @@ int insert_device(simlod_t* h, const int4* pts, uint64_t n, cudaStream_t s) {
   const unsigned long long base = h->base;
   const uint32_t nodes0 = h->n_nodes;
   const unsigned gp = std::max(1u, std::min<unsigned>(grid_for(h, n, PBLOCK), (unsigned)PHASE_MIN_BLOCKS * h->sm_count));
+  const unsigned full = (unsigned)PHASE_MIN_BLOCKS * h->sm_count;
+  const uint32_t max_iters = h->cfg.max_expand_iters ? h->cfg.max_expand_iters
+                                                      : h->cfg.root_log2 + 1;
   int rc;
   rc = launch(h, K_COUNT, s, [&] {
     k_count1<<<gp, PBLOCK, PHASE_SMEM_BYTES, s>>>(c, pts, n, nodes0);
   });
   if (rc) return poison(h, rc);
   rc = launch(h, K_DECIDE, s, [&] {
-    k_decide<<<grid_for(h, 32ull * nodes0, BLOCK), BLOCK, 0, s>>>(c, 0, nodes0, -1);
+    k_decide<<<grid_for(h, 32ull * nodes0, BLOCK), BLOCK, 0, s>>>(c, 0, nodes0);
   });
   if (rc) return poison(h, rc);
-  if ((rc = read_ctl(h, s))) return poison(h, rc);
   const Ctl& t = *h->ctl_host;
-  if (t.error) return poison(h, error_from_bits(t.error));
-  if (t.reject) {
-    rc = launch(h, K_END, s, [&] { k_end_rejected<<<1, 1, 0, s>>>(c); });
-    if (rc) return poison(h, rc);
-    return SIMLOD_ERR_OUT_OF_BOUNDS;
-  }
-  const uint32_t max_iters = h->cfg.max_expand_iters ? h->cfg.max_expand_iters
-                                                      : h->cfg.root_log2 + 1;
-  // s: split-list range of the previous round, n: nodes it created,
-  // t_hi: spill tasks (all made by the first decide round)
-  uint32_t s_lo = 0, s_hi = t.split_count, n_lo = nodes0, n_hi = t.n_nodes,
-           t_hi = t.ntasks, iters = 1;
-  while (s_hi > s_lo) {
-    if (iters >= max_iters) return poison(h, SIMLOD_ERR_ITER_CAP);
-    const int in_list = iters >= 2 ? (int)((iters - 2) & 1u) : -1;
-    const int out_list = (int)((iters - 1) & 1u);
-    const uint32_t n_in = in_list >= 0 ? h->ctl_host->mv_count[in_list] : 0u;
-    const uint64_t units = (in_list < 0 ? (n + 31) / 32 + (uint64_t)t_hi * ((c.C + 31) / 32)
-                                        : ((uint64_t)n_in + 31) / 32) +
-                           (uint64_t)(s_hi - s_lo) * 64;
-    const unsigned ga =
-        std::max(1u, std::min<unsigned>(grid_for(h, units * 32, PBLOCK), (unsigned)PHASE_MIN_BLOCKS * h->sm_count));
-    const uint32_t nn = n_hi;
+  for (uint32_t r = 0;; ++r) {
     rc = launch(h, K_ADVANCE, s, [&] {
-      k_advance<<<ga, PBLOCK, PHASE_SMEM_BYTES, s>>>(c, pts, n, nn, t_hi, s_lo, s_hi, in_list,
-                                                     n_in, out_list);
+      k_hist<<<full, PBLOCK, PHASE_SMEM_BYTES, s>>>(c, pts, n, r);
+      k_build<<<full, PBLOCK, 0, s>>>(c, r, max_iters);
     });
     if (rc) return poison(h, rc);
-    ++iters;
-    const uint64_t cand = n_hi - n_lo;
-    const int zero_list = iters >= 3 ? (int)((iters - 1) & 1u) : -1;
     rc = launch(h, K_DECIDE, s, [&] {
-      k_decide<<<grid_for(h, 32 * cand, BLOCK), BLOCK, 0, s>>>(c, n_lo, n_hi, zero_list);
+      k_decide_new<<<full * 2, BLOCK, 0, s>>>(c, r);
     });
+    if (rc) return poison(h, rc);
+    rc = launch(h, K_CLAIM, s, [&] {
+      k_claim<<<full, PBLOCK, PHASE_SMEM_BYTES, s>>>(c, pts, n, base, nodes0, r);
+    });
+    if (rc) return poison(h, rc);
+    rc = launch(h, K_DECIDE, s, [&] { k_alloc_voxels<<<full * 2, BLOCK, 0, s>>>(c, r); });
     if (rc) return poison(h, rc);
     if ((rc = read_ctl(h, s))) return poison(h, rc);
-    if (h->ctl_host->error) return poison(h, error_from_bits(h->ctl_host->error));
-    if (h->ctl_host->ntasks != t_hi) return poison(h, SIMLOD_ERR_CUDA);
-    s_lo = s_hi;
-    s_hi = h->ctl_host->split_count;
-    n_lo = n_hi;
-    n_hi = h->ctl_host->n_nodes;
+    if (t.error) return poison(h, error_from_bits(t.error));
+    if (t.reject) {
+      rc = launch(h, K_END, s, [&] { k_end_rejected<<<1, 1, 0, s>>>(c); });
+      if (rc) return poison(h, rc);
+      return SIMLOD_ERR_OUT_OF_BOUNDS;
+    }
+    if (t.split_count == round_end(&t, r)) break;
+    if (r + 1u >= MAX_ROUNDS) return poison(h, SIMLOD_ERR_CUDA);
   }
-  const uint32_t n_spill = std::min<uint32_t>(h->ctl_host->spill_count, c.spill_cap);
-  const uint32_t nodes1 = h->ctl_host->n_nodes;
-  rc = launch(h, K_CLAIM, s, [&] {
-    k_claim<<<gp, PBLOCK, PHASE_SMEM_BYTES, s>>>(c, pts, n, base, n_spill, nodes0);
-  });
-  if (rc) return poison(h, rc);
-  // chunks for the new voxels of the inner nodes
-  rc = launch(h, K_DECIDE, s, [&] {
-    k_decide<<<grid_for(h, 32ull * nodes1, BLOCK), BLOCK, 0, s>>>(c, 0, nodes1, -1);
-  });
-  if (rc) return poison(h, rc);
-  if ((rc = read_ctl(h, s))) return poison(h, rc);
-  if (h->ctl_host->error) return poison(h, error_from_bits(h->ctl_host->error));
-  const uint32_t n_tasks = h->ctl_host->ntasks;
-  const uint32_t n_keys = std::min<uint32_t>(h->ctl_host->nkeys, c.backlog_cap);
-  const int pool_top = h->ctl_host->pool_top;
-  const uint64_t work =
-      std::max<uint64_t>(std::max<uint64_t>(std::max<uint64_t>(n, n_spill), n_tasks), n_keys);
+  const uint32_t t_hi = t.ntasks;
+  const uint32_t n_keys = std::min<uint32_t>(t.nkeys, c.backlog_cap);
+  const int pool_top = t.pool_top;
+  const uint64_t work = std::max<uint64_t>(std::max<uint64_t>(n, (uint64_t)t_hi * c.C), n_keys);
   rc = launch(h, K_STORE, s, [&] {
-    k_store<<<grid_for(h, work, BLOCK), BLOCK, 0, s>>>(c, pts, n, base, n_spill, n_tasks,
-                                                      n_keys, pool_top);
+    k_store<<<grid_for(h, work, BLOCK), BLOCK, 0, s>>>(c, pts, n, base, t_hi, n_keys, pool_top);
   });
-  if (rc) return poison(h, rc);
-  rc = launch(h, K_END, s, [&] { k_end<<<1, 1, 0, s>>>(c, n, iters); });
   if (rc) return poison(h, rc);
   h->base += n;
   h->n_nodes = h->ctl_host->n_nodes;
@@ -745,10 +780,8 @@ int finish_fused(simlod_t* h, uint32_t* consumed) {
 
 int init_octree(simlod_t* h, cudaStream_t s, bool clear_hash, bool wait) {
   const Ctx& c = h->ctx;
-  if (clear_hash) {
-    k_fill_hash<<<grid_for(h, h->lay.hash_slots, BLOCK), BLOCK, 0, s>>>(c.hash, h->lay.hash_slots);
-    if (cudaGetLastError() != cudaSuccess) return SIMLOD_ERR_CUDA;
-  }
+  k_clear_tables<<<(unsigned)h->sm_count * 8, BLOCK, 0, s>>>(c, clear_hash ? 1 : 0);
+  if (cudaGetLastError() != cudaSuccess) return SIMLOD_ERR_CUDA;
   k_init<<<1, 1, 0, s>>>(c);
   if (cudaGetLastError() != cudaSuccess) return SIMLOD_ERR_CUDA;
   if (wait && cudaStreamSynchronize(s) != cudaSuccess) return SIMLOD_ERR_CUDA;
@@ -819,7 +852,7 @@ SIMLOD_API int simlod_create(const simlod_config* cfg, void* d_arena, size_t are
   memset(h->ctl_host, 0, sizeof(Ctl));
   if (cudaFuncSetAttribute(k_count1, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            PHASE_SMEM_BYTES) != cudaSuccess ||
-      cudaFuncSetAttribute(k_advance, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      cudaFuncSetAttribute(k_hist, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            PHASE_SMEM_BYTES) != cudaSuccess ||
       cudaFuncSetAttribute(k_claim, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            PHASE_SMEM_BYTES) != cudaSuccess ||
@@ -833,7 +866,7 @@ SIMLOD_API int simlod_create(const simlod_config* cfg, void* d_arena, size_t are
   // shared-memory share of the unified L1/shared storage, in percent
   cudaFuncSetAttribute(k_fused, cudaFuncAttributePreferredSharedMemoryCarveout, SL_CARVEOUT);
   cudaFuncSetAttribute(k_count1, cudaFuncAttributePreferredSharedMemoryCarveout, SL_CARVEOUT);
-  cudaFuncSetAttribute(k_advance, cudaFuncAttributePreferredSharedMemoryCarveout, SL_CARVEOUT);
+  cudaFuncSetAttribute(k_hist, cudaFuncAttributePreferredSharedMemoryCarveout, SL_CARVEOUT);
   cudaGetLastError();
 #endif
   int coop = 0, bpsm = 0;
@@ -1374,7 +1407,7 @@ SIMLOD_API int simlod_restore(simlod_t* h, const simlod_snapshot_t* snap, void* 
       const int64_t c = find(Key{pk.level + 1, 2 * pk.ix + (o & 1), 2 * pk.iy + ((o >> 1) & 1),
                                  2 * pk.iz + ((o >> 2) & 1)});
       if (c < 0 || rec_of.size() >= n) return SIMLOD_ERR_INVALID_ARG;
-      up[rec_of.size()] = (uint32_t)q | ((uint32_t)pk.level << MV_NODE_BITS);
+      up[rec_of.size()] = (uint32_t)q | ((uint32_t)pk.level << NODE_BITS);
       rec_of.push_back((uint32_t)c);
     }
   }
@@ -1410,7 +1443,7 @@ SIMLOD_API int simlod_restore(simlod_t* h, const simlod_snapshot_t* snap, void* 
     NodeMeta m;
     memset(&m, 0, sizeof(m));
     m.up = up[id];
-    m.up_grid = id ? gridref[up[id] & MV_NODE_MASK] : NONE;
+    m.up_grid = id ? gridref[up[id] & NODE_MASK] : NONE;
     for (int a = 0; a < 3; ++a) m.min[a] = rec.min[a];
     m.level = rec.level;
     m.st_tail = NONE;
