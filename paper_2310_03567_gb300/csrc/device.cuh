@@ -158,7 +158,7 @@ enum : uint32_t {
 struct PlainRound {
   uint32_t s_lo, K, inner, d, lvl0, n_lo;
 };
-constexpr uint32_t MAX_ROUNDS = 32;  // a round builds at least one of 31 levels
+constexpr uint32_t MAX_ROUNDS = 33;  // from 1; a round builds at least one of 31 levels
 
 struct Ctl {
   unsigned long long base;                  // gidx of the next accepted point

@@ -93,12 +93,11 @@ __global__ void __launch_bounds__(BLOCK) k_decide(Ctx c, uint32_t n_lo, uint32_t
 
 // The plain form's kernels after the first decide. All are enqueued before the
 // host has seen anything of the update: what they need is in the control
-// block, and they leave at once when the batch was rejected, an error came up
-// or (hist, build, decide_new) no leaf splits. One round of them covers most
-// updates; k_claim and k_alloc_voxels also leave when a leaf still has to
-// split, and the host, which reads the control block then, enqueues another
-// round and them again. A wait for the host per round (7 per update of a
-// clustered scan) took longer than the kernels between.
+// block, and they leave at once when the batch was rejected or an error came
+// up. hist, build and decide_new leave when no leaf splits, claim and
+// alloc_voxels when one still has to: the host, which reads the control block
+// then, enqueues another round and them again. A wait for the host per round
+// (7 per update of a clustered scan) took longer than the kernels between.
 // (All threads of the block call and get one answer: another block of the
 // same kernel may set the error meanwhile.)
 __device__ __forceinline__ bool plain_stop(const Ctx& c) {
@@ -106,9 +105,10 @@ __device__ __forceinline__ bool plain_stop(const Ctx& c) {
                           (vload(&c.ctl->reject) != 0u || vload(&c.ctl->error) != 0u)) != 0;
 }
 
-// First split entry after round r and the inner nodes it built (after its
-// build; split_inner stays until the next one).
+// First split entry after round r (from 1) and the inner nodes it built (after
+// its build; split_inner stays until the next one).
 __host__ __device__ __forceinline__ uint32_t round_end(const Ctl* t, uint32_t r) {
+  if (r == 0u) return 0u;
   const volatile PlainRound& p = t->round[r];
   return p.s_lo + p.K + (*static_cast<const volatile unsigned int*>(&t->split_inner) - p.inner);
 }
@@ -117,17 +117,17 @@ __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_hist(Ctx c, const 
                                                                   uint64_t n, uint32_t r) {
   extern __shared__ uint32_t smem[];
   if (plain_stop(c)) return;
-  const uint32_t s_lo = r ? round_end(c.ctl, r - 1u) : 0u;
+  const uint32_t s_lo = round_end(c.ctl, r - 1u);
   const uint32_t K = vload(&c.ctl->split_count) - s_lo, n_nodes = vload(&c.ctl->n_nodes);
   const uint32_t d = hist_depth(c, K, n + vload(&c.ctl->spill_count), vload(&c.ctl->split_most));
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    const uint32_t lvl0 = r ? c.ctl->round[r - 1u].lvl0 + c.ctl->round[r - 1u].d : 0u;
+    const uint32_t lvl0 = r > 1u ? c.ctl->round[r - 1u].lvl0 + c.ctl->round[r - 1u].d : 0u;
     c.ctl->round[r] = PlainRound{s_lo, K, vload(&c.ctl->split_inner), d, lvl0, n_nodes};
   }
   if (K == 0u) return;
   node_cache_load(c, smem, 0, n_nodes);
   phase_hist(c, smem, node_cache_at(smem, n_nodes), pts, n, vload(&c.ctl->ntasks), s_lo, K, d,
-             r == 0u);
+             r == 1u);
 }
 
 __global__ void __launch_bounds__(PBLOCK) k_build(Ctx c, uint32_t r, uint32_t max_iters) {
@@ -394,6 +394,7 @@ struct simlod {
   int fused_grid;           // blocks of k_fused launches
   int fused_max_per_sm;     // co-resident k_fused blocks per SM
   sl_variant_info var[SL_N_VARIANTS];  // kernel instances of the batched form
+  bool plain_split;         // the last plain update split leaves
   bool mirror_stale;        // a fused launch ran since the last control-block read
   unsigned long long rejected_async_seen;  // fused-launch rejections already reported
   BatchDesc* desc_host;     // pinned staging of the batch table
@@ -680,21 +681,25 @@ int insert_device(simlod_t* h, const int4* pts, uint64_t n, cudaStream_t s) {
   });
   if (rc) return poison(h, rc);
   const Ctl& t = *h->ctl_host;
-  for (uint32_t r = 0;; ++r) {
-    rc = launch(h, K_ADVANCE, s, [&] {
-      k_hist<<<full, PBLOCK, PHASE_SMEM_BYTES, s>>>(c, pts, n, r);
-      k_build<<<full, PBLOCK, 0, s>>>(c, r, max_iters);
-    });
-    if (rc) return poison(h, rc);
-    rc = launch(h, K_DECIDE, s, [&] {
-      k_decide_new<<<full * 2, BLOCK, 0, s>>>(c, r);
-    });
-    if (rc) return poison(h, rc);
+  // an update after one that split leaves begins with a round of the expansion
+  // at once; else the first claim finds out whether one is needed
+  for (uint32_t r = h->plain_split ? 1u : 0u;; ++r) {
+    if (r) {
+      rc = launch(h, K_ADVANCE, s, [&] {
+        k_hist<<<full, PBLOCK, PHASE_SMEM_BYTES, s>>>(c, pts, n, r);
+        k_build<<<full, PBLOCK, 0, s>>>(c, r, max_iters);
+      });
+      if (rc) return poison(h, rc);
+      rc = launch(h, K_DECIDE, s, [&] {
+        k_decide_new<<<full, BLOCK, 0, s>>>(c, r);
+      });
+      if (rc) return poison(h, rc);
+    }
     rc = launch(h, K_CLAIM, s, [&] {
-      k_claim<<<full, PBLOCK, PHASE_SMEM_BYTES, s>>>(c, pts, n, base, nodes0, r);
+      k_claim<<<r ? full : gp, PBLOCK, PHASE_SMEM_BYTES, s>>>(c, pts, n, base, nodes0, r);
     });
     if (rc) return poison(h, rc);
-    rc = launch(h, K_DECIDE, s, [&] { k_alloc_voxels<<<full * 2, BLOCK, 0, s>>>(c, r); });
+    rc = launch(h, K_DECIDE, s, [&] { k_alloc_voxels<<<full, BLOCK, 0, s>>>(c, r); });
     if (rc) return poison(h, rc);
     if ((rc = read_ctl(h, s))) return poison(h, rc);
     if (t.error) return poison(h, error_from_bits(t.error));
@@ -706,6 +711,7 @@ int insert_device(simlod_t* h, const int4* pts, uint64_t n, cudaStream_t s) {
     if (t.split_count == round_end(&t, r)) break;
     if (r + 1u >= MAX_ROUNDS) return poison(h, SIMLOD_ERR_CUDA);
   }
+  h->plain_split = t.split_count != 0u;
   const uint32_t t_hi = t.ntasks;
   const uint32_t n_keys = std::min<uint32_t>(t.nkeys, c.backlog_cap);
   const int pool_top = t.pool_top;
