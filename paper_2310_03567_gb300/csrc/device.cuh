@@ -194,6 +194,8 @@ struct Ctl {
   unsigned long long st_decompacted;     // arrays turned back into chunk lists by an insert
   unsigned long long compact_now;        // nodes that are arrays now
   unsigned long long compact_chunks_now; // chunks those arrays stand in for
+  unsigned long long compact_need;       // bytes the candidates of a compaction need
+  unsigned long long compact_from;       // the bump pointer before it
   unsigned int store_blocks;             // plain form: blocks that finished the store
   PlainRound round[MAX_ROUNDS];
 };

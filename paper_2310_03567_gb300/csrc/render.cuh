@@ -146,8 +146,10 @@ __device__ __forceinline__ void splat(const View& v, int4 r, unsigned long long*
 
 // A piece of a drawn node: records [first, first + n) of the chunk or array
 // at ref. At most C records, so that a node's records spread over many warps.
+// (Compaction: n records of the chunk at ref that go to records first, ... of
+// the array at arr.)
 struct DrawUnit {
-  uint32_t ref, first, n, pad;
+  uint32_t ref, first, n, arr;
 };
 static_assert(sizeof(DrawUnit) == sizeof(SpillTask), "draw units use the spill-task region");
 
@@ -183,18 +185,68 @@ __device__ __forceinline__ void put_unit(const Ctx& c, const View& v, DrawUnit* 
     w.ref = __shfl_sync(FULL_MASK, u.ref, l);
     w.first = __shfl_sync(FULL_MASK, u.first, l);
     w.n = __shfl_sync(FULL_MASK, u.n, l);
-    w.pad = 0;
+    w.arr = 0;
     draw_records(c, v, w, 0, w.n, fb);
   }
 }
 
+// The chunks of one node, in list order: all 32 lanes call, and so does f(on, j,
+// ref) for 32 chunks at a time (lane with `on`: chunk j is at ref). A leaf's
+// chunks are in its directory (dir != nullptr). An inner node's chunk list has
+// to be walked, one memory round trip per link; the chunks of one allocation
+// lie one after another in the data region, so the warp reads the next links
+// of 32 such successors at once and keeps as many as the list confirms (a link
+// that points elsewhere ends the run: the walk goes on from there). Returns how
+// many chunks it found; fewer than nch when the list is broken (an error).
+template <typename F>
+__device__ __forceinline__ uint32_t walk_chunks(const Ctx& c, uint32_t head, uint32_t nch,
+                                                const uint32_t* dir, F&& f) {
+  const uint32_t lane = lane_id();
+  if (dir) {
+    for (uint32_t j0 = 0; j0 < nch; j0 += 32u) {
+      const bool in = j0 + lane < nch;
+      const uint32_t ref = in ? dir[j0 + lane] : NONE;
+      const bool ok = in && ref_ok(c, ref, c.chunk_bytes);
+      if (in && !ok) set_error(c, E_INTERNAL);
+      f(ok, j0 + lane, ref);
+      const unsigned bad = __ballot_sync(FULL_MASK, in && !ok);
+      if (bad) return j0 + (uint32_t)__ffs(bad) - 1u;
+    }
+    return nch;
+  }
+  uint32_t ref = head, j0 = 0;
+  while (j0 < nch) {
+    const uint32_t mine = ref + lane * c.chunk_units;
+    const bool in = j0 + lane < nch && ref != NONE && ref_ok(c, mine, c.chunk_bytes);
+    const uint32_t nxt = in ? *chunk_next(c, mine) : NONE;
+    // the run: lanes whose predecessors' links all lead to the next lane
+    const unsigned brk = __ballot_sync(FULL_MASK, !in || nxt != mine + c.chunk_units);
+    const uint32_t run = brk ? (uint32_t)__ffs(brk) : 32u;  // lanes before run are in the list
+    const bool ok = __shfl_sync(FULL_MASK, in ? 1 : 0, (int)run - 1) != 0;
+    f(lane < run && in, j0 + lane, mine);
+    if (lane < run && j0 + lane < nch && !in) set_error(c, E_INTERNAL);
+    if (!ok) return min(j0 + run - 1u, nch);
+    j0 += run;
+    ref = __shfl_sync(FULL_MASK, nxt, (int)run - 1);
+  }
+  return nch;
+}
+
+// Directory of a leaf whose chunks are all in it, else nullptr.
+__device__ __forceinline__ const uint32_t* leaf_dir(const Ctx& c, uint32_t id, const NodeMeta& m) {
+  return c.child[id] == NONE && m.n_chunks <= c.dir_cap && ref_ok(c, m.dir, c.dir_bytes)
+             ? dir_entries(c, m.dir)
+             : nullptr;
+}
+
+// Records of chunk j of a node with n records.
+__device__ __forceinline__ uint32_t chunk_fill(const Ctx& c, uint32_t j, uint32_t n) {
+  const unsigned long long at = (unsigned long long)j * c.C;
+  return at < n ? (uint32_t)min((unsigned long long)c.C, n - at) : 0u;
+}
+
 // One warp per drawn node: cut its records into draw units of one chunk (or C
-// records of a compacted node's array). A leaf's chunks are in its directory.
-// An inner node's chunk list has to be walked, one memory round trip per
-// link; the chunks of one allocation lie one after another in the data
-// region, so the warp reads the next links of 32 such successors at once and
-// keeps as many as the list confirms (a link that points elsewhere ends the
-// run: the walk goes on from there).
+// records of a compacted node's array).
 __global__ void k_render_units(Ctx c, View v, const uint32_t* vis, DrawUnit* units,
                                unsigned long long* fb) {
   const uint32_t nv = min(vload(&c.ctl->vis_count), c.max_nodes);
@@ -206,7 +258,7 @@ __global__ void k_render_units(Ctx c, View v, const uint32_t* vis, DrawUnit* uni
     const uint32_t id = vis[k];
     const uint32_t n = c.num[id];
     const NodeMeta& m = c.meta[id];
-    const uint32_t head = m.head, compact = m.compact, mdir = m.dir;
+    const uint32_t head = m.head, compact = m.compact;
     const uint32_t nch = compact ? (uint32_t)(((unsigned long long)n + c.C - 1) / c.C)
                                  : m.n_chunks;
     samples += n;
@@ -214,55 +266,23 @@ __global__ void k_render_units(Ctx c, View v, const uint32_t* vis, DrawUnit* uni
     uint32_t u0 = 0;
     if (lane == 0) u0 = atomicAdd(&c.ctl->draw_units, nch);
     u0 = __shfl_sync(FULL_MASK, u0, 0);
-    auto records_of = [&](uint32_t j) -> uint32_t {  // records of the node's chunk j
-      const unsigned long long at = (unsigned long long)j * c.C;
-      return at < n ? (uint32_t)min((unsigned long long)c.C, n - at) : 0u;
-    };
-    const bool by_dir = !compact && c.child[id] == NONE && nch <= c.dir_cap &&
-                        ref_ok(c, mdir, c.dir_bytes);
-    if (compact || by_dir) {
-      const bool arr_ok = !compact || array_ok(c, head, n);
-      if (!arr_ok && lane == 0) set_error(c, E_INTERNAL);
-      const uint32_t* dir = by_dir ? dir_entries(c, mdir) : nullptr;
-      for (uint32_t j0 = 0; j0 < nch; j0 += 32u) {
-        const uint32_t j = j0 + lane;
-        const bool in = j < nch;
-        DrawUnit u{0, 0, 0, 0};
-        if (in && arr_ok) {
-          u.ref = compact ? head : dir[j];
-          u.first = compact ? j * c.C : 0u;
-          u.n = records_of(j);
-          if (!compact && !ref_ok(c, u.ref, c.chunk_bytes)) {
-            set_error(c, E_INTERNAL);
-            u = DrawUnit{0, 0, 0, 0};
-          }
-        }
-        put_unit(c, v, units, in, (uint64_t)u0 + j, u, fb);
+    uint32_t got = 0;
+    if (!compact) {
+      got = walk_chunks(c, head, nch, leaf_dir(c, id, m), [&](bool on, uint32_t j, uint32_t ref) {
+        put_unit(c, v, units, on, (uint64_t)u0 + j, DrawUnit{ref, 0, chunk_fill(c, j, n), 0}, fb);
+      });
+    } else if (array_ok(c, head, n)) {
+      for (; got < nch; got += 32u) {
+        const uint32_t j = got + lane;
+        put_unit(c, v, units, j < nch, (uint64_t)u0 + j,
+                 DrawUnit{head, j * c.C, chunk_fill(c, j, n), 0}, fb);
       }
-      continue;
+    } else if (lane == 0) {
+      set_error(c, E_INTERNAL);
     }
-    uint32_t ref = head, j0 = 0;
-    while (j0 < nch) {
-      const uint32_t mine = ref + lane * c.chunk_units;
-      const bool in = j0 + lane < nch && ref != NONE && ref_ok(c, mine, c.chunk_bytes);
-      const uint32_t nxt = in ? *chunk_next(c, mine) : NONE;
-      // the run: lanes whose predecessors' links all lead to the next lane
-      const unsigned brk = __ballot_sync(FULL_MASK, !in || nxt != mine + c.chunk_units);
-      const uint32_t run = brk ? (uint32_t)__ffs(brk) : 32u;  // lanes before run are in the list
-      const bool ok = __shfl_sync(FULL_MASK, in ? 1 : 0, (int)run - 1) != 0;
-      const bool on = lane < run && j0 + lane < nch;
-      DrawUnit u{mine, 0, records_of(j0 + lane), 0};
-      if (!in) u = DrawUnit{0, 0, 0, 0};
-      if (on && !in) set_error(c, E_INTERNAL);
-      put_unit(c, v, units, on, (uint64_t)u0 + j0 + lane, u, fb);
-      j0 += run;
-      if (!ok) {  // a broken list: the rest of the reserved units draw nothing
-        for (uint32_t j = j0 + lane; j < nch; j += 32u)
-          if ((uint64_t)u0 + j < c.max_chunks) units[(uint64_t)u0 + j] = DrawUnit{0, 0, 0, 0};
-        break;
-      }
-      ref = __shfl_sync(FULL_MASK, nxt, (int)run - 1);
-    }
+    // a broken list: the rest of the reserved units draw nothing
+    for (uint32_t j = got + lane; j < nch; j += 32u)
+      if ((uint64_t)u0 + j < c.max_chunks) units[(uint64_t)u0 + j] = DrawUnit{0, 0, 0, 0};
   }
   if (lane == 0 && samples) atomicAdd(&c.ctl->render_samples, samples);
 }

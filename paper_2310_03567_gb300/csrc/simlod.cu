@@ -223,37 +223,71 @@ __global__ void k_check_nested(Ctx c) {
 }
 
 // Compaction of cold nodes (the paper's closing direction: nodes that are no
-// longer modified become non-growable arrays). One warp per node: a node with
-// records in two or more chunks that has received none in the last `idle`
-// updates gets one contiguous array (records, then aux words) from the data
-// region, its records are copied over in order, and its chunks go back to
-// the pool. Space the data region cannot give is skipped without an error.
-__global__ void k_compact(Ctx c, uint32_t idle) {
+// longer modified become non-growable arrays). A node with records in two or
+// more chunks that has received none in the last `idle` updates gets one
+// contiguous array (records, then aux words) from the data region, its records
+// are copied over in order, and its chunks go back to the pool. Space the data
+// region cannot give is skipped without an error.
+// Three kernels: the bytes that all candidates need together; one warp per
+// candidate takes its array and cuts its chunk list into copies of one chunk;
+// the copies, several warps to a chunk. (One warp per node did all of it
+// before: 3.4 ms for the 12M-point building scan, of which the longest nodes'
+// copies were most, and a compare-and-swap loop on the bump pointer per node,
+// which is only needed now when the region cannot hold all of them.)
+__device__ __forceinline__ bool compact_candidate(const Ctx& c, uint32_t id, uint32_t idle,
+                                                  unsigned long long now) {
+  const NodeMeta& m = c.meta[id];
+  return !m.compact && c.num[id] != 0u && m.n_chunks >= 2u &&
+         (unsigned long long)m.touched + idle <= now;
+}
+
+__global__ void k_compact_need(Ctx c, uint32_t idle) {
+  const uint32_t n_nodes = min(vload(&c.ctl->n_nodes), c.max_nodes);
+  const unsigned long long now = vload(&c.ctl->st_batches);
+  unsigned long long bytes = 0;
+  for (uint64_t id = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; id < n_nodes;
+       id += (uint64_t)gridDim.x * blockDim.x)
+    if (compact_candidate(c, (uint32_t)id, idle, now)) bytes += array_bytes(c.num[id]);
+  for (int d = 16; d; d >>= 1) bytes += __shfl_down_sync(FULL_MASK, bytes, d);
+  if ((threadIdx.x & 31u) == 0u && bytes) atomicAdd(&c.ctl->compact_need, bytes);
+  if (blockIdx.x == 0 && threadIdx.x == 0) c.ctl->compact_from = vload(&c.ctl->bump);
+}
+
+__global__ void k_compact_plan(Ctx c, uint32_t idle, DrawUnit* units) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
   const uint64_t nwarps = (uint64_t)gridDim.x * blockDim.x / 32;
   const uint32_t n_nodes = min(vload(&c.ctl->n_nodes), c.max_nodes);
   const unsigned long long now = vload(&c.ctl->st_batches);
+  const bool all_fit = vload(&c.ctl->compact_need) <= c.data_bytes - c.ctl->compact_from;
   for (uint64_t id = warp; id < n_nodes; id += nwarps) {
+    if (!compact_candidate(c, (uint32_t)id, idle, now)) continue;
     NodeMeta& m = c.meta[id];
-    const uint32_t n = c.num[id], nch = m.n_chunks;
-    if (m.compact || n == 0 || nch < 2 || (unsigned long long)m.touched + idle > now) continue;
+    const uint32_t n = c.num[id], nch = m.n_chunks, head = m.head;
+    const uint32_t* dir = leaf_dir(c, (uint32_t)id, m);
     const unsigned long long bytes = array_bytes(n);
     unsigned long long off = ~0ull;
     int p0 = 0;
+    uint32_t u0 = 0;
     if (lane == 0) {
-      unsigned long long b = vload(&c.ctl->bump);
-      while (b + bytes <= c.data_bytes) {
-        const unsigned long long seen = atomicCAS(&c.ctl->bump, b, b + bytes);
-        if (seen == b) {
-          off = b;
-          break;
+      if (all_fit) {
+        off = atomicAdd(&c.ctl->bump, bytes);
+      } else {
+        unsigned long long b = vload(&c.ctl->bump);
+        while (b + bytes <= c.data_bytes) {
+          const unsigned long long seen = atomicCAS(&c.ctl->bump, b, b + bytes);
+          if (seen == b) {
+            off = b;
+            break;
+          }
+          b = seen;
         }
-        b = seen;
       }
       if (off != ~0ull) {
         p0 = atomicAdd(&c.ctl->pool_top, (int)nch);
-        if (p0 < 0 || (unsigned long long)p0 + nch > c.max_chunks) {
+        u0 = atomicAdd(&c.ctl->draw_units, nch);
+        if (p0 < 0 || (unsigned long long)p0 + nch > c.max_chunks ||
+            (unsigned long long)u0 + nch > c.max_chunks) {
           set_error(c, E_POOL);
           off = ~0ull;
         }
@@ -261,28 +295,15 @@ __global__ void k_compact(Ctx c, uint32_t idle) {
     }
     off = __shfl_sync(FULL_MASK, off, 0);
     p0 = __shfl_sync(FULL_MASK, p0, 0);
+    u0 = __shfl_sync(FULL_MASK, u0, 0);
     if (off == ~0ull) continue;
     const uint32_t arr = (uint32_t)(off / REF_BYTES);
-    int4* drec = array_recs(c, arr);
-    uint32_t* daux = array_aux(c, arr, n);
-    uint32_t ref = m.head, idx = 0;
-    for (uint32_t j = 0; j < nch && idx < n; ++j) {
-      if (!ref_ok(c, ref, c.chunk_bytes)) {
-        if (lane == 0) set_error(c, E_INTERNAL);
-        break;
-      }
-      const uint32_t nxt = *chunk_next(c, ref);
-      const uint32_t cnt = min(c.C, n - idx);
-      const int4* srec = chunk_recs(c, ref);
-      const uint32_t* saux = chunk_aux(c, ref);
-      for (uint32_t q = lane; q < cnt; q += 32) {
-        drec[idx + q] = srec[q];
-        daux[idx + q] = saux[q];
-      }
-      if (lane == 0) c.pool[p0 + (int)j] = ref;
-      idx += cnt;
-      ref = nxt;
-    }
+    const uint32_t got = walk_chunks(c, head, nch, dir, [&](bool on, uint32_t j, uint32_t ref) {
+      if (!on) return;
+      units[u0 + j] = DrawUnit{ref, j * c.C, chunk_fill(c, j, n), arr};
+      c.pool[p0 + (int)j] = ref;
+    });
+    for (uint32_t j = got + lane; j < nch; j += 32u) units[u0 + j] = DrawUnit{0, 0, 0, 0};
     __syncwarp();
     if (lane == 0) {
       uint32_t* hdr = reinterpret_cast<uint32_t*>(ref_ptr(c, arr));
@@ -294,6 +315,29 @@ __global__ void k_compact(Ctx c, uint32_t idle) {
       atomicAdd(&c.ctl->st_compact_chunks, (unsigned long long)nch);
       atomicAdd(&c.ctl->compact_now, 1ull);
       atomicAdd(&c.ctl->compact_chunks_now, (unsigned long long)nch);
+    }
+  }
+}
+
+// Copy the units, `parts` warps per unit (parts * part >= C).
+__global__ void k_compact_copy(Ctx c, const DrawUnit* units, uint32_t parts, uint32_t part) {
+  const uint64_t nu = min((uint64_t)vload(&c.ctl->draw_units), (uint64_t)c.max_chunks);
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
+  const uint64_t nwarps = (uint64_t)gridDim.x * blockDim.x / 32;
+  for (uint64_t w = warp; w < nu * parts; w += nwarps) {
+    const DrawUnit u = units[w / parts];
+    const uint32_t lo = (uint32_t)(w % parts) * part, hi = min(lo + part, u.n);
+    if (lo >= hi) continue;
+    const uint32_t cap = reinterpret_cast<const uint32_t*>(ref_ptr(c, u.arr))[1];
+    const int4* srec = chunk_recs(c, u.ref);
+    const uint32_t* saux = chunk_aux(c, u.ref);
+    int4* drec = array_recs(c, u.arr) + u.first;
+    uint32_t* daux = array_aux(c, u.arr, cap) + u.first;
+#pragma unroll 4
+    for (uint32_t q = lo + lane; q < hi; q += 32) {
+      drec[q] = __ldcg(srec + q);
+      daux[q] = __ldcg(saux + q);
     }
   }
 }
@@ -642,6 +686,12 @@ unsigned grid_for(const simlod_t* h, uint64_t work, uint64_t per_block) {
   return (unsigned)blocks;
 }
 
+// Warps per unit of C records (about 256 records each) and records per warp.
+void unit_parts(uint32_t C, uint32_t* parts, uint32_t* part) {
+  *parts = std::min<uint32_t>(16u, (C + 255u) / 256u);
+  *part = ((C + *parts - 1u) / *parts + 31u) / 32u * 32u;
+}
+
 // Read the control block (waits for the stream).
 int read_ctl(simlod_t* h, cudaStream_t s) {
   if (cudaMemcpyAsync(h->ctl_host, h->ctx.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s) !=
@@ -691,7 +741,7 @@ int insert_device(simlod_t* h, const int4* pts, uint64_t n, cudaStream_t s) {
       });
       if (rc) return poison(h, rc);
       rc = launch(h, K_DECIDE, s, [&] {
-        k_decide_new<<<full, BLOCK, 0, s>>>(c, r);
+        k_decide_new<<<full * 2, BLOCK, 0, s>>>(c, r);
       });
       if (rc) return poison(h, rc);
     }
@@ -699,7 +749,7 @@ int insert_device(simlod_t* h, const int4* pts, uint64_t n, cudaStream_t s) {
       k_claim<<<r ? full : gp, PBLOCK, PHASE_SMEM_BYTES, s>>>(c, pts, n, base, nodes0, r);
     });
     if (rc) return poison(h, rc);
-    rc = launch(h, K_DECIDE, s, [&] { k_alloc_voxels<<<full, BLOCK, 0, s>>>(c, r); });
+    rc = launch(h, K_DECIDE, s, [&] { k_alloc_voxels<<<full * 2, BLOCK, 0, s>>>(c, r); });
     if (rc) return poison(h, rc);
     if ((rc = read_ctl(h, s))) return poison(h, rc);
     if (t.error) return poison(h, error_from_bits(t.error));
@@ -1604,7 +1654,16 @@ SIMLOD_API int simlod_compact(simlod_t* h, uint32_t idle_updates, void* stream) 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   h->last_stream = s;
   const Ctx& c = h->ctx;
-  k_compact<<<(unsigned)h->sm_count * 4, BLOCK, 0, s>>>(c, idle_updates);
+  if (cudaMemsetAsync(&c.ctl->compact_need, 0, sizeof(unsigned long long), s) != cudaSuccess ||
+      cudaMemsetAsync(&c.ctl->draw_units, 0, sizeof(unsigned int), s) != cudaSuccess)
+    return poison(h, SIMLOD_ERR_CUDA);
+  DrawUnit* units = reinterpret_cast<DrawUnit*>(c.tasks);  // dead between updates
+  uint32_t parts, part;
+  unit_parts(c.C, &parts, &part);
+  const unsigned grid = (unsigned)h->sm_count * 8;
+  k_compact_need<<<grid, BLOCK, 0, s>>>(c, idle_updates);
+  k_compact_plan<<<grid, BLOCK, 0, s>>>(c, idle_updates, units);
+  k_compact_copy<<<grid, BLOCK, 0, s>>>(c, units, parts, part);
   return cudaGetLastError() == cudaSuccess ? SIMLOD_OK : poison(h, SIMLOD_ERR_CUDA);
 }
 
@@ -1636,8 +1695,8 @@ SIMLOD_API int simlod_render(simlod_t* h, const float view_proj[16], uint32_t wi
   // the spill tasks are dead between updates (the render is ordered after
   // them): their region, one entry per chunk, holds the draw units
   DrawUnit* units = reinterpret_cast<DrawUnit*>(c.tasks);
-  const uint32_t parts = std::min<uint32_t>(16u, (c.C + 255u) / 256u);
-  const uint32_t part = ((c.C + parts - 1u) / parts + 31u) / 32u * 32u;
+  uint32_t parts, part;
+  unit_parts(c.C, &parts, &part);
   const unsigned grid = (unsigned)h->sm_count * 8;
   return launch(h, K_RENDER, s, [&] {
     k_render_select<<<grid, BLOCK, 0, s>>>(c, v, vis, fb, (uint64_t)width * height, clear);
