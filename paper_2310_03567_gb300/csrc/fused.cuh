@@ -37,14 +37,23 @@ struct PlanSeg {
   uint32_t n, dst;
 };
 
-// Per-launch control words of the fused kernel (arena).
+// A short batch list travels in the launch itself: a table in device memory
+// costs a copy before every launch (and the host waits for the one before it).
+constexpr uint32_t INLINE_BATCHES = 16;
+struct BatchList {
+  BatchDesc d[INLINE_BATCHES];
+};
+
+// Control words of the fused kernel (arena). All zero between launches: the
+// last block to leave a launch clears them (a memset before every launch was
+// 2 us of the stream), but for `consumed`, which the host reads.
 struct FusedCtl {
   // block arrivals at grid barriers since the launch began (gridDim.x per
   // barrier); bit 63 (BAR_ABORT) aborts the launch
   unsigned long long bar;
   unsigned int consumed;  // batches fully handled (applied or rejected)
   unsigned int stop;      // the frame budget ran out
-  unsigned int rejected;  // batches rejected in this launch
+  unsigned int left;      // blocks that have left the launch
   unsigned int pad[11];
 };
 static_assert(sizeof(FusedCtl) == 64, "FusedCtl size");
@@ -189,13 +198,13 @@ struct PhaseClock {
 //
 // ready != nullptr: update b starts once ready[b] != 0 (its points were copied
 // by another stream, which then set the flag).
-__global__ void __launch_bounds__(FUSED_BLOCK, PHASE_MIN_BLOCKS) k_fused(Ctx c, const BatchDesc* batches,
-                                                        uint32_t n_batches, FusedCtl* f,
-                                                        unsigned long long budget_ns,
-                                                        uint32_t max_iters,
-                                                        const unsigned int* n_dev,
-                                                        const PlanSeg* segs,
-                                                        const unsigned int* ready) {
+//
+// batches == nullptr: the list is `list`, in the kernel's parameters.
+__device__ __forceinline__ void fused_body(const Ctx& c, const BatchDesc* batches,
+                                           const BatchList& list, uint32_t n_batches, FusedCtl* f,
+                                           unsigned long long budget_ns, uint32_t max_iters,
+                                           const unsigned int* n_dev, const PlanSeg* segs,
+                                           const unsigned int* ready) {
   const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const uint64_t nthreads = (uint64_t)gridDim.x * blockDim.x;
   const uint64_t warp0 = tid / 32, nwarps = nthreads / 32;
@@ -219,7 +228,7 @@ __global__ void __launch_bounds__(FUSED_BLOCK, PHASE_MIN_BLOCKS) k_fused(Ctx c, 
     // first batch reads them directly: no barrier has filled the view yet)
     if (b ? SL_CV(stop, &f->stop) : vload(&f->stop)) return;
     if (ready && !wait_ready(c, f, ready + b)) return;
-    BatchDesc bd = batches[b];
+    BatchDesc bd = batches ? batches[b] : list.d[b];
     const unsigned long long base = b ? SL_CV(base, &c.ctl->base) : vload(&c.ctl->base);
     const uint32_t nodes0 = b ? SL_CV(n_nodes, &c.ctl->n_nodes) : vload(&c.ctl->n_nodes);
     bool rejected = false;
@@ -250,7 +259,6 @@ __global__ void __launch_bounds__(FUSED_BLOCK, PHASE_MIN_BLOCKS) k_fused(Ctx c, 
         if (tid == 0) {
           phase_end_rejected(c);
           c.ctl->st_rejected_async += 1;
-          f->rejected += 1;
         }
       } else {
         // s_hi: splits so far, [n_lo, n_hi): nodes the last build created, t_hi:
@@ -290,19 +298,24 @@ __global__ void __launch_bounds__(FUSED_BLOCK, PHASE_MIN_BLOCKS) k_fused(Ctx c, 
         const ClaimArgs ca{nodes0, (uint32_t)(SL_CV(bump0, &c.ctl->bump0) / REF_BYTES),
                            SL_CV(open, &c.ctl->open),
                            claim_near_mask(c, bd.n + n_spill, SL_CV(key_rate, &c.ctl->key_rate))};
-        phase_claim(c, smem, node_cache_at(smem, n_hi), bd.pts, bd.n, base, t_hi, s_hi, ca, warp0,
-                    nwarps);
-        if (!grid_barrier(c, f)) return;
-        clk.tick(c, PH_CLAIM);
-        phase_decide(c, 0, n_hi, warp0, nwarps);  // chunks for the new voxels
+        uint32_t n_keys = 0;
+        if (n_hi > 1u) {  // (an octree of one leaf has no voxels)
+          phase_claim(c, smem, node_cache_at(smem, n_hi), bd.pts, bd.n, base, t_hi, s_hi, ca,
+                      warp0, nwarps);
+          if (!grid_barrier(c, f, vw)) return;
+          clk.tick(c, PH_CLAIM);
+          n_keys = min(SL_CV(nkeys, &c.ctl->nkeys), c.backlog_cap);
+          if (n_keys) phase_decide(c, 0, n_hi, warp0, nwarps);  // chunks for the new voxels
+        }
         phase_store(c, smem, bd.pts, bd.n, base, t_hi, tid, nthreads);
         if (!grid_barrier(c, f, vw)) return;
         clk.tick(c, PH_STORE);
-        const uint32_t n_keys = min(SL_CV(nkeys, &c.ctl->nkeys), c.backlog_cap);
-        phase_store_voxels(c, smem, t_hi, n_keys, SL_CV(pool_top, &c.ctl->pool_top), tid,
-                           nthreads);
-        if (!grid_barrier(c, f)) return;
-        clk.tick(c, PH_STORE);
+        if (n_keys || t_hi) {
+          phase_store_voxels(c, smem, t_hi, n_keys, SL_CV(pool_top, &c.ctl->pool_top), tid,
+                             nthreads);
+          if (!grid_barrier(c, f)) return;
+          clk.tick(c, PH_STORE);
+        }
         if (tid == 0) phase_end(c, bd.n);
       }
     }
@@ -337,6 +350,23 @@ __global__ void __launch_bounds__(FUSED_BLOCK, PHASE_MIN_BLOCKS) k_fused(Ctx c, 
   if (blockIdx.x == 0 && threadIdx.x == 0)
     atomicAdd(&c.ctl->phase_ns[PH_LAUNCH], globaltimer_ns() - t_begin);
 #undef SL_CV
+}
+
+__global__ void __launch_bounds__(FUSED_BLOCK, PHASE_MIN_BLOCKS)
+    k_fused(Ctx c, const BatchDesc* batches, const __grid_constant__ BatchList list,
+            uint32_t n_batches, FusedCtl* f, unsigned long long budget_ns, uint32_t max_iters,
+            const unsigned int* n_dev, const PlanSeg* segs, const unsigned int* ready) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) f->consumed = 0;
+  fused_body(c, batches, list, n_batches, f, budget_ns, max_iters, n_dev, segs, ready);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(&f->left, 1u) + 1u == gridDim.x) {
+      f->bar = 0;
+      f->stop = 0;
+      f->left = 0;
+    }
+  }
 }
 
 // ------------------------------------------------------------ batched form

@@ -44,6 +44,11 @@ extern "C" int SL_VARIANT_LAUNCH(const sl_fused_launch* a) {
   Ctx c;
   memcpy(&c, a->ctx, sizeof(Ctx));
   const BatchDesc* bt = static_cast<const BatchDesc*>(a->batches);
+  BatchList list{};
+  if (!bt) {
+    if (a->list_bytes != sizeof(BatchList)) return (int)cudaErrorInvalidValue;
+    memcpy(&list, a->list, sizeof(BatchList));
+  }
   uint32_t n = a->n_batches;
   FusedCtl* f = static_cast<FusedCtl*>(a->fctl);
   unsigned long long budget = a->budget_ns;
@@ -51,7 +56,7 @@ extern "C" int SL_VARIANT_LAUNCH(const sl_fused_launch* a) {
   const unsigned int* n_dev = a->n_dev;
   const PlanSeg* segs = static_cast<const PlanSeg*>(a->segs);
   const unsigned int* ready = a->ready;
-  void* args[] = {&c, &bt, &n, &f, &budget, &max_iters, &n_dev, &segs, &ready};
+  void* args[] = {&c, &bt, &list, &n, &f, &budget, &max_iters, &n_dev, &segs, &ready};
   return (int)cudaLaunchCooperativeKernel((const void*)k_fused, dim3(a->grid), dim3(FUSED_BLOCK),
                                           args, PHASE_SMEM_BYTES,
                                           static_cast<cudaStream_t>(a->stream));

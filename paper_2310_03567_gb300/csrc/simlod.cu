@@ -26,8 +26,9 @@ namespace {
 constexpr int BLOCK = 256;
 constexpr int PBLOCK = PHASE_BLOCK;  // count / advance kernels (one node-table cache per block)
 
-__global__ void k_init(Ctx c) {
+__global__ void k_init(Ctx c, FusedCtl* f) {
   if (blockIdx.x == 0 && threadIdx.x == 0) {
+    memset(f, 0, sizeof(FusedCtl));  // (an error outside a launch leaves its abort bit there)
     Ctl* t = c.ctl;
     unsigned long long phase_ns[8];  // diagnostics survive a reset
     for (int k = 0; k < 8; ++k) phase_ns[k] = t->phase_ns[k];
@@ -369,6 +370,11 @@ int fused_launch_0(const sl_fused_launch* a) {
   Ctx c;
   memcpy(&c, a->ctx, sizeof(Ctx));
   const BatchDesc* bt = static_cast<const BatchDesc*>(a->batches);
+  BatchList list{};
+  if (!bt) {
+    if (a->list_bytes != sizeof(BatchList)) return (int)cudaErrorInvalidValue;
+    memcpy(&list, a->list, sizeof(BatchList));
+  }
   uint32_t n = a->n_batches;
   FusedCtl* f = static_cast<FusedCtl*>(a->fctl);
   unsigned long long budget = a->budget_ns;
@@ -376,7 +382,7 @@ int fused_launch_0(const sl_fused_launch* a) {
   const unsigned int* n_dev = a->n_dev;
   const PlanSeg* segs = static_cast<const PlanSeg*>(a->segs);
   const unsigned int* ready = a->ready;
-  void* args[] = {&c, &bt, &n, &f, &budget, &max_iters, &n_dev, &segs, &ready};
+  void* args[] = {&c, &bt, &list, &n, &f, &budget, &max_iters, &n_dev, &segs, &ready};
   return (int)cudaLaunchCooperativeKernel((const void*)k_fused, dim3(a->grid), dim3(FUSED_BLOCK),
                                           args, PHASE_SMEM_BYTES,
                                           static_cast<cudaStream_t>(a->stream));
@@ -788,30 +794,48 @@ int launch_fused(simlod_t* h, const simlod_point* const* d_batches, const uint64
     total += counts[k];
   }
   if (h->base + total > (1ull << 32)) return SIMLOD_ERR_TOO_MANY_POINTS;
+  BatchList list{};
+  const bool small = n <= INLINE_BATCHES;
   // the staging table may still feed the previous copy
-  if (cudaEventSynchronize(h->desc_done) != cudaSuccess) return poison(h, SIMLOD_ERR_CUDA);
-  for (uint32_t k = 0; k < n; ++k)
-    h->desc_host[k] = BatchDesc{reinterpret_cast<const int4*>(d_batches[k]), counts[k], 0, 0};
+  if (!small && cudaEventSynchronize(h->desc_done) != cudaSuccess)
+    return poison(h, SIMLOD_ERR_CUDA);
+  uint64_t largest = 0;
+  for (uint32_t k = 0; k < n; ++k) {
+    (small ? list.d : h->desc_host)[k] =
+        BatchDesc{reinterpret_cast<const int4*>(d_batches[k]), counts[k], 0, 0};
+    largest = std::max(largest, counts[k]);
+  }
   h->last_stream = s;
-  if (cudaMemcpyAsync(h->batches_dev, h->desc_host, sizeof(BatchDesc) * n,
-                      cudaMemcpyHostToDevice, s) != cudaSuccess ||
-      cudaEventRecord(h->desc_done, s) != cudaSuccess ||
-      cudaMemsetAsync(h->fctl_dev, 0, sizeof(FusedCtl), s) != cudaSuccess)
+  if (!small && (cudaMemcpyAsync(h->batches_dev, h->desc_host, sizeof(BatchDesc) * n,
+                                 cudaMemcpyHostToDevice, s) != cudaSuccess ||
+                 cudaEventRecord(h->desc_done, s) != cudaSuccess))
     return poison(h, SIMLOD_ERR_CUDA);
   Ctx c = h->ctx;
   c.progress = h->prog_dev;
-  const BatchDesc* bt = h->batches_dev;
-  FusedCtl* f = h->fctl_dev;
-  uint32_t max_iters = h->cfg.max_expand_iters ? h->cfg.max_expand_iters : h->cfg.root_log2 + 1;
-  const unsigned int* n_dev = nullptr;
-  const PlanSeg* segs = nullptr;
-  void* args[] = {&c, &bt, &n, &f, &budget_ns, &max_iters, &n_dev, &segs, &ready};
-  cudaError_t le = cudaSuccess;
-  int rc = launch(h, K_FUSED, s, [&] {
-    le = cudaLaunchCooperativeKernel((const void*)k_fused, dim3(h->fused_grid),
-                                     dim3(FUSED_BLOCK), args, PHASE_SMEM_BYTES, s);
-  });
-  if (rc || le != cudaSuccess) return poison(h, SIMLOD_ERR_CUDA);
+  sl_fused_launch a;
+  a.ctx = &c;
+  a.ctx_bytes = sizeof(Ctx);
+  a.batches = small ? nullptr : h->batches_dev;
+  a.list = &list;
+  a.list_bytes = sizeof(BatchList);
+  a.n_batches = n;
+  a.fctl = h->fctl_dev;
+  a.budget_ns = budget_ns;
+  a.max_iters = h->cfg.max_expand_iters ? h->cfg.max_expand_iters : h->cfg.root_log2 + 1;
+  a.n_dev = nullptr;
+  a.segs = nullptr;
+  a.ready = ready;
+  // a block per SM and a point per thread: more blocks only make the grid
+  // barriers longer (16 launches of 4,096 points: 0.32 against 0.36 ms). An
+  // update may re-insert points of the octree too, at most all of them
+  const uint64_t work = std::max<uint64_t>(largest, h->base / 8);
+  const uint64_t want =
+      std::max<uint64_t>((uint64_t)h->sm_count, (work + FUSED_BLOCK - 1) / FUSED_BLOCK);
+  a.grid = (unsigned)std::min<uint64_t>(want, (uint64_t)h->fused_grid);
+  a.stream = s;
+  int le = (int)cudaSuccess;
+  int rc = launch(h, K_FUSED, s, [&] { le = fused_launch_0(&a); });
+  if (rc || le != (int)cudaSuccess) return poison(h, SIMLOD_ERR_CUDA);
   h->base += total;  // upper bound until the next control-block read
   h->mirror_stale = true;
   h->prog_submitted += n;
@@ -838,7 +862,7 @@ int init_octree(simlod_t* h, cudaStream_t s, bool clear_hash, bool wait) {
   const Ctx& c = h->ctx;
   k_clear_tables<<<(unsigned)h->sm_count * 8, BLOCK, 0, s>>>(c, clear_hash ? 1 : 0);
   if (cudaGetLastError() != cudaSuccess) return SIMLOD_ERR_CUDA;
-  k_init<<<1, 1, 0, s>>>(c);
+  k_init<<<1, 1, 0, s>>>(c, h->fctl_dev);
   if (cudaGetLastError() != cudaSuccess) return SIMLOD_ERR_CUDA;
   if (wait && cudaStreamSynchronize(s) != cudaSuccess) return SIMLOD_ERR_CUDA;
   h->base = 0;
@@ -1112,13 +1136,13 @@ int plan_enqueue(simlod_plan_t* P, cudaStream_t s) {
   k_plan_validate<<<vg, BLOCK, 0, s>>>(c, P->in, P->tile0, P->n, P->bad);
   k_plan_groups<<<1, 1, 0, s>>>(c, P->in, P->n, P->bad, P->p.merge_points, P->groups, P->segs,
                                 P->n_groups);
-  if (cudaGetLastError() != cudaSuccess ||
-      cudaMemsetAsync(h->fctl_dev, 0, sizeof(FusedCtl), s) != cudaSuccess)
-    return SIMLOD_ERR_CUDA;
+  if (cudaGetLastError() != cudaSuccess) return SIMLOD_ERR_CUDA;
   sl_fused_launch a;
   a.ctx = &c;
   a.ctx_bytes = sizeof(Ctx);
   a.batches = P->groups;
+  a.list = nullptr;
+  a.list_bytes = 0;
   a.n_batches = P->n;
   a.fctl = h->fctl_dev;
   a.budget_ns = NO_BUDGET;

@@ -26,7 +26,9 @@ struct sl_variant_info {
 struct sl_fused_launch {
   const void* ctx;
   size_t ctx_bytes;
-  const void* batches;
+  const void* batches;  // nullptr: the list (a BatchList, list_bytes long)
+  const void* list;
+  size_t list_bytes;
   uint32_t n_batches;
   void* fctl;
   unsigned long long budget_ns;
