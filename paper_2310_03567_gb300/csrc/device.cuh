@@ -82,9 +82,6 @@ constexpr uint32_t CHUNK_HEADER = 16;
 #ifndef SL_CTL_SPREAD
 #define SL_CTL_SPREAD 1
 #endif
-#ifndef SL_STORE_PREFETCH
-#define SL_STORE_PREFETCH 1
-#endif
 #ifndef SL_COUNT_PREFETCH
 #define SL_COUNT_PREFETCH 1
 #endif
@@ -96,9 +93,6 @@ constexpr uint32_t CHUNK_HEADER = 16;
 #endif
 #ifndef SL_STORE_UNROLL
 #define SL_STORE_UNROLL 2
-#endif
-#ifndef SL_STORE_BLOCK
-#define SL_STORE_BLOCK 1
 #endif
 #ifndef SL_BLOCK_TALLY
 #define SL_BLOCK_TALLY 1
@@ -125,7 +119,7 @@ constexpr uint32_t TALLY_SLOTS = 1u << TALLY_LOG2;
 constexpr int CLAIM_U = SL_CLAIM_UNROLL;  // units of 32 points a warp claims for at once
 constexpr uint32_t CLAIM_QUEUE = 32 * (CLAIM_U + 1);  // points that wait for their next claim
 constexpr uint32_t SMEM_WBUF = NODE_CACHE;            // in u32 words
-constexpr uint32_t SMEM_QUEUE = SMEM_WBUF + (PHASE_BLOCK / 32) * WBUF;
+constexpr uint32_t SMEM_QUEUE = SMEM_WBUF + (PHASE_BLOCK / 32) * WBUF * 2;
 constexpr uint32_t SMEM_TALLY = SMEM_QUEUE + (PHASE_BLOCK / 32) * CLAIM_QUEUE * 6;
 constexpr uint32_t PHASE_SMEM_BYTES = 4 * (SMEM_TALLY + 2 * TALLY_SLOTS);
 
@@ -268,7 +262,7 @@ struct Ctx {
   uint32_t* hist;     // counts of the cubes below split leaves; zero between updates
   uint32_t* hist_up;  //   their sums per inner level, and the list of inner nodes
   HSlot* hash;
-  uint32_t* keys;     // backlog: table slots of this update's new cells
+  uint2* keys;        // backlog: table slot and node of this update's new cells
   uint8_t* data;
   unsigned long long data_bytes;
   int4* staging;
@@ -276,6 +270,7 @@ struct Ctx {
   uint32_t rlog2, T, C, G;
   uint32_t chunk_bytes, chunk_units, grid_bytes, dir_bytes, dir_cap;
   uint32_t hash_mask;
+  uint32_t C_mul, C_shift;  // division by C (div_C)
   uint32_t max_nodes, max_chunks, spill_cap, backlog_cap, max_splits;
   uint64_t max_batch;
   uint64_t hist_words;
@@ -628,14 +623,14 @@ __device__ __forceinline__ LaneRun lane_run(bool on, T v) {
 // Per-warp staging of the table slots of new cells (shared memory), flushed
 // to the backlog with one atomic per flush.
 struct WarpBuf {
-  uint32_t* buf;   // WBUF entries of this warp
+  uint2* buf;      // WBUF entries (slot, node) of this warp
   uint32_t n;      // staged entries (the same value in every lane)
   uint32_t* smem;  // the block's dynamic shared memory (tally cache)
 };
 
 __device__ __forceinline__ WarpBuf warp_buf(uint32_t* smem) {
   WarpBuf wb;
-  wb.buf = smem + SMEM_WBUF + (threadIdx.x / 32) * WBUF;
+  wb.buf = reinterpret_cast<uint2*>(smem + SMEM_WBUF) + (threadIdx.x / 32) * WBUF;
   wb.n = 0;
   wb.smem = smem;
   return wb;
@@ -718,7 +713,7 @@ __device__ __forceinline__ void warp_claim(const Ctx& c, WarpBuf& wb, const bool
     if (wb.n + ni > WBUF) warp_flush(c, wb);
     const LaneRun r = lane_run(inst[j], node[j]);
     if (inst[j]) {
-      wb.buf[wb.n + __popc(mi & ((1u << lane) - 1u))] = h[j];
+      wb.buf[wb.n + __popc(mi & ((1u << lane) - 1u))] = make_uint2(h[j], node[j]);
       if (r.head) tally_add(c.cnt, wb.smem, node[j], r.end - lane);
     }
     wb.n += ni;
@@ -1501,266 +1496,225 @@ __device__ void phase_rollback(const Ctx& c, uint32_t n_nodes, uint64_t t0, uint
 
 // -------------------------------------------------------------- phase: store
 
-// All 32 lanes call with U items each (warp-uniform). Every valid item gets
-// the next free slot of its node in this update: the node's records before
-// the update (st_base) + a running per-node cursor, one atomicAdd per
-// distinct node per warp and item index; the store map then turns the slot
-// into (chunk ref, index in chunk). The map (st_nch, st_tail, st_seq,
-// st_base) is one 16-byte load per item, issued with the cursor atomics.
-// Invalid items, and items whose slot has no chunk, get ref NONE (the latter
-// raise E_INTERNAL).
-template <int U>
-__device__ __forceinline__ void warp_place(const Ctx& c, const bool (&valid)[U],
-                                           const uint32_t (&node)[U], uint32_t (&ref)[U],
-                                           uint32_t (&q)[U]) {
-  const uint32_t lane = lane_id();
-  uint4 map[U];
-  uint32_t rank[U], cur[U];
-  int leader[U];
-#pragma unroll
-  for (int j = 0; j < U; ++j) {
-    map[j] = valid[j] ? *reinterpret_cast<const uint4*>(&c.meta[node[j]].st_nch)
-                      : make_uint4(0, NONE, 0, 0);
-  }
-  // exact groups here (a match over the warp): the cursor atomics return a
-  // value, and in dense regions the lanes of one node are not contiguous, so
-  // one reservation per lane run would queue many more of them on one counter
-#pragma unroll
-  for (int j = 0; j < U; ++j) {
-    const unsigned m = __ballot_sync(FULL_MASK, valid[j]);
-    leader[j] = 0;
-    rank[j] = 0;
-    cur[j] = 0;
-    if (valid[j]) {
-      const unsigned grp = __match_any_sync(m, node[j]);
-      leader[j] = __ffs(grp) - 1;
-      rank[j] = __popc(grp & ((1u << lane) - 1u));
-      if ((int)lane == leader[j]) cur[j] = atomicAdd(&c.scur[node[j]], (uint32_t)__popc(grp));
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < U; ++j) {
-    cur[j] = __shfl_sync(FULL_MASK, cur[j], leader[j]);
-    ref[j] = NONE;
-    q[j] = 0;
-    if (valid[j]) {
-      const uint32_t slot = map[j].w + cur[j] + rank[j];
-      const uint32_t k = slot / c.C;
-      q[j] = slot - k * c.C;
-      if (k + 1u == map[j].x) {
-        ref[j] = map[j].y;
-      } else if (k >= map[j].x) {
-        const unsigned long long at = (unsigned long long)map[j].z + (k - map[j].x);
-        if (at < c.max_chunks) ref[j] = c.alloc_refs[at];
-      }
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < U; ++j) {
-    if (valid[j] && !ref_ok(c, ref[j], c.chunk_bytes)) {
-      set_error(c, E_INTERNAL);
-      ref[j] = NONE;
-    }
-  }
+// n / C for any 32-bit n: multiply, add and shift by the constants that Granlund
+// and Montgomery ("Division by invariant integers using multiplication", 1994)
+// give for a divisor (div_constants).
+__device__ __forceinline__ uint32_t div_C(const Ctx& c, uint32_t n) {
+  if (c.C == 1u) return n;
+  const uint32_t t = __umulhi(c.C_mul, n);
+  return (t + ((n - t) >> 1)) >> c.C_shift;
 }
 
-// Block form of warp_place (all threads of the block call; loops are
-// block-uniform): items of the whole block reserve their slots per node in a
-// shared-memory table first (256 slots, direct-mapped, in the tally region),
-// then one thread per table entry takes the node's range with one global
-// atomicAdd. In dense regions many warps of a block store into the same few
-// nodes; their returning atomics on one counter would queue at one L2 slice.
-// Items whose table slot holds another node take the warp path.
-constexpr uint32_t PLACE_SLOTS = 256;
-
-template <int U>
-__device__ __forceinline__ void block_place(const Ctx& c, uint32_t* smem, const bool (&valid)[U],
-                                            const uint32_t (&node)[U], uint32_t (&ref)[U],
-                                            uint32_t (&q)[U]) {
-  const uint32_t lane = lane_id();
-  uint32_t* tn = smem + SMEM_TALLY;  // node of each table slot
-  uint32_t* tc = tn + PLACE_SLOTS;   // items of the block for it
-  uint32_t* tb = tc + PLACE_SLOTS;   // the range it got
-  uint4 map[U];
-  uint32_t sl[U], rank[U], cur[U];
-  int leader[U];
-#pragma unroll
-  for (int j = 0; j < U; ++j) {
-    map[j] = valid[j] ? *reinterpret_cast<const uint4*>(&c.meta[node[j]].st_nch)
-                      : make_uint4(0, NONE, 0, 0);
-    sl[j] = NONE;
-    rank[j] = 0;
-    if (valid[j]) {
-      const uint32_t h = (node[j] * 0x9E3779B1u) >> 24;  // PLACE_SLOTS = 2^8
-      const uint32_t old = tn[h] == node[j] ? node[j] : atomicCAS(tn + h, NONE, node[j]);
-      if (old == NONE || old == node[j]) {
-        sl[j] = h;
-        rank[j] = atomicAdd(tc + h, 1u);
-      }
-    }
-  }
-  // items without a table slot: exact groups of the warp, one global atomic each
-#pragma unroll
-  for (int j = 0; j < U; ++j) {
-    const bool fb = valid[j] && sl[j] == NONE;
-    const unsigned m = __ballot_sync(FULL_MASK, fb);
-    leader[j] = 0;
-    cur[j] = 0;
-    if (fb) {
-      const unsigned grp = __match_any_sync(m, node[j]);
-      leader[j] = __ffs(grp) - 1;
-      rank[j] = __popc(grp & ((1u << lane) - 1u));
-      if ((int)lane == leader[j]) cur[j] = atomicAdd(&c.scur[node[j]], (uint32_t)__popc(grp));
-    }
-    cur[j] = __shfl_sync(FULL_MASK, cur[j], leader[j]);
-  }
-  __syncthreads();
-  for (uint32_t t = threadIdx.x; t < PLACE_SLOTS; t += blockDim.x) {
-    const uint32_t nd = tn[t];
-    if (nd != NONE) tb[t] = atomicAdd(&c.scur[nd], tc[t]);
-    tn[t] = NONE;  // every thread has passed its table lookups (barrier above)
-    tc[t] = 0;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int j = 0; j < U; ++j) {
-    ref[j] = NONE;
-    q[j] = 0;
-    if (valid[j]) {
-      const uint32_t slot = map[j].w + (sl[j] != NONE ? tb[sl[j]] : cur[j]) + rank[j];
-      const uint32_t k = slot / c.C;
-      q[j] = slot - k * c.C;
-      if (k + 1u == map[j].x) {
-        ref[j] = map[j].y;
-      } else if (k >= map[j].x) {
-        const unsigned long long at = (unsigned long long)map[j].z + (k - map[j].x);
-        if (at < c.max_chunks) ref[j] = c.alloc_refs[at];
-      }
-      if (!ref_ok(c, ref[j], c.chunk_bytes)) {
-        set_error(c, E_INTERNAL);
-        ref[j] = NONE;
-      }
-    }
-  }
+inline void div_constants(uint32_t d, uint32_t* mul, uint32_t* shift) {  // d >= 1
+  uint32_t l = 0;
+  while ((1ull << l) < d) ++l;
+  *mul = (uint32_t)(((1ull << 32) * ((1ull << l) - d)) / d + 1ull);
+  *shift = l ? l - 1u : 0u;
 }
 
-// All threads of the block call: an empty block placement table.
-__device__ __forceinline__ void block_place_init(uint32_t* smem) {
-  for (uint32_t t = threadIdx.x; t < PLACE_SLOTS; t += blockDim.x) {
-    smem[SMEM_TALLY + t] = NONE;
-    smem[SMEM_TALLY + PLACE_SLOTS + t] = 0;
+// Slots of the items that one block stores (the table lies over the staging,
+// queue and tally regions, which the store phases do not use): the block
+// counts its items per node, takes one range per node with one atomicAdd on
+// the node's store cursor, and its threads then place the items in the ranges
+// with shared-memory atomics. With one range per node and round of 1,024
+// items (the form before) the returning atomics on a few cursors and the two
+// block barriers of every round were the phase: 50 of 54 stalled cycles per
+// instruction waited for memory, at 12 % of the issue slots and of DRAM.
+constexpr uint32_t PLACE_WORDS = SMEM_TALLY + 2 * TALLY_SLOTS - SMEM_WBUF;
+constexpr uint32_t place_log2(uint32_t words) {
+  uint32_t l = 0;
+  while ((5u << (l + 1u)) <= words) ++l;
+  return l;
+}
+constexpr uint32_t PLACE_LOG2 = place_log2(PLACE_WORDS);
+constexpr uint32_t PLACE_SLOTS = 1u << PLACE_LOG2;
+constexpr int PLACE_PROBES = 6;  // then the item's own atomic takes its slot
+
+struct PlaceTable {
+  uint32_t *node, *next;       // node, NONE: free; items counted, then next slot
+  uint32_t *nch, *tail, *seq;  // the node's store map
+};
+
+__device__ __forceinline__ PlaceTable place_table(uint32_t* smem) {
+  uint32_t* w = smem + SMEM_WBUF;
+  return PlaceTable{w, w + PLACE_SLOTS, w + 2 * PLACE_SLOTS, w + 3 * PLACE_SLOTS,
+                    w + 4 * PLACE_SLOTS};
+}
+
+__device__ __forceinline__ uint32_t place_home(uint32_t node) {
+  return (node * 0x9E3779B1u) >> (32u - PLACE_LOG2);
+}
+
+// The node's entry, made if there is none (pass 1); NONE after PLACE_PROBES.
+__device__ __forceinline__ uint32_t place_insert(const PlaceTable& t, uint32_t node) {
+  uint32_t h = place_home(node);
+  for (int p = 0; p < PLACE_PROBES; ++p) {
+    uint32_t old = t.node[h];
+    if (old == NONE) old = atomicCAS(t.node + h, NONE, node);
+    if (old == NONE || old == node) return h;
+    h = (h + 1u) & (PLACE_SLOTS - 1u);
   }
-  __syncthreads();
+  return NONE;
+}
+
+__device__ __forceinline__ uint32_t place_find(const PlaceTable& t, uint32_t node) {
+  uint32_t h = place_home(node);
+  for (int p = 0; p < PLACE_PROBES; ++p) {
+    if (t.node[h] == node) return h;
+    h = (h + 1u) & (PLACE_SLOTS - 1u);
+  }
+  return NONE;
 }
 
 __device__ __forceinline__ void put_rec(const Ctx& c, uint32_t ref, uint32_t q, int4 rec,
                                         uint32_t aux) {
-  if (ref == NONE) return;
   chunk_recs(c, ref)[q] = rec;
   chunk_aux(c, ref)[q] = aux;
 }
 
 constexpr int STORE_U = SL_STORE_UNROLL;
-static_assert(3 * 256 <= 2 * TALLY_SLOTS, "the block placement table fits the tally region");
 
-// Slots for U items per lane: per block in the persistent kernel (smem), per
-// warp in the plain form's kernels (smem == nullptr).
-template <int U>
-__device__ __forceinline__ void place_items(const Ctx& c, uint32_t* smem, const bool (&valid)[U],
-                                            const uint32_t (&node)[U], uint32_t (&ref)[U],
-                                            uint32_t (&q)[U]) {
-#if SL_STORE_BLOCK
-  if (smem) {
-    block_place<U>(c, smem, valid, node, ref, q);
-    return;
+struct StoreItem {
+  uint32_t node;         // NONE: nothing
+  int4 rec;
+  uint32_t aux;
+  uint32_t slot, gref;   // voxels: claim-table slot and occupancy grid
+};
+
+// All threads of the block call. The block takes a contiguous range of the
+// `units` (32 items each). node_of(w): the lane's node in unit w, NONE for
+// none. load(w, node, item): its record. done(item): after its record is in
+// place. Equal nodes of a run of lanes share one reservation. Each warp carries
+// STORE_U units at a time.
+template <typename NodeOf, typename Load, typename Done>
+__device__ __forceinline__ void place_units(const Ctx& c, uint32_t* smem, uint64_t units,
+                                            NodeOf&& node_of, Load&& load, Done&& done) {
+  constexpr int U = STORE_U;
+  const PlaceTable t = place_table(smem);
+  const uint32_t lane = lane_id();
+  const uint64_t per = (units + gridDim.x - 1) / gridDim.x;
+  const uint64_t first = blockIdx.x * per, last = (blockIdx.x + 1ull) * per;
+  const uint64_t lo = first + threadIdx.x / 32, hi = last < units ? last : units;
+  const uint32_t wpb = blockDim.x / 32;
+  if (first >= units) return;  // (all threads of the block alike)
+  __syncthreads();             // the regions' last use is over
+  for (uint32_t i = threadIdx.x; i < PLACE_SLOTS; i += blockDim.x) {
+    t.node[i] = NONE;
+    t.next[i] = 0;
   }
-#endif
-  warp_place<U>(c, valid, node, ref, q);
+  __syncthreads();
+  for (uint64_t w = lo; w < hi; w += wpb) {
+    const uint32_t node = node_of(w);
+    const LaneRun r = lane_run(node != NONE, node);
+    if (r.head) {
+      const uint32_t h = place_insert(t, node);
+      if (h != NONE) atomicAdd(t.next + h, r.end - lane);
+    }
+  }
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < PLACE_SLOTS; i += blockDim.x) {
+    const uint32_t node = t.node[i];
+    if (node == NONE) continue;
+    const uint4 map = *reinterpret_cast<const uint4*>(&c.meta[node].st_nch);
+    t.next[i] = map.w + atomicAdd(&c.scur[node], t.next[i]);
+    t.nch[i] = map.x;
+    t.tail[i] = map.y;
+    t.seq[i] = map.z;
+  }
+  __syncthreads();
+  for (uint64_t w0 = lo; w0 < hi; w0 += U * wpb) {
+    StoreItem it[U];
+    uint32_t slot[U];
+    uint32_t nch[U], tail[U], seq[U];
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const uint64_t w = w0 + j * wpb;
+      it[j] = StoreItem{w < hi ? node_of(w) : NONE, make_int4(0, 0, 0, 0), 0, 0, 0};
+    }
+#pragma unroll
+    for (int j = 0; j < U; ++j)
+      if (it[j].node != NONE) load(w0 + j * wpb, it[j]);
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const LaneRun r = lane_run(it[j].node != NONE, it[j].node);
+      uint32_t at = 0;
+      nch[j] = seq[j] = 0;
+      tail[j] = NONE;
+      if (it[j].node != NONE) {
+        const uint32_t h = place_find(t, it[j].node);
+        if (h != NONE) {
+          if (r.head) at = atomicAdd(t.next + h, r.end - lane);
+          nch[j] = t.nch[h];
+          tail[j] = t.tail[h];
+          seq[j] = t.seq[h];
+        } else {
+          const uint4 map = *reinterpret_cast<const uint4*>(&c.meta[it[j].node].st_nch);
+          if (r.head) at = map.w + atomicAdd(&c.scur[it[j].node], r.end - lane);
+          nch[j] = map.x;
+          tail[j] = map.y;
+          seq[j] = map.z;
+        }
+      }
+      slot[j] = __shfl_sync(FULL_MASK, at, (int)r.first) + lane - r.first;
+    }
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      if (it[j].node == NONE) continue;
+      const uint32_t k = div_C(c, slot[j]), q = slot[j] - k * c.C;
+      uint32_t ref = NONE;
+      if (k + 1u == nch[j]) {
+        ref = tail[j];
+      } else if (k >= nch[j]) {
+        const unsigned long long a = (unsigned long long)seq[j] + (k - nch[j]);
+        if (a < c.max_chunks) ref = c.alloc_refs[a];
+      }
+      if (!ref_ok(c, ref, c.chunk_bytes)) {
+        set_error(c, E_INTERNAL);
+        continue;
+      }
+      put_rec(c, ref, q, it[j].rec, it[j].aux);
+      done(it[j]);
+    }
+  }
 }
 
 // Store the batch points and the re-inserted points (of the spill tasks
-// [0, t_hi), still in their old chunks), each at the next free slot of its leaf. Loops are block-uniform so
-// that a block's items share their slot reservations; each lane carries
-// STORE_U items at a time so that their L2 round trips overlap.
+// [0, t_hi), still in their old chunks), each at the next free slot of its leaf.
 __device__ void phase_store(const Ctx& c, uint32_t* smem, const int4* pts, uint64_t n,
-                            unsigned long long base, uint32_t t_hi, uint64_t t0,
-                            uint64_t nthreads) {
-  constexpr int U = STORE_U;
-  // block-uniform loops: item j of thread t in round b is b + j * nthreads + t
-  const uint64_t blk = t0 - threadIdx.x, stride = nthreads;
-  const uint64_t me = threadIdx.x;
-#if SL_STORE_BLOCK
-  if (smem) block_place_init(smem);
-#endif
-#if SL_STORE_PREFETCH
-  // the next round's cursors and points load while this round is placed
-  uint32_t node_n[U];
-  int4 p_n[U];
-#pragma unroll
-  for (int j = 0; j < U; ++j) {
-    const uint64_t i = blk + j * stride + me;
-    node_n[j] = i < n ? c.b_cur[i] : 0u;
-    p_n[j] = i < n ? __ldcg(pts + i) : make_int4(0, 0, 0, 0);
-  }
-#endif
-  for (uint64_t b0 = blk; b0 < n; b0 += U * stride) {
-    bool valid[U];
-    uint32_t node[U], ref[U], q[U];
-    int4 p[U];
-#pragma unroll
-    for (int j = 0; j < U; ++j) {
-      const uint64_t i = b0 + j * stride + me;
-      valid[j] = i < n;
-#if SL_STORE_PREFETCH
-      node[j] = node_n[j];
-      p[j] = p_n[j];
-      const uint64_t inext = i + (uint64_t)U * stride;
-      node_n[j] = inext < n ? c.b_cur[inext] : 0u;
-      p_n[j] = inext < n ? __ldcg(pts + inext) : make_int4(0, 0, 0, 0);
-#else
-      node[j] = valid[j] ? c.b_cur[i] : 0u;
-      p[j] = valid[j] ? __ldcg(pts + i) : make_int4(0, 0, 0, 0);
-#endif
-      if (valid[j] && node[j] >= c.max_nodes) {
-        set_error(c, E_INTERNAL);
-        valid[j] = false;
-      }
-    }
-    place_items<U>(c, smem, valid, node, ref, q);
-#pragma unroll
-    for (int j = 0; j < U; ++j) put_rec(c, ref[j], q[j], p[j], (uint32_t)(base + b0 + j * stride + me));
-  }
-  const uint32_t parts = task_units(c);
-  const uint64_t n_re = (uint64_t)t_hi * parts * 32u;  // (lanes past a task's end idle)
-  for (uint64_t b0 = blk; b0 < n_re; b0 += U * stride) {
-    bool valid[U];
-    uint32_t node[U], ref[U], q[U], g[U];
-    int4 r[U];
-#pragma unroll
-    for (int j = 0; j < U; ++j) {
-      const uint64_t e = b0 + j * stride + me;
-      valid[j] = false;
-      node[j] = g[j] = 0u;
-      r[j] = make_int4(0, 0, 0, 0);
-      if (e < n_re) {
+                            unsigned long long base, uint32_t t_hi) {
+  const uint32_t lane = lane_id(), parts = task_units(c);
+  auto checked = [&](uint32_t node) -> uint32_t {
+    if (node < c.max_nodes) return node;
+    set_error(c, E_INTERNAL);
+    return NONE;
+  };
+  auto none = [](const StoreItem&) {};
+  place_units(
+      c, smem, (n + 31) / 32,
+      [&](uint64_t w) -> uint32_t {
+        const uint64_t i = w * 32 + lane;
+        return i < n ? checked(c.b_cur[i]) : NONE;
+      },
+      [&](uint64_t w, StoreItem& it) {
+        it.rec = __ldcg(pts + w * 32 + lane);
+        it.aux = (uint32_t)(base + w * 32 + lane);
+      },
+      none);
+  place_units(
+      c, smem, (uint64_t)t_hi * parts,
+      [&](uint64_t w) -> uint32_t {
         SpillTask tk;
-        uint32_t at;
-        valid[j] = task_point(c, (uint32_t)(e / 32u), parts, tk, at);
-        if (valid[j]) {
-          node[j] = c.sp_cur[tk.dst + at];
-          r[j] = chunk_recs(c, tk.ref)[at];
-          g[j] = chunk_aux(c, tk.ref)[at];
-        }
-      }
-      if (valid[j] && node[j] >= c.max_nodes) {
-        set_error(c, E_INTERNAL);
-        valid[j] = false;
-      }
-    }
-    place_items<U>(c, smem, valid, node, ref, q);
-#pragma unroll
-    for (int j = 0; j < U; ++j) put_rec(c, ref[j], q[j], r[j], g[j]);
-  }
+        uint32_t q;
+        return task_point(c, (uint32_t)w, parts, tk, q) ? checked(c.sp_cur[tk.dst + q]) : NONE;
+      },
+      [&](uint64_t w, StoreItem& it) {
+        SpillTask tk;
+        uint32_t q;
+        if (!task_point(c, (uint32_t)w, parts, tk, q)) return;
+        it.rec = chunk_recs(c, tk.ref)[q];
+        it.aux = chunk_aux(c, tk.ref)[q];
+      },
+      none);
 }
 
 // Store the n_keys new voxels, each at the next free slot of its node, set
@@ -1769,58 +1723,41 @@ __device__ void phase_store(const Ctx& c, uint32_t* smem, const int4* pts, uint6
 // raises it).
 __device__ void phase_store_voxels(const Ctx& c, uint32_t* smem, uint32_t n_tasks, uint32_t n_keys,
                                    int pool_top, uint64_t t0, uint64_t nthreads) {
-  constexpr int U = STORE_U;
-  const uint64_t blk = t0 - threadIdx.x, stride = nthreads;
-  const uint64_t me = threadIdx.x;
-#if SL_STORE_BLOCK
-  if (smem) block_place_init(smem);
-#endif
+  const uint32_t lane = lane_id();
   const uint32_t G = c.G, cmask = (1u << (3u * G)) - 1u, amask = (1u << G) - 1u;
-  for (uint64_t b0 = blk; b0 < n_keys; b0 += U * stride) {
-    bool valid[U];
-    uint32_t node[U], ref[U], q[U], cell[U], gref[U], rgba[U];
-    HSlot* sl[U];
-#pragma unroll
-    for (int j = 0; j < U; ++j) {
-      const uint64_t e = b0 + j * stride + me;
-      valid[j] = e < n_keys;
-      sl[j] = valid[j] ? c.hash + c.keys[e] : nullptr;
-    }
-#pragma unroll
-    for (int j = 0; j < U; ++j) {
-      const ulonglong2 kv = valid[j] ? *reinterpret_cast<const ulonglong2*>(sl[j])
-                                     : make_ulonglong2(0ull, 0ull);
-      rgba[j] = (uint32_t)kv.y;
-      node[j] = (uint32_t)(kv.x >> (3u * G));
-      cell[j] = (uint32_t)kv.x & cmask;
-    }
-    int4 nm[U];  // the node's min corner and level (voxel centre), loaded with its grid ref
-#pragma unroll
-    for (int j = 0; j < U; ++j) {
-      const bool in = valid[j] && node[j] < c.max_nodes;
-      gref[j] = in ? c.gridref[node[j]] : NONE;
-      nm[j] = in ? *reinterpret_cast<const int4*>(&c.meta[node[j]].min[0]) : make_int4(0, 0, 0, 0);
-      const bool ok = valid[j] && ref_ok(c, gref[j], c.grid_bytes);
-      if (valid[j] && !ok) set_error(c, E_INTERNAL);
-      valid[j] = ok;
-    }
-    place_items<U>(c, smem, valid, node, ref, q);
-#pragma unroll
-    for (int j = 0; j < U; ++j) {
-      if (!valid[j]) continue;
-      const uint32_t L = c.rlog2 - (uint32_t)nm[j].w;
-      const uint32_t cx = cell[j] & amask, cy = (cell[j] >> G) & amask, cz = cell[j] >> (2u * G);
-      // Section 3.4: the voxel is a point at the (floor of the) cell centre
-      int4 v;
-      v.x = nm[j].x + (int32_t)(((2ull * cx + 1ull) << L) >> (G + 1u));
-      v.y = nm[j].y + (int32_t)(((2ull * cy + 1ull) << L) >> (G + 1u));
-      v.z = nm[j].z + (int32_t)(((2ull * cz + 1ull) << L) >> (G + 1u));
-      v.w = (int32_t)rgba[j];
-      put_rec(c, ref[j], q[j], v, cell[j]);
-      atomicOr(grid_words(c, gref[j]) + (cell[j] >> 5), 1u << (cell[j] & 31u));
-      *reinterpret_cast<ulonglong2*>(sl[j]) = make_ulonglong2(HASH_EMPTY, HASH_EMPTY);
-    }
-  }
+  place_units(
+      c, smem, ((uint64_t)n_keys + 31) / 32,
+      [&](uint64_t w) -> uint32_t {
+        const uint64_t e = w * 32 + lane;
+        if (e >= n_keys) return NONE;
+        const uint32_t node = c.keys[e].y;
+        if (node < c.max_nodes) return node;
+        set_error(c, E_INTERNAL);
+        return NONE;
+      },
+      [&](uint64_t w, StoreItem& it) {
+        it.slot = c.keys[w * 32 + lane].x;
+        it.gref = c.gridref[it.node];
+        const ulonglong2 kv = *reinterpret_cast<const ulonglong2*>(c.hash + it.slot);
+        // the node's min corner and level
+        const int4 nm = *reinterpret_cast<const int4*>(&c.meta[it.node].min[0]);
+        const uint32_t L = c.rlog2 - (uint32_t)nm.w;
+        it.aux = (uint32_t)kv.x & cmask;  // the cell
+        const uint32_t cx = it.aux & amask, cy = (it.aux >> G) & amask, cz = it.aux >> (2u * G);
+        // Section 3.4: the voxel is a point at the (floor of the) cell centre
+        it.rec = make_int4(nm.x + (int32_t)(((2ull * cx + 1ull) << L) >> (G + 1u)),
+                           nm.y + (int32_t)(((2ull * cy + 1ull) << L) >> (G + 1u)),
+                           nm.z + (int32_t)(((2ull * cz + 1ull) << L) >> (G + 1u)), (int32_t)kv.y);
+        if (!ref_ok(c, it.gref, c.grid_bytes)) {
+          set_error(c, E_INTERNAL);
+          it.gref = NONE;
+        }
+      },
+      [&](const StoreItem& it) {
+        if (it.gref != NONE)
+          atomicOr(grid_words(c, it.gref) + (it.aux >> 5), 1u << (it.aux & 31u));
+        *reinterpret_cast<ulonglong2*>(c.hash + it.slot) = make_ulonglong2(HASH_EMPTY, HASH_EMPTY);
+      });
   const int top = pool_top > 0 ? pool_top : 0;
   if ((unsigned long long)top + n_tasks > c.max_chunks) {
     if (t0 == 0) set_error(c, E_POOL);

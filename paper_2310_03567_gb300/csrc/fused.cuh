@@ -307,7 +307,7 @@ __device__ __forceinline__ void fused_body(const Ctx& c, const BatchDesc* batche
           n_keys = min(SL_CV(nkeys, &c.ctl->nkeys), c.backlog_cap);
           if (n_keys) phase_decide(c, 0, n_hi, warp0, nwarps);  // chunks for the new voxels
         }
-        phase_store(c, smem, bd.pts, bd.n, base, t_hi, tid, nthreads);
+        phase_store(c, smem, bd.pts, bd.n, base, t_hi);
         if (!grid_barrier(c, f, vw)) return;
         clk.tick(c, PH_STORE);
         if (n_keys || t_hi) {

@@ -171,13 +171,14 @@ __global__ void __launch_bounds__(BLOCK) k_alloc_voxels(Ctx c, uint32_t r) {
 
 // The points and, their nodes' chunks being there too, the voxels; the last
 // block closes the update (a launch of its own took 5 us).
-__global__ void __launch_bounds__(BLOCK) k_store(Ctx c, const int4* pts, uint64_t n,
+__global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_store(Ctx c, const int4* pts, uint64_t n,
                                                   unsigned long long base, uint32_t t_hi,
                                                   uint32_t n_keys, int pool_top) {
+  extern __shared__ uint32_t smem[];
   const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   const uint64_t nt = (uint64_t)gridDim.x * blockDim.x;
-  phase_store(c, nullptr, pts, n, base, t_hi, t0, nt);
-  phase_store_voxels(c, nullptr, t_hi, n_keys, pool_top, t0, nt);
+  phase_store(c, smem, pts, n, base, t_hi);
+  phase_store_voxels(c, smem, t_hi, n_keys, pool_top, t0, nt);
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0 && atomicAdd(&c.ctl->store_blocks, 1u) + 1u == gridDim.x) {
@@ -553,7 +554,7 @@ bool plan_layout(const simlod_config* c, size_t arena_bytes, Layout* L) {
   L->scur = take(4 * N);
   L->vis = take(4 * N);
   L->hash = take(sizeof(HSlot) * L->hash_slots);
-  L->keys = take(sizeof(uint32_t) * c->backlog_capacity);
+  L->keys = take(sizeof(uint2) * c->backlog_capacity);
   L->staging = take(16 * B);
   const size_t fixed = align_up(o, 256);
   if (arena_bytes < fixed) return false;
@@ -599,7 +600,7 @@ void make_ctx(simlod_t* h) {
   c.hist_words = L.hist_words;
   c.scur = reinterpret_cast<uint32_t*>(a + L.scur);
   c.hash = reinterpret_cast<HSlot*>(a + L.hash);
-  c.keys = reinterpret_cast<uint32_t*>(a + L.keys);
+  c.keys = reinterpret_cast<uint2*>(a + L.keys);
   c.staging = reinterpret_cast<int4*>(a + L.staging);
   c.data = a + L.data;
   c.data_bytes = L.data_bytes;
@@ -608,6 +609,7 @@ void make_ctx(simlod_t* h) {
   c.rlog2 = g.root_log2;
   c.T = g.leaf_capacity;
   c.C = g.chunk_points;
+  div_constants(c.C, &c.C_mul, &c.C_shift);
   c.G = g.grid_log2;
   c.chunk_bytes = chunk_bytes_of(&g);
   c.chunk_units = c.chunk_bytes / REF_BYTES;
@@ -773,7 +775,8 @@ int insert_device(simlod_t* h, const int4* pts, uint64_t n, cudaStream_t s) {
   const int pool_top = t.pool_top;
   const uint64_t work = std::max<uint64_t>(std::max<uint64_t>(n, (uint64_t)t_hi * c.C), n_keys);
   rc = launch(h, K_STORE, s, [&] {
-    k_store<<<grid_for(h, work, BLOCK), BLOCK, 0, s>>>(c, pts, n, base, t_hi, n_keys, pool_top);
+    k_store<<<std::min(full, grid_for(h, work, PBLOCK)), PBLOCK, PHASE_SMEM_BYTES, s>>>(
+        c, pts, n, base, t_hi, n_keys, pool_top);
   });
   if (rc) return poison(h, rc);
   h->base += n;
@@ -935,6 +938,8 @@ SIMLOD_API int simlod_create(const simlod_config* cfg, void* d_arena, size_t are
       cudaFuncSetAttribute(k_hist, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            PHASE_SMEM_BYTES) != cudaSuccess ||
       cudaFuncSetAttribute(k_claim, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           PHASE_SMEM_BYTES) != cudaSuccess ||
+      cudaFuncSetAttribute(k_store, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            PHASE_SMEM_BYTES) != cudaSuccess ||
       cudaFuncSetAttribute(k_fused, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            PHASE_SMEM_BYTES) != cudaSuccess) {
