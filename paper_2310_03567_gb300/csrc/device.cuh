@@ -86,10 +86,7 @@ constexpr uint32_t CHUNK_HEADER = 16;
 #define SL_COUNT_PREFETCH 1
 #endif
 #ifndef SL_COUNT_UNROLL
-#define SL_COUNT_UNROLL 1
-#endif
-#ifndef SL_CLAIM_UNROLL
-#define SL_CLAIM_UNROLL 1
+#define SL_COUNT_UNROLL 2
 #endif
 #ifndef SL_STORE_UNROLL
 #define SL_STORE_UNROLL 2
@@ -116,7 +113,9 @@ constexpr uint32_t TALLY_LOG2 = 9;                      // block tally cache: 51
 constexpr uint32_t TALLY_SLOTS = 1u << TALLY_LOG2;
 // dynamic shared memory of the phase blocks: node cache, new-cell staging,
 // claim queues, block tally cache
-constexpr int CLAIM_U = SL_CLAIM_UNROLL;  // units of 32 points a warp claims for at once
+// units of 32 points a warp claims for at once (two: 0.99 against 0.94 ms of
+// claims on a 16M-point terrain, and spills)
+constexpr int CLAIM_U = 1;
 constexpr uint32_t CLAIM_QUEUE = 32 * (CLAIM_U + 1);  // points that wait for their next claim
 constexpr uint32_t SMEM_WBUF = NODE_CACHE;            // in u32 words
 constexpr uint32_t SMEM_QUEUE = SMEM_WBUF + (PHASE_BLOCK / 32) * WBUF * 2;
@@ -270,7 +269,9 @@ struct Ctx {
   uint32_t rlog2, T, C, G;
   uint32_t chunk_bytes, chunk_units, grid_bytes, dir_bytes, dir_cap;
   uint32_t hash_mask;
-  uint32_t C_mul, C_shift;  // division by C (div_C)
+  uint32_t C_mul, C_shift;  // division by C (div_by)
+  uint32_t parts, P_mul, P_shift;  // 32-record units per chunk, and division by them
+  uint32_t chunk_lim, grid_lim;    // first references whose chunk or grid would not fit
   uint32_t max_nodes, max_chunks, spill_cap, backlog_cap, max_splits;
   uint64_t max_batch;
   uint64_t hist_words;
@@ -301,6 +302,22 @@ __device__ __forceinline__ unsigned long long fmix64(unsigned long long k) {
 __device__ __forceinline__ void set_error(const Ctx& c, uint32_t bits) {
   atomicOr(&c.ctl->error, bits);
   atomicOr(c.launch_bar, BAR_ABORT);
+}
+
+// n / d for any 32-bit n: multiply, add and shift by the constants that Granlund
+// and Montgomery ("Division by invariant integers using multiplication", 1994)
+// give for a divisor (div_constants).
+__device__ __forceinline__ uint32_t div_by(uint32_t n, uint32_t d, uint32_t mul, uint32_t shift) {
+  if (d == 1u) return n;
+  const uint32_t t = __umulhi(mul, n);
+  return (t + ((n - t) >> 1)) >> shift;
+}
+
+inline void div_constants(uint32_t d, uint32_t* mul, uint32_t* shift) {  // d >= 1
+  uint32_t l = 0;
+  while ((1ull << l) < d) ++l;
+  *mul = (uint32_t)(((1ull << 32) * ((1ull << l) - d)) / d + 1ull);
+  *shift = l ? l - 1u : 0u;
 }
 
 __device__ __forceinline__ uint8_t* ref_ptr(const Ctx& c, uint32_t ref) {
@@ -339,6 +356,10 @@ __device__ __forceinline__ bool ref_ok(const Ctx& c, uint32_t ref, uint32_t byte
   return ref != NONE && (unsigned long long)ref * REF_BYTES + bytes <= c.data_bytes;
 }
 
+// References below these limits hold a whole chunk or grid (NONE never does).
+__device__ __forceinline__ bool chunk_ok(const Ctx& c, uint32_t ref) { return ref < c.chunk_lim; }
+__device__ __forceinline__ bool grid_ok(const Ctx& c, uint32_t ref) { return ref < c.grid_lim; }
+
 // An array of cap records at ref stays inside the data region.
 __device__ __forceinline__ bool array_ok(const Ctx& c, uint32_t ref, uint32_t cap) {
   return ref != NONE && (unsigned long long)ref * REF_BYTES + array_bytes(cap) <= c.data_bytes;
@@ -369,17 +390,19 @@ __device__ __forceinline__ uint32_t octant(uint32_t rx, uint32_t ry, uint32_t rz
   return ((rx >> s) & 1u) | (((ry >> s) & 1u) << 1) | (((rz >> s) & 1u) << 2);
 }
 
-// Cell of a point in the 2^G grid of a node of side 2^L: per axis
+// Cell of a point in the 2^G grid of a node of side 2^L (L <= 31): per axis
 // ((p - min) << G) >> L, where p - min is the low L bits of the root-relative
-// coordinate (Section 3.3).
-__device__ __forceinline__ uint32_t cell_axis(uint32_t r, uint32_t L, uint32_t G) {
-  uint32_t local = (L >= 32u) ? r : (r & ((1u << L) - 1u));
-  return (L >= G) ? (local >> (L - G)) : (local << (G - L));
-}
-
+// coordinate (Section 3.3); the result's G bits are those of r shifted by
+// L - G, whichever way.
 __device__ __forceinline__ uint32_t cell_index(uint32_t rx, uint32_t ry, uint32_t rz, uint32_t L,
                                                uint32_t G) {
-  return cell_axis(rx, L, G) | (cell_axis(ry, L, G) << G) | (cell_axis(rz, L, G) << (2u * G));
+  const uint32_t m = (1u << G) - 1u;
+  if (L >= G) {
+    const uint32_t sh = L - G;
+    return ((rx >> sh) & m) | (((ry >> sh) & m) << G) | (((rz >> sh) & m) << (2u * G));
+  }
+  const uint32_t sh = G - L;
+  return ((rx << sh) & m) | (((ry << sh) & m) << G) | (((rz << sh) & m) << (2u * G));
 }
 
 // ------------------------------------------------------- node-table cache
@@ -732,9 +755,9 @@ __device__ __forceinline__ void warp_tally(uint32_t* counters, uint32_t* smem, b
 // consecutive units are dealt out to the warps in turn (chunk q to warp q mod
 // nwarps), so that a warp's units are neighbours in the stream while the work
 // stays spread over the grid.
-__device__ __forceinline__ uint64_t warp_unit(uint64_t warp0, uint64_t nwarps, uint64_t k,
+__device__ __forceinline__ uint32_t warp_unit(uint32_t warp0, uint32_t nwarps, uint32_t k,
                                               uint32_t chl) {
-  return ((warp0 + (k >> chl) * nwarps) << chl) + (k & ((1ull << chl) - 1ull));
+  return ((warp0 + (k >> chl) * nwarps) << chl) + (k & ((1u << chl) - 1u));
 }
 
 // log2 of the count phase's chunk for `units` units: the largest power of two
@@ -743,9 +766,11 @@ __device__ __forceinline__ uint64_t warp_unit(uint64_t warp0, uint64_t nwarps, u
 // nodes and cells (measured on the clustered stream: 15.1 against 18.7 ms of
 // count phase with chunks of 4); batches too small to give every warp several
 // chunks keep single units (1M-point batches slowed down with chunks of 8).
-__device__ __forceinline__ uint32_t count_chunk_log2(uint64_t units, uint64_t nwarps) {
+__device__ __forceinline__ uint32_t count_chunk_log2(uint32_t units, uint32_t nwarps) {
   uint32_t chl = 0;
-  while (chl < SL_COUNT_CHUNK_MAX && units >= (nwarps * SL_COUNT_CHUNK_DIV) << (chl + 1)) ++chl;
+  while (chl < SL_COUNT_CHUNK_MAX &&
+         units >= (uint64_t)(nwarps * SL_COUNT_CHUNK_DIV) << (chl + 1))
+    ++chl;
   return chl;
 }
 
@@ -754,7 +779,7 @@ __device__ __forceinline__ uint32_t count_chunk_log2(uint64_t units, uint64_t nw
 // Iteration 1 for the batch points [0, n): descend and count. `smem` holds
 // PHASE_SMEM_BYTES of dynamic shared memory.
 __device__ void phase_count1(const Ctx& c, uint32_t* smem, const NodeCache nc, const int4* pts,
-                             uint64_t n, uint64_t warp0, uint64_t nwarps) {
+                             uint32_t n, uint32_t warp0, uint32_t nwarps) {
   constexpr int U = COUNT_U;
   tally_init(smem);
   __syncthreads();  // also publishes the caller's node-cache writes
@@ -766,21 +791,21 @@ __device__ void phase_count1(const Ctx& c, uint32_t* smem, const NodeCache nc, c
   int4 pn[U];
 #pragma unroll
   for (int j = 0; j < U; ++j) {
-    const uint64_t i = warp_unit(warp0, nwarps, j, chl) * 32 + lane;
+    const uint32_t i = warp_unit(warp0, nwarps, j, chl) * 32 + lane;
     pn[j] = i < n ? __ldcg(pts + i) : make_int4(0, 0, 0, 0);
   }
-  for (uint64_t k0 = 0; warp_unit(warp0, nwarps, k0, chl) * 32 < n; k0 += U) {
+  for (uint32_t k0 = 0; warp_unit(warp0, nwarps, k0, chl) * 32 < n; k0 += U) {
     bool valid[U], walking[U];
     uint32_t rx[U], ry[U], rz[U], node[U], L[U];
-    uint64_t iu[U];
+    uint32_t iu[U];
     bool any = false;
 #pragma unroll
     for (int j = 0; j < U; ++j) {
-      const uint64_t i = warp_unit(warp0, nwarps, k0 + j, chl) * 32 + lane;
+      const uint32_t i = warp_unit(warp0, nwarps, k0 + j, chl) * 32 + lane;
       iu[j] = i;
       valid[j] = i < n;
       const int4 p = pn[j];
-      const uint64_t inext = warp_unit(warp0, nwarps, k0 + j + U, chl) * 32 + lane;
+      const uint32_t inext = warp_unit(warp0, nwarps, k0 + j + U, chl) * 32 + lane;
       pn[j] = inext < n ? __ldcg(pts + inext) : make_int4(0, 0, 0, 0);
       if (!rel_coords(c, p, rx[j], ry[j], rz[j]) && valid[j]) {
         atomicOr(&c.ctl->reject, 1u);
@@ -823,16 +848,13 @@ __device__ void phase_count1(const Ctx& c, uint32_t* smem, const NodeCache nc, c
 
 // The spill tasks as units of 32 re-inserted points (a unit never crosses into
 // the next task).
-__device__ __forceinline__ uint32_t task_units(const Ctx& c) { return (c.C + 31u) / 32u; }
-
 // Lane's re-inserted point of unit u of the tasks [0, t_hi): its task, its
 // place in the task's chunk; false past the end of the task.
-__device__ __forceinline__ bool task_point(const Ctx& c, uint32_t u, uint32_t parts, SpillTask& tk,
-                                           uint32_t& q) {
-  const uint32_t t = u / parts;
-  q = (u - t * parts) * 32u + lane_id();
+__device__ __forceinline__ bool task_point(const Ctx& c, uint32_t u, SpillTask& tk, uint32_t& q) {
+  const uint32_t t = div_by(u, c.parts, c.P_mul, c.P_shift);
+  q = (u - t * c.parts) * 32u + lane_id();
   tk = c.tasks[t];
-  if (!ref_ok(c, tk.ref, c.chunk_bytes) || tk.n > c.C || tk.node >= c.max_nodes ||
+  if (!chunk_ok(c, tk.ref) || tk.n > c.C || tk.node >= c.max_nodes ||
       (unsigned long long)tk.dst + tk.n > c.spill_cap) {
     if (lane_id() == 0) set_error(c, E_INTERNAL);
     return false;
@@ -890,7 +912,7 @@ __host__ __device__ __forceinline__ uint32_t hist_depth(const Ctx& c, uint32_t K
 // point's cursor is its leaf; later the leaf is looked up (only leaves of the
 // lowest level of the round before split again, which is rare).
 __device__ void phase_hist(const Ctx& c, uint32_t* smem, const NodeCache nc, const int4* pts,
-                           uint64_t n, uint32_t t_hi, uint32_t s_lo, uint32_t K, uint32_t d,
+                           uint32_t n, uint32_t t_hi, uint32_t s_lo, uint32_t K, uint32_t d,
                            bool first) {
   tally_init(smem);
   __syncthreads();  // also publishes the caller's node-cache writes
@@ -898,22 +920,22 @@ __device__ void phase_hist(const Ctx& c, uint32_t* smem, const NodeCache nc, con
     if (blockIdx.x == 0 && threadIdx.x == 0) set_error(c, E_INTERNAL);
     return;  // (the same in every thread)
   }
-  const uint32_t lane = lane_id(), parts = task_units(c);
-  const uint64_t us = (uint64_t)t_hi * parts, units = us + (n + 31) / 32;
+  const uint32_t lane = lane_id();
+  const uint32_t us = t_hi * c.parts, units = us + (n + 31u) / 32u;
   // every block takes one range of neighbouring units: its points fall into
   // few cubes, whose counts its tally cache adds up (a shuffled building scan
   // of 40M points: 1.03 against 1.47 ms a pass with the units dealt out)
-  const uint64_t per = (units + gridDim.x - 1) / gridDim.x;
-  const uint64_t last = (blockIdx.x + 1ull) * per, end = last < units ? last : units;
-  for (uint64_t w = blockIdx.x * per + threadIdx.x / 32; w < end; w += blockDim.x / 32) {
+  const uint32_t per = (units + gridDim.x - 1u) / gridDim.x;
+  const uint32_t last = (blockIdx.x + 1u) * per, end = last < units ? last : units;
+  for (uint32_t w = blockIdx.x * per + threadIdx.x / 32u; w < end; w += blockDim.x / 32) {
     bool on = false, have = false;
     uint32_t cur = 0;
-    uint64_t i = 0;
+    uint32_t i = 0;
     int4 p = make_int4(0, 0, 0, 0);
     if (w < us) {
       SpillTask tk;
       uint32_t q;
-      on = have = task_point(c, (uint32_t)w, parts, tk, q);
+      on = have = task_point(c, w, tk, q);
       if (on) {
         p = chunk_recs(c, tk.ref)[q];
         cur = tk.node;
@@ -1087,7 +1109,7 @@ __device__ __forceinline__ void zero_grids(const Ctx& c, uint32_t s_hi, uint64_t
   for (uint64_t w = warp0; w < uz; w += nwarps) {
     const uint32_t id = c.splits[(uint32_t)(w / zpg)];
     const uint32_t gref = id < c.max_nodes ? c.gridref[id] : NONE;
-    if (!ref_ok(c, gref, c.grid_bytes)) {
+    if (!grid_ok(c, gref)) {
       if (lane == 0) set_error(c, E_INTERNAL);
       continue;
     }
@@ -1124,15 +1146,15 @@ struct ClaimArgs {
 };
 
 // All 32 lanes call: lanes with on[j] sample the grid of their node's parent.
-// SORTED: the items are units of consecutive batch points or of re-inserted
-// ones. gidx grows with the lane in the former, so that of a run of lanes in
-// one cell only the first has to claim, and the others are done (unless the
-// voxels do not nest). Points that have to go on join the queue, naming the
-// parent.
+// SORTED: the items are units of consecutive batch points or (respill) of
+// re-inserted ones of one chunk. A lane whose neighbour lane is in the same
+// cell with a lower index is done (unless the voxels do not nest); in a unit of
+// batch points the index grows with the lane, so only the left one can have
+// it. Points that have to go on join the queue, naming the parent.
 template <int N, bool SORTED>
 __device__ __forceinline__ void claim_level(const Ctx& c, WarpBuf& wb, ClaimQueue& cq,
                                             const ClaimArgs& a, const bool (&on)[N],
-                                            const ClaimItem (&it)[N]) {
+                                            const ClaimItem (&it)[N], bool respill) {
   const uint32_t lane = lane_id();
   uint32_t par[N], word[N], cell[N];
   bool want[N], more[N];
@@ -1150,7 +1172,7 @@ __device__ __forceinline__ void claim_level(const Ctx& c, WarpBuf& wb, ClaimQueu
     want[j] = false;
     if (up[j].x != NONE) {
       cell[j] = cell_index(it[j].rx, it[j].ry, it[j].rz, c.rlog2 - (up[j].x >> NODE_BITS), c.G);
-      if (!ref_ok(c, up[j].y, c.grid_bytes) || par[j] >= c.max_nodes) {
+      if (!grid_ok(c, up[j].y) || par[j] >= c.max_nodes) {
         set_error(c, E_INTERNAL);
       } else {
         want[j] = true;
@@ -1168,9 +1190,22 @@ __device__ __forceinline__ void claim_level(const Ctx& c, WarpBuf& wb, ClaimQueu
     val[j] = ((unsigned long long)it[j].gidx << 32) | it[j].rgba;
     lead[j] = want[j];
     if (SORTED) {
-      const LaneRun r = lane_run(want[j], key[j]);  // all lanes take part
-      // (a head wants its claim)
-      lead[j] = (it[j].node & RESPILL) || a.open ? want[j] : r.head;
+      // a neighbour lane in the same cell with a lower index: done
+      const unsigned wm = __ballot_sync(FULL_MASK, want[j]);
+      const uint32_t pc = __shfl_up_sync(FULL_MASK, cell[j], 1);
+      const uint32_t pp = __shfl_up_sync(FULL_MASK, par[j], 1);
+      const uint32_t pg = __shfl_up_sync(FULL_MASK, it[j].gidx, 1);
+      const bool left = lane != 0u && ((wm >> (lane - 1u)) & 1u) && pc == cell[j] &&
+                        pp == par[j] && pg < it[j].gidx;
+      bool beaten = left;
+      if (respill) {
+        const uint32_t nc2 = __shfl_down_sync(FULL_MASK, cell[j], 1);
+        const uint32_t np = __shfl_down_sync(FULL_MASK, par[j], 1);
+        const uint32_t ng = __shfl_down_sync(FULL_MASK, it[j].gidx, 1);
+        beaten = beaten || (lane != 31u && ((wm >> (lane + 1u)) & 1u) && nc2 == cell[j] &&
+                            np == par[j] && ng < it[j].gidx);
+      }
+      lead[j] = want[j] && (!beaten || a.open);
     }
   }
   warp_claim<N>(c, wb, lead, key, val, par, a.near, more);
@@ -1209,7 +1244,7 @@ __device__ __forceinline__ void claim_drain(const Ctx& c, WarpBuf& wb, ClaimQueu
                         q[4 * CLAIM_QUEUE], q[5 * CLAIM_QUEUE]};
     }
     __syncwarp();
-    claim_level<1, false>(c, wb, cq, a, on, it);
+    claim_level<1, false>(c, wb, cq, a, on, it, false);
   }
 }
 
@@ -1219,8 +1254,8 @@ __device__ __forceinline__ void claim_drain(const Ctx& c, WarpBuf& wb, ClaimQueu
 // points come first: they have the lowest indices, so batch points stop at
 // them. Each warp loads the next unit's points and cursors while it claims.
 __device__ void phase_claim(const Ctx& c, uint32_t* smem, const NodeCache nc, const int4* pts,
-                            uint64_t n, unsigned long long base, uint32_t t_hi, uint32_t s_hi,
-                            const ClaimArgs& a, uint64_t warp0, uint64_t nwarps) {
+                            uint32_t n, unsigned long long base, uint32_t t_hi, uint32_t s_hi,
+                            const ClaimArgs& a, uint32_t warp0, uint32_t nwarps) {
   constexpr int U = CLAIM_U;
   tally_init(smem);
   __syncthreads();  // also publishes the caller's node-cache writes
@@ -1229,26 +1264,26 @@ __device__ void phase_claim(const Ctx& c, uint32_t* smem, const NodeCache nc, co
   ClaimQueue cq;
   cq.q = smem + SMEM_QUEUE + (threadIdx.x / 32) * CLAIM_QUEUE * 6;
   cq.n = 0;
-  const uint32_t lane = lane_id(), parts = task_units(c);
+  const uint32_t lane = lane_id();
   // units [0, us) are re-inserted points, the rest batch points
-  const uint64_t us = (uint64_t)t_hi * parts, units = us + (n + 31) / 32;
+  const uint32_t us = t_hi * c.parts, units = us + (n + 31u) / 32u;
   const uint32_t chl = count_chunk_log2(units, nwarps);
   int4 pn[U];
   uint32_t curn[U], gn[U];
-  auto load = [&](uint64_t w, int4& p, uint32_t& cur, uint32_t& g) {  // cur = NONE: no point
+  auto load = [&](uint32_t w, int4& p, uint32_t& cur, uint32_t& g) {  // cur = NONE: no point
     p = make_int4(0, 0, 0, 0);
     cur = NONE;
     g = 0;
     if (w < us) {
       SpillTask tk;
       uint32_t q;
-      if (task_point(c, (uint32_t)w, parts, tk, q)) {
+      if (task_point(c, w, tk, q)) {
         p = chunk_recs(c, tk.ref)[q];
         g = chunk_aux(c, tk.ref)[q];
         cur = tk.node | RESPILL;
       }
     } else {
-      const uint64_t i = (w - us) * 32 + lane;
+      const uint32_t i = (w - us) * 32 + lane;
       if (i < n) {
         p = __ldcg(pts + i);
         g = (uint32_t)(base + i);
@@ -1258,12 +1293,12 @@ __device__ void phase_claim(const Ctx& c, uint32_t* smem, const NodeCache nc, co
   };
 #pragma unroll
   for (int j = 0; j < U; ++j) load(warp_unit(warp0, nwarps, j, chl), pn[j], curn[j], gn[j]);
-  for (uint64_t k = 0; warp_unit(warp0, nwarps, k, chl) < units; k += U) {
+  for (uint32_t k = 0; warp_unit(warp0, nwarps, k, chl) < units; k += U) {
     bool on[U];
     ClaimItem it[U];
 #pragma unroll
     for (int j = 0; j < U; ++j) {
-      const uint64_t w = warp_unit(warp0, nwarps, k + j, chl);
+      const uint32_t w = warp_unit(warp0, nwarps, k + j, chl);
       on[j] = curn[j] != NONE;
       it[j] = ClaimItem{curn[j], 0, 0, 0, (uint32_t)pn[j].w, gn[j]};
       rel_coords(c, pn[j], it[j].rx, it[j].ry, it[j].rz);
@@ -1272,15 +1307,15 @@ __device__ void phase_claim(const Ctx& c, uint32_t* smem, const NodeCache nc, co
         const uint32_t cur = it[j].node & ~RESPILL;
         const uint32_t leaf = walk_down(c, nc, cur, it[j].rx, it[j].ry, it[j].rz);
         if (w < us) {
-          const uint32_t t = (uint32_t)w / parts;
-          c.sp_cur[c.tasks[t].dst + ((uint32_t)w - t * parts) * 32u + lane] = leaf;
+          const uint32_t t = div_by(w, c.parts, c.P_mul, c.P_shift);
+          c.sp_cur[c.tasks[t].dst + (w - t * c.parts) * 32u + lane] = leaf;
         } else if (leaf != cur) {
           c.b_cur[(w - us) * 32 + lane] = leaf;
         }
         it[j].node = leaf | (it[j].node & RESPILL);
       }
     }
-    claim_level<U, true>(c, wb, cq, a, on, it);
+    claim_level<U, true>(c, wb, cq, a, on, it, warp_unit(warp0, nwarps, k, chl) < us);
     claim_drain(c, wb, cq, a, 31u);
   }
   claim_drain(c, wb, cq, a, 0u);
@@ -1496,22 +1531,6 @@ __device__ void phase_rollback(const Ctx& c, uint32_t n_nodes, uint64_t t0, uint
 
 // -------------------------------------------------------------- phase: store
 
-// n / C for any 32-bit n: multiply, add and shift by the constants that Granlund
-// and Montgomery ("Division by invariant integers using multiplication", 1994)
-// give for a divisor (div_constants).
-__device__ __forceinline__ uint32_t div_C(const Ctx& c, uint32_t n) {
-  if (c.C == 1u) return n;
-  const uint32_t t = __umulhi(c.C_mul, n);
-  return (t + ((n - t) >> 1)) >> c.C_shift;
-}
-
-inline void div_constants(uint32_t d, uint32_t* mul, uint32_t* shift) {  // d >= 1
-  uint32_t l = 0;
-  while ((1ull << l) < d) ++l;
-  *mul = (uint32_t)(((1ull << 32) * ((1ull << l) - d)) / d + 1ull);
-  *shift = l ? l - 1u : 0u;
-}
-
 // Slots of the items that one block stores (the table lies over the staging,
 // queue and tally regions, which the store phases do not use): the block
 // counts its items per node, takes one range per node with one atomicAdd on
@@ -1587,14 +1606,14 @@ struct StoreItem {
 // place. Equal nodes of a run of lanes share one reservation. Each warp carries
 // STORE_U units at a time.
 template <typename NodeOf, typename Load, typename Done>
-__device__ __forceinline__ void place_units(const Ctx& c, uint32_t* smem, uint64_t units,
+__device__ __forceinline__ void place_units(const Ctx& c, uint32_t* smem, uint32_t units,
                                             NodeOf&& node_of, Load&& load, Done&& done) {
   constexpr int U = STORE_U;
   const PlaceTable t = place_table(smem);
   const uint32_t lane = lane_id();
-  const uint64_t per = (units + gridDim.x - 1) / gridDim.x;
-  const uint64_t first = blockIdx.x * per, last = (blockIdx.x + 1ull) * per;
-  const uint64_t lo = first + threadIdx.x / 32, hi = last < units ? last : units;
+  const uint32_t per = (units + gridDim.x - 1u) / gridDim.x;
+  const uint32_t first = blockIdx.x * per, last = first + per;
+  const uint32_t lo = first + threadIdx.x / 32u, hi = last < units ? last : units;
   const uint32_t wpb = blockDim.x / 32;
   if (first >= units) return;  // (all threads of the block alike)
   __syncthreads();             // the regions' last use is over
@@ -1603,7 +1622,7 @@ __device__ __forceinline__ void place_units(const Ctx& c, uint32_t* smem, uint64
     t.next[i] = 0;
   }
   __syncthreads();
-  for (uint64_t w = lo; w < hi; w += wpb) {
+  for (uint32_t w = lo; w < hi; w += wpb) {
     const uint32_t node = node_of(w);
     const LaneRun r = lane_run(node != NONE, node);
     if (r.head) {
@@ -1622,13 +1641,13 @@ __device__ __forceinline__ void place_units(const Ctx& c, uint32_t* smem, uint64
     t.seq[i] = map.z;
   }
   __syncthreads();
-  for (uint64_t w0 = lo; w0 < hi; w0 += U * wpb) {
+  for (uint32_t w0 = lo; w0 < hi; w0 += U * wpb) {
     StoreItem it[U];
     uint32_t slot[U];
     uint32_t nch[U], tail[U], seq[U];
 #pragma unroll
     for (int j = 0; j < U; ++j) {
-      const uint64_t w = w0 + j * wpb;
+      const uint32_t w = w0 + j * wpb;
       it[j] = StoreItem{w < hi ? node_of(w) : NONE, make_int4(0, 0, 0, 0), 0, 0, 0};
     }
 #pragma unroll
@@ -1660,7 +1679,7 @@ __device__ __forceinline__ void place_units(const Ctx& c, uint32_t* smem, uint64
 #pragma unroll
     for (int j = 0; j < U; ++j) {
       if (it[j].node == NONE) continue;
-      const uint32_t k = div_C(c, slot[j]), q = slot[j] - k * c.C;
+      const uint32_t k = div_by(slot[j], c.C, c.C_mul, c.C_shift), q = slot[j] - k * c.C;
       uint32_t ref = NONE;
       if (k + 1u == nch[j]) {
         ref = tail[j];
@@ -1668,7 +1687,7 @@ __device__ __forceinline__ void place_units(const Ctx& c, uint32_t* smem, uint64
         const unsigned long long a = (unsigned long long)seq[j] + (k - nch[j]);
         if (a < c.max_chunks) ref = c.alloc_refs[a];
       }
-      if (!ref_ok(c, ref, c.chunk_bytes)) {
+      if (!chunk_ok(c, ref)) {
         set_error(c, E_INTERNAL);
         continue;
       }
@@ -1680,41 +1699,43 @@ __device__ __forceinline__ void place_units(const Ctx& c, uint32_t* smem, uint64
 
 // Store the batch points and the re-inserted points (of the spill tasks
 // [0, t_hi), still in their old chunks), each at the next free slot of its leaf.
-__device__ void phase_store(const Ctx& c, uint32_t* smem, const int4* pts, uint64_t n,
+__device__ void phase_store(const Ctx& c, uint32_t* smem, const int4* pts, uint32_t n,
                             unsigned long long base, uint32_t t_hi) {
-  const uint32_t lane = lane_id(), parts = task_units(c);
-  auto checked = [&](uint32_t node) -> uint32_t {
-    if (node < c.max_nodes) return node;
-    set_error(c, E_INTERNAL);
-    return NONE;
-  };
-  auto none = [](const StoreItem&) {};
+  const uint32_t lane = lane_id();
+  // units [0, us) are re-inserted points, the rest batch points
+  const uint32_t us = t_hi * c.parts;
   place_units(
-      c, smem, (n + 31) / 32,
-      [&](uint64_t w) -> uint32_t {
-        const uint64_t i = w * 32 + lane;
-        return i < n ? checked(c.b_cur[i]) : NONE;
+      c, smem, us + (n + 31u) / 32u,
+      [&](uint32_t w) -> uint32_t {
+        uint32_t node = NONE;
+        if (w < us) {
+          SpillTask tk;
+          uint32_t q;
+          if (!task_point(c, w, tk, q)) return NONE;
+          node = c.sp_cur[tk.dst + q];
+        } else {
+          const uint32_t i = (w - us) * 32u + lane;
+          if (i >= n) return NONE;
+          node = c.b_cur[i];
+        }
+        if (node < c.max_nodes) return node;
+        set_error(c, E_INTERNAL);
+        return NONE;
       },
-      [&](uint64_t w, StoreItem& it) {
-        it.rec = __ldcg(pts + w * 32 + lane);
-        it.aux = (uint32_t)(base + w * 32 + lane);
+      [&](uint32_t w, StoreItem& it) {
+        if (w < us) {
+          SpillTask tk;
+          uint32_t q;
+          if (!task_point(c, w, tk, q)) return;
+          it.rec = chunk_recs(c, tk.ref)[q];
+          it.aux = chunk_aux(c, tk.ref)[q];
+        } else {
+          const uint32_t i = (w - us) * 32u + lane;
+          it.rec = __ldcg(pts + i);
+          it.aux = (uint32_t)(base + i);
+        }
       },
-      none);
-  place_units(
-      c, smem, (uint64_t)t_hi * parts,
-      [&](uint64_t w) -> uint32_t {
-        SpillTask tk;
-        uint32_t q;
-        return task_point(c, (uint32_t)w, parts, tk, q) ? checked(c.sp_cur[tk.dst + q]) : NONE;
-      },
-      [&](uint64_t w, StoreItem& it) {
-        SpillTask tk;
-        uint32_t q;
-        if (!task_point(c, (uint32_t)w, parts, tk, q)) return;
-        it.rec = chunk_recs(c, tk.ref)[q];
-        it.aux = chunk_aux(c, tk.ref)[q];
-      },
-      none);
+      [](const StoreItem&) {});
 }
 
 // Store the n_keys new voxels, each at the next free slot of its node, set
@@ -1726,17 +1747,17 @@ __device__ void phase_store_voxels(const Ctx& c, uint32_t* smem, uint32_t n_task
   const uint32_t lane = lane_id();
   const uint32_t G = c.G, cmask = (1u << (3u * G)) - 1u, amask = (1u << G) - 1u;
   place_units(
-      c, smem, ((uint64_t)n_keys + 31) / 32,
-      [&](uint64_t w) -> uint32_t {
-        const uint64_t e = w * 32 + lane;
+      c, smem, n_keys / 32u + (n_keys % 32u ? 1u : 0u),
+      [&](uint32_t w) -> uint32_t {
+        const uint32_t e = w * 32u + lane;
         if (e >= n_keys) return NONE;
         const uint32_t node = c.keys[e].y;
         if (node < c.max_nodes) return node;
         set_error(c, E_INTERNAL);
         return NONE;
       },
-      [&](uint64_t w, StoreItem& it) {
-        it.slot = c.keys[w * 32 + lane].x;
+      [&](uint32_t w, StoreItem& it) {
+        it.slot = c.keys[w * 32u + lane].x;
         it.gref = c.gridref[it.node];
         const ulonglong2 kv = *reinterpret_cast<const ulonglong2*>(c.hash + it.slot);
         // the node's min corner and level
@@ -1748,7 +1769,7 @@ __device__ void phase_store_voxels(const Ctx& c, uint32_t* smem, uint32_t n_task
         it.rec = make_int4(nm.x + (int32_t)(((2ull * cx + 1ull) << L) >> (G + 1u)),
                            nm.y + (int32_t)(((2ull * cy + 1ull) << L) >> (G + 1u)),
                            nm.z + (int32_t)(((2ull * cz + 1ull) << L) >> (G + 1u)), (int32_t)kv.y);
-        if (!ref_ok(c, it.gref, c.grid_bytes)) {
+        if (!grid_ok(c, it.gref)) {
           set_error(c, E_INTERNAL);
           it.gref = NONE;
         }

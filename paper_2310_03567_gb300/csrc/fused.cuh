@@ -207,7 +207,7 @@ __device__ __forceinline__ void fused_body(const Ctx& c, const BatchDesc* batche
                                            const unsigned int* ready) {
   const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const uint64_t nthreads = (uint64_t)gridDim.x * blockDim.x;
-  const uint64_t warp0 = tid / 32, nwarps = nthreads / 32;
+  const uint32_t warp0 = (uint32_t)(tid / 32), nwarps = (uint32_t)(nthreads / 32);
   const unsigned long long t_begin = globaltimer_ns();
   extern __shared__ uint32_t smem[];  // node-table cache (PHASE_SMEM_BYTES)
   PhaseClock clk{t_begin};
@@ -248,7 +248,7 @@ __device__ __forceinline__ void fused_body(const Ctx& c, const BatchDesc* batche
       bd.pts = c.staging;
     }
     if (bd.n) {
-      phase_count1(c, smem, node_cache_at(smem, nodes0), bd.pts, bd.n, warp0, nwarps);
+      phase_count1(c, smem, node_cache_at(smem, nodes0), bd.pts, (uint32_t)bd.n, warp0, nwarps);
       if (!grid_barrier(c, f, vw)) return;
       clk.tick(c, PH_COUNT);
       rejected = SL_CV(reject, &c.ctl->reject) != 0u;  // set only by the count round
@@ -276,7 +276,7 @@ __device__ __forceinline__ void fused_body(const Ctx& c, const BatchDesc* batche
           if (K == 0u) break;
           const uint32_t d = hist_depth(c, K, bd.n + SL_CV(spill_count, &c.ctl->spill_count),
                                         SL_CV(split_most, &c.ctl->split_most));
-          phase_hist(c, smem, node_cache_at(smem, n_hi), bd.pts, bd.n, t_hi, s_hi, K, d, first);
+          phase_hist(c, smem, node_cache_at(smem, n_hi), bd.pts, (uint32_t)bd.n, t_hi, s_hi, K, d, first);
           if (!grid_barrier(c, f)) return;
           phase_build(c, s_hi, K, d, lvl0, max_iters);
           if (!grid_barrier(c, f, vw)) return;
@@ -300,14 +300,14 @@ __device__ __forceinline__ void fused_body(const Ctx& c, const BatchDesc* batche
                            claim_near_mask(c, bd.n + n_spill, SL_CV(key_rate, &c.ctl->key_rate))};
         uint32_t n_keys = 0;
         if (n_hi > 1u) {  // (an octree of one leaf has no voxels)
-          phase_claim(c, smem, node_cache_at(smem, n_hi), bd.pts, bd.n, base, t_hi, s_hi, ca,
+          phase_claim(c, smem, node_cache_at(smem, n_hi), bd.pts, (uint32_t)bd.n, base, t_hi, s_hi, ca,
                       warp0, nwarps);
           if (!grid_barrier(c, f, vw)) return;
           clk.tick(c, PH_CLAIM);
           n_keys = min(SL_CV(nkeys, &c.ctl->nkeys), c.backlog_cap);
-          if (n_keys) phase_decide(c, 0, n_hi, warp0, nwarps);  // chunks for the new voxels
         }
-        phase_store(c, smem, bd.pts, bd.n, base, t_hi);
+        phase_store(c, smem, bd.pts, (uint32_t)bd.n, base, t_hi);
+        if (n_keys) phase_decide(c, 0, n_hi, warp0, nwarps);  // chunks for the new voxels
         if (!grid_barrier(c, f, vw)) return;
         clk.tick(c, PH_STORE);
         if (n_keys || t_hi) {

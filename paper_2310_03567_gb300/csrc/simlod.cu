@@ -610,10 +610,17 @@ void make_ctx(simlod_t* h) {
   c.T = g.leaf_capacity;
   c.C = g.chunk_points;
   div_constants(c.C, &c.C_mul, &c.C_shift);
+  c.parts = (c.C + 31u) / 32u;
+  div_constants(c.parts, &c.P_mul, &c.P_shift);
   c.G = g.grid_log2;
   c.chunk_bytes = chunk_bytes_of(&g);
   c.chunk_units = c.chunk_bytes / REF_BYTES;
   c.grid_bytes = grid_bytes_of(&g);
+  auto ref_limit = [&](uint64_t bytes) -> uint32_t {
+    return L.data_bytes < bytes ? 0u : (uint32_t)((L.data_bytes - bytes) / REF_BYTES + 1u);
+  };
+  c.chunk_lim = ref_limit(c.chunk_bytes);
+  c.grid_lim = ref_limit(c.grid_bytes);
   c.dir_bytes = dir_bytes_of(&g);
   c.dir_cap = dir_cap_of(&g);
   c.hash_mask = (uint32_t)(L.hash_slots - 1);
