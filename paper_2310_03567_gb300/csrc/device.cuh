@@ -1001,11 +1001,17 @@ __device__ void phase_build(const Ctx& c, uint32_t s_lo, uint32_t K, uint32_t d,
     const int32_t rm[3] = {m.min[0], m.min[1], m.min[2]};
     if (threadIdx.x == 0) s_n = s_deep = 0;
     for (uint32_t j = d; j-- > 0;) {
-      const uint32_t* below = j + 1u == d ? hist : up + level_first(j + 1u);
+      const uint32_t* below = up + level_first(j + 1u);
+      const uint4* bins4 = reinterpret_cast<const uint4*>(hist);
       for (uint32_t q = threadIdx.x; q < (1u << (3u * j)); q += blockDim.x) {
         uint32_t t = 0;
+        if (j + 1u == d) {
+          const uint4 a = bins4[2u * q], b = bins4[2u * q + 1u];
+          t = a.x + a.y + a.z + a.w + b.x + b.y + b.z + b.w;
+        } else {
 #pragma unroll
-        for (uint32_t o = 0; o < 8; ++o) t += below[8u * q + o];
+          for (uint32_t o = 0; o < 8; ++o) t += below[8u * q + o];
+        }
         up[level_first(j) + q] = t;
       }
       __syncthreads();
