@@ -3,12 +3,15 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <memory>
 #include <new>
+#include <thread>
 #include <vector>
 
 #include "device.cuh"
@@ -1433,6 +1436,40 @@ SIMLOD_API int simlod_set_wait_limits(simlod_t* h, uint64_t barrier_ns, uint64_t
   return SIMLOD_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// Host side of checkpoints: f(k) for every node k in [0, n), on several threads
+// when there are enough records (a node's records are unpacked, sorted or
+// packed by one thread). f does not throw.
+template <typename F>
+void for_each_node(uint64_t n, uint64_t records, F&& f) {
+  constexpr uint64_t GRAIN = 4, PER_THREAD = 1u << 15;
+  std::atomic<uint64_t> next{0};
+  auto work = [&] {
+    for (uint64_t k; (k = next.fetch_add(GRAIN, std::memory_order_relaxed)) < n;)
+      for (uint64_t i = k; i < std::min(k + GRAIN, n); ++i) f(i);
+  };
+  const uint64_t want = std::min<uint64_t>(
+      {records / PER_THREAD, std::max(1u, std::thread::hardware_concurrency()), 16u});
+  std::thread pool[16];
+  uint64_t made = 0;
+  try {
+    while (made + 1u < want) {
+      pool[made] = std::thread(work);
+      ++made;
+    }
+  } catch (...) {  // no more threads: the ones there are do the work
+  }
+  work();
+  for (uint64_t t = 0; t < made; ++t) pool[t].join();
+}
+
+}  // namespace
+
+extern "C" {
+
 // ----------------------------------------------------------------- restore
 
 SIMLOD_API int simlod_restore(simlod_t* h, const simlod_snapshot_t* snap, void* stream) {
@@ -1515,21 +1552,24 @@ SIMLOD_API int simlod_restore(simlod_t* h, const simlod_snapshot_t* snap, void* 
   }
   if (bytes > h->lay.data_bytes) return SIMLOD_ERR_ARENA_FULL;
   if (chunks > h->lay.max_chunks) return SIMLOD_ERR_ARENA_FULL;
-  std::vector<uint8_t> data;
-  try {
-    data.assign(bytes, 0);
-  } catch (const std::bad_alloc&) {
-    return SIMLOD_ERR_INVALID_ARG;
-  }
+  // (not zeroed: every byte that is read later is written below)
+  std::unique_ptr<uint8_t[]> image(new (std::nothrow) uint8_t[bytes + 1]);
+  if (!image) return SIMLOD_ERR_INVALID_ARG;
+  uint8_t* const data = image.get();
   std::vector<uint32_t> child(n), gridref(n), num(n), zeros(n, 0);
   std::vector<NodeMeta> meta(n);
+  std::vector<uint64_t> place(n);  // a node's grid or directory; its chunks follow
   uint64_t bump = 0;
-  auto take = [&](uint64_t b) {
-    const uint64_t at = bump;
-    bump += b;
-    return at;
-  };
   for (uint64_t id = 0; id < n; ++id) {
+    const simlod_node_rec& rec = nodes[rec_of[id]];
+    place[id] = bump;
+    gridref[id] = rec.is_inner ? (uint32_t)(bump / REF_BYTES) : NONE;
+    child[id] = rec.is_inner ? first_child[id] : NONE;
+    num[id] = (uint32_t)(rec.is_inner ? rec.n_voxels : rec.n_points);
+    bump += (rec.is_inner ? gb : db) + rec.n_chunks * cb;
+  }
+  std::atomic<bool> bad{false};
+  for_each_node(n, snap->n_points + snap->n_voxels, [&](uint64_t id) {
     const uint32_t r = rec_of[id];
     const simlod_node_rec& rec = nodes[r];
     NodeMeta m;
@@ -1540,37 +1580,38 @@ SIMLOD_API int simlod_restore(simlod_t* h, const simlod_snapshot_t* snap, void* 
     m.level = rec.level;
     m.st_tail = NONE;
     m.head = m.tail = NONE;
+    uint64_t at = place[id];
     uint32_t* dir = nullptr;
     if (rec.is_inner) {
-      const uint64_t go = take(gb);
-      uint32_t* words = reinterpret_cast<uint32_t*>(data.data() + go);
+      uint32_t* words = reinterpret_cast<uint32_t*>(data + at);
+      memset(words, 0, gb);
       for (uint64_t q = vo[r]; q < vo[r + 1]; ++q) {
         const uint32_t cell = snap->voxels[q].cell;
-        if (cell >> (3 * G)) return SIMLOD_ERR_INVALID_ARG;
+        if (cell >> (3 * G)) {
+          bad = true;
+          return;
+        }
         words[cell >> 5] |= 1u << (cell & 31u);
       }
-      gridref[id] = (uint32_t)(go / REF_BYTES);
-      child[id] = first_child[id];
-      num[id] = (uint32_t)rec.n_voxels;
       m.dir = NONE;
+      at += gb;
     } else {
-      const uint64_t d = take(db);
-      dir = reinterpret_cast<uint32_t*>(data.data() + d);
-      gridref[id] = NONE;
-      child[id] = NONE;
-      num[id] = (uint32_t)rec.n_points;
-      m.dir = (uint32_t)(d / REF_BYTES);
+      dir = reinterpret_cast<uint32_t*>(data + at);
+      memset(dir, 0, db);
+      m.dir = (uint32_t)(at / REF_BYTES);
+      at += db;
     }
     const uint64_t cnt = rec.is_inner ? rec.n_voxels : rec.n_points;
-    uint32_t prev = NONE;
-    for (uint64_t j = 0; j < rec.n_chunks; ++j) {
-      const uint64_t co = take(cb);
-      const uint32_t ref = (uint32_t)(co / REF_BYTES);
-      uint8_t* ch = data.data() + co;
-      *reinterpret_cast<uint32_t*>(ch) = NONE;
+    for (uint64_t j = 0; j < rec.n_chunks; ++j, at += cb) {
+      const uint32_t ref = (uint32_t)(at / REF_BYTES);
+      uint8_t* ch = data + at;
+      memset(ch, 0, CHUNK_HEADER);
+      *reinterpret_cast<uint32_t*>(ch) =
+          j + 1 < rec.n_chunks ? (uint32_t)((at + cb) / REF_BYTES) : NONE;
       int4* recs = reinterpret_cast<int4*>(ch + CHUNK_HEADER);
       uint32_t* aux = reinterpret_cast<uint32_t*>(ch + CHUNK_HEADER + 16ull * C);
-      for (uint64_t q = 0; q < C && j * C + q < cnt; ++q) {
+      const uint64_t fill = std::min<uint64_t>(C, cnt - j * C);
+      for (uint64_t q = 0; q < fill; ++q) {
         if (rec.is_inner) {
           const simlod_voxel_rec& v = snap->voxels[vo[r] + j * C + q];
           recs[q] = make_int4(v.x, v.y, v.z, (int)v.rgba);
@@ -1581,15 +1622,14 @@ SIMLOD_API int simlod_restore(simlod_t* h, const simlod_snapshot_t* snap, void* 
           aux[q] = p.gidx;
         }
       }
-      if (prev == NONE) m.head = ref;
-      else *reinterpret_cast<uint32_t*>(data.data() + (uint64_t)prev * REF_BYTES) = ref;
+      if (j == 0) m.head = ref;
       if (dir && j < dcap) dir[j] = ref;
-      prev = ref;
+      m.tail = ref;
     }
-    m.tail = prev;
     m.n_chunks = (uint32_t)rec.n_chunks;
     meta[id] = m;
-  }
+  });
+  if (bad) return SIMLOD_ERR_INVALID_ARG;
   // start from an empty octree (clears a poisoned state and the claim table)
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const bool dirty = h->sticky != 0;
@@ -1618,7 +1658,7 @@ SIMLOD_API int simlod_restore(simlod_t* h, const simlod_snapshot_t* snap, void* 
       cudaMemcpy(c.scur, zeros.data(), 4 * n, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(c.meta, meta.data(), sizeof(NodeMeta) * n, cudaMemcpyHostToDevice) !=
           cudaSuccess ||
-      (bump && cudaMemcpy(c.data, data.data(), bump, cudaMemcpyHostToDevice) != cudaSuccess) ||
+      (bump && cudaMemcpy(c.data, data, bump, cudaMemcpyHostToDevice) != cudaSuccess) ||
       cudaMemcpy(c.ctl, &t, sizeof(Ctl), cudaMemcpyHostToDevice) != cudaSuccess)
     return poison(h, SIMLOD_ERR_CUDA);
   k_check_nested<<<(unsigned)std::min<uint64_t>(n, (uint64_t)h->sm_count * 8), BLOCK, 0, s>>>(c);
@@ -1751,14 +1791,9 @@ SIMLOD_API int simlod_snapshot(simlod_t* h, simlod_snapshot_t* snap) {
   if (t.error) return poison(h, error_from_bits(t.error));
   const uint32_t n = t.n_nodes;
   std::vector<uint32_t> child(n), num(n);
-  std::vector<NodeMeta> meta(n);
-  std::vector<uint8_t> data(t.bump);
   const Ctx& c = h->ctx;
   if (cudaMemcpy(child.data(), c.child, 4ull * n, cudaMemcpyDeviceToHost) != cudaSuccess ||
-      cudaMemcpy(num.data(), c.num, 4ull * n, cudaMemcpyDeviceToHost) != cudaSuccess ||
-      cudaMemcpy(meta.data(), c.meta, sizeof(NodeMeta) * n, cudaMemcpyDeviceToHost) !=
-          cudaSuccess ||
-      (t.bump && cudaMemcpy(data.data(), c.data, t.bump, cudaMemcpyDeviceToHost) != cudaSuccess))
+      cudaMemcpy(num.data(), c.num, 4ull * n, cudaMemcpyDeviceToHost) != cudaSuccess)
     return poison(h, SIMLOD_ERR_CUDA);
   uint64_t np = 0, nv = 0;
   for (uint32_t i = 0; i < n; ++i) (child[i] == NONE ? np : nv) += num[i];
@@ -1769,7 +1804,16 @@ SIMLOD_API int simlod_snapshot(simlod_t* h, simlod_snapshot_t* snap) {
   if (!snap->nodes || snap->nodes_capacity < n || (np && (!snap->points ||
       snap->points_capacity < np)) || (nv && (!snap->voxels || snap->voxels_capacity < nv)))
     return SIMLOD_ERR_INVALID_ARG;
-  const uint32_t C = h->cfg.chunk_points, G = h->cfg.grid_log2;
+  std::vector<NodeMeta> meta(n);
+  std::unique_ptr<uint8_t[]> image(new (std::nothrow) uint8_t[t.bump + 1]);
+  if (!image) return SIMLOD_ERR_INVALID_ARG;
+  const uint8_t* const data = image.get();
+  const uint64_t data_size = t.bump;
+  if (cudaMemcpy(meta.data(), c.meta, sizeof(NodeMeta) * n, cudaMemcpyDeviceToHost) !=
+          cudaSuccess ||
+      (t.bump && cudaMemcpy(image.get(), c.data, t.bump, cudaMemcpyDeviceToHost) != cudaSuccess))
+    return poison(h, SIMLOD_ERR_CUDA);
+  const uint32_t C = h->cfg.chunk_points;
   struct Key {
     uint32_t level, ix, iy, iz, id;
   };
@@ -1788,9 +1832,15 @@ SIMLOD_API int simlod_snapshot(simlod_t* h, simlod_snapshot_t* snap) {
     return a.iz < b.iz;
   });
   const uint64_t chunk_bytes = chunk_bytes_of(&h->cfg);
+  std::vector<uint64_t> first(n);  // of a node's points or voxels among the output's
   uint64_t po = 0, vo = 0;
-  int bad = 0;
   for (uint32_t k = 0; k < n; ++k) {
+    uint64_t& o = child[keys[k].id] != NONE ? vo : po;
+    first[k] = o;
+    o += num[keys[k].id];
+  }
+  std::atomic<bool> bad{false};
+  for_each_node(n, np + nv, [&](uint64_t k) {
     const uint32_t i = keys[k].id;
     const NodeMeta& m = meta[i];
     const bool inner = child[i] != NONE;
@@ -1804,23 +1854,23 @@ SIMLOD_API int simlod_snapshot(simlod_t* h, simlod_snapshot_t* snap) {
     r.n_points = inner ? 0 : num[i];
     r.n_voxels = inner ? num[i] : 0;
     uint64_t walked = 0, idx = 0;
+    auto put = [&](const int4& v, uint32_t aux) {
+      if (inner) {
+        snap->voxels[first[k] + idx] = simlod_voxel_rec{aux, v.x, v.y, v.z, (uint32_t)v.w};
+      } else {
+        snap->points[first[k] + idx] = simlod_point_rec{v.x, v.y, v.z, (uint32_t)v.w, aux};
+      }
+    };
     if (m.compact) {  // one contiguous array (simlod_compact)
       const uint64_t off = (uint64_t)m.head * REF_BYTES;
       const uint64_t cap = num[i];
-      if (m.head == NONE || off + CHUNK_HEADER + 20 * cap > data.size()) {
-        bad = 1;
+      if (m.head == NONE || off + CHUNK_HEADER + 20 * cap > data_size) {
+        bad = true;
       } else {
-        const int4* recs = reinterpret_cast<const int4*>(data.data() + off + CHUNK_HEADER);
+        const int4* recs = reinterpret_cast<const int4*>(data + off + CHUNK_HEADER);
         const uint32_t* aux =
-            reinterpret_cast<const uint32_t*>(data.data() + off + CHUNK_HEADER + 16 * cap);
-        for (; idx < cap; ++idx) {
-          const int4 v = recs[idx];
-          if (inner) {
-            snap->voxels[vo + idx] = simlod_voxel_rec{aux[idx], v.x, v.y, v.z, (uint32_t)v.w};
-          } else {
-            snap->points[po + idx] = simlod_point_rec{v.x, v.y, v.z, (uint32_t)v.w, aux[idx]};
-          }
-        }
+            reinterpret_cast<const uint32_t*>(data + off + CHUNK_HEADER + 16 * cap);
+        for (; idx < cap; ++idx) put(recs[idx], aux[idx]);
       }
       walked = (num[i] + C - 1) / C;  // the chunks the node would take
     }
@@ -1828,36 +1878,26 @@ SIMLOD_API int simlod_snapshot(simlod_t* h, simlod_snapshot_t* snap) {
     for (uint32_t ref = m.compact ? NONE : m.head; ref != NONE && walked <= m.n_chunks;
          ++walked) {
       const uint64_t off = (uint64_t)ref * REF_BYTES;
-      if (off + chunk_bytes > data.size()) {
-        bad = 1;
+      if (off + chunk_bytes > data_size) {
+        bad = true;
         break;
       }
-      const uint8_t* ch = data.data() + off;
+      const uint8_t* ch = data + off;
       const int4* recs = reinterpret_cast<const int4*>(ch + CHUNK_HEADER);
       const uint32_t* aux = reinterpret_cast<const uint32_t*>(ch + CHUNK_HEADER + 16ull * C);
-      for (uint32_t q = 0; q < C && idx < num[i]; ++q, ++idx) {
-        const int4 v = recs[q];
-        if (inner) {
-          snap->voxels[vo + idx] = simlod_voxel_rec{aux[q], v.x, v.y, v.z, (uint32_t)v.w};
-        } else {
-          snap->points[po + idx] = simlod_point_rec{v.x, v.y, v.z, (uint32_t)v.w, aux[q]};
-        }
-      }
+      for (uint32_t q = 0; q < C && idx < num[i]; ++q, ++idx) put(recs[q], aux[q]);
       ref = *reinterpret_cast<const uint32_t*>(ch);
     }
-    if (idx != num[i]) bad = 1;
+    if (idx != num[i]) bad = true;
     r.n_chunks = walked;
     if (inner) {
-      std::sort(snap->voxels + vo, snap->voxels + vo + num[i],
+      std::sort(snap->voxels + first[k], snap->voxels + first[k] + num[i],
                 [](const simlod_voxel_rec& a, const simlod_voxel_rec& b) { return a.cell < b.cell; });
-      vo += num[i];
     } else {
-      std::sort(snap->points + po, snap->points + po + num[i],
+      std::sort(snap->points + first[k], snap->points + first[k] + num[i],
                 [](const simlod_point_rec& a, const simlod_point_rec& b) { return a.gidx < b.gidx; });
-      po += num[i];
     }
-  }
-  (void)G;
+  });
   return bad ? SIMLOD_ERR_CUDA : SIMLOD_OK;
 }
 
