@@ -78,7 +78,7 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
 // next one) into the block's shared copy, so that one load per block, not
 // one per warp, reaches the control block's L2 lines.
 struct CtlView {
-  unsigned long long base, bump0;
+  unsigned long long bump0;
   uint32_t n_nodes, key_rate, open, reject, split_count, split_inner, split_most, ntasks, spill_count, nkeys, stop;
   int pool_top;
 };
@@ -118,7 +118,6 @@ __device__ __forceinline__ bool grid_barrier(const Ctx& c, FusedCtl* f, CtlView*
     asm volatile("fence.acq_rel.gpu;" ::: "memory");
 #if SL_CTL_VIEW
     if (ok && view) {
-      view->base = vload(&c.ctl->base);
       view->bump0 = vload(&c.ctl->bump0);
       view->key_rate = vload(&c.ctl->key_rate);
       view->open = vload(&c.ctl->open);
@@ -222,15 +221,14 @@ __device__ __forceinline__ void fused_body(const Ctx& c, const BatchDesc* batche
   CtlView* const vw = nullptr;
 #define SL_CV(field, addr) vload(addr)
 #endif
+  // counters that every thread follows by itself from batch to batch
+  unsigned long long base = vload(&c.ctl->base);
+  uint32_t nodes0 = vload(&c.ctl->n_nodes);
   for (uint32_t b = 0; b < nb; ++b) {
-    // every value read here was written before the last barrier and is not
-    // written again before the next one, so all threads decide alike (the
-    // first batch reads them directly: no barrier has filled the view yet)
-    if (b ? SL_CV(stop, &f->stop) : vload(&f->stop)) return;
+    // (with a budget, every batch ends with a barrier that fills the view)
+    if (b && budget_ns != NO_BUDGET && SL_CV(stop, &f->stop)) return;
     if (ready && !wait_ready(c, f, ready + b)) return;
     BatchDesc bd = batches ? batches[b] : list.d[b];
-    const unsigned long long base = b ? SL_CV(base, &c.ctl->base) : vload(&c.ctl->base);
-    const uint32_t nodes0 = b ? SL_CV(n_nodes, &c.ctl->n_nodes) : vload(&c.ctl->n_nodes);
     bool rejected = false;
     if (bd.nseg && bd.n) {
       // merged update: gather its batches into the staging buffer
@@ -316,7 +314,11 @@ __device__ __forceinline__ void fused_body(const Ctx& c, const BatchDesc* batche
           if (!grid_barrier(c, f)) return;
           clk.tick(c, PH_STORE);
         }
+        // the next batch's count round reads nothing that this changes, and a
+        // barrier follows it
         if (tid == 0) phase_end(c, bd.n);
+        base += bd.n;
+        nodes0 = n_hi;
       }
     }
     if (tid == 0) {
@@ -344,7 +346,10 @@ __device__ __forceinline__ void fused_body(const Ctx& c, const BatchDesc* batche
                      : "memory");
       }
     }
-    if (!grid_barrier(c, f, vw)) return;  // the next batch reads stop, base and n_nodes
+    // the next batch must not set the reject flag before it is cleared, and
+    // all blocks decide alike on a budget stop; else it may begin at once (a
+    // barrier per update was 3 % of a stream of 1M-point batches)
+    if (b + 1u < nb && (rejected || budget_ns != NO_BUDGET) && !grid_barrier(c, f, vw)) return;
     clk.tick(c, PH_END);
   }
   if (blockIdx.x == 0 && threadIdx.x == 0)
