@@ -777,12 +777,29 @@ __device__ __forceinline__ uint32_t count_chunk_log2(uint32_t units, uint32_t nw
 // ------------------------------------------------------------ phase: count1
 
 // Iteration 1 for the batch points [0, n): descend and count. `smem` holds
-// PHASE_SMEM_BYTES of dynamic shared memory.
+// PHASE_SMEM_BYTES of dynamic shared memory. Every block first writes down where
+// the top JUMP levels lead each of their 8^JUMP cubes to (node | level <<
+// NODE_BITS, in the queue region): a point's first steps are one lookup.
+constexpr uint32_t JUMP = 3;
+static_assert((1u << (3u * JUMP)) <= (PHASE_BLOCK / 32) * CLAIM_QUEUE * 6, "the jump table fits");
 __device__ void phase_count1(const Ctx& c, uint32_t* smem, const NodeCache nc, const int4* pts,
                              uint32_t n, uint32_t warp0, uint32_t nwarps) {
   constexpr int U = COUNT_U;
   tally_init(smem);
   __syncthreads();  // also publishes the caller's node-cache writes
+  uint32_t* jump = smem + SMEM_QUEUE;
+  const uint32_t jl = c.rlog2 < JUMP ? c.rlog2 : JUMP, top = c.rlog2 - jl;
+  for (uint32_t t = threadIdx.x; t < (1u << (3u * jl)); t += blockDim.x) {
+    const uint32_t m = (1u << jl) - 1u;
+    uint32_t node = 0, lvl = 0;
+    for (uint32_t ch = node_child(c, nc, 0u); ch != NONE && lvl < jl && ch + 8u <= c.max_nodes;
+         ch = node_child(c, nc, node)) {
+      node = ch + octant(t & m, (t >> jl) & m, t >> (2u * jl), jl - lvl);
+      ++lvl;
+    }
+    jump[t] = node | (lvl << NODE_BITS);
+  }
+  __syncthreads();
   const uint32_t lane = lane_id();
   // each warp carries U units of 32 points (warp_unit k, k + 1, ...) at a
   // time so that their descents overlap; the next units' points are loaded
@@ -811,8 +828,11 @@ __device__ void phase_count1(const Ctx& c, uint32_t* smem, const NodeCache nc, c
         atomicOr(&c.ctl->reject, 1u);
         valid[j] = false;
       }
-      node[j] = 0;
-      L[j] = c.rlog2;
+      const uint32_t e = valid[j] ? jump[(rx[j] >> top) | ((ry[j] >> top) << jl) |
+                                         ((rz[j] >> top) << (2u * jl))]
+                                  : 0u;
+      node[j] = e & NODE_MASK;
+      L[j] = c.rlog2 - (e >> NODE_BITS);
       walking[j] = valid[j];
       any = any || walking[j];
     }
