@@ -1367,22 +1367,24 @@ __device__ __forceinline__ uint32_t pool_take(const Ctx& c, uint32_t k, int* fir
 // them, note them in a leaf's directory and record the store map for this
 // update. Lane 0 takes the allocator atomics; the lanes link the new chunks
 // in parallel (chunk q's successor is chunk q + 1 of the same allocation).
-__device__ void alloc_chunks(const Ctx& c, uint32_t id, uint32_t total, bool leaf) {
+__device__ void alloc_chunks(const Ctx& c, uint32_t id, uint32_t total, bool leaf, uint32_t num,
+                             const uint4& chunks) {
   const uint32_t lane = lane_id();
   NodeMeta& m = c.meta[id];
-  const uint32_t have = m.n_chunks, tail = m.tail, mdir = m.dir;
+  const uint32_t have = chunks.x, tail = chunks.z, mdir = chunks.w;
   const uint32_t need = (uint32_t)(((unsigned long long)total + c.C - 1) / c.C);
   const uint32_t k = need > have ? need - have : 0u;
   uint32_t seq = 0, from_pool = 0, ok = 1;
   int pfirst = 0;
   unsigned long long off = 0;
   if (lane == 0 && k) {
+    // (both on their way before either is looked at)
     seq = atomicAdd(&c.ctl->alloc_seq, k);
+    from_pool = pool_take(c, k, &pfirst);
     if ((unsigned long long)seq + k > c.max_chunks) {
       set_error(c, E_ALLOC_REFS);
       ok = 0;
     } else {
-      from_pool = pool_take(c, k, &pfirst);
       const uint32_t rest = k - from_pool;
       if (rest) {
         off = atomicAdd(&c.ctl->bump, (unsigned long long)rest * c.chunk_bytes);
@@ -1404,7 +1406,7 @@ __device__ void alloc_chunks(const Ctx& c, uint32_t id, uint32_t total, bool lea
     m.st_nch = have;
     m.st_tail = tail;
     m.st_seq = k ? seq : 0u;
-    m.st_base = c.num[id];
+    m.st_base = num;
     m.touched = (uint32_t)c.ctl->st_batches + 1u;
     c.scur[id] = 0;
   }
@@ -1494,7 +1496,7 @@ __device__ void restore_chunks(const Ctx& c, uint32_t id, bool leaf) {
     m.head = m.tail = NONE;
   }
   __syncwarp();
-  alloc_chunks(c, id, n, leaf);
+  alloc_chunks(c, id, n, leaf, n, make_uint4(0, NONE, NONE, m.dir));
   __syncwarp();
   const uint32_t seq = m.st_seq, nch = m.n_chunks;
   if (nch != (n + c.C - 1) / c.C || (unsigned long long)seq + nch > c.max_chunks) {
@@ -1518,22 +1520,39 @@ __device__ void restore_chunks(const Ctx& c, uint32_t id, bool leaf) {
   __syncwarp();
 }
 
+// A node's n_chunks, head, tail and dir, loaded where it stands (the compiler
+// would move the load behind the test of the node's count).
+__device__ __forceinline__ uint4 chunk_words(const Ctx& c, uint32_t id) {
+  static_assert(offsetof(NodeMeta, n_chunks) == 16 && offsetof(NodeMeta, dir) == 28,
+                "the chunk words are one aligned 16-byte load");
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(&c.meta[id].n_chunks)
+               : "memory");
+  return v;
+}
+
 // All 32 lanes of a warp call for one candidate node (a leaf: inner nodes have
-// no counts before the claim phase).
+// no counts before the claim phase). What a node with a count needs is loaded
+// with the count: most of this phase is the chain of one node's round trips.
 __device__ __forceinline__ void decide_node(const Ctx& c, uint32_t id) {
-  const uint32_t k = c.cnt[id];
+  const uint32_t k = vload(c.cnt + id);
+  uint4 chunks = chunk_words(c, id);
+  const uint32_t child = vload(c.child + id), num = vload(c.num + id);
+  const uint32_t level = vload(&c.meta[id].level), compact = vload(&c.meta[id].compact);
   if (k == 0) return;
-  const bool leaf = c.child[id] == NONE;
-  if (c.meta[id].compact) restore_chunks(c, id, leaf);
-  const uint32_t total = c.num[id] + k;
-  if (leaf) {
-    const uint32_t L = c.rlog2 - c.meta[id].level;
-    if (total > c.T && L > 0) {
-      split_leaf(c, id, total);
-      return;
-    }
+  const bool leaf = child == NONE;
+  if (compact) {
+    restore_chunks(c, id, leaf);
+    chunks = chunk_words(c, id);
   }
-  alloc_chunks(c, id, total, leaf);
+  const uint32_t total = num + k;
+  if (leaf && total > c.T && c.rlog2 > level) {
+    split_leaf(c, id, total);
+    return;
+  }
+  alloc_chunks(c, id, total, leaf, num, chunks);
   __syncwarp();
   if (lane_id() == 0) {
     c.num[id] = total;
