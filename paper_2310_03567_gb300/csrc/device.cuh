@@ -288,6 +288,14 @@ constexpr unsigned long long BAR_ABORT = 1ull << 63;
 
 // ------------------------------------------------------------------ helpers
 
+// First thing in a kernel that may be launched before the one in front of it
+// has ended (launch_next): let the kernel behind be placed too, then wait until
+// the one in front has ended and its writes are visible. Returns at once in a
+// kernel that was launched the plain way.
+__device__ __forceinline__ void after_previous() {
+  asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
+}
+
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31u; }
 
 __device__ __forceinline__ unsigned long long fmix64(unsigned long long k) {

@@ -103,6 +103,7 @@ __device__ __forceinline__ bool node_drawn(const Ctx& c, const View& v, uint32_t
 // while the node tests wait for the node table.
 __global__ void k_render_select(Ctx c, View v, uint32_t* vis, unsigned long long* fb,
                                 uint64_t n_px, int clear) {
+  after_previous();
   const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   if (clear) {
@@ -249,6 +250,7 @@ __device__ __forceinline__ uint32_t chunk_fill(const Ctx& c, uint32_t j, uint32_
 // records of a compacted node's array).
 __global__ void k_render_units(Ctx c, View v, const uint32_t* vis, DrawUnit* units,
                                unsigned long long* fb) {
+  after_previous();
   const uint32_t nv = min(vload(&c.ctl->vis_count), c.max_nodes);
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
@@ -297,6 +299,7 @@ __global__ void k_render_units(Ctx c, View v, const uint32_t* vis, DrawUnit* uni
 // millions of samples, the 64-bit minimums on the frame in L2.
 __global__ void k_render_draw(Ctx c, View v, const DrawUnit* units, uint32_t parts, uint32_t part,
                               unsigned long long* fb) {
+  after_previous();
   const uint64_t nu = min((uint64_t)vload(&c.ctl->draw_units), (uint64_t)c.max_chunks);
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
   const uint64_t nwarps = (uint64_t)gridDim.x * blockDim.x / 32;

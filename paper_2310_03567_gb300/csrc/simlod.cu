@@ -77,6 +77,7 @@ __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_count1(Ctx c, cons
                                                                     uint64_t n, uint32_t n_nodes) {
   extern __shared__ uint32_t smem[];
   const uint64_t warps_per_block = blockDim.x / 32;
+  after_previous();
   node_cache_load(c, smem, 0, n_nodes);
   phase_count1(c, smem, node_cache_at(smem, n_nodes), pts, n,
                blockIdx.x * warps_per_block + threadIdx.x / 32,
@@ -86,6 +87,7 @@ __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_count1(Ctx c, cons
 // Decide / allocate; after the first count round of a rejected batch (no
 // thread changes the reject flag during this kernel) undo that round instead.
 __global__ void __launch_bounds__(BLOCK) k_decide(Ctx c, uint32_t n_lo, uint32_t n_hi) {
+  after_previous();
   const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   const uint64_t nt = (uint64_t)gridDim.x * blockDim.x;
   if (*reinterpret_cast<volatile unsigned int*>(&c.ctl->reject)) {
@@ -120,6 +122,7 @@ __host__ __device__ __forceinline__ uint32_t round_end(const Ctl* t, uint32_t r)
 __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_hist(Ctx c, const int4* pts,
                                                                   uint64_t n, uint32_t r) {
   extern __shared__ uint32_t smem[];
+  after_previous();
   if (plain_stop(c)) return;
   const uint32_t s_lo = round_end(c.ctl, r - 1u);
   const uint32_t K = vload(&c.ctl->split_count) - s_lo, n_nodes = vload(&c.ctl->n_nodes);
@@ -135,6 +138,7 @@ __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_hist(Ctx c, const 
 }
 
 __global__ void __launch_bounds__(PBLOCK) k_build(Ctx c, uint32_t r, uint32_t max_iters) {
+  after_previous();
   if (plain_stop(c)) return;
   const PlainRound* p = &c.ctl->round[r];
   if (vload(&p->K)) phase_build(c, vload(&p->s_lo), vload(&p->K), vload(&p->d), vload(&p->lvl0),
@@ -142,6 +146,7 @@ __global__ void __launch_bounds__(PBLOCK) k_build(Ctx c, uint32_t r, uint32_t ma
 }
 
 __global__ void __launch_bounds__(BLOCK) k_decide_new(Ctx c, uint32_t r) {
+  after_previous();
   if (plain_stop(c) || vload(&c.ctl->round[r].K) == 0u) return;
   phase_decide(c, vload(&c.ctl->round[r].n_lo), vload(&c.ctl->n_nodes),
                (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) / 32,
@@ -152,6 +157,7 @@ __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_claim(Ctx c, const
                                                      unsigned long long base, uint32_t nodes0,
                                                      uint32_t r) {
   extern __shared__ uint32_t smem[];
+  after_previous();
   if (plain_stop(c) || vload(&c.ctl->split_count) != round_end(c.ctl, r)) return;
   const uint32_t s_hi = vload(&c.ctl->split_count), t_hi = vload(&c.ctl->ntasks);
   const uint64_t wpb = blockDim.x / 32;
@@ -166,6 +172,7 @@ __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_claim(Ctx c, const
 
 // Chunks for the new voxels of the inner nodes.
 __global__ void __launch_bounds__(BLOCK) k_alloc_voxels(Ctx c, uint32_t r) {
+  after_previous();
   if (plain_stop(c) || vload(&c.ctl->split_count) != round_end(c.ctl, r)) return;
   phase_decide(c, 0, vload(&c.ctl->n_nodes),
                (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) / 32,
@@ -247,6 +254,7 @@ __device__ __forceinline__ bool compact_candidate(const Ctx& c, uint32_t id, uin
 }
 
 __global__ void k_compact_need(Ctx c, uint32_t idle) {
+  after_previous();
   const uint32_t n_nodes = min(vload(&c.ctl->n_nodes), c.max_nodes);
   const unsigned long long now = vload(&c.ctl->st_batches);
   unsigned long long bytes = 0;
@@ -259,6 +267,7 @@ __global__ void k_compact_need(Ctx c, uint32_t idle) {
 }
 
 __global__ void k_compact_plan(Ctx c, uint32_t idle, DrawUnit* units) {
+  after_previous();
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
   const uint64_t nwarps = (uint64_t)gridDim.x * blockDim.x / 32;
@@ -326,6 +335,7 @@ __global__ void k_compact_plan(Ctx c, uint32_t idle, DrawUnit* units) {
 
 // Copy the units, `parts` warps per unit (parts * part >= C).
 __global__ void k_compact_copy(Ctx c, const DrawUnit* units, uint32_t parts, uint32_t part) {
+  after_previous();
   const uint64_t nu = min((uint64_t)vload(&c.ctl->draw_units), (uint64_t)c.max_chunks);
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
@@ -696,6 +706,29 @@ int launch(simlod_t* h, int kernel, cudaStream_t s, Launch&& fn) {
   return err == cudaSuccess ? SIMLOD_OK : SIMLOD_ERR_CUDA;
 }
 
+// Launch a kernel that begins with after_previous() behind another of this
+// library: its blocks may be placed while the last blocks of the one before
+// still run, and wait there for its end (programmatic dependent launch), so that
+// the launch itself costs nothing between short kernels. Plain launches while
+// the stream is captured.
+template <typename... P, typename... A>
+void launch_next(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                 A&&... args) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cap = cudaStreamCaptureStatusActive;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 unsigned grid_for(const simlod_t* h, uint64_t work, uint64_t per_block) {
   uint64_t blocks = (work + per_block - 1) / per_block;
   uint64_t cap = (uint64_t)h->sm_count * 8;
@@ -745,7 +778,7 @@ int insert_device(simlod_t* h, const int4* pts, uint64_t n, cudaStream_t s) {
   });
   if (rc) return poison(h, rc);
   rc = launch(h, K_DECIDE, s, [&] {
-    k_decide<<<grid_for(h, 32ull * nodes0, BLOCK), BLOCK, 0, s>>>(c, 0, nodes0);
+    launch_next(k_decide, grid_for(h, 32ull * nodes0, BLOCK), BLOCK, 0, s, c, 0u, nodes0);
   });
   if (rc) return poison(h, rc);
   const Ctl& t = *h->ctl_host;
@@ -754,20 +787,20 @@ int insert_device(simlod_t* h, const int4* pts, uint64_t n, cudaStream_t s) {
   for (uint32_t r = h->plain_split ? 1u : 0u;; ++r) {
     if (r) {
       rc = launch(h, K_ADVANCE, s, [&] {
-        k_hist<<<full, PBLOCK, PHASE_SMEM_BYTES, s>>>(c, pts, n, r);
-        k_build<<<full, PBLOCK, 0, s>>>(c, r, max_iters);
+        launch_next(k_hist, full, PBLOCK, PHASE_SMEM_BYTES, s, c, pts, n, r);
+        launch_next(k_build, full, PBLOCK, 0, s, c, r, max_iters);
       });
       if (rc) return poison(h, rc);
       rc = launch(h, K_DECIDE, s, [&] {
-        k_decide_new<<<full * 2, BLOCK, 0, s>>>(c, r);
+        launch_next(k_decide_new, full * 2, BLOCK, 0, s, c, r);
       });
       if (rc) return poison(h, rc);
     }
     rc = launch(h, K_CLAIM, s, [&] {
-      k_claim<<<r ? full : gp, PBLOCK, PHASE_SMEM_BYTES, s>>>(c, pts, n, base, nodes0, r);
+      launch_next(k_claim, r ? full : gp, PBLOCK, PHASE_SMEM_BYTES, s, c, pts, n, base, nodes0, r);
     });
     if (rc) return poison(h, rc);
-    rc = launch(h, K_DECIDE, s, [&] { k_alloc_voxels<<<full * 2, BLOCK, 0, s>>>(c, r); });
+    rc = launch(h, K_DECIDE, s, [&] { launch_next(k_alloc_voxels, full * 2, BLOCK, 0, s, c, r); });
     if (rc) return poison(h, rc);
     if ((rc = read_ctl(h, s))) return poison(h, rc);
     if (t.error) return poison(h, error_from_bits(t.error));
@@ -1738,8 +1771,8 @@ SIMLOD_API int simlod_compact(simlod_t* h, uint32_t idle_updates, void* stream) 
   unit_parts(c.C, &parts, &part);
   const unsigned grid = (unsigned)h->sm_count * 8;
   k_compact_need<<<grid, BLOCK, 0, s>>>(c, idle_updates);
-  k_compact_plan<<<grid, BLOCK, 0, s>>>(c, idle_updates, units);
-  k_compact_copy<<<grid, BLOCK, 0, s>>>(c, units, parts, part);
+  launch_next(k_compact_plan, grid, BLOCK, 0, s, c, idle_updates, units);
+  launch_next(k_compact_copy, grid, BLOCK, 0, s, c, units, parts, part);
   return cudaGetLastError() == cudaSuccess ? SIMLOD_OK : poison(h, SIMLOD_ERR_CUDA);
 }
 
@@ -1776,8 +1809,8 @@ SIMLOD_API int simlod_render(simlod_t* h, const float view_proj[16], uint32_t wi
   const unsigned grid = (unsigned)h->sm_count * 8;
   return launch(h, K_RENDER, s, [&] {
     k_render_select<<<grid, BLOCK, 0, s>>>(c, v, vis, fb, (uint64_t)width * height, clear);
-    k_render_units<<<grid, BLOCK, 0, s>>>(c, v, vis, units, fb);
-    k_render_draw<<<grid, BLOCK, 0, s>>>(c, v, units, parts, part, fb);
+    launch_next(k_render_units, grid, BLOCK, 0, s, c, v, vis, units, fb);
+    launch_next(k_render_draw, grid, BLOCK, 0, s, c, v, units, parts, part, fb);
   });
 }
 
