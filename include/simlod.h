@@ -287,7 +287,7 @@ typedef struct {
   uint32_t max_blocks_per_sm;  /* that fit on the current device */
   uint32_t node_cache;         /* node-table entries mirrored in shared memory */
   uint32_t store_unroll;       /* records per thread in flight while storing */
-  uint32_t descent_group;      /* tree levels whose occupancy words load together */
+  uint32_t descent_group;      /* units of 32 points whose descents a warp overlaps */
   uint32_t smem_bytes;         /* dynamic shared memory per block */
 } simlod_variant_desc;
 /* Parameters of kernel instance `variant` on the current device;

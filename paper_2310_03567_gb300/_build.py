@@ -28,9 +28,9 @@ OBJ_DIR = os.path.join(PKG_DIR, "build", platform.machine())
 
 # Instances of the persistent update kernel beyond the one built into
 # simlod.cu (instance 0: 512 threads, 2 blocks per SM, 4,096 cached nodes,
-# store unroll 2, descent group 2), each built from fused_variant.cu:
+# store unroll 2, count unroll 2), each built from fused_variant.cu:
 # (threads per block, blocks per SM, node-cache entries, store unroll,
-# descent group). The batched form's autotuner picks among all of them.
+# count unroll). The batched form's autotuner picks among all of them.
 VARIANTS = [
     (256, 4, 2048, 2, 2),
     (1024, 1, 8192, 2, 2),
@@ -71,7 +71,7 @@ def library_headers() -> list[str]:
 
 def _common_flags(extra: list[str] | None = None) -> list[str]:
     # Plain global loads may be cached in L1. The persistent kernel re-reads
-    # node tables, split lists, mover lists and grids that other blocks wrote
+    # node tables, split lists, histograms and grids that other blocks wrote
     # before a grid barrier; at every barrier thread 0 of each block takes a
     # GPU-scope acquire fence after the other blocks' release, and the block
     # barrier that follows orders it before every thread's later loads, so
@@ -86,12 +86,12 @@ def _common_flags(extra: list[str] | None = None) -> list[str]:
 
 def variant_flags(k: int) -> list[str]:
     """Defines of kernel instance k >= 1 (fused_variant.cu)."""
-    block, per_sm, cache, store_u, group = VARIANTS[k - 1]
+    block, per_sm, cache, store_u, count_u = VARIANTS[k - 1]
     return [f"-DSL_NS=sl_v{k}", f"-DSL_VARIANT_INFO=sl_fused_variant_info_{k}",
             f"-DSL_VARIANT_LAUNCH=sl_fused_variant_launch_{k}",
             f"-DSL_PHASE_BLOCK={block}", f"-DSL_PHASE_MIN_BLOCKS={per_sm}",
             f"-DSL_NODE_CACHE={cache}", f"-DSL_STORE_UNROLL={store_u}",
-            f"-DSL_COUNT_UNROLL={group}"]
+            f"-DSL_COUNT_UNROLL={count_u}"]
 
 
 def compile_commands(extra: list[str] | None = None, obj_dir: str = OBJ_DIR):

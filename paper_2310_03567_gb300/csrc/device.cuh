@@ -39,7 +39,7 @@
 // an update are listed (the backlog of Section 5.2) and cleared by store.
 //
 // Descents read the node table (first child) from a copy in shared memory of the first NODE_CACHE nodes (the node ids of the upper
-// levels are the smallest): the plain form's count / advance kernels load it,
+// levels are the smallest): the plain form's kernels load it,
 // the persistent kernel loads it once and patches it after every decide
 // round with the nodes that split or were created.
 // Per-node counters are summed per block in shared memory before they reach
@@ -76,15 +76,6 @@ constexpr uint32_t CHUNK_HEADER = 16;
 #ifndef SL_PHASE_MIN_BLOCKS
 #define SL_PHASE_MIN_BLOCKS 2
 #endif
-#ifndef SL_CTL_VIEW
-#define SL_CTL_VIEW 1
-#endif
-#ifndef SL_CTL_SPREAD
-#define SL_CTL_SPREAD 1
-#endif
-#ifndef SL_COUNT_PREFETCH
-#define SL_COUNT_PREFETCH 1
-#endif
 #ifndef SL_COUNT_UNROLL
 #define SL_COUNT_UNROLL 2
 #endif
@@ -107,7 +98,7 @@ constexpr int COUNT_U = SL_COUNT_UNROLL;               // count units a warp car
 #define SL_WBUF 128
 #endif
 constexpr uint32_t WBUF = SL_WBUF;                      // new-cell slots staged per warp
-constexpr int PHASE_BLOCK = SL_PHASE_BLOCK;            // threads of count / advance / fused blocks
+constexpr int PHASE_BLOCK = SL_PHASE_BLOCK;            // threads of a phase block
 constexpr int PHASE_MIN_BLOCKS = SL_PHASE_MIN_BLOCKS;  // resident blocks per SM they aim for
 constexpr uint32_t TALLY_LOG2 = 9;                      // block tally cache: 512 nodes
 constexpr uint32_t TALLY_SLOTS = 1u << TALLY_LOG2;
@@ -139,11 +130,7 @@ enum : uint32_t {
 // The counters that warps all over the grid change with atomics inside a
 // phase (SL_HOT) each start a 128-byte line of their own, so that their
 // atomics spread over several L2 slices instead of queueing at one.
-#if SL_CTL_SPREAD
 #define SL_HOT alignas(128)
-#else
-#define SL_HOT
-#endif
 // An expansion round of the plain form, whose kernels find here what the ones
 // before them left: split entries [s_lo, s_lo + K) are built d levels deep
 // below lvl0 levels of earlier rounds, which made `inner` inner nodes; the
@@ -198,7 +185,7 @@ static_assert(sizeof(Ctl) % 16 == 0, "Ctl size");
 // Phases of the fused form, for its phase clock.
 enum : int { PH_COUNT = 0, PH_DECIDE, PH_ADVANCE, PH_STORE, PH_END, PH_CLAIM, PH_LAUNCH, PH_OTHER };
 
-// Per-node metadata that the count/advance hot loops do not touch.
+// Per-node metadata that the descents do not touch.
 struct NodeMeta {
   int32_t min[3];
   uint32_t level;
@@ -297,15 +284,6 @@ __device__ __forceinline__ void after_previous() {
 }
 
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31u; }
-
-__device__ __forceinline__ unsigned long long fmix64(unsigned long long k) {
-  k ^= k >> 33;
-  k *= 0xff51afd7ed558ccdull;
-  k ^= k >> 33;
-  k *= 0xc4ceb9fe1a85ec53ull;
-  k ^= k >> 33;
-  return k;
-}
 
 __device__ __forceinline__ void set_error(const Ctx& c, uint32_t bits) {
   atomicOr(&c.ctl->error, bits);

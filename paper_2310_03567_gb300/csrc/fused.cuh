@@ -116,7 +116,6 @@ __device__ __forceinline__ bool grid_barrier(const Ctx& c, FusedCtl* f, CtlView*
       }
     }
     asm volatile("fence.acq_rel.gpu;" ::: "memory");
-#if SL_CTL_VIEW
     if (ok && view) {
       view->bump0 = vload(&c.ctl->bump0);
       view->key_rate = vload(&c.ctl->key_rate);
@@ -132,7 +131,6 @@ __device__ __forceinline__ bool grid_barrier(const Ctx& c, FusedCtl* f, CtlView*
       view->pool_top = vload(&c.ctl->pool_top);
       view->stop = vload(&f->stop);
     }
-#endif
     s_ok = ok;
   }
   __syncthreads();
@@ -213,20 +211,14 @@ __device__ __forceinline__ void fused_body(const Ctx& c, const BatchDesc* batche
   const uint32_t nb = n_dev ? min(vload(n_dev), n_batches) : n_batches;
   // the node-table cache is loaded once and patched after every decide round
   node_cache_load(c, smem, 0, vload(&c.ctl->n_nodes));
-#if SL_CTL_VIEW
   __shared__ CtlView cv;  // control values after the last barrier that filled it
   CtlView* const vw = &cv;
-#define SL_CV(field, addr) (cv.field)
-#else
-  CtlView* const vw = nullptr;
-#define SL_CV(field, addr) vload(addr)
-#endif
   // counters that every thread follows by itself from batch to batch
   unsigned long long base = vload(&c.ctl->base);
   uint32_t nodes0 = vload(&c.ctl->n_nodes);
   for (uint32_t b = 0; b < nb; ++b) {
     // (with a budget, every batch ends with a barrier that fills the view)
-    if (b && budget_ns != NO_BUDGET && SL_CV(stop, &f->stop)) return;
+    if (b && budget_ns != NO_BUDGET && cv.stop) return;
     if (ready && !wait_ready(c, f, ready + b)) return;
     BatchDesc bd = batches ? batches[b] : list.d[b];
     bool rejected = false;
@@ -249,7 +241,7 @@ __device__ __forceinline__ void fused_body(const Ctx& c, const BatchDesc* batche
       phase_count1(c, smem, node_cache_at(smem, nodes0), bd.pts, (uint32_t)bd.n, warp0, nwarps);
       if (!grid_barrier(c, f, vw)) return;
       clk.tick(c, PH_COUNT);
-      rejected = SL_CV(reject, &c.ctl->reject) != 0u;  // set only by the count round
+      rejected = cv.reject != 0u;  // set only by the count round
       if (rejected) {
         phase_rollback(c, nodes0, tid, nthreads);
         if (!grid_barrier(c, f)) return;  // all have read the flag before it is cleared
@@ -266,14 +258,14 @@ __device__ __forceinline__ void fused_body(const Ctx& c, const BatchDesc* batche
           phase_decide(c, n_lo, n_hi, warp0, nwarps);
           if (!grid_barrier(c, f, vw)) return;
           clk.tick(c, PH_DECIDE);
-          const uint32_t K = SL_CV(split_count, &c.ctl->split_count) - s_hi;
-          const uint32_t nt = SL_CV(ntasks, &c.ctl->ntasks);
+          const uint32_t K = cv.split_count - s_hi;
+          const uint32_t nt = cv.ntasks;
           const bool first = n_lo == 0u;
           if (first) t_hi = nt;
           else if (nt != t_hi && tid == 0) set_error(c, E_INTERNAL);
           if (K == 0u) break;
-          const uint32_t d = hist_depth(c, K, bd.n + SL_CV(spill_count, &c.ctl->spill_count),
-                                        SL_CV(split_most, &c.ctl->split_most));
+          const uint32_t d = hist_depth(c, K, bd.n + cv.spill_count,
+                                        cv.split_most);
           phase_hist(c, smem, node_cache_at(smem, n_hi), bd.pts, (uint32_t)bd.n, t_hi, s_hi, K, d, first);
           if (!grid_barrier(c, f)) return;
           phase_build(c, s_hi, K, d, lvl0, max_iters);
@@ -281,10 +273,10 @@ __device__ __forceinline__ void fused_body(const Ctx& c, const BatchDesc* batche
           clk.tick(c, PH_ADVANCE);
           // the entries so far: not split_count, which the next decide raises
           // while a late block still reads its view
-          const uint32_t inner = SL_CV(split_inner, &c.ctl->split_inner);
+          const uint32_t inner = cv.split_inner;
           const uint32_t sc = s_hi + K + (inner - inner0);
           inner0 = inner;
-          const uint32_t nn = SL_CV(n_nodes, &c.ctl->n_nodes);
+          const uint32_t nn = cv.n_nodes;
           node_cache_patch(c, smem, s_hi, sc, n_hi, nn);
           s_hi = sc;
           n_lo = n_hi;
@@ -292,24 +284,24 @@ __device__ __forceinline__ void fused_body(const Ctx& c, const BatchDesc* batche
           lvl0 += d;
         }
         // (the last decide round's barrier filled the view)
-        const uint32_t n_spill = min(SL_CV(spill_count, &c.ctl->spill_count), c.spill_cap);
-        const ClaimArgs ca{nodes0, (uint32_t)(SL_CV(bump0, &c.ctl->bump0) / REF_BYTES),
-                           SL_CV(open, &c.ctl->open),
-                           claim_near_mask(c, bd.n + n_spill, SL_CV(key_rate, &c.ctl->key_rate))};
+        const uint32_t n_spill = min(cv.spill_count, c.spill_cap);
+        const ClaimArgs ca{nodes0, (uint32_t)(cv.bump0 / REF_BYTES),
+                           cv.open,
+                           claim_near_mask(c, bd.n + n_spill, cv.key_rate)};
         uint32_t n_keys = 0;
         if (n_hi > 1u) {  // (an octree of one leaf has no voxels)
           phase_claim(c, smem, node_cache_at(smem, n_hi), bd.pts, (uint32_t)bd.n, base, t_hi, s_hi, ca,
                       warp0, nwarps);
           if (!grid_barrier(c, f, vw)) return;
           clk.tick(c, PH_CLAIM);
-          n_keys = min(SL_CV(nkeys, &c.ctl->nkeys), c.backlog_cap);
+          n_keys = min(cv.nkeys, c.backlog_cap);
         }
         phase_store(c, smem, bd.pts, (uint32_t)bd.n, base, t_hi);
         if (n_keys) phase_decide(c, 0, n_hi, warp0, nwarps);  // chunks for the new voxels
         if (!grid_barrier(c, f, vw)) return;
         clk.tick(c, PH_STORE);
         if (n_keys || t_hi) {
-          phase_store_voxels(c, smem, t_hi, n_keys, SL_CV(pool_top, &c.ctl->pool_top), tid,
+          phase_store_voxels(c, smem, t_hi, n_keys, cv.pool_top, tid,
                              nthreads);
           if (!grid_barrier(c, f)) return;
           clk.tick(c, PH_STORE);
@@ -354,7 +346,6 @@ __device__ __forceinline__ void fused_body(const Ctx& c, const BatchDesc* batche
   }
   if (blockIdx.x == 0 && threadIdx.x == 0)
     atomicAdd(&c.ctl->phase_ns[PH_LAUNCH], globaltimer_ns() - t_begin);
-#undef SL_CV
 }
 
 __global__ void __launch_bounds__(FUSED_BLOCK, PHASE_MIN_BLOCKS)

@@ -1,8 +1,8 @@
 // One more instance of the persistent update kernel (k_fused), compiled with
 // other launch-shape knobs than the instance built into simlod.cu: threads
 // per block, resident blocks per SM, node-cache entries, store unroll and
-// descent group (SL_PHASE_BLOCK, SL_PHASE_MIN_BLOCKS, SL_NODE_CACHE,
-// SL_STORE_UNROLL, SL_DESCENT_GROUP). The build compiles this file once per
+// count unroll (SL_PHASE_BLOCK, SL_PHASE_MIN_BLOCKS, SL_NODE_CACHE,
+// SL_STORE_UNROLL, SL_COUNT_UNROLL). The build compiles this file once per
 // instance with those values, a namespace of its own (SL_NS) and the names of
 // its two entry points (SL_VARIANT_INFO, SL_VARIANT_LAUNCH); the host code of
 // simlod.cu calls them through variant.h. The arithmetic is the same in every

@@ -27,7 +27,7 @@ using namespace sl;
 namespace {
 
 constexpr int BLOCK = 256;
-constexpr int PBLOCK = PHASE_BLOCK;  // count / advance kernels (one node-table cache per block)
+constexpr int PBLOCK = PHASE_BLOCK;  // phase kernels (one node-table cache per block)
 
 __global__ void k_init(Ctx c, FusedCtl* f) {
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -990,13 +990,6 @@ SIMLOD_API int simlod_create(const simlod_config* cfg, void* d_arena, size_t are
     delete h;
     return SIMLOD_ERR_CUDA;
   }
-#ifdef SL_CARVEOUT
-  // shared-memory share of the unified L1/shared storage, in percent
-  cudaFuncSetAttribute(k_fused, cudaFuncAttributePreferredSharedMemoryCarveout, SL_CARVEOUT);
-  cudaFuncSetAttribute(k_count1, cudaFuncAttributePreferredSharedMemoryCarveout, SL_CARVEOUT);
-  cudaFuncSetAttribute(k_hist, cudaFuncAttributePreferredSharedMemoryCarveout, SL_CARVEOUT);
-  cudaGetLastError();
-#endif
   int coop = 0, bpsm = 0;
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
   if (coop && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, k_fused, FUSED_BLOCK,

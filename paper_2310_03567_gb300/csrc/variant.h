@@ -15,7 +15,7 @@ struct sl_variant_info {
   uint32_t min_blocks;     // resident blocks per SM the registers are sized for
   uint32_t node_cache;     // node-table entries mirrored in shared memory
   uint32_t store_unroll;   // items per thread in flight in the store phase
-  uint32_t descent_group;  // tree levels whose grid words load together
+  uint32_t descent_group;  // units of 32 points whose descents a warp overlaps
   uint32_t smem_bytes;     // dynamic shared memory per block
   int32_t max_per_sm;      // blocks per SM that fit on this device (0 = none)
 };
