@@ -6,7 +6,7 @@
  * arriving batch of points is counted into the current leaves, leaves holding
  * more than T points split into 8 children until no leaf spills (Section 5.1),
  * every point samples a voxel in the 128^3 occupancy grid of each inner node
- * on its way down (Section 5.2), chunks are allocated from a pool and a bump
+ * above it (Section 5.2), chunks are allocated from a pool and a bump
  * allocator (Sections 3.2, 3.4, 5.3) and points and voxels are stored into
  * linked chunks of C records (Section 5.4).
  *
@@ -180,12 +180,11 @@ SIMLOD_API int simlod_create(const simlod_config* cfg, void* d_arena, size_t are
  * point ever accepted gets gidx k. n = 0 is a no-op.
  *
  * The work runs on `stream`, in stream order after earlier work there. The
- * call enqueues the update up to the allocation of its chunks, waits for the
- * stream once (a read of the control block; once more for every further
- * histogram round of an unusually deep split), then enqueues the final store
- * and returns without waiting for it. d_pts must therefore stay valid
- * and unchanged until `stream` has passed the insert (record an event or
- * synchronise). Returns SIMLOD_ERR_OUT_OF_BOUNDS, with the octree and the
+ * call enqueues the update, waits once until its allocations are made (a read
+ * of the control block; once more for every further histogram round of an
+ * unusually deep split) and returns without waiting for the final store.
+ * d_pts must therefore stay valid and unchanged until `stream` has passed the
+ * insert (record an event or synchronise). Returns SIMLOD_ERR_OUT_OF_BOUNDS, with the octree and the
  * gidx counter unchanged, when any point lies outside the root cube. Calls on
  * one handle must be ordered: use one stream, or order the streams. */
 SIMLOD_API int simlod_insert_batch(simlod_t* h, const simlod_point* d_pts, uint64_t n,

@@ -180,13 +180,19 @@ __global__ void __launch_bounds__(BLOCK) k_alloc_voxels(Ctx c, uint32_t r) {
 }
 
 // The points and, their nodes' chunks being there too, the voxels; the last
-// block closes the update (a launch of its own took 5 us).
+// block closes the update (a launch of its own took 5 us). Enqueued behind the
+// host's copy of the control block, so that it runs while the host looks at it
+// (ten updates of 100k uniform points 918 instead of 946 us); it leaves, too,
+// when the update does not go through as it stands.
 __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_store(Ctx c, const int4* pts, uint64_t n,
-                                                  unsigned long long base, uint32_t t_hi,
-                                                  uint32_t n_keys, int pool_top) {
+                                                  unsigned long long base, uint32_t r) {
   extern __shared__ uint32_t smem[];
+  if (plain_stop(c) || vload(&c.ctl->split_count) != round_end(c.ctl, r)) return;
   const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   const uint64_t nt = (uint64_t)gridDim.x * blockDim.x;
+  const uint32_t t_hi = vload(&c.ctl->ntasks);
+  const uint32_t n_keys = min(vload(&c.ctl->nkeys), c.backlog_cap);
+  const int pool_top = vload(&c.ctl->pool_top);
   phase_store(c, smem, pts, n, base, t_hi);
   phase_store_voxels(c, smem, t_hi, n_keys, pool_top, t0, nt);
   __threadfence();
@@ -463,6 +469,7 @@ struct simlod {
   unsigned long long rejected_async_seen;  // fused-launch rejections already reported
   BatchDesc* desc_host;     // pinned staging of the batch table
   cudaEvent_t desc_done;    // the last batch-table copy has finished
+  cudaEvent_t ctl_copied;   // the plain form's copy of the control block has arrived
   FusedCtl* fctl_host;      // pinned mirror of the fused control words
   uint32_t* one_host;       // pinned word holding 1: the source of ready-flag copies
   uint32_t* prog_host;      // mapped pinned words: [0] batches of persistent launches
@@ -802,7 +809,19 @@ int insert_device(simlod_t* h, const int4* pts, uint64_t n, cudaStream_t s) {
     if (rc) return poison(h, rc);
     rc = launch(h, K_DECIDE, s, [&] { launch_next(k_alloc_voxels, full * 2, BLOCK, 0, s, c, r); });
     if (rc) return poison(h, rc);
-    if ((rc = read_ctl(h, s))) return poison(h, rc);
+    // the host waits for the copy of the control block, not for the store
+    if (cudaMemcpyAsync(h->ctl_host, c.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s) !=
+            cudaSuccess ||
+        cudaEventRecord(h->ctl_copied, s) != cudaSuccess)
+      return poison(h, SIMLOD_ERR_CUDA);
+    rc = launch(h, K_STORE, s, [&] {
+      k_store<<<r ? full : gp, PBLOCK, PHASE_SMEM_BYTES, s>>>(c, pts, n, base, r);
+    });
+    if (rc) return poison(h, rc);
+    if ((h->timing ? cudaStreamSynchronize(s) : cudaEventSynchronize(h->ctl_copied)) !=
+        cudaSuccess)
+      return poison(h, SIMLOD_ERR_CUDA);
+    if (h->timing) harvest_timing(h);
     if (t.error) return poison(h, error_from_bits(t.error));
     if (t.reject) {
       rc = launch(h, K_END, s, [&] { k_end_rejected<<<1, 1, 0, s>>>(c); });
@@ -813,15 +832,6 @@ int insert_device(simlod_t* h, const int4* pts, uint64_t n, cudaStream_t s) {
     if (r + 1u >= MAX_ROUNDS) return poison(h, SIMLOD_ERR_CUDA);
   }
   h->plain_split = t.split_count != 0u;
-  const uint32_t t_hi = t.ntasks;
-  const uint32_t n_keys = std::min<uint32_t>(t.nkeys, c.backlog_cap);
-  const int pool_top = t.pool_top;
-  const uint64_t work = std::max<uint64_t>(std::max<uint64_t>(n, (uint64_t)t_hi * c.C), n_keys);
-  rc = launch(h, K_STORE, s, [&] {
-    k_store<<<std::min(full, grid_for(h, work, PBLOCK)), PBLOCK, PHASE_SMEM_BYTES, s>>>(
-        c, pts, n, base, t_hi, n_keys, pool_top);
-  });
-  if (rc) return poison(h, rc);
   h->base += n;
   h->n_nodes = h->ctl_host->n_nodes;
   return SIMLOD_OK;
@@ -1008,6 +1018,7 @@ SIMLOD_API int simlod_create(const simlod_config* cfg, void* d_arena, size_t are
       cudaMallocHost(reinterpret_cast<void**>(&h->fctl_host), sizeof(FusedCtl)) != cudaSuccess ||
       cudaMallocHost(reinterpret_cast<void**>(&h->one_host), sizeof(uint32_t)) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->desc_done, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&h->ctl_copied, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->flags_clear, cudaEventDisableTiming) != cudaSuccess) {
     simlod_destroy(h);
     return SIMLOD_ERR_CUDA;
@@ -1972,6 +1983,7 @@ SIMLOD_API int simlod_destroy(simlod_t* h) {
   if (h->one_host) cudaFreeHost(h->one_host);
   if (h->prog_host) cudaFreeHost(h->prog_host);
   if (h->desc_done) cudaEventDestroy(h->desc_done);
+  if (h->ctl_copied) cudaEventDestroy(h->ctl_copied);
   if (h->flags_clear) cudaEventDestroy(h->flags_clear);
   delete h;
   return SIMLOD_OK;
