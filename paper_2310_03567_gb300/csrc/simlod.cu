@@ -100,8 +100,8 @@ __global__ void __launch_bounds__(BLOCK) k_decide(Ctx c, uint32_t n_lo, uint32_t
 // The plain form's kernels after the first decide. All are enqueued before the
 // host has seen anything of the update: what they need is in the control
 // block, and they leave at once when the batch was rejected or an error came
-// up. hist, build and decide_new leave when no leaf splits, claim and
-// alloc_voxels when one still has to: the host, which reads the control block
+// up. hist, build and decide_new leave when no leaf splits, claim, alloc_voxels
+// and store when one still has to: the host, which reads the control block
 // then, enqueues another round and them again. A wait for the host per round
 // (7 per update of a clustered scan) took longer than the kernels between.
 // (All threads of the block call and get one answer: another block of the
