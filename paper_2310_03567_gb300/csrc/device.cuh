@@ -283,11 +283,22 @@ __device__ __forceinline__ void after_previous() {
   asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
 }
 
+template <typename T>
+__device__ __forceinline__ T vload(const T* p) {
+  return *reinterpret_cast<const volatile T*>(p);
+}
+
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31u; }
 
 __device__ __forceinline__ void set_error(const Ctx& c, uint32_t bits) {
   atomicOr(&c.ctl->error, bits);
   atomicOr(c.launch_bar, BAR_ABORT);
+}
+
+// All 32 lanes call and get one answer: a device error has left the octree half
+// updated (the host learns of it at its next look at the control block).
+__device__ __forceinline__ bool update_failed(const Ctx& c) {
+  return __any_sync(FULL_MASK, vload(&c.ctl->error) != 0u);
 }
 
 // n / d for any 32-bit n: multiply, add and shift by the constants that Granlund
@@ -479,11 +490,6 @@ __device__ __forceinline__ uint32_t node_child(const Ctx& c, NodeCache nc, uint3
 }
 
 // -------------------------------------------------------- voxel claims
-
-template <typename T>
-__device__ __forceinline__ T vload(const T* p) {
-  return *reinterpret_cast<const volatile T*>(p);
-}
 
 // Key and value of a claim-table slot in one 16-byte load. Within an update
 // a slot's value only decreases once its key is set (the store phase empties

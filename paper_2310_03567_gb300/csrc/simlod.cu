@@ -252,6 +252,10 @@ __global__ void k_check_nested(Ctx c) {
 // before: 3.4 ms for the 12M-point building scan, of which the longest nodes'
 // copies were most, and a compare-and-swap loop on the bump pointer per node,
 // which is only needed now when the region cannot hold all of them.)
+// An octree whose last update failed half way, which the host may not know yet,
+// stays as it is: its bump pointer can lie behind the data region's end (an
+// allocation adds to it before it looks), and node ids that were reserved have
+// no metadata.
 __device__ __forceinline__ bool compact_candidate(const Ctx& c, uint32_t id, uint32_t idle,
                                                   unsigned long long now) {
   const NodeMeta& m = c.meta[id];
@@ -261,6 +265,7 @@ __device__ __forceinline__ bool compact_candidate(const Ctx& c, uint32_t id, uin
 
 __global__ void k_compact_need(Ctx c, uint32_t idle) {
   after_previous();
+  if (update_failed(c)) return;
   const uint32_t n_nodes = min(vload(&c.ctl->n_nodes), c.max_nodes);
   const unsigned long long now = vload(&c.ctl->st_batches);
   unsigned long long bytes = 0;
@@ -274,12 +279,15 @@ __global__ void k_compact_need(Ctx c, uint32_t idle) {
 
 __global__ void k_compact_plan(Ctx c, uint32_t idle, DrawUnit* units) {
   after_previous();
+  if (update_failed(c)) return;
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
   const uint64_t nwarps = (uint64_t)gridDim.x * blockDim.x / 32;
   const uint32_t n_nodes = min(vload(&c.ctl->n_nodes), c.max_nodes);
   const unsigned long long now = vload(&c.ctl->st_batches);
-  const bool all_fit = vload(&c.ctl->compact_need) <= c.data_bytes - c.ctl->compact_from;
+  const unsigned long long from = c.ctl->compact_from;
+  const bool all_fit =
+      from <= c.data_bytes && vload(&c.ctl->compact_need) <= c.data_bytes - from;
   for (uint64_t id = warp; id < n_nodes; id += nwarps) {
     if (!compact_candidate(c, (uint32_t)id, idle, now)) continue;
     NodeMeta& m = c.meta[id];
@@ -292,6 +300,7 @@ __global__ void k_compact_plan(Ctx c, uint32_t idle, DrawUnit* units) {
     if (lane == 0) {
       if (all_fit) {
         off = atomicAdd(&c.ctl->bump, bytes);
+        if (off + bytes > c.data_bytes) off = ~0ull;
       } else {
         unsigned long long b = vload(&c.ctl->bump);
         while (b + bytes <= c.data_bytes) {
@@ -305,11 +314,13 @@ __global__ void k_compact_plan(Ctx c, uint32_t idle, DrawUnit* units) {
       }
       if (off != ~0ull) {
         p0 = atomicAdd(&c.ctl->pool_top, (int)nch);
-        u0 = atomicAdd(&c.ctl->draw_units, nch);
-        if (p0 < 0 || (unsigned long long)p0 + nch > c.max_chunks ||
-            (unsigned long long)u0 + nch > c.max_chunks) {
+        if (p0 < 0 || (unsigned long long)p0 + nch > c.max_chunks) {
           set_error(c, E_POOL);
           off = ~0ull;
+        } else {
+          // taken only with the pool's room: every unit below draw_units is
+          // written, and there are never more of them than pool entries
+          u0 = atomicAdd(&c.ctl->draw_units, nch);
         }
       }
     }
