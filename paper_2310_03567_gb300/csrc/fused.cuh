@@ -46,10 +46,11 @@ struct BatchList {
 
 // Control words of the fused kernel (arena). All zero between launches: the
 // last block to leave a launch clears them (a memset before every launch was
-// 2 us of the stream), but for `consumed`, which the host reads.
+// 2 us of the stream), but for `consumed`, which the host reads, and the abort
+// bit of a launch that failed.
 struct FusedCtl {
   // block arrivals at grid barriers since the launch began (gridDim.x per
-  // barrier); bit 63 (BAR_ABORT) aborts the launch
+  // barrier); bit 63 (BAR_ABORT) aborts the launch and those behind it
   unsigned long long bar;
   unsigned int consumed;  // batches fully handled (applied or rejected)
   unsigned int stop;      // the frame budget ran out
@@ -210,7 +211,8 @@ __device__ __forceinline__ void fused_body(const Ctx& c, const BatchDesc* batche
   PhaseClock clk{t_begin};
   const uint32_t nb = n_dev ? min(vload(n_dev), n_batches) : n_batches;
   // the node-table cache is loaded once and patched after every decide round
-  node_cache_load(c, smem, 0, vload(&c.ctl->n_nodes));
+  // (after a failed update the node count can lie above the table's end)
+  node_cache_load(c, smem, 0, min(vload(&c.ctl->n_nodes), c.max_nodes));
   __shared__ CtlView cv;  // control values after the last barrier that filled it
   CtlView* const vw = &cv;
   // counters that every thread follows by itself from batch to batch
@@ -358,7 +360,12 @@ __global__ void __launch_bounds__(FUSED_BLOCK, PHASE_MIN_BLOCKS)
   if (threadIdx.x == 0) {
     __threadfence();
     if (atomicAdd(&f->left, 1u) + 1u == gridDim.x) {
-      f->bar = 0;
+      // all but the abort bit, which stays until the octree is reset: a launch
+      // enqueued behind one that failed, before the host has seen the error,
+      // leaves at its first barrier, and until then it only counts, inside the
+      // node table (a look at the error at the start of every launch made the
+      // compiler spill or cost 0.3 to 0.8 % of an update)
+      atomicAnd(&f->bar, BAR_ABORT);
       f->stop = 0;
       f->left = 0;
     }
@@ -409,6 +416,7 @@ __global__ void k_plan_groups(Ctx c, const PlanInput* in, uint32_t n_in, const u
                               unsigned long long merge, BatchDesc* groups, PlanSeg* segs,
                               unsigned int* n_groups) {
   if (blockIdx.x != 0 || threadIdx.x != 0) return;
+  if (vload(&c.ctl->error) != 0u) return;  // an earlier update failed: no updates
   uint32_t ng = 0, ns = 0, rejected = 0;
   BatchDesc g{nullptr, 0, 0, 0};
   auto close = [&]() {

@@ -73,12 +73,22 @@ __global__ void k_clear_tables(Ctx c, int always) {
   for (uint64_t i = t0; i < c.hist_words; i += nt) c.hist[i] = 0;
 }
 
+// The batch was rejected, or an update (this one or one before it) failed: the
+// plain form's kernels leave. All threads of the block call and get one answer:
+// another block of the same kernel may set the error meanwhile.
+__device__ __forceinline__ bool plain_stop(const Ctx& c) {
+  return __syncthreads_or(threadIdx.x == 0 &&
+                          (vload(&c.ctl->reject) | vload(&c.ctl->error)) != 0u) != 0;
+}
+
 __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_count1(Ctx c, const int4* pts,
                                                                     uint64_t n, uint32_t n_nodes) {
   extern __shared__ uint32_t smem[];
   const uint64_t warps_per_block = blockDim.x / 32;
   after_previous();
+  const uint32_t err = threadIdx.x == 0 ? vload(&c.ctl->error) : 0u;
   node_cache_load(c, smem, 0, n_nodes);
+  if (__syncthreads_or(err != 0u)) return;
   phase_count1(c, smem, node_cache_at(smem, n_nodes), pts, n,
                blockIdx.x * warps_per_block + threadIdx.x / 32,
                (uint64_t)gridDim.x * warps_per_block);
@@ -90,8 +100,8 @@ __global__ void __launch_bounds__(BLOCK) k_decide(Ctx c, uint32_t n_lo, uint32_t
   after_previous();
   const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   const uint64_t nt = (uint64_t)gridDim.x * blockDim.x;
-  if (*reinterpret_cast<volatile unsigned int*>(&c.ctl->reject)) {
-    phase_rollback(c, n_hi, t0, nt);
+  if (plain_stop(c)) {
+    if (vload(&c.ctl->reject) != 0u) phase_rollback(c, n_hi, t0, nt);
     return;
   }
   phase_decide(c, n_lo, n_hi, t0 / 32, nt / 32);
@@ -104,13 +114,6 @@ __global__ void __launch_bounds__(BLOCK) k_decide(Ctx c, uint32_t n_lo, uint32_t
 // and store when one still has to: the host, which reads the control block
 // then, enqueues another round and them again. A wait for the host per round
 // (7 per update of a clustered scan) took longer than the kernels between.
-// (All threads of the block call and get one answer: another block of the
-// same kernel may set the error meanwhile.)
-__device__ __forceinline__ bool plain_stop(const Ctx& c) {
-  return __syncthreads_or(threadIdx.x == 0 &&
-                          (vload(&c.ctl->reject) != 0u || vload(&c.ctl->error) != 0u)) != 0;
-}
-
 // First split entry after round r (from 1) and the inner nodes it built (after
 // its build; split_inner stays until the next one).
 __host__ __device__ __forceinline__ uint32_t round_end(const Ctl* t, uint32_t r) {

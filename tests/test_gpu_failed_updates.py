@@ -43,3 +43,60 @@ def test_compaction_behind_a_failed_update(what):
     assert 0 < st["batches"] < len(batches)
     assert st["compacted_total"] == st["compact_nodes"] == 0
     works_after_reset(tree)
+
+
+def alone(what):
+    """Counters after the failing launch with nothing behind it."""
+    tree, batches, status = failing(what)
+    tree.insert_many(batches)
+    assert tree.sync() == status
+    return tree.stats()
+
+
+@pytest.mark.parametrize("what", ["arena", "nodes"])
+@pytest.mark.parametrize("behind", ["one", "many", "budget", "hostfed", "plan", "rejected"])
+def test_update_behind_a_failed_update(what, behind):
+    want = alone(what)
+    tree, batches, status = failing(what)
+    ptrs = [b.data_ptr() for b in batches]
+    counts = [len(b) for b in batches]
+    plan = tree.plan(ptrs, counts, merge_points=20_000) if behind == "plan" else None
+    out = PTS[:10].copy()
+    out["z"][4] = -1  # outside the root cube
+    bad = simlod.points_tensor(out)
+    host = [b.cpu().pin_memory() for b in batches[:3]]
+    dst = torch.empty((15_000, 16), dtype=torch.uint8, device="cuda")
+    ready = torch.zeros(3, dtype=torch.int32, device="cuda")
+    copies = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    tree.insert_many(batches)
+    for _ in range(2):
+        if behind == "one":
+            tree.insert_many(batches[:1])
+        elif behind == "many":
+            tree.insert_many(batches)
+        elif behind == "budget":
+            assert tree.insert_many_ptrs(ptrs, counts, budget_ns=10 ** 9) == simlod.OK
+        elif behind == "hostfed":
+            tree.insert_many_host(host, dst, ready, copies)
+        elif behind == "plan":
+            assert plan.run() == simlod.OK
+        else:
+            tree.insert_many([bad])
+    assert tree.sync() == status
+    got = tree.stats()
+    for k in ("batches", "points", "rejected_batches", "splits", "voxels", "last_points"):
+        assert got[k] == want[k], k
+    works_after_reset(tree)
+    if plan:
+        plan.close()
+
+
+def test_plain_update_behind_a_failed_update():
+    tree, batches, status = failing("nodes")
+    want = alone("nodes")
+    tree.insert_many(batches)
+    assert tree.insert(batches[0], check=False) == status
+    assert tree.insert(batches[0], check=False) == simlod.ERR_POISONED
+    assert tree.stats()["batches"] == want["batches"]
+    works_after_reset(tree)
