@@ -106,6 +106,8 @@ __global__ void k_render_select(Ctx c, View v, uint32_t* vis, unsigned long long
   after_previous();
   const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  // (nothing writes these during the frame: plain loads, most of them from L1)
+  const uint32_t err = c.ctl->error, n_nodes = c.ctl->n_nodes;
   if (clear) {
     // the frame is 8-byte aligned; 16-byte stores from its first 16-byte boundary
     const uint64_t head = (reinterpret_cast<uintptr_t>(fb) & 15u) ? 1u : 0u;
@@ -117,7 +119,9 @@ __global__ void k_render_select(Ctx c, View v, uint32_t* vis, unsigned long long
       if ((n_px - head) & 1u) fb[n_px - 1u] = ~0ull;
     }
   }
-  const uint32_t n = vload(&c.ctl->n_nodes);
+  // an octree whose last update failed is not drawn: ids that a failing build
+  // reserved have no metadata (the host learns of the error at its next look)
+  const uint32_t n = __any_sync(FULL_MASK, err != 0u) ? 0u : n_nodes;
   const uint32_t lane = threadIdx.x & 31u;
   for (uint64_t b = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); b < n; b += stride) {
     const uint64_t id = b + lane;

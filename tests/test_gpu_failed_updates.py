@@ -100,3 +100,22 @@ def test_plain_update_behind_a_failed_update():
     assert tree.insert(batches[0], check=False) == simlod.ERR_POISONED
     assert tree.stats()["batches"] == want["batches"]
     works_after_reset(tree)
+
+
+@pytest.mark.parametrize("what", ["arena", "nodes"])
+@pytest.mark.parametrize("clear", [True, False])
+def test_frame_behind_a_failed_update(what, clear):
+    # the frame is cleared as asked, and no node is drawn
+    tree, batches, status = failing(what)
+    side = float(1 << 16)
+    cam = simlod.view_proj([side * 0.1] * 3, [side / 2] * 3, 90.0, 2.0)
+    frame = torch.full((128, 256), 77, dtype=torch.int64, device="cuda")
+    tree.insert_many(batches)
+    tree.render(cam, frame, clear=clear)
+    assert tree.sync() == status
+    assert bool((frame == (-1 if clear else 77)).all())
+    st = tree.stats()
+    assert st["render_nodes"] == st["render_samples"] == 0
+    works_after_reset(tree)
+    tree.render(cam, frame)
+    assert tree.sync() == simlod.OK and bool((frame != -1).any())
