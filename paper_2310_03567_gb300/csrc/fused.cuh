@@ -145,6 +145,7 @@ __device__ __forceinline__ bool grid_barrier(const Ctx& c, FusedCtl* f, CtlView*
 // launch was aborted.
 __device__ __forceinline__ bool wait_ready(const Ctx& c, FusedCtl* f, const unsigned int* flag) {
   __shared__ int s_ok;
+  __syncthreads();  // behind an empty batch the last answer may still be being read
   if (threadIdx.x == 0) {
     int ok = 1;
     unsigned int v;

@@ -60,3 +60,20 @@ def test_a_launch_after_an_aborted_one(synced):
     assert tree.sync() == simlod.OK
     want = oracle.static_build(oracle.Config.make(**KW), pts[:6_000])
     assert_snapshots_equal(tree.snapshot(), want)
+
+
+@pytest.mark.parametrize("sizes", [(0, 0, 3_000, 0, 0, 0, 5_000, 0), (0,) * 20 + (4_000, 0, 0, 1)])
+def test_host_fed_lists_with_empty_batches(sizes):
+    # nothing but the wait for its flag stands between an empty batch and the next
+    tree, pts = make(), synth.uniform(10, 1 << 16, 2 * sum(sizes))
+    for lo in (0, sum(sizes)):
+        cut = np.split(pts[lo:lo + sum(sizes)], np.cumsum(sizes)[:-1])
+        host = [torch.from_numpy(np.ascontiguousarray(b).view(np.uint8).reshape(-1, 16)).pin_memory()
+                for b in cut]
+        dst = torch.empty((sum(sizes), 16), dtype=torch.uint8, device="cuda")
+        ready = torch.empty(len(sizes), dtype=torch.int32, device="cuda")
+        tree.insert_many_host(host, dst, ready, torch.cuda.Stream())
+        assert tree.sync() == simlod.OK
+    assert tree.progress() == (2 * len(sizes), 2 * len(sizes))
+    want = oracle.static_build(oracle.Config.make(**KW), pts)
+    assert_snapshots_equal(tree.snapshot(), want)
