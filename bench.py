@@ -644,7 +644,7 @@ def run_ours(args):
         "fused_phase_ms_per_step": phases,
         "render_1080p": render,
         "batched": batched,
-        "gpu_launches": 3 * args.steps,  # reset (two kernels) and the update
+        "gpu_launches": 2 * args.steps,  # the reset and the update
         "e2e": {"value": job_points / e2e_s / 1e6, "unit": UNIT,
                 # points, the batch table (24 B per batch) and, host-fed, a
                 # 4-byte ready flag per batch

@@ -29,14 +29,41 @@ namespace {
 constexpr int BLOCK = 256;
 constexpr int PBLOCK = PHASE_BLOCK;  // phase kernels (one node-table cache per block)
 
-__global__ void k_init(Ctx c, FusedCtl* f) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    memset(f, 0, sizeof(FusedCtl));  // (an error outside a launch leaves its abort bit there)
+// Empty the octree. The claim table and the histograms are emptied too, always
+// or when an update failed half way since they were last empty (a handle that is
+// reset without having been asked for its status does not know). The last block
+// to have looked at the error starts the control block anew. (A look by eight
+// blocks per SM and a launch of one thread behind it were 14.5 us a reset; this is
+// 6.2, which is what the host takes to enqueue it.)
+__global__ void __launch_bounds__(BLOCK) k_reset(Ctx c, FusedCtl* f, int always) {
+  __shared__ uint32_t s_flag;
+  if (threadIdx.x == 0) s_flag = always || vload(&c.ctl->error) != 0u;
+  __syncthreads();
+  if (s_flag) {
+    const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    const uint64_t nt = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t i = t0; i <= c.hash_mask; i += nt) {
+      c.hash[i].key = HASH_EMPTY;
+      c.hash[i].val = HASH_EMPTY;
+    }
+    for (uint64_t i = t0; i < c.hist_words; i += nt) c.hist[i] = 0;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_flag = atomicAdd(&f->left, 1u) + 1u == gridDim.x;  // zero between launches
+  }
+  __syncthreads();
+  if (!s_flag) return;
+  // diagnostics (phase_ns) survive a reset
+  constexpr uint32_t ns0 = offsetof(Ctl, phase_ns) / 4, ns1 = ns0 + sizeof(Ctl::phase_ns) / 4;
+  uint32_t* words = reinterpret_cast<uint32_t*>(c.ctl);
+  for (uint32_t i = threadIdx.x; i < sizeof(Ctl) / 4; i += blockDim.x)
+    if (i < ns0 || i >= ns1) words[i] = 0;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    memset(f, 0, sizeof(FusedCtl));  // (a failed launch leaves its abort bit there)
     Ctl* t = c.ctl;
-    unsigned long long phase_ns[8];  // diagnostics survive a reset
-    for (int k = 0; k < 8; ++k) phase_ns[k] = t->phase_ns[k];
-    memset(t, 0, sizeof(Ctl));
-    for (int k = 0; k < 8; ++k) t->phase_ns[k] = phase_ns[k];
     t->n_nodes = 1;
     t->bump = c.dir_bytes;  // the root's chunk directory is the first data ref
     t->bump0 = t->bump;
@@ -57,20 +84,6 @@ __global__ void k_init(Ctx c, FusedCtl* f) {
     c.cnt[0] = 0;
     c.num[0] = 0;
   }
-}
-
-// Empty the claim table and the histograms: always, or when an update failed
-// half way since they were last empty (a handle that is reset without having
-// been asked for its status does not know).
-__global__ void k_clear_tables(Ctx c, int always) {
-  if (!always && vload(&c.ctl->error) == 0u) return;
-  const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  const uint64_t nt = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t i = t0; i <= c.hash_mask; i += nt) {
-    c.hash[i].key = HASH_EMPTY;
-    c.hash[i].val = HASH_EMPTY;
-  }
-  for (uint64_t i = t0; i < c.hist_words; i += nt) c.hist[i] = 0;
 }
 
 // The batch was rejected, or an update (this one or one before it) failed: the
@@ -930,9 +943,9 @@ int finish_fused(simlod_t* h, uint32_t* consumed) {
 
 int init_octree(simlod_t* h, cudaStream_t s, bool clear_hash, bool wait) {
   const Ctx& c = h->ctx;
-  k_clear_tables<<<(unsigned)h->sm_count * 8, BLOCK, 0, s>>>(c, clear_hash ? 1 : 0);
-  if (cudaGetLastError() != cudaSuccess) return SIMLOD_ERR_CUDA;
-  k_init<<<1, 1, 0, s>>>(c, h->fctl_dev);
+  // (a block per SM is enough to look; all of them when there is something to do)
+  k_reset<<<(unsigned)h->sm_count * (clear_hash ? 8u : 1u), BLOCK, 0, s>>>(c, h->fctl_dev,
+                                                                          clear_hash ? 1 : 0);
   if (cudaGetLastError() != cudaSuccess) return SIMLOD_ERR_CUDA;
   if (wait && cudaStreamSynchronize(s) != cudaSuccess) return SIMLOD_ERR_CUDA;
   h->base = 0;
@@ -1048,9 +1061,11 @@ SIMLOD_API int simlod_create(const simlod_config* cfg, void* d_arena, size_t are
   }
   h->prog_host[0] = h->prog_host[1] = 0u;
   h->prog_submitted = 0u;
-  // the arena is the caller's memory: start from a zeroed control block
+  // the arena is the caller's memory: start from zeroed control blocks
   if (cudaMemsetAsync(h->ctx.ctl, 0, sizeof(Ctl), static_cast<cudaStream_t>(stream)) !=
-      cudaSuccess) {
+          cudaSuccess ||
+      cudaMemsetAsync(h->fctl_dev, 0, sizeof(FusedCtl), static_cast<cudaStream_t>(stream)) !=
+          cudaSuccess) {
     simlod_destroy(h);
     return SIMLOD_ERR_CUDA;
   }
