@@ -1557,12 +1557,34 @@ __device__ __forceinline__ void decide_node(const Ctx& c, uint32_t id) {
   }
 }
 
-// Candidates, one warp each: the node id range [n_lo, n_hi). In the expansion
-// rounds these are leaves; after the claim phase the counts left are the inner
-// nodes' new voxels, which get their chunks here.
-__device__ void phase_decide(const Ctx& c, uint32_t n_lo, uint32_t n_hi, uint64_t warp0,
-                             uint64_t nwarps) {
-  for (uint64_t w = n_lo + warp0; w < n_hi; w += nwarps) decide_node(c, (uint32_t)w);
+// Candidates: the node id range [n_lo, n_hi). In the expansion rounds these are
+// leaves; after the claim phase the counts left are the inner nodes' new voxels,
+// which get their chunks here. One warp per node. From DECIDE_SCAN nodes per warp
+// on, a warp first reads the counts of its next 32 nodes at once and visits those
+// that have one: a small update of a large octree then pays a round trip per 32
+// nodes (4,096 points into 300k nodes 36 against 52 us, into 104k nodes 33 against
+// 38; both looks at the nodes used to load five words of each). Below that the
+// look would only come in front of the node's own loads.
+constexpr uint32_t DECIDE_SCAN = 2;
+__device__ void phase_decide(const Ctx& c, uint32_t n_lo, uint32_t n_hi, uint32_t warp0,
+                             uint32_t nwarps) {
+  const bool scan = n_hi - n_lo > DECIDE_SCAN * nwarps;
+  uint32_t seen = n_lo + warp0;  // scan: the warp's first node not looked at yet
+  unsigned some = 0;             // which of the last 32 looked at are to be visited
+#pragma unroll 1
+  for (uint32_t w = seen; w < n_hi; w += nwarps) {
+    if (scan) {
+      while (some == 0u && seen < n_hi) {
+        const uint32_t id = seen + lane_id() * nwarps;
+        some = __ballot_sync(FULL_MASK, id < n_hi && __ldcg(c.cnt + id) != 0u);
+        seen += 32u * nwarps;
+      }
+      if (some == 0u) break;
+      w = seen - (33u - (uint32_t)__ffs(some)) * nwarps;
+      some &= some - 1u;
+    }
+    decide_node(c, w);
+  }
 }
 
 // The batch was rejected (a point outside the root cube): undo the counts of
