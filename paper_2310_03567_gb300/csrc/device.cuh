@@ -912,14 +912,18 @@ __device__ __forceinline__ uint32_t spread5(uint32_t x) {
 // levels for every leaf cost more counts than that saves (terrain: build 0.30
 // against 0.11 ms a pass; mixed batches: histogram 0.68 against 0.51 ms), 1 and
 // 2 levels more than the factors took a second round too often (clustered
-// scan: 1.72 and 1.57 against 1.50 ms). hist_words has room for one level.
-constexpr uint32_t HIST_DEPTH = 5;
+// scan: 1.72 and 1.57 against 1.50 ms). A leaf of more than 2^HIST_WIDE times T
+// points gets 3 levels again: its subtree would be thousands of nodes, which one
+// block would write (2M even points into leaves of 100: 0.08 against 0.34 ms).
+// hist_words has room for one level.
+constexpr uint32_t HIST_DEPTH = 5, HIST_WIDE = 9;
 __host__ __device__ __forceinline__ uint32_t hist_depth(const Ctx& c, uint32_t K, uint64_t n,
                                                         uint32_t most) {
   const uint64_t want = n < 32768u ? 32768u : n;
   const uint64_t lim = want < c.hist_words ? want : c.hist_words;
   uint32_t aim = 3, d = 1;
   while (aim < HIST_DEPTH && ((unsigned long long)c.T << (2u * (aim - 2u))) < most) ++aim;
+  if ((most >> HIST_WIDE) > c.T) aim = 3;
   while (d < aim && ((uint64_t)K << (3u * (d + 1u))) <= lim) ++d;
   return d;
 }
@@ -994,6 +998,146 @@ __device__ void phase_hist(const Ctx& c, uint32_t* smem, const NodeCache nc, con
 // 0 .. d-1 in this order, then the list of the inner nodes among them.
 __device__ __forceinline__ uint32_t level_first(uint32_t j) { return ((1u << (3u * j)) - 1u) / 7u; }
 
+// A split leaf that a build turns into a subtree.
+struct BuildRoot {
+  uint32_t id, level, L;  // L: log2 size
+  int32_t min[3];
+};
+
+__device__ __forceinline__ BuildRoot build_root(const Ctx& c, uint32_t id) {
+  const NodeMeta& m = c.meta[id];
+  return BuildRoot{id, m.level, c.rlog2 - m.level, {m.min[0], m.min[1], m.min[2]}};
+}
+
+// Node `kid` at the octant path `path`, j + 1 levels below the root: a child of
+// `up` (whose grid is up_grid); an inner node with children at `first` and a
+// grid, or (first = NONE) a leaf of n points with a directory.
+__device__ __forceinline__ void build_node(const Ctx& c, const BuildRoot& r, uint32_t kid,
+                                           uint32_t j, uint32_t path, uint32_t up,
+                                           uint32_t up_grid, uint32_t first, uint32_t grid,
+                                           uint32_t dir, uint32_t n) {
+  NodeMeta cm;
+  for (uint32_t a = 0; a < 3; ++a) {
+    cm.min[a] = r.min[a];
+#pragma unroll 1
+    for (uint32_t l = 0; l <= j; ++l)  // octant digits, the topmost first
+      cm.min[a] += (int32_t)(((path >> (3u * (j - l) + a)) & 1u) << (r.L - 1u - l));
+  }
+  cm.level = r.level + j + 1u;
+  cm.n_chunks = 0;
+  cm.head = cm.tail = NONE;
+  cm.dir = first == NONE ? dir : NONE;
+  cm.st_nch = 0;
+  cm.st_tail = NONE;
+  cm.st_seq = 0;
+  cm.st_base = 0;
+  cm.touched = 0;
+  cm.compact = 0;
+  cm.up = up | ((r.level + j) << NODE_BITS);
+  cm.up_grid = up_grid;
+  c.meta[kid] = cm;
+  c.child[kid] = first;
+  c.gridref[kid] = first == NONE ? NONE : grid;
+  c.cnt[kid] = first == NONE ? n : 0u;
+  c.num[kid] = 0;
+}
+
+// Room for ns inner nodes' children, directories and grids, and for the list
+// entries of all but the root. False (and an error) when there is none.
+struct BuildRoom {
+  uint32_t node0, entry;
+  unsigned long long data;
+};
+
+__device__ __forceinline__ bool build_room(const Ctx& c, uint32_t ns, uint32_t rounds,
+                                           uint32_t max_iters, BuildRoom& b) {
+  const unsigned long long bytes = (unsigned long long)ns * (8u * c.dir_bytes + c.grid_bytes);
+  b.node0 = atomicAdd(&c.ctl->n_nodes, 8u * ns);
+  b.data = atomicAdd(&c.ctl->bump, bytes);
+  b.entry = ns > 1u ? atomicAdd(&c.ctl->split_count, ns - 1u) : 0u;
+  if (ns > 1u) atomicAdd(&c.ctl->split_inner, ns - 1u);
+  if (rounds >= max_iters) set_error(c, E_ITER_CAP);
+  else if ((unsigned long long)b.node0 + 8ull * ns > c.max_nodes ||
+           (unsigned long long)b.entry + ns > c.max_splits)
+    set_error(c, E_NODES);
+  else if (b.data + bytes > c.data_bytes) set_error(c, E_ARENA);
+  else return true;
+  return false;
+}
+
+// The build for histograms of one or two levels, which are what many leaves that
+// split together get (hist_depth): one warp per leaf. Lanes 4q to 4q + 3 hold the
+// points of child q; with two levels a child of more than T points is an inner
+// node too, with the next 8 of the node ids. (2M even points in 500k batches into
+// leaves of one point: histograms and builds 2.2 ms, with a block and its barriers
+// per leaf 9.0; of 10 points 0.18 against 0.95.)
+__device__ void phase_build_warps(const Ctx& c, uint32_t s_lo, uint32_t K, uint32_t d,
+                                  uint32_t lvl0, uint32_t max_iters, uint32_t warp0,
+                                  uint32_t nwarps) {
+  const uint32_t lane = lane_id();
+  uint32_t deepest = 0;
+  for (uint32_t k = warp0; k < K; k += nwarps) {
+    uint32_t* hist = c.hist + ((uint64_t)k << (3u * d));
+    const BuildRoot r = build_root(c, c.splits[s_lo + k]);
+    uint32_t sum;
+    if (d == 1u) {
+      sum = hist[lane >> 2];
+    } else {
+      const uint2 b = reinterpret_cast<const uint2*>(hist)[lane];
+      sum = b.x + b.y;
+      sum += __shfl_xor_sync(FULL_MASK, sum, 1);
+      sum += __shfl_xor_sync(FULL_MASK, sum, 2);
+    }
+    const unsigned deep = __ballot_sync(  // bit 4q: child q is an inner node
+        FULL_MASK, (lane & 3u) == 0u && d > 1u && r.L > 1u && sum > c.T);
+    const uint32_t ns = 1u + (uint32_t)__popc(deep);
+    const uint32_t rounds = lvl0 + (ns > 1u ? 2u : 1u);
+    deepest = rounds > deepest ? rounds : deepest;
+    BuildRoom b{0, 0, 0};
+    bool ok = false;
+    if (lane == 0) ok = build_room(c, ns, rounds, max_iters, b);
+    ok = __shfl_sync(FULL_MASK, (int)ok, 0) != 0;
+    if (ok) {
+      b.node0 = __shfl_sync(FULL_MASK, b.node0, 0);
+      b.entry = __shfl_sync(FULL_MASK, b.entry, 0);
+      b.data = __shfl_sync(FULL_MASK, b.data, 0);
+      const unsigned long long grid0 = b.data + (unsigned long long)ns * 8u * c.dir_bytes;
+      auto grid_of = [&](uint32_t e) -> uint32_t {
+        return (uint32_t)((grid0 + (unsigned long long)e * c.grid_bytes) / REF_BYTES);
+      };
+      auto number = [&](uint32_t q) -> uint32_t {  // of inner child q; the root is 0
+        return 1u + (uint32_t)__popc(deep & ((1u << (4u * q)) - 1u));
+      };
+#pragma unroll 1
+      for (uint32_t t0 = 0; t0 < 8u * ns; t0 += 32u) {
+        const uint32_t t = t0 + lane, e = t >> 3, o = t & 7u;
+        const uint32_t n0 = __shfl_sync(FULL_MASK, sum, (int)(4u * o));
+        if (t >= 8u * ns) continue;
+        const uint32_t dir =
+            (uint32_t)((b.data + (unsigned long long)t * c.dir_bytes) / REF_BYTES);
+        const bool in = e == 0u && ((deep >> (4u * o)) & 1u);
+        const uint32_t f = number(o);
+        unsigned rest = deep;
+#pragma unroll 1
+        for (uint32_t x = 1; x < e; ++x) rest &= rest - 1u;
+        const uint32_t q = (uint32_t)(__ffs(rest) - 1) >> 2;  // e > 0: the e-th inner child
+        const uint32_t path = e == 0u ? o : 8u * q + o;
+        build_node(c, r, b.node0 + t, e == 0u ? 0u : 1u, path, e == 0u ? r.id : b.node0 + q,
+                   grid_of(e), in ? b.node0 + 8u * f : NONE, grid_of(f), dir,
+                   e == 0u ? n0 : hist[path]);
+      }
+      if ((deep >> lane) & 1u) c.splits[b.entry + number(lane >> 2) - 1u] = b.node0 + (lane >> 2);
+      if (lane == 0) {
+        c.child[r.id] = b.node0;
+        c.gridref[r.id] = grid_of(0);
+      }
+    }
+    __syncwarp();  // all counts have been read
+    if (lane < (2u << (3u * (d - 1u)))) reinterpret_cast<uint4*>(hist)[lane] = make_uint4(0, 0, 0, 0);
+  }
+  if (lane == 0 && deepest) atomicMax(&c.ctl->iters, deepest + 1u);
+}
+
 // One block per split leaf (entries [s_lo, s_lo + K)): sum its cube counts
 // level by level, make every cube with more than T points an inner node (8
 // children with chunk directories, and a grid each, zeroed in the claim
@@ -1005,6 +1149,12 @@ __device__ __forceinline__ uint32_t level_first(uint32_t j) { return ((1u << (3u
 // (128 KB at d = 5) from L2, which the other blocks do at the same time.
 __device__ void phase_build(const Ctx& c, uint32_t s_lo, uint32_t K, uint32_t d, uint32_t lvl0,
                             uint32_t max_iters) {
+  if (d <= 2u) {
+    const uint32_t wpb = blockDim.x / 32u;
+    phase_build_warps(c, s_lo, K, d, lvl0, max_iters, blockIdx.x * wpb + threadIdx.x / 32u,
+                      gridDim.x * wpb);
+    return;
+  }
   __shared__ uint32_t s_n, s_deep, s_node, s_entry, s_ok;
   __shared__ unsigned long long s_data;
   const uint32_t U = level_first(d), bins = 1u << (3u * d);
@@ -1012,10 +1162,7 @@ __device__ void phase_build(const Ctx& c, uint32_t s_lo, uint32_t K, uint32_t d,
     uint32_t* hist = c.hist + ((uint64_t)k << (3u * d));
     uint32_t* up = c.hist_up + (uint64_t)k * 2u * U;
     uint32_t* list = up + U;
-    const uint32_t root = c.splits[s_lo + k];
-    const NodeMeta& m = c.meta[root];
-    const uint32_t L = c.rlog2 - m.level, level = m.level;
-    const int32_t rm[3] = {m.min[0], m.min[1], m.min[2]};
+    const BuildRoot r = build_root(c, c.splits[s_lo + k]);
     if (threadIdx.x == 0) s_n = s_deep = 0;
     for (uint32_t j = d; j-- > 0;) {
       const uint32_t* below = up + level_first(j + 1u);
@@ -1037,7 +1184,7 @@ __device__ void phase_build(const Ctx& c, uint32_t s_lo, uint32_t K, uint32_t d,
     for (uint32_t i = threadIdx.x; i < U; i += blockDim.x) {
       uint32_t j = 0;
       while (level_first(j + 1u) <= i) ++j;
-      if (i == 0 || (up[i] > c.T && L > j)) {
+      if (i == 0 || (up[i] > c.T && r.L > j)) {
         const uint32_t e = atomicAdd(&s_n, 1u);
         atomicMax(&s_deep, j);
         list[e] = i;
@@ -1047,20 +1194,13 @@ __device__ void phase_build(const Ctx& c, uint32_t s_lo, uint32_t K, uint32_t d,
     __syncthreads();
     const uint32_t ns = s_n;
     if (threadIdx.x == 0) {
-      const unsigned long long bytes = (unsigned long long)ns * (8u * c.dir_bytes + c.grid_bytes);
       const uint32_t rounds = lvl0 + s_deep + 1u;
-      s_node = atomicAdd(&c.ctl->n_nodes, 8u * ns);
-      s_data = atomicAdd(&c.ctl->bump, bytes);
-      s_entry = ns > 1u ? atomicAdd(&c.ctl->split_count, ns - 1u) : 0u;
-      if (ns > 1u) atomicAdd(&c.ctl->split_inner, ns - 1u);
+      BuildRoom b;
+      s_ok = build_room(c, ns, rounds, max_iters, b);
+      s_node = b.node0;
+      s_data = b.data;
+      s_entry = b.entry;
       atomicMax(&c.ctl->iters, rounds + 1u);
-      s_ok = 0;
-      if (rounds >= max_iters) set_error(c, E_ITER_CAP);
-      else if ((unsigned long long)s_node + 8ull * ns > c.max_nodes ||
-               (unsigned long long)s_entry + ns > c.max_splits)
-        set_error(c, E_NODES);
-      else if (s_data + bytes > c.data_bytes) set_error(c, E_ARENA);
-      else s_ok = 1;
     }
     __syncthreads();
     if (s_ok) {
@@ -1069,44 +1209,24 @@ __device__ void phase_build(const Ctx& c, uint32_t s_lo, uint32_t K, uint32_t d,
       auto grid_of = [&](uint32_t e) -> uint32_t {
         return (uint32_t)((grid0 + (unsigned long long)e * c.grid_bytes) / REF_BYTES);
       };
+#pragma unroll 1
       for (uint32_t t = threadIdx.x; t < 8u * ns; t += blockDim.x) {
         const uint32_t e = t >> 3, o = t & 7u, i = list[e];
         uint32_t j = 0;
         while (level_first(j + 1u) <= i) ++j;
         const uint32_t q = i - level_first(j);
         const uint32_t id =
-            j == 0 ? root : node0 + 8u * (up[level_first(j - 1u) + (q >> 3)] & ~SPLIT_MARK) + (q & 7u);
+            j == 0 ? r.id : node0 + 8u * (up[level_first(j - 1u) + (q >> 3)] & ~SPLIT_MARK) + (q & 7u);
         const uint32_t path = 8u * q + o, kid = node0 + t;
         const uint32_t w = j + 1u == d ? hist[path] : up[level_first(j + 1u) + path];
         const bool inner = j + 1u < d && (w & SPLIT_MARK);
-        NodeMeta cm;
-        for (uint32_t a = 0; a < 3; ++a) {
-          cm.min[a] = rm[a];
-          for (uint32_t l = 0; l <= j; ++l)  // octant digits, the topmost first
-            cm.min[a] += (int32_t)(((path >> (3u * (j - l) + a)) & 1u) << (L - 1u - l));
-        }
-        cm.level = level + j + 1u;
-        cm.n_chunks = 0;
-        cm.head = cm.tail = NONE;
-        cm.dir = inner ? NONE
-                       : (uint32_t)((s_data + (unsigned long long)t * c.dir_bytes) / REF_BYTES);
-        cm.st_nch = 0;
-        cm.st_tail = NONE;
-        cm.st_seq = 0;
-        cm.st_base = 0;
-        cm.touched = 0;
-        cm.compact = 0;
-        cm.up = id | ((level + j) << NODE_BITS);
-        cm.up_grid = grid_of(e);
-        c.meta[kid] = cm;
-        c.child[kid] = inner ? node0 + 8u * (w & ~SPLIT_MARK) : NONE;
-        c.gridref[kid] = inner ? grid_of(w & ~SPLIT_MARK) : NONE;
-        c.cnt[kid] = inner ? 0u : w;
-        c.num[kid] = 0;
+        const uint32_t x = w & ~SPLIT_MARK;  // an inner node's number
+        build_node(c, r, kid, j, path, id, grid_of(e), inner ? node0 + 8u * x : NONE, grid_of(x),
+                   (uint32_t)((s_data + (unsigned long long)t * c.dir_bytes) / REF_BYTES), w);
         if (o == 0) {
           if (j == 0) {
-            c.child[root] = node0 + 8u * e;
-            c.gridref[root] = grid_of(e);
+            c.child[r.id] = node0 + 8u * e;
+            c.gridref[r.id] = grid_of(e);
           } else {
             // entry numbers without the root's
             const uint32_t re = up[0] & ~SPLIT_MARK;
