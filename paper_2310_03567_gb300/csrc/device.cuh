@@ -1436,7 +1436,12 @@ __device__ void phase_claim(const Ctx& c, uint32_t* smem, const NodeCache nc, co
   };
 #pragma unroll
   for (int j = 0; j < U; ++j) load(warp_unit(warp0, nwarps, j, chl), pn[j], curn[j], gn[j]);
-  for (uint32_t k = 0; warp_unit(warp0, nwarps, k, chl) < units; k += U) {
+  // (the last time round there are no points, and the queue is emptied: one copy
+  // of the drain, 10 KB of code less than with a second one behind the loop. The
+  // persistent kernel's phases share the instruction caches: a 16M-point terrain
+  // 2.248 against 2.266 ms)
+  for (uint32_t k = 0, more = 1; more; k += U) {
+    more = warp_unit(warp0, nwarps, k, chl) < units;
     bool on[U];
     ClaimItem it[U];
 #pragma unroll
@@ -1459,9 +1464,8 @@ __device__ void phase_claim(const Ctx& c, uint32_t* smem, const NodeCache nc, co
       }
     }
     claim_level<U, true>(c, wb, cq, a, on, it, warp_unit(warp0, nwarps, k, chl) < us);
-    claim_drain(c, wb, cq, a, 31u);
+    claim_drain(c, wb, cq, a, more ? 31u : 0u);
   }
-  claim_drain(c, wb, cq, a, 0u);
   warp_flush(c, wb);
   tally_flush(c.cnt, smem);
 }
