@@ -127,46 +127,72 @@ __global__ void __launch_bounds__(BLOCK) k_decide(Ctx c, uint32_t n_lo, uint32_t
 // and store when one still has to: the host, which reads the control block
 // then, enqueues another round and them again. A wait for the host per round
 // (7 per update of a clustered scan) took longer than the kernels between.
-// First split entry after round r (from 1) and the inner nodes it built (after
-// its build; split_inner stays until the next one).
-__host__ __device__ __forceinline__ uint32_t round_end(const Ctl* t, uint32_t r) {
-  if (r == 0u) return 0u;
-  const volatile PlainRound& p = t->round[r];
-  return p.s_lo + p.K + (*static_cast<const volatile unsigned int*>(&t->split_inner) - p.inner);
+// What such a kernel finds in the control block: loaded by one thread of the
+// block, all at once (one after another, by every thread, the loads were five round
+// trips in front of a claim). r: the last round whose end counts.
+struct PlainView {
+  unsigned long long bump0;
+  uint32_t stop, end, split_count, split_inner, split_most, ntasks, n_nodes, spill_count, nkeys;
+  uint32_t open, key_rate;
+  int pool_top;
+  PlainRound round;
+};
+
+__device__ __forceinline__ const PlainView& plain_view(const Ctx& c, uint32_t r) {
+  __shared__ PlainView v;
+  if (threadIdx.x == 0) {
+    const Ctl* t = c.ctl;
+    const PlainRound* p = &t->round[r];
+    v.stop = vload(&t->reject) | vload(&t->error);
+    v.split_count = vload(&t->split_count);
+    v.split_inner = vload(&t->split_inner);
+    v.split_most = vload(&t->split_most);
+    v.ntasks = vload(&t->ntasks);
+    v.n_nodes = vload(&t->n_nodes);
+    v.spill_count = vload(&t->spill_count);
+    v.nkeys = vload(&t->nkeys);
+    v.bump0 = vload(&t->bump0);
+    v.open = vload(&t->open);
+    v.key_rate = vload(&t->key_rate);
+    v.pool_top = vload(&t->pool_top);
+    v.round = PlainRound{vload(&p->s_lo), vload(&p->K),    vload(&p->inner),
+                         vload(&p->d),    vload(&p->lvl0), vload(&p->n_lo)};
+    v.end = r ? v.round.s_lo + v.round.K + (v.split_inner - v.round.inner) : 0u;
+  }
+  __syncthreads();
+  return v;
 }
 
 __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_hist(Ctx c, const int4* pts,
                                                                   uint64_t n, uint32_t r) {
   extern __shared__ uint32_t smem[];
   after_previous();
-  if (plain_stop(c)) return;
-  const uint32_t s_lo = round_end(c.ctl, r - 1u);
-  const uint32_t K = vload(&c.ctl->split_count) - s_lo, n_nodes = vload(&c.ctl->n_nodes);
-  const uint32_t d = hist_depth(c, K, n + vload(&c.ctl->spill_count), vload(&c.ctl->split_most));
+  const PlainView& v = plain_view(c, r - 1u);
+  if (v.stop) return;
+  const uint32_t s_lo = v.end, K = v.split_count - s_lo;
+  const uint32_t d = hist_depth(c, K, n + v.spill_count, v.split_most);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    const uint32_t lvl0 = r > 1u ? c.ctl->round[r - 1u].lvl0 + c.ctl->round[r - 1u].d : 0u;
-    c.ctl->round[r] = PlainRound{s_lo, K, vload(&c.ctl->split_inner), d, lvl0, n_nodes};
+    const uint32_t lvl0 = r > 1u ? v.round.lvl0 + v.round.d : 0u;
+    c.ctl->round[r] = PlainRound{s_lo, K, v.split_inner, d, lvl0, v.n_nodes};
   }
   if (K == 0u) return;
-  node_cache_load(c, smem, 0, n_nodes);
-  phase_hist(c, smem, node_cache_at(smem, n_nodes), pts, n, vload(&c.ctl->ntasks), s_lo, K, d,
-             r == 1u);
+  node_cache_load(c, smem, 0, v.n_nodes);
+  phase_hist(c, smem, node_cache_at(smem, v.n_nodes), pts, n, v.ntasks, s_lo, K, d, r == 1u);
 }
 
 __global__ void __launch_bounds__(PBLOCK) k_build(Ctx c, uint32_t r, uint32_t max_iters) {
   after_previous();
-  if (plain_stop(c)) return;
-  const PlainRound* p = &c.ctl->round[r];
-  if (vload(&p->K)) phase_build(c, vload(&p->s_lo), vload(&p->K), vload(&p->d), vload(&p->lvl0),
-                                max_iters);
+  const PlainView& v = plain_view(c, r);
+  if (v.stop || v.round.K == 0u) return;
+  phase_build(c, v.round.s_lo, v.round.K, v.round.d, v.round.lvl0, max_iters);
 }
 
 __global__ void __launch_bounds__(BLOCK) k_decide_new(Ctx c, uint32_t r) {
   after_previous();
-  if (plain_stop(c) || vload(&c.ctl->round[r].K) == 0u) return;
-  phase_decide(c, vload(&c.ctl->round[r].n_lo), vload(&c.ctl->n_nodes),
-               (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) / 32,
-               (uint64_t)gridDim.x * blockDim.x / 32);
+  const PlainView& v = plain_view(c, r);
+  if (v.stop || v.round.K == 0u) return;
+  phase_decide(c, v.round.n_lo, v.n_nodes, (blockIdx.x * blockDim.x + threadIdx.x) / 32,
+               gridDim.x * blockDim.x / 32);
 }
 
 __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_claim(Ctx c, const int4* pts, uint64_t n,
@@ -174,25 +200,24 @@ __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_claim(Ctx c, const
                                                      uint32_t r) {
   extern __shared__ uint32_t smem[];
   after_previous();
-  if (plain_stop(c) || vload(&c.ctl->split_count) != round_end(c.ctl, r)) return;
-  const uint32_t s_hi = vload(&c.ctl->split_count), t_hi = vload(&c.ctl->ntasks);
-  const uint64_t wpb = blockDim.x / 32;
-  if (s_hi == 0u && blockIdx.x * wpb * 32u >= n) return;  // nothing for this block
-  const uint32_t n_nodes = vload(&c.ctl->n_nodes);
-  const ClaimArgs a{nodes0, (uint32_t)(vload(&c.ctl->bump0) / REF_BYTES), vload(&c.ctl->open),
-                    claim_near_mask(c, n + vload(&c.ctl->spill_count), vload(&c.ctl->key_rate))};
-  node_cache_load(c, smem, 0, n_nodes);
-  phase_claim(c, smem, node_cache_at(smem, n_nodes), pts, n, base, t_hi, s_hi, a,
-              blockIdx.x * wpb + threadIdx.x / 32, (uint64_t)gridDim.x * wpb);
+  const PlainView& v = plain_view(c, r);
+  if (v.stop || v.split_count != v.end) return;
+  const uint32_t wpb = blockDim.x / 32;
+  if (v.split_count == 0u && (uint64_t)blockIdx.x * wpb * 32u >= n) return;  // nothing to do
+  const ClaimArgs a{nodes0, (uint32_t)(v.bump0 / REF_BYTES), v.open,
+                    claim_near_mask(c, n + v.spill_count, v.key_rate)};
+  node_cache_load(c, smem, 0, v.n_nodes);
+  phase_claim(c, smem, node_cache_at(smem, v.n_nodes), pts, n, base, v.ntasks, v.split_count, a,
+              blockIdx.x * wpb + threadIdx.x / 32, gridDim.x * wpb);
 }
 
 // Chunks for the new voxels of the inner nodes.
 __global__ void __launch_bounds__(BLOCK) k_alloc_voxels(Ctx c, uint32_t r) {
   after_previous();
-  if (plain_stop(c) || vload(&c.ctl->split_count) != round_end(c.ctl, r)) return;
-  phase_decide(c, 0, vload(&c.ctl->n_nodes),
-               (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) / 32,
-               (uint64_t)gridDim.x * blockDim.x / 32);
+  const PlainView& v = plain_view(c, r);
+  if (v.stop || v.split_count != v.end) return;
+  phase_decide(c, 0, v.n_nodes, (blockIdx.x * blockDim.x + threadIdx.x) / 32,
+               gridDim.x * blockDim.x / 32);
 }
 
 // The points and, their nodes' chunks being there too, the voxels; the last
@@ -203,12 +228,12 @@ __global__ void __launch_bounds__(BLOCK) k_alloc_voxels(Ctx c, uint32_t r) {
 __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_store(Ctx c, const int4* pts, uint64_t n,
                                                   unsigned long long base, uint32_t r) {
   extern __shared__ uint32_t smem[];
-  if (plain_stop(c) || vload(&c.ctl->split_count) != round_end(c.ctl, r)) return;
+  const PlainView& v = plain_view(c, r);
+  if (v.stop || v.split_count != v.end) return;
   const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   const uint64_t nt = (uint64_t)gridDim.x * blockDim.x;
-  const uint32_t t_hi = vload(&c.ctl->ntasks);
-  const uint32_t n_keys = min(vload(&c.ctl->nkeys), c.backlog_cap);
-  const int pool_top = vload(&c.ctl->pool_top);
+  const uint32_t t_hi = v.ntasks, n_keys = min(v.nkeys, c.backlog_cap);
+  const int pool_top = v.pool_top;
   phase_store(c, smem, pts, n, base, t_hi);
   phase_store_voxels(c, smem, t_hi, n_keys, pool_top, t0, nt);
   __threadfence();
@@ -743,13 +768,11 @@ int launch(simlod_t* h, int kernel, cudaStream_t s, Launch&& fn) {
 // Launch a kernel that begins with after_previous() behind another of this
 // library: its blocks may be placed while the last blocks of the one before
 // still run, and wait there for its end (programmatic dependent launch), so that
-// the launch itself costs nothing between short kernels. Plain launches while
-// the stream is captured.
+// the launch itself costs nothing between short kernels. overlap = false: a plain
+// launch.
 template <typename... P, typename... A>
-void launch_next(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
-                 A&&... args) {
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cap = cudaStreamCaptureStatusActive;
+void launch_next(bool overlap, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
+                 cudaStream_t s, A&&... args) {
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
@@ -759,8 +782,14 @@ void launch_next(void (*kernel)(P...), unsigned grid, unsigned block, size_t sme
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = &attr;
-  cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+  cfg.numAttrs = overlap ? 1 : 0;
   cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// Renders and compactions may be captured: plain launches then.
+bool captured(cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
 }
 
 unsigned grid_for(const simlod_t* h, uint64_t work, uint64_t per_block) {
@@ -792,6 +821,12 @@ int read_ctl(simlod_t* h, cudaStream_t s) {
   return SIMLOD_OK;
 }
 
+// First split entry behind round r (0: none yet) and the inner nodes that it built.
+uint32_t round_end(const Ctl* t, uint32_t r) {
+  const PlainRound& p = t->round[r];
+  return r ? p.s_lo + p.K + (t->split_inner - p.inner) : 0u;
+}
+
 int insert_device(simlod_t* h, const int4* pts, uint64_t n, cudaStream_t s) {
   if (h->mirror_stale) {
     int r0 = read_ctl(h, h->last_stream);
@@ -812,7 +847,7 @@ int insert_device(simlod_t* h, const int4* pts, uint64_t n, cudaStream_t s) {
   });
   if (rc) return poison(h, rc);
   rc = launch(h, K_DECIDE, s, [&] {
-    launch_next(k_decide, grid_for(h, 32ull * nodes0, BLOCK), BLOCK, 0, s, c, 0u, nodes0);
+    launch_next(true, k_decide, grid_for(h, 32ull * nodes0, BLOCK), BLOCK, 0, s, c, 0u, nodes0);
   });
   if (rc) return poison(h, rc);
   const Ctl& t = *h->ctl_host;
@@ -821,20 +856,20 @@ int insert_device(simlod_t* h, const int4* pts, uint64_t n, cudaStream_t s) {
   for (uint32_t r = h->plain_split ? 1u : 0u;; ++r) {
     if (r) {
       rc = launch(h, K_ADVANCE, s, [&] {
-        launch_next(k_hist, full, PBLOCK, PHASE_SMEM_BYTES, s, c, pts, n, r);
-        launch_next(k_build, full, PBLOCK, 0, s, c, r, max_iters);
+        launch_next(true, k_hist, full, PBLOCK, PHASE_SMEM_BYTES, s, c, pts, n, r);
+        launch_next(true, k_build, full, PBLOCK, 0, s, c, r, max_iters);
       });
       if (rc) return poison(h, rc);
       rc = launch(h, K_DECIDE, s, [&] {
-        launch_next(k_decide_new, full * 2, BLOCK, 0, s, c, r);
+        launch_next(true, k_decide_new, full * 2, BLOCK, 0, s, c, r);
       });
       if (rc) return poison(h, rc);
     }
     rc = launch(h, K_CLAIM, s, [&] {
-      launch_next(k_claim, r ? full : gp, PBLOCK, PHASE_SMEM_BYTES, s, c, pts, n, base, nodes0, r);
+      launch_next(true, k_claim, r ? full : gp, PBLOCK, PHASE_SMEM_BYTES, s, c, pts, n, base, nodes0, r);
     });
     if (rc) return poison(h, rc);
-    rc = launch(h, K_DECIDE, s, [&] { launch_next(k_alloc_voxels, full * 2, BLOCK, 0, s, c, r); });
+    rc = launch(h, K_DECIDE, s, [&] { launch_next(true, k_alloc_voxels, full * 2, BLOCK, 0, s, c, r); });
     if (rc) return poison(h, rc);
     // the host waits for the copy of the control block, not for the store
     if (cudaMemcpyAsync(h->ctl_host, c.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s) !=
@@ -1803,9 +1838,10 @@ SIMLOD_API int simlod_compact(simlod_t* h, uint32_t idle_updates, void* stream) 
   uint32_t parts, part;
   unit_parts(c.C, &parts, &part);
   const unsigned grid = (unsigned)h->sm_count * 8;
+  const bool overlap = !captured(s);
   k_compact_need<<<grid, BLOCK, 0, s>>>(c, idle_updates);
-  launch_next(k_compact_plan, grid, BLOCK, 0, s, c, idle_updates, units);
-  launch_next(k_compact_copy, grid, BLOCK, 0, s, c, units, parts, part);
+  launch_next(overlap, k_compact_plan, grid, BLOCK, 0, s, c, idle_updates, units);
+  launch_next(overlap, k_compact_copy, grid, BLOCK, 0, s, c, units, parts, part);
   return cudaGetLastError() == cudaSuccess ? SIMLOD_OK : poison(h, SIMLOD_ERR_CUDA);
 }
 
@@ -1840,10 +1876,11 @@ SIMLOD_API int simlod_render(simlod_t* h, const float view_proj[16], uint32_t wi
   uint32_t parts, part;
   unit_parts(c.C, &parts, &part);
   const unsigned grid = (unsigned)h->sm_count * 8;
+  const bool overlap = !captured(s);
   return launch(h, K_RENDER, s, [&] {
     k_render_select<<<grid, BLOCK, 0, s>>>(c, v, vis, fb, (uint64_t)width * height, clear);
-    launch_next(k_render_units, grid, BLOCK, 0, s, c, v, vis, units, fb);
-    launch_next(k_render_draw, grid, BLOCK, 0, s, c, v, units, parts, part, fb);
+    launch_next(overlap, k_render_units, grid, BLOCK, 0, s, c, v, vis, units, fb);
+    launch_next(overlap, k_render_draw, grid, BLOCK, 0, s, c, v, units, parts, part, fb);
   });
 }
 
