@@ -150,7 +150,8 @@ __device__ __forceinline__ void splat(const View& v, int4 r, unsigned long long*
 }
 
 // A piece of a drawn node: records [first, first + n) of the chunk or array
-// at ref. At most C records, so that a node's records spread over many warps.
+// at ref, a chunk's or about as many, so that a node's records spread over many
+// warps.
 // (Compaction: n records of the chunk at ref that go to records first, ... of
 // the array at arr.)
 struct DrawUnit {
@@ -250,50 +251,122 @@ __device__ __forceinline__ uint32_t chunk_fill(const Ctx& c, uint32_t j, uint32_
   return at < n ? (uint32_t)min((unsigned long long)c.C, n - at) : 0u;
 }
 
-// One warp per drawn node: cut its records into draw units of one chunk (or C
-// records of a compacted node's array).
-__global__ void k_render_units(Ctx c, View v, const uint32_t* vis, DrawUnit* units,
+// All 32 lanes call: draw the n records of up to 32 chunks at once, C of them in
+// each but the last; lane j holds the reference of chunk j (of those in `have`).
+__device__ __forceinline__ void draw_chunks(const Ctx& c, const View& v, uint32_t ref,
+                                            unsigned have, uint32_t n, unsigned long long* fb) {
+#pragma unroll 2
+  for (uint32_t q0 = 0; q0 < n; q0 += 32u) {
+    const uint32_t q = q0 + lane_id(), j = div_by(q, c.C, c.C_mul, c.C_shift);
+    const uint32_t from = __shfl_sync(FULL_MASK, ref, (int)(j & 31u));
+    if (q < n && ((have >> (j & 31u)) & 1u)) splat(v, __ldcg(chunk_recs(c, from) + (q - j * c.C)), fb);
+  }
+}
+
+// Cut the drawn nodes' records into draw units of one chunk, or `piece` records of
+// a compacted node's array. A warp looks at up to 32 nodes at once, one per lane
+// (fewer nodes than warps: one node a warp); the block takes their unit numbers
+// with one atomic, and each lane hands out the chunks of its own node when it need
+// not follow a list of them. The other nodes are walked one after another by all
+// lanes; chunks of less than a warp's records are drawn on the way. (A warp and an
+// atomic per node, and a unit for every chunk: a frame of 17,764 nodes of 60 points
+// 61 us, of 282k nodes of 4 points 296, where one warp had drawn each in 45 and 252.)
+constexpr uint32_t LANE_CHUNKS = 4;
+__global__ void k_render_units(Ctx c, View v, const uint32_t* vis, DrawUnit* units, uint32_t piece,
                                unsigned long long* fb) {
+  __shared__ uint32_t s_first[32], s_u0;
   after_previous();
   const uint32_t nv = min(vload(&c.ctl->vis_count), c.max_nodes);
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
-  const uint64_t nwarps = (uint64_t)gridDim.x * blockDim.x / 32;
+  const uint32_t lane = threadIdx.x & 31u, wi = threadIdx.x / 32u, wpb = blockDim.x / 32u;
+  const uint64_t nwarps = (uint64_t)gridDim.x * wpb;
   unsigned long long samples = 0;
-  for (uint64_t k = warp; k < nv; k += nwarps) {
-    const uint32_t id = vis[k];
-    const uint32_t n = c.num[id];
-    const NodeMeta& m = c.meta[id];
-    const uint32_t head = m.head, compact = m.compact;
-    const uint32_t nch = compact ? (uint32_t)(((unsigned long long)n + c.C - 1) / c.C)
-                                 : m.n_chunks;
-    samples += n;
-    if (n == 0 || nch == 0) continue;
-    uint32_t u0 = 0;
-    if (lane == 0) u0 = atomicAdd(&c.ctl->draw_units, nch);
-    u0 = __shfl_sync(FULL_MASK, u0, 0);
-    uint32_t got = 0;
-    if (!compact) {
-      got = walk_chunks(c, head, nch, leaf_dir(c, id, m), [&](bool on, uint32_t j, uint32_t ref) {
-        put_unit(c, v, units, on, (uint64_t)u0 + j, DrawUnit{ref, 0, chunk_fill(c, j, n), 0}, fb);
-      });
-    } else if (array_ok(c, head, n)) {
-      for (; got < nch; got += 32u) {
-        const uint32_t j = got + lane;
-        put_unit(c, v, units, j < nch, (uint64_t)u0 + j,
-                 DrawUnit{head, j * c.C, chunk_fill(c, j, n), 0}, fb);
-      }
-    } else if (lane == 0) {
-      set_error(c, E_INTERNAL);
+  for (uint64_t b = (uint64_t)blockIdx.x * wpb; b < nv; b += 32u * nwarps) {
+    const uint64_t k = b + wi + lane * nwarps;
+    uint32_t n = 0, nch = 0, head = NONE;
+    bool compact = false;
+    const uint32_t* dir = nullptr;
+    if (k < nv) {
+      const uint32_t id = vis[k];
+      const NodeMeta& m = c.meta[id];
+      n = c.num[id];
+      head = m.head;
+      compact = m.compact != 0u;
+      nch = compact ? (uint32_t)(((unsigned long long)n + piece - 1) / piece) : m.n_chunks;
+      if (n == 0) nch = 0;
+      if (!compact) dir = leaf_dir(c, id, m);
+      samples += n;
     }
-    // a broken list: the rest of the reserved units draw nothing
-    for (uint32_t j = got + lane; j < nch; j += 32u)
-      if ((uint64_t)u0 + j < c.max_chunks) units[(uint64_t)u0 + j] = DrawUnit{0, 0, 0, 0};
+    const bool own = nch == 1u ? !compact : dir && nch <= LANE_CHUNKS;
+    const uint32_t take = own || compact || c.C >= 32u ? nch : 0u;  // units
+    uint32_t upto = take;  // of the lanes up to this one
+    for (uint32_t d = 1; d < 32u; d <<= 1) {
+      const uint32_t o = __shfl_up_sync(FULL_MASK, upto, d);
+      if (lane >= d) upto += o;
+    }
+    if (lane == 31u) s_first[wi] = upto;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      uint32_t all = 0;
+      for (uint32_t w = 0; w < wpb; ++w) {
+        const uint32_t t = s_first[w];
+        s_first[w] = all;
+        all += t;
+      }
+      s_u0 = all ? atomicAdd(&c.ctl->draw_units, all) : 0u;
+    }
+    __syncthreads();
+    const uint32_t u0 = s_u0 + s_first[wi] + upto - take;  // the first of this lane's node
+    __syncthreads();
+    for (uint32_t j = 0; __any_sync(FULL_MASK, own && j < nch); ++j) {
+      const bool on = own && j < nch;
+      const uint32_t ref = !on ? NONE : nch == 1u ? head : dir[j];
+      const bool ok = on && ref_ok(c, ref, c.chunk_bytes);
+      if (on && !ok) set_error(c, E_INTERNAL);
+      put_unit(c, v, units, on, (uint64_t)u0 + j,
+               ok ? DrawUnit{ref, 0, chunk_fill(c, j, n), 0} : DrawUnit{0, 0, 0, 0}, fb);
+    }
+    for (unsigned rest = __ballot_sync(FULL_MASK, nch != 0u && !own); rest; rest &= rest - 1u) {
+      const int l = __ffs(rest) - 1;
+      const uint32_t ln = __shfl_sync(FULL_MASK, n, l), lnch = __shfl_sync(FULL_MASK, nch, l);
+      const uint32_t lhead = __shfl_sync(FULL_MASK, head, l);
+      const uint32_t ltake = __shfl_sync(FULL_MASK, take, l);
+      const uint64_t lu = __shfl_sync(FULL_MASK, u0, l);
+      const uint32_t* ldir = reinterpret_cast<const uint32_t*>(
+          __shfl_sync(FULL_MASK, reinterpret_cast<unsigned long long>(dir), l));
+      uint32_t got = 0;
+      if (!__shfl_sync(FULL_MASK, (int)compact, l)) {
+        got = walk_chunks(c, lhead, lnch, ldir, [&](bool on, uint32_t j, uint32_t ref) {
+          if (ltake) {
+            put_unit(c, v, units, on, lu + j, DrawUnit{ref, 0, chunk_fill(c, j, ln), 0}, fb);
+          } else {
+            const unsigned have = __ballot_sync(FULL_MASK, on);
+            const unsigned long long first = (unsigned long long)(j - lane) * c.C;
+            if (first < ln)
+              draw_chunks(c, v, ref, have,
+                          min(ln - (uint32_t)first, (32u - (uint32_t)__clz(have)) * c.C), fb);
+          }
+        });
+      } else if (array_ok(c, lhead, ln)) {
+        for (; got < lnch; got += 32u) {
+          const uint32_t j = got + lane;
+          const unsigned long long at = (unsigned long long)j * piece;
+          put_unit(c, v, units, j < lnch, lu + j,
+                   DrawUnit{lhead, (uint32_t)at, at < ln ? min(piece, ln - (uint32_t)at) : 0u, 0},
+                   fb);
+        }
+      } else if (lane == 0) {
+        set_error(c, E_INTERNAL);
+      }
+      // a broken list: the rest of the reserved units draw nothing
+      for (uint32_t j = got + lane; j < ltake; j += 32u)
+        if (lu + j < c.max_chunks) units[lu + j] = DrawUnit{0, 0, 0, 0};
+    }
   }
+  for (uint32_t d = 16; d; d >>= 1) samples += __shfl_down_sync(FULL_MASK, samples, d);
   if (lane == 0 && samples) atomicAdd(&c.ctl->render_samples, samples);
 }
 
-// Splat the units, `parts` warps per unit (parts * part >= C): about 256
+// Splat the units, `parts` warps per unit (parts * part >= C and the pieces): about 256
 // records a warp, so that a frame of a few nodes with tens of thousands of
 // records each fills the GPU. One warp per node (the first form) left the
 // longest node's chain of loads in charge: 0.43 ms for 3 nodes of 65k points

@@ -800,10 +800,11 @@ unsigned grid_for(const simlod_t* h, uint64_t work, uint64_t per_block) {
   return (unsigned)blocks;
 }
 
-// Warps per unit of C records (about 256 records each) and records per warp.
+// Warps per unit of C records (about 256 records each) and records per warp, which
+// are at least 256 together.
 void unit_parts(uint32_t C, uint32_t* parts, uint32_t* part) {
   *parts = std::min<uint32_t>(16u, (C + 255u) / 256u);
-  *part = ((C + *parts - 1u) / *parts + 31u) / 32u * 32u;
+  *part = ((std::max(C, 256u) + *parts - 1u) / *parts + 31u) / 32u * 32u;
 }
 
 // Read the control block (waits for the stream).
@@ -1879,7 +1880,7 @@ SIMLOD_API int simlod_render(simlod_t* h, const float view_proj[16], uint32_t wi
   const bool overlap = !captured(s);
   return launch(h, K_RENDER, s, [&] {
     k_render_select<<<grid, BLOCK, 0, s>>>(c, v, vis, fb, (uint64_t)width * height, clear);
-    launch_next(overlap, k_render_units, grid, BLOCK, 0, s, c, v, vis, units, fb);
+    launch_next(overlap, k_render_units, grid, BLOCK, 0, s, c, v, vis, units, parts * part, fb);
     launch_next(overlap, k_render_draw, grid, BLOCK, 0, s, c, v, units, parts, part, fb);
   });
 }

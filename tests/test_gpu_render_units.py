@@ -50,3 +50,68 @@ def test_frames_for_any_chunk_size(C, T, batch, compact):
         assert st["render_nodes"] == nd
         assert st["render_samples"] == int(np.where(
             snap.nodes["is_inner"] == 1, snap.nodes["n_voxels"], snap.nodes["n_points"])[drawn].sum())
+
+
+def test_pieces_beyond_the_unit_region_are_drawn_at_once():
+    # 1,000 chunks of one octant become an array of 1,000 pieces, and as many
+    # points of another octant take the chunks it gave back: 2,000 units in a
+    # region that has room for fewer
+    C, per = 256, 256_000
+    kw = dict(root_log2=20, leaf_capacity=per + 100, chunk_points=C, grid_log2=1)
+    cfg = simlod.default_config(max_batch_points=1 << 19, spill_capacity=1 << 16,
+                                backlog_capacity=1 << 12, max_nodes=1 << 10, **kw)
+    lo = synth.uniform(5, 1 << 19, per)
+    hi = synth.uniform(6, 1 << 19, per)
+    for f in "xyz":
+        hi[f] += 1 << 19
+    tree = simlod.Octree(cfg, simlod.make_arena(cfg, 10_570_000), stream=torch.cuda.Stream())
+    tree.insert_many([simlod.points_tensor(np.concatenate([lo, hi[:200]]))])
+    tree.compact()
+    tree.insert_many([simlod.points_tensor(hi[200:])])
+    assert tree.sync() == simlod.OK
+    st = tree.stats()
+    assert st["compact_nodes"] == 1 and st["compact_chunks"] == per // C
+    assert st["data_bytes"] // (20 * C + 256) < 2 * per // C  # chunks in the data region
+    ocfg = oracle.Config.make(**kw)
+    snap = oracle.static_build(ocfg, np.concatenate([lo, hi]))
+    eye, tgt, fov = CAMS[0]
+    W, H = 211, 97
+    m = look_at_perspective(eye, tgt, fov, W / H)
+    fb = torch.empty((H, W), dtype=torch.int64, device="cuda")
+    tree.render(m, fb)
+    assert tree.sync() == simlod.OK
+    want, drawn, nd = oracle.render(ocfg, snap, m, W, H)
+    assert np.array_equal(fb.cpu().numpy().view(np.uint64), want)
+    assert tree.stats()["render_nodes"] == nd
+
+
+def test_captured_frames_and_compactions():
+    # a captured render draws the octree as it is at each replay, a captured
+    # compaction compacts it
+    kw = dict(root_log2=20, leaf_capacity=700, chunk_points=50, grid_log2=5)
+    cfg = simlod.default_config(max_batch_points=1 << 16, spill_capacity=1 << 18,
+                                backlog_capacity=1 << 18, max_nodes=1 << 14, **kw)
+    pts = synth.uniform(7, 1 << 20, 40_000)
+    tree = simlod.Octree(cfg, simlod.make_arena(cfg, 256 << 20))
+    eye, tgt, fov = CAMS[0]
+    m = look_at_perspective(eye, tgt, fov, 2.0)
+    fb, direct = (torch.empty((128, 256), dtype=torch.int64, device="cuda") for _ in range(2))
+    tree.render(m, direct)
+    tree.compact()
+    torch.cuda.synchronize()
+    frame, pack = torch.cuda.CUDAGraph(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(frame):
+        tree.render(m, fb)
+    with torch.cuda.graph(pack):
+        tree.compact()
+    for lo in (0, 20_000):
+        tree.insert(simlod.points_tensor(pts[lo:lo + 20_000]))
+        pack.replay()
+        frame.replay()
+        tree.render(m, direct)
+        assert tree.sync() == simlod.OK
+        assert tree.stats()["compact_nodes"] > 0
+        assert torch.equal(fb, direct) and bool((fb != -1).any())
+    ocfg = oracle.Config.make(**kw)
+    want, _, _ = oracle.render(ocfg, oracle.static_build(ocfg, pts), m, 256, 128)
+    assert np.array_equal(fb.cpu().numpy().view(np.uint64), want)
