@@ -154,6 +154,7 @@ struct Ctl {
   unsigned int reject;                      // out-of-cube point seen in this update
   SL_HOT unsigned int spill_count;          // re-inserted points of this update
   SL_HOT unsigned int nkeys;                // new voxels (backlog entries) of this update
+  PlainRound round[2];                      // plain form: round r is round[r & 1]
   SL_HOT unsigned int alloc_seq;            // alloc_refs entries of this update
   SL_HOT unsigned int split_count;          // split-list entries of this update
   unsigned int split_inner;                 //   those made by the builds (inner nodes below the
@@ -178,7 +179,6 @@ struct Ctl {
   unsigned long long compact_need;       // bytes the candidates of a compaction need
   unsigned long long compact_from;       // the bump pointer before it
   unsigned int store_blocks;             // plain form: blocks that finished the store
-  PlainRound round[MAX_ROUNDS];
 };
 #undef SL_HOT
 static_assert(sizeof(Ctl) % 16 == 0, "Ctl size");
@@ -249,7 +249,8 @@ struct Ctx {
   uint32_t* hist;     // counts of the cubes below split leaves; zero between updates
   uint32_t* hist_up;  //   their sums per inner level, and the list of inner nodes
   HSlot* hash;
-  uint2* keys;        // backlog: table slot and node of this update's new cells
+  uint32_t* keys;     // backlog: table slots of this update's new cells
+  uint32_t* key_node; //   and the nodes of the first key_nodes of them
   uint8_t* data;
   unsigned long long data_bytes;
   int4* staging;
@@ -260,7 +261,7 @@ struct Ctx {
   uint32_t C_mul, C_shift;  // division by C (div_by)
   uint32_t parts, P_mul, P_shift;  // 32-record units per chunk, and division by them
   uint32_t chunk_lim, grid_lim;    // first references whose chunk or grid would not fit
-  uint32_t max_nodes, max_chunks, spill_cap, backlog_cap, max_splits;
+  uint32_t max_nodes, max_chunks, spill_cap, backlog_cap, key_nodes, max_splits;
   uint64_t max_batch;
   uint64_t hist_words;
   unsigned long long* launch_bar;  // barrier word of the persistent launch (abort bit)
@@ -661,7 +662,9 @@ __device__ __forceinline__ void warp_flush(const Ctx& c, WarpBuf& wb) {
   e0 = __shfl_sync(FULL_MASK, e0, 0);
   for (uint32_t k = lane_id(); k < wb.n; k += 32) {
     const uint32_t e = e0 + k;
-    if (e < c.backlog_cap) c.keys[e] = wb.buf[k];
+    const uint2 at = wb.buf[k];  // slot, node
+    if (e < c.key_nodes) c.key_node[e] = at.y;
+    if (e < c.backlog_cap) c.keys[e] = at.x;
     else set_error(c, E_BACKLOG);
   }
   wb.n = 0;
@@ -1939,13 +1942,15 @@ __device__ void phase_store_voxels(const Ctx& c, uint32_t* smem, uint32_t n_task
       [&](uint32_t w) -> uint32_t {
         const uint32_t e = w * 32u + lane;
         if (e >= n_keys) return NONE;
-        const uint32_t node = c.keys[e].y;
+        // (where the arena leaves no room for the list of nodes, from the slot)
+        const uint32_t node = e < c.key_nodes ? c.key_node[e]
+                                              : (uint32_t)(c.hash[c.keys[e]].key >> (3u * G));
         if (node < c.max_nodes) return node;
         set_error(c, E_INTERNAL);
         return NONE;
       },
       [&](uint32_t w, StoreItem& it) {
-        it.slot = c.keys[w * 32u + lane].x;
+        it.slot = c.keys[w * 32u + lane];
         it.gref = c.gridref[it.node];
         const ulonglong2 kv = *reinterpret_cast<const ulonglong2*>(c.hash + it.slot);
         // the node's min corner and level

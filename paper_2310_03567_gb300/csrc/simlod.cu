@@ -142,7 +142,7 @@ __device__ __forceinline__ const PlainView& plain_view(const Ctx& c, uint32_t r)
   __shared__ PlainView v;
   if (threadIdx.x == 0) {
     const Ctl* t = c.ctl;
-    const PlainRound* p = &t->round[r];
+    const PlainRound* p = &t->round[r & 1u];
     v.stop = vload(&t->reject) | vload(&t->error);
     v.split_count = vload(&t->split_count);
     v.split_inner = vload(&t->split_inner);
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_hist(Ctx c, const 
   const uint32_t d = hist_depth(c, K, n + v.spill_count, v.split_most);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     const uint32_t lvl0 = r > 1u ? v.round.lvl0 + v.round.d : 0u;
-    c.ctl->round[r] = PlainRound{s_lo, K, v.split_inner, d, lvl0, v.n_nodes};
+    c.ctl->round[r & 1u] = PlainRound{s_lo, K, v.split_inner, d, lvl0, v.n_nodes};
   }
   if (K == 0u) return;
   node_cache_load(c, smem, 0, v.n_nodes);
@@ -496,8 +496,8 @@ static const char* const kKernelNames[SIMLOD_N_KERNELS] = {
 
 struct Layout {
   size_t ctl, fctl, batches, child, gridref, cnt, num, meta, pool, pending, alloc_refs, splits,
-      tasks, sp_cur, b_cur, hist, hist_up, scur, vis, hash, keys, staging, data, end;
-  uint64_t hash_slots, hist_words, max_chunks, max_splits, data_bytes;
+      tasks, sp_cur, b_cur, hist, scratch, scur, hash, keys, key_node, staging, data, end;
+  uint64_t hash_slots, hist_words, key_nodes, max_chunks, max_splits, data_bytes;
 };
 
 struct simlod {
@@ -592,6 +592,29 @@ uint32_t grid_bytes_of(const simlod_config* c) {
   return (uint32_t)align_up(std::max<uint64_t>(bits / 8, 1), REF_BYTES);
 }
 
+// The largest fixed part: what the kernels that moved points level by level placed
+// in front of the data region (8-byte split entries, two lists of movers and the
+// records of re-inserted points). Callers may keep arenas of the size that was
+// asked for then; the histograms and the backlog's nodes take what the smaller
+// regions of today leave of it.
+uint64_t fixed_bound(const simlod_config* c, uint64_t hash_slots) {
+  const uint64_t N = c->max_nodes, B = c->max_batch_points, S = c->spill_capacity;
+  uint64_t o = 0;
+  for (uint64_t bytes : {(uint64_t)1408, (uint64_t)sizeof(FusedCtl),
+                         (uint64_t)sizeof(BatchDesc) * MAX_FUSED_BATCHES, 4 * N, 4 * N, 4 * N, 4 * N,
+                         (uint64_t)sizeof(NodeMeta) * N, 8 * (N / 8 + 1), 4 * S, 4 * B, 8 * (B + S),
+                         8 * (B + S), 16 * S, 4 * S, 4 * N, 4 * N, (uint64_t)sizeof(HSlot) * hash_slots,
+                         4 * c->backlog_capacity, 16 * B})
+    o = align_up(o, 256) + bytes;
+  return align_up(o, 256);
+}
+
+// Sums and lists of the builds for `words` counts: less than 2 / 7 of them per leaf,
+// whatever the depth. They share a region with the renderer's list of drawn nodes.
+uint64_t scratch_bytes(const simlod_config* c, uint64_t words) {
+  return std::max<uint64_t>(4 * c->max_nodes, 8 * (words / 7 + 1));
+}
+
 // Place every region; the data region (grids and chunks) takes what is left
 // and pool / pending / alloc_refs hold one entry per chunk that fits in it.
 bool plan_layout(const simlod_config* c, size_t arena_bytes, Layout* L) {
@@ -604,30 +627,44 @@ bool plan_layout(const simlod_config* c, size_t arena_bytes, Layout* L) {
   const uint64_t N = c->max_nodes, B = c->max_batch_points, S = c->spill_capacity;
   L->max_splits = N / 8 + 1;
   L->hash_slots = next_pow2(2 * c->backlog_capacity);
-  L->ctl = take(sizeof(Ctl));
-  L->fctl = take(sizeof(FusedCtl));
-  L->batches = take(sizeof(BatchDesc) * MAX_FUSED_BATCHES);
-  L->child = take(4 * N);
-  L->gridref = take(4 * N);
-  L->cnt = take(4 * N);
-  L->num = take(4 * N);
-  L->meta = take(sizeof(NodeMeta) * N);
-  L->splits = take(4 * L->max_splits);
-  L->sp_cur = take(4 * S);
-  L->b_cur = take(4 * B);
   // an update splits at most (B + S) / (T + 1) leaves, each with the 8 counts
   // of one level; more levels where there is room for a count per moving point
-  const uint64_t leaves = std::min<uint64_t>(L->max_splits, (B + S) / (c->leaf_capacity + 1ull) + 1);
-  L->hist_words = std::max<uint64_t>(8 * leaves, std::min<uint64_t>(std::max<uint64_t>(B + S, 32768), 32u << 20));
-  L->hist_words = align_up(L->hist_words, 64);
-  L->hist = take(4 * L->hist_words);
-  // sums and list: 2 (8^d - 1) / 7 words for 8^d counts
-  L->hist_up = take(8 * (L->hist_words / 7 + leaves));
-  L->scur = take(4 * N);
-  L->vis = take(4 * N);
-  L->hash = take(sizeof(HSlot) * L->hash_slots);
-  L->keys = take(sizeof(uint2) * c->backlog_capacity);
-  L->staging = take(16 * B);
+  const uint64_t leaves =
+      std::min<uint64_t>(L->max_splits, (B + S) / (c->leaf_capacity + 1ull) + 1);
+  const uint64_t least = align_up(8 * leaves, 64);
+  const uint64_t want = std::max<uint64_t>(
+      least, align_up(std::min<uint64_t>(std::max<uint64_t>(B + S, 32768), 32u << 20), 64));
+  auto place = [&](uint64_t hist_words, uint64_t key_nodes) {
+    o = 0;
+    L->hist_words = hist_words;
+    L->key_nodes = key_nodes;
+    L->ctl = take(sizeof(Ctl));
+    L->fctl = take(sizeof(FusedCtl));
+    L->batches = take(sizeof(BatchDesc) * MAX_FUSED_BATCHES);
+    L->child = take(4 * N);
+    L->gridref = take(4 * N);
+    L->cnt = take(4 * N);
+    L->num = take(4 * N);
+    L->meta = take(sizeof(NodeMeta) * N);
+    L->splits = take(4 * L->max_splits);
+    L->sp_cur = take(4 * S);
+    L->b_cur = take(4 * B);
+    L->hist = take(4 * hist_words);
+    L->scratch = take(scratch_bytes(c, hist_words));
+    L->scur = take(4 * N);
+    L->hash = take(sizeof(HSlot) * L->hash_slots);
+    L->keys = take(4 * c->backlog_capacity);
+    L->key_node = take(4 * key_nodes);
+    L->staging = take(16 * B);
+    return align_up(o, 256);
+  };
+  const uint64_t bound = fixed_bound(c, L->hash_slots);
+  // (1,024: the regions' alignment; a count and its share of the sums: 6 bytes)
+  uint64_t used = place(least, 0) + 1024;
+  const uint64_t room = bound > used ? bound - used : 0;
+  const uint64_t words = std::min<uint64_t>(want, least + room / 6 / 64 * 64);
+  used = place(words, 0) + 1024;
+  place(words, std::min<uint64_t>(c->backlog_capacity, bound > used ? (bound - used) / 4 : 0));
   const size_t fixed = align_up(o, 256);
   if (arena_bytes < fixed) return false;
   const uint64_t cb = chunk_bytes_of(c);
@@ -668,11 +705,13 @@ void make_ctx(simlod_t* h) {
   c.sp_cur = reinterpret_cast<uint32_t*>(a + L.sp_cur);
   c.b_cur = reinterpret_cast<uint32_t*>(a + L.b_cur);
   c.hist = reinterpret_cast<uint32_t*>(a + L.hist);
-  c.hist_up = reinterpret_cast<uint32_t*>(a + L.hist_up);
+  c.hist_up = reinterpret_cast<uint32_t*>(a + L.scratch);
   c.hist_words = L.hist_words;
   c.scur = reinterpret_cast<uint32_t*>(a + L.scur);
   c.hash = reinterpret_cast<HSlot*>(a + L.hash);
-  c.keys = reinterpret_cast<uint2*>(a + L.keys);
+  c.keys = reinterpret_cast<uint32_t*>(a + L.keys);
+  c.key_node = reinterpret_cast<uint32_t*>(a + L.key_node);
+  c.key_nodes = (uint32_t)L.key_nodes;
   c.staging = reinterpret_cast<int4*>(a + L.staging);
   c.data = a + L.data;
   c.data_bytes = L.data_bytes;
@@ -824,7 +863,7 @@ int read_ctl(simlod_t* h, cudaStream_t s) {
 
 // First split entry behind round r (0: none yet) and the inner nodes that it built.
 uint32_t round_end(const Ctl* t, uint32_t r) {
-  const PlainRound& p = t->round[r];
+  const PlainRound& p = t->round[r & 1u];
   return r ? p.s_lo + p.K + (t->split_inner - p.inner) : 0u;
 }
 
@@ -1864,7 +1903,7 @@ SIMLOD_API int simlod_render(simlod_t* h, const float view_proj[16], uint32_t wi
   v.width = width;
   v.height = height;
   const Ctx& c = h->ctx;
-  uint32_t* vis = reinterpret_cast<uint32_t*>(h->arena + h->lay.vis);
+  uint32_t* vis = reinterpret_cast<uint32_t*>(h->arena + h->lay.scratch);
   unsigned long long* fb = reinterpret_cast<unsigned long long*>(d_framebuffer);
   // the sample count and the two list counters are neighbours
   static_assert(offsetof(Ctl, vis_count) == offsetof(Ctl, render_samples) + 8 &&
