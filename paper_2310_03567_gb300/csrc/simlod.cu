@@ -127,9 +127,9 @@ __global__ void __launch_bounds__(BLOCK) k_decide(Ctx c, uint32_t n_lo, uint32_t
 // and store when one still has to: the host, which reads the control block
 // then, enqueues another round and them again. A wait for the host per round
 // (7 per update of a clustered scan) took longer than the kernels between.
-// What such a kernel finds in the control block: loaded by one thread of the
+// What such a kernel needs from the control block is loaded by one thread of the
 // block, all at once (one after another, by every thread, the loads were five round
-// trips in front of a claim). r: the last round whose end counts.
+// trips in front of a claim). r: the last round whose end counts; more: the rest.
 struct PlainView {
   unsigned long long bump0;
   uint32_t stop, end, split_count, split_inner, split_most, ntasks, n_nodes, spill_count, nkeys;
@@ -138,36 +138,36 @@ struct PlainView {
   PlainRound round;
 };
 
-__device__ __forceinline__ const PlainView& plain_view(const Ctx& c, uint32_t r) {
-  __shared__ PlainView v;
+template <typename More>
+__device__ __forceinline__ void plain_view(const Ctx& c, uint32_t r, PlainView& v, More&& more) {
   if (threadIdx.x == 0) {
     const Ctl* t = c.ctl;
     const PlainRound* p = &t->round[r & 1u];
     v.stop = vload(&t->reject) | vload(&t->error);
     v.split_count = vload(&t->split_count);
     v.split_inner = vload(&t->split_inner);
-    v.split_most = vload(&t->split_most);
-    v.ntasks = vload(&t->ntasks);
     v.n_nodes = vload(&t->n_nodes);
-    v.spill_count = vload(&t->spill_count);
-    v.nkeys = vload(&t->nkeys);
-    v.bump0 = vload(&t->bump0);
-    v.open = vload(&t->open);
-    v.key_rate = vload(&t->key_rate);
-    v.pool_top = vload(&t->pool_top);
-    v.round = PlainRound{vload(&p->s_lo), vload(&p->K),    vload(&p->inner),
-                         vload(&p->d),    vload(&p->lvl0), vload(&p->n_lo)};
+    v.round.s_lo = vload(&p->s_lo);
+    v.round.K = vload(&p->K);
+    v.round.inner = vload(&p->inner);
+    more(t, p);
     v.end = r ? v.round.s_lo + v.round.K + (v.split_inner - v.round.inner) : 0u;
   }
   __syncthreads();
-  return v;
 }
 
 __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_hist(Ctx c, const int4* pts,
                                                                   uint64_t n, uint32_t r) {
   extern __shared__ uint32_t smem[];
+  __shared__ PlainView v;
   after_previous();
-  const PlainView& v = plain_view(c, r - 1u);
+  plain_view(c, r - 1u, v, [&](const Ctl* t, const PlainRound* p) {
+    v.spill_count = vload(&t->spill_count);
+    v.split_most = vload(&t->split_most);
+    v.ntasks = vload(&t->ntasks);
+    v.round.d = vload(&p->d);
+    v.round.lvl0 = vload(&p->lvl0);
+  });
   if (v.stop) return;
   const uint32_t s_lo = v.end, K = v.split_count - s_lo;
   const uint32_t d = hist_depth(c, K, n + v.spill_count, v.split_most);
@@ -181,15 +181,20 @@ __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_hist(Ctx c, const 
 }
 
 __global__ void __launch_bounds__(PBLOCK) k_build(Ctx c, uint32_t r, uint32_t max_iters) {
+  __shared__ PlainView v;
   after_previous();
-  const PlainView& v = plain_view(c, r);
+  plain_view(c, r, v, [&](const Ctl*, const PlainRound* p) {
+    v.round.d = vload(&p->d);
+    v.round.lvl0 = vload(&p->lvl0);
+  });
   if (v.stop || v.round.K == 0u) return;
   phase_build(c, v.round.s_lo, v.round.K, v.round.d, v.round.lvl0, max_iters);
 }
 
 __global__ void __launch_bounds__(BLOCK) k_decide_new(Ctx c, uint32_t r) {
+  __shared__ PlainView v;
   after_previous();
-  const PlainView& v = plain_view(c, r);
+  plain_view(c, r, v, [&](const Ctl*, const PlainRound* p) { v.round.n_lo = vload(&p->n_lo); });
   if (v.stop || v.round.K == 0u) return;
   phase_decide(c, v.round.n_lo, v.n_nodes, (blockIdx.x * blockDim.x + threadIdx.x) / 32,
                gridDim.x * blockDim.x / 32);
@@ -199,8 +204,15 @@ __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_claim(Ctx c, const
                                                      unsigned long long base, uint32_t nodes0,
                                                      uint32_t r) {
   extern __shared__ uint32_t smem[];
+  __shared__ PlainView v;
   after_previous();
-  const PlainView& v = plain_view(c, r);
+  plain_view(c, r, v, [&](const Ctl* t, const PlainRound*) {
+    v.ntasks = vload(&t->ntasks);
+    v.spill_count = vload(&t->spill_count);
+    v.bump0 = vload(&t->bump0);
+    v.open = vload(&t->open);
+    v.key_rate = vload(&t->key_rate);
+  });
   if (v.stop || v.split_count != v.end) return;
   const uint32_t wpb = blockDim.x / 32;
   if (v.split_count == 0u && (uint64_t)blockIdx.x * wpb * 32u >= n) return;  // nothing to do
@@ -213,8 +225,9 @@ __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_claim(Ctx c, const
 
 // Chunks for the new voxels of the inner nodes.
 __global__ void __launch_bounds__(BLOCK) k_alloc_voxels(Ctx c, uint32_t r) {
+  __shared__ PlainView v;
   after_previous();
-  const PlainView& v = plain_view(c, r);
+  plain_view(c, r, v, [](const Ctl*, const PlainRound*) {});
   if (v.stop || v.split_count != v.end) return;
   phase_decide(c, 0, v.n_nodes, (blockIdx.x * blockDim.x + threadIdx.x) / 32,
                gridDim.x * blockDim.x / 32);
@@ -228,7 +241,12 @@ __global__ void __launch_bounds__(BLOCK) k_alloc_voxels(Ctx c, uint32_t r) {
 __global__ void __launch_bounds__(PBLOCK, PHASE_MIN_BLOCKS) k_store(Ctx c, const int4* pts, uint64_t n,
                                                   unsigned long long base, uint32_t r) {
   extern __shared__ uint32_t smem[];
-  const PlainView& v = plain_view(c, r);
+  __shared__ PlainView v;
+  plain_view(c, r, v, [&](const Ctl* t, const PlainRound*) {
+    v.ntasks = vload(&t->ntasks);
+    v.nkeys = vload(&t->nkeys);
+    v.pool_top = vload(&t->pool_top);
+  });
   if (v.stop || v.split_count != v.end) return;
   const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   const uint64_t nt = (uint64_t)gridDim.x * blockDim.x;
