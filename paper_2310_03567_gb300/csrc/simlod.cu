@@ -1789,12 +1789,13 @@ SIMLOD_API int simlod_restore(simlod_t* h, const simlod_snapshot_t* snap, void* 
     meta[id] = m;
   });
   if (bad) return SIMLOD_ERR_INVALID_ARG;
-  // start from an empty octree (clears a poisoned state and the claim table)
+  // start from an empty octree (clears a poisoned state; the claim table and the
+  // histograms are empty unless an update failed)
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const bool dirty = h->sticky != 0;
   if (dirty) cudaStreamSynchronize(h->last_stream);
   h->sticky = 0;
-  int rc = init_octree(h, s, true, false);
+  int rc = init_octree(h, s, dirty, false);
   if (rc) return poison(h, rc);
   if (cudaStreamSynchronize(s) != cudaSuccess) return poison(h, SIMLOD_ERR_CUDA);
   Ctl t;

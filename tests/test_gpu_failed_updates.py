@@ -119,3 +119,22 @@ def test_frame_behind_a_failed_update(what, clear):
     works_after_reset(tree)
     tree.render(cam, frame)
     assert tree.sync() == simlod.OK and bool((frame != -1).any())
+
+
+@pytest.mark.parametrize("what", ["arena", "nodes"])
+@pytest.mark.parametrize("synced", [True, False])
+def test_restore_behind_a_failed_update(what, synced):
+    # the failed update's counts and claims are gone with its octree, whether its
+    # status has been read or not
+    tree, batches, status = failing(what)
+    tree.insert_many(batches[:1])
+    snap = tree.snapshot()
+    tree.reset()
+    tree.insert_many(batches)
+    if synced:
+        assert tree.sync() == status
+    tree.restore(snap)
+    tree.insert_many(batches[1:2])
+    assert tree.sync() == simlod.OK
+    want = oracle.static_build(oracle.Config.make(**KW), PTS[:10_000])
+    assert_snapshots_equal(tree.snapshot(), want)
