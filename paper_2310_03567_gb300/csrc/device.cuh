@@ -38,10 +38,10 @@
 // lowest arrival index wins regardless of thread timing. The table entries of
 // an update are listed (the backlog of Section 5.2) and cleared by store.
 //
-// Descents read the node table (first child) from a copy in shared memory of the first NODE_CACHE nodes (the node ids of the upper
-// levels are the smallest): the plain form's kernels load it,
-// the persistent kernel loads it once and patches it after every decide
-// round with the nodes that split or were created.
+// Descents read the node table (first child) from a copy in shared memory of the
+// first NODE_CACHE nodes (the node ids of the upper levels are the smallest): the
+// plain form's kernels load it, the persistent kernel loads it once and patches it
+// after every build with the nodes that split or were created.
 // Per-node counters are summed per block in shared memory before they reach
 // the global counters (the block tally cache).
 #pragma once
@@ -102,12 +102,9 @@ constexpr int PHASE_BLOCK = SL_PHASE_BLOCK;            // threads of a phase blo
 constexpr int PHASE_MIN_BLOCKS = SL_PHASE_MIN_BLOCKS;  // resident blocks per SM they aim for
 constexpr uint32_t TALLY_LOG2 = 9;                      // block tally cache: 512 nodes
 constexpr uint32_t TALLY_SLOTS = 1u << TALLY_LOG2;
+constexpr uint32_t CLAIM_QUEUE = 64;  // points of a warp that wait for their next claim
 // dynamic shared memory of the phase blocks: node cache, new-cell staging,
 // claim queues, block tally cache
-// units of 32 points a warp claims for at once (two: 0.99 against 0.94 ms of
-// claims on a 16M-point terrain, and spills)
-constexpr int CLAIM_U = 1;
-constexpr uint32_t CLAIM_QUEUE = 32 * (CLAIM_U + 1);  // points that wait for their next claim
 constexpr uint32_t SMEM_WBUF = NODE_CACHE;            // in u32 words
 constexpr uint32_t SMEM_QUEUE = SMEM_WBUF + (PHASE_BLOCK / 32) * WBUF * 2;
 constexpr uint32_t SMEM_TALLY = SMEM_QUEUE + (PHASE_BLOCK / 32) * CLAIM_QUEUE * 6;
@@ -671,72 +668,43 @@ __device__ __forceinline__ void warp_flush(const Ctx& c, WarpBuf& wb) {
   __syncwarp();
 }
 
-// All 32 lanes call. Lanes with lead[j] offer val[j] for key[j] (a cell of
-// node[j]) to the update's claim table, where the lowest value wins. The
-// first probes of all N items are issued together (their loads, then their
-// compare-and-swaps), so the items pay about two L2 round trips together. A
-// key new in this update is staged for the backlog and counted towards its
-// node's new voxels. on[j] becomes true in lanes that met no lower value.
-template <int N>
-__device__ __forceinline__ void warp_claim(const Ctx& c, WarpBuf& wb, const bool (&lead)[N],
-                                           const unsigned long long (&key)[N],
-                                           const unsigned long long (&val)[N],
-                                           const uint32_t (&node)[N], uint32_t near,
-                                           bool (&on)[N]) {
+// All 32 lanes call. Lanes with `lead` offer val for key (a cell of `node`) to the
+// update's claim table, where the lowest value wins. A key new in this update is
+// staged for the backlog and counted towards its node's new voxels. `on` becomes
+// true in lanes that met no lower value.
+__device__ __forceinline__ void warp_claim(const Ctx& c, WarpBuf& wb, bool lead,
+                                           unsigned long long key, unsigned long long val,
+                                           uint32_t node, uint32_t near, bool& on) {
   const uint32_t lane = lane_id();
-  bool cas[N], inst[N];
-  uint32_t h[N];
-  unsigned long long k0[N], v0[N];
-#pragma unroll
-  for (int j = 0; j < N; ++j) {
-    h[j] = claim_slot(key[j], near);
-    k0[j] = v0[j] = 0ull;
-    if (lead[j]) {
-      const ulonglong2 kv = slot_load(c.hash + h[j]);
-      k0[j] = kv.x;
-      v0[j] = kv.y;
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < N; ++j) {
-    cas[j] = lead[j] && k0[j] == HASH_EMPTY;
-    if (cas[j]) {
-      const ulonglong2 kv = slot_cas(c.hash + h[j], key[j], val[j]);
-      k0[j] = kv.x;
-      v0[j] = kv.y;
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < N; ++j) {
-    inst[j] = false;
-    if (lead[j]) {
-      if (cas[j] && k0[j] == HASH_EMPTY) {
-        inst[j] = on[j] = true;
-      } else if (k0[j] == key[j]) {
-        if (v0[j] > val[j]) {
-          on[j] = true;
-          atomicMin(&c.hash[h[j]].val, val[j]);
-        }
-      } else {
-        const int got = hash_claim_rest(c, key[j], val[j], near, h[j]);
-        inst[j] = got == CLAIM_NEW;
-        if (got != CLAIM_BEATEN) on[j] = true;
+  uint32_t h = claim_slot(key, near);
+  bool inst = false;
+  if (lead) {
+    ulonglong2 kv = slot_load(c.hash + h);
+    const bool cas = kv.x == HASH_EMPTY;
+    if (cas) kv = slot_cas(c.hash + h, key, val);
+    if (cas && kv.x == HASH_EMPTY) {
+      inst = on = true;
+    } else if (kv.x == key) {
+      if (kv.y > val) {
+        on = true;
+        atomicMin(&c.hash[h].val, val);
       }
+    } else {
+      const int got = hash_claim_rest(c, key, val, near, h);
+      inst = got == CLAIM_NEW;
+      if (got != CLAIM_BEATEN) on = true;
     }
   }
-#pragma unroll
-  for (int j = 0; j < N; ++j) {
-    const unsigned mi = __ballot_sync(FULL_MASK, inst[j]);
-    if (mi == 0u) continue;
-    const uint32_t ni = (uint32_t)__popc(mi);
-    if (wb.n + ni > WBUF) warp_flush(c, wb);
-    const LaneRun r = lane_run(inst[j], node[j]);
-    if (inst[j]) {
-      wb.buf[wb.n + __popc(mi & ((1u << lane) - 1u))] = make_uint2(h[j], node[j]);
-      if (r.head) tally_add(c.cnt, wb.smem, node[j], r.end - lane);
-    }
-    wb.n += ni;
+  const unsigned mi = __ballot_sync(FULL_MASK, inst);
+  if (mi == 0u) return;
+  const uint32_t ni = (uint32_t)__popc(mi);
+  if (wb.n + ni > WBUF) warp_flush(c, wb);
+  const LaneRun r = lane_run(inst, node);
+  if (inst) {
+    wb.buf[wb.n + __popc(mi & ((1u << lane) - 1u))] = make_uint2(h, node);
+    if (r.head) tally_add(c.cnt, wb.smem, node, r.end - lane);
   }
+  wb.n += ni;
 }
 
 // All 32 lanes call. Lanes with `valid` add one to counters[i] (one addition
@@ -1291,87 +1259,68 @@ struct ClaimArgs {
   uint32_t nodes0, grid0, open, near;
 };
 
-// All 32 lanes call: lanes with on[j] sample the grid of their node's parent.
-// SORTED: the items are units of consecutive batch points or (respill) of
+// All 32 lanes call: lanes with `on` sample the grid of their node's parent.
+// SORTED: the items are a unit of consecutive batch points or (respill) of
 // re-inserted ones of one chunk. A lane whose neighbour lane is in the same
 // cell with a lower index is done (unless the voxels do not nest); in a unit of
 // batch points the index grows with the lane, so only the left one can have
 // it. Points that have to go on join the queue, naming the parent.
-template <int N, bool SORTED>
+template <bool SORTED>
 __device__ __forceinline__ void claim_level(const Ctx& c, WarpBuf& wb, ClaimQueue& cq,
-                                            const ClaimArgs& a, const bool (&on)[N],
-                                            const ClaimItem (&it)[N], bool respill) {
+                                            const ClaimArgs& a, bool on, const ClaimItem& it,
+                                            bool respill) {
   const uint32_t lane = lane_id();
-  uint32_t par[N], word[N], cell[N];
-  bool want[N], more[N];
-  unsigned long long key[N], val[N];
-  uint2 up[N];
-#pragma unroll
-  for (int j = 0; j < N; ++j) {
-    up[j] = on[j] ? *reinterpret_cast<const uint2*>(&c.meta[it[j].node & NODE_MASK].up)
-                  : make_uint2(NONE, 0u);
-  }
-#pragma unroll
-  for (int j = 0; j < N; ++j) {
-    par[j] = up[j].x & NODE_MASK;
-    word[j] = cell[j] = 0;
-    want[j] = false;
-    if (up[j].x != NONE) {
-      cell[j] = cell_index(it[j].rx, it[j].ry, it[j].rz, c.rlog2 - (up[j].x >> NODE_BITS), c.G);
-      if (!grid_ok(c, up[j].y) || par[j] >= c.max_nodes) {
-        set_error(c, E_INTERNAL);
-      } else {
-        want[j] = true;
-        // a grid of this update's own splits is empty until the store
-        if (up[j].y < a.grid0) word[j] = grid_words(c, up[j].y)[cell[j] >> 5];
-      }
+  const uint2 up = on ? *reinterpret_cast<const uint2*>(&c.meta[it.node & NODE_MASK].up)
+                      : make_uint2(NONE, 0u);
+  const uint32_t par = up.x & NODE_MASK;
+  uint32_t word = 0, cell = 0;
+  bool want = false;
+  if (up.x != NONE) {
+    cell = cell_index(it.rx, it.ry, it.rz, c.rlog2 - (up.x >> NODE_BITS), c.G);
+    if (!grid_ok(c, up.y) || par >= c.max_nodes) {
+      set_error(c, E_INTERNAL);
+    } else {
+      want = true;
+      // a grid of this update's own splits is empty until the store
+      if (up.y < a.grid0) word = grid_words(c, up.y)[cell >> 5];
     }
   }
-  bool lead[N];
-#pragma unroll
-  for (int j = 0; j < N; ++j) {
-    more[j] = want[j] && a.open != 0u;
-    want[j] = want[j] && ((word[j] >> (cell[j] & 31u)) & 1u) == 0u;
-    key[j] = ((unsigned long long)par[j] << (3u * c.G)) | cell[j];
-    val[j] = ((unsigned long long)it[j].gidx << 32) | it[j].rgba;
-    lead[j] = want[j];
-    if (SORTED) {
-      // a neighbour lane in the same cell with a lower index: done
-      const unsigned wm = __ballot_sync(FULL_MASK, want[j]);
-      const uint32_t pc = __shfl_up_sync(FULL_MASK, cell[j], 1);
-      const uint32_t pp = __shfl_up_sync(FULL_MASK, par[j], 1);
-      const uint32_t pg = __shfl_up_sync(FULL_MASK, it[j].gidx, 1);
-      const bool left = lane != 0u && ((wm >> (lane - 1u)) & 1u) && pc == cell[j] &&
-                        pp == par[j] && pg < it[j].gidx;
-      bool beaten = left;
-      if (respill) {
-        const uint32_t nc2 = __shfl_down_sync(FULL_MASK, cell[j], 1);
-        const uint32_t np = __shfl_down_sync(FULL_MASK, par[j], 1);
-        const uint32_t ng = __shfl_down_sync(FULL_MASK, it[j].gidx, 1);
-        beaten = beaten || (lane != 31u && ((wm >> (lane + 1u)) & 1u) && nc2 == cell[j] &&
-                            np == par[j] && ng < it[j].gidx);
-      }
-      lead[j] = want[j] && (!beaten || a.open);
+  bool more = want && a.open != 0u;
+  want = want && ((word >> (cell & 31u)) & 1u) == 0u;
+  const unsigned long long key = ((unsigned long long)par << (3u * c.G)) | cell;
+  const unsigned long long val = ((unsigned long long)it.gidx << 32) | it.rgba;
+  bool lead = want;
+  if (SORTED) {
+    // a neighbour lane in the same cell with a lower index: done
+    const unsigned wm = __ballot_sync(FULL_MASK, want);
+    const uint32_t pc = __shfl_up_sync(FULL_MASK, cell, 1);
+    const uint32_t pp = __shfl_up_sync(FULL_MASK, par, 1);
+    const uint32_t pg = __shfl_up_sync(FULL_MASK, it.gidx, 1);
+    bool beaten = lane != 0u && ((wm >> (lane - 1u)) & 1u) && pc == cell && pp == par &&
+                  pg < it.gidx;
+    if (respill) {
+      const uint32_t nc2 = __shfl_down_sync(FULL_MASK, cell, 1);
+      const uint32_t np = __shfl_down_sync(FULL_MASK, par, 1);
+      const uint32_t ng = __shfl_down_sync(FULL_MASK, it.gidx, 1);
+      beaten = beaten || (lane != 31u && ((wm >> (lane + 1u)) & 1u) && nc2 == cell && np == par &&
+                          ng < it.gidx);
     }
+    lead = want && (!beaten || a.open);
   }
-  warp_claim<N>(c, wb, lead, key, val, par, a.near, more);
-#pragma unroll
-  for (int j = 0; j < N; ++j) {
-    // a re-inserted point sampled the grids above its old leaf when it came
-    if ((it[j].node & RESPILL) && par[j] < a.nodes0) more[j] = false;
-    const unsigned mm = __ballot_sync(FULL_MASK, more[j]);
-    if (mm == 0u) continue;
-    if (more[j]) {
-      uint32_t* q = cq.q + cq.n + __popc(mm & ((1u << lane) - 1u));
-      q[0] = par[j] | (it[j].node & RESPILL);
-      q[CLAIM_QUEUE] = it[j].rx;
-      q[2 * CLAIM_QUEUE] = it[j].ry;
-      q[3 * CLAIM_QUEUE] = it[j].rz;
-      q[4 * CLAIM_QUEUE] = it[j].rgba;
-      q[5 * CLAIM_QUEUE] = it[j].gidx;
-    }
-    cq.n += (uint32_t)__popc(mm);
+  warp_claim(c, wb, lead, key, val, par, a.near, more);
+  // a re-inserted point sampled the grids above its old leaf when it came
+  if ((it.node & RESPILL) && par < a.nodes0) more = false;
+  const unsigned mm = __ballot_sync(FULL_MASK, more);
+  if (more) {
+    uint32_t* q = cq.q + cq.n + __popc(mm & ((1u << lane) - 1u));
+    q[0] = par | (it.node & RESPILL);
+    q[CLAIM_QUEUE] = it.rx;
+    q[2 * CLAIM_QUEUE] = it.ry;
+    q[3 * CLAIM_QUEUE] = it.rz;
+    q[4 * CLAIM_QUEUE] = it.rgba;
+    q[5 * CLAIM_QUEUE] = it.gidx;
   }
+  cq.n += (uint32_t)__popc(mm);
   __syncwarp();
 }
 
@@ -1382,15 +1331,15 @@ __device__ __forceinline__ void claim_drain(const Ctx& c, WarpBuf& wb, ClaimQueu
   while (cq.n > keep) {
     const uint32_t k = cq.n < 32u ? cq.n : 32u;
     cq.n -= k;
-    const bool on[1] = {lane_id() < k};
-    ClaimItem it[1] = {{0, 0, 0, 0, 0, 0}};
-    if (on[0]) {
+    const bool on = lane_id() < k;
+    ClaimItem it{0, 0, 0, 0, 0, 0};
+    if (on) {
       const uint32_t* q = cq.q + cq.n + lane_id();
-      it[0] = ClaimItem{q[0], q[CLAIM_QUEUE], q[2 * CLAIM_QUEUE], q[3 * CLAIM_QUEUE],
-                        q[4 * CLAIM_QUEUE], q[5 * CLAIM_QUEUE]};
+      it = ClaimItem{q[0], q[CLAIM_QUEUE], q[2 * CLAIM_QUEUE], q[3 * CLAIM_QUEUE],
+                     q[4 * CLAIM_QUEUE], q[5 * CLAIM_QUEUE]};
     }
     __syncwarp();
-    claim_level<1, false>(c, wb, cq, a, on, it, false);
+    claim_level<false>(c, wb, cq, a, on, it, false);
   }
 }
 
@@ -1402,7 +1351,6 @@ __device__ __forceinline__ void claim_drain(const Ctx& c, WarpBuf& wb, ClaimQueu
 __device__ void phase_claim(const Ctx& c, uint32_t* smem, const NodeCache nc, const int4* pts,
                             uint32_t n, unsigned long long base, uint32_t t_hi, uint32_t s_hi,
                             const ClaimArgs& a, uint32_t warp0, uint32_t nwarps) {
-  constexpr int U = CLAIM_U;
   tally_init(smem);
   __syncthreads();  // also publishes the caller's node-cache writes
   zero_grids(c, s_hi, warp0, nwarps);
@@ -1414,8 +1362,8 @@ __device__ void phase_claim(const Ctx& c, uint32_t* smem, const NodeCache nc, co
   // units [0, us) are re-inserted points, the rest batch points
   const uint32_t us = t_hi * c.parts, units = us + (n + 31u) / 32u;
   const uint32_t chl = count_chunk_log2(units, nwarps);
-  int4 pn[U];
-  uint32_t curn[U], gn[U];
+  int4 pn;
+  uint32_t curn, gn;
   auto load = [&](uint32_t w, int4& p, uint32_t& cur, uint32_t& g) {  // cur = NONE: no point
     p = make_int4(0, 0, 0, 0);
     cur = NONE;
@@ -1437,36 +1385,30 @@ __device__ void phase_claim(const Ctx& c, uint32_t* smem, const NodeCache nc, co
       }
     }
   };
-#pragma unroll
-  for (int j = 0; j < U; ++j) load(warp_unit(warp0, nwarps, j, chl), pn[j], curn[j], gn[j]);
+  load(warp_unit(warp0, nwarps, 0, chl), pn, curn, gn);
   // (the last time round there are no points, and the queue is emptied: one copy
   // of the drain, 10 KB of code less than with a second one behind the loop. The
   // persistent kernel's phases share the instruction caches: a 16M-point terrain
   // 2.248 against 2.266 ms)
-  for (uint32_t k = 0, more = 1; more; k += U) {
-    more = warp_unit(warp0, nwarps, k, chl) < units;
-    bool on[U];
-    ClaimItem it[U];
-#pragma unroll
-    for (int j = 0; j < U; ++j) {
-      const uint32_t w = warp_unit(warp0, nwarps, k + j, chl);
-      on[j] = curn[j] != NONE;
-      it[j] = ClaimItem{curn[j], 0, 0, 0, (uint32_t)pn[j].w, gn[j]};
-      rel_coords(c, pn[j], it[j].rx, it[j].ry, it[j].rz);
-      load(warp_unit(warp0, nwarps, k + j + U, chl), pn[j], curn[j], gn[j]);
-      if (on[j]) {
-        const uint32_t cur = it[j].node & ~RESPILL;
-        const uint32_t leaf = walk_down(c, nc, cur, it[j].rx, it[j].ry, it[j].rz);
-        if (w < us) {
-          const uint32_t t = div_by(w, c.parts, c.P_mul, c.P_shift);
-          c.sp_cur[c.tasks[t].dst + (w - t * c.parts) * 32u + lane] = leaf;
-        } else if (leaf != cur) {
-          c.b_cur[(w - us) * 32 + lane] = leaf;
-        }
-        it[j].node = leaf | (it[j].node & RESPILL);
+  for (uint32_t k = 0, more = 1; more; ++k) {
+    const uint32_t w = warp_unit(warp0, nwarps, k, chl);
+    more = w < units;
+    const bool on = curn != NONE;
+    ClaimItem it{curn, 0, 0, 0, (uint32_t)pn.w, gn};
+    rel_coords(c, pn, it.rx, it.ry, it.rz);
+    load(warp_unit(warp0, nwarps, k + 1u, chl), pn, curn, gn);
+    if (on) {
+      const uint32_t cur = it.node & ~RESPILL;
+      const uint32_t leaf = walk_down(c, nc, cur, it.rx, it.ry, it.rz);
+      if (w < us) {
+        const uint32_t t = div_by(w, c.parts, c.P_mul, c.P_shift);
+        c.sp_cur[c.tasks[t].dst + (w - t * c.parts) * 32u + lane] = leaf;
+      } else if (leaf != cur) {
+        c.b_cur[(w - us) * 32 + lane] = leaf;
       }
+      it.node = leaf | (it.node & RESPILL);
     }
-    claim_level<U, true>(c, wb, cq, a, on, it, warp_unit(warp0, nwarps, k, chl) < us);
+    claim_level<true>(c, wb, cq, a, on, it, w < us);
     claim_drain(c, wb, cq, a, more ? 31u : 0u);
   }
   warp_flush(c, wb);

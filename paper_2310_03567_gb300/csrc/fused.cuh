@@ -80,7 +80,8 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
 // one per warp, reaches the control block's L2 lines.
 struct CtlView {
   unsigned long long bump0;
-  uint32_t n_nodes, key_rate, open, reject, split_count, split_inner, split_most, ntasks, spill_count, nkeys, stop;
+  uint32_t n_nodes, key_rate, open, reject, split_count, split_inner, split_most, ntasks;
+  uint32_t spill_count, nkeys, stop;
   int pool_top;
 };
 

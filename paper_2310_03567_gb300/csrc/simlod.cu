@@ -895,8 +895,8 @@ int insert_device(simlod_t* h, const int4* pts, uint64_t n, cudaStream_t s) {
   const Ctx& c = h->ctx;
   const unsigned long long base = h->base;
   const uint32_t nodes0 = h->n_nodes;
-  const unsigned gp = std::max(1u, std::min<unsigned>(grid_for(h, n, PBLOCK), (unsigned)PHASE_MIN_BLOCKS * h->sm_count));
   const unsigned full = (unsigned)PHASE_MIN_BLOCKS * h->sm_count;
+  const unsigned gp = std::max(1u, std::min<unsigned>(grid_for(h, n, PBLOCK), full));
   const uint32_t max_iters = h->cfg.max_expand_iters ? h->cfg.max_expand_iters
                                                       : h->cfg.root_log2 + 1;
   int rc;
