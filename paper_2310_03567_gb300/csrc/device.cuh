@@ -246,8 +246,8 @@ struct Ctx {
   uint32_t* hist;     // counts of the cubes below split leaves; zero between updates
   uint32_t* hist_up;  //   their sums per inner level, and the list of inner nodes
   HSlot* hash;
-  uint32_t* keys;     // backlog: table slots of this update's new cells
-  uint32_t* key_node; //   and the nodes of the first key_nodes of them
+  uint2* keys;        // backlog: table slot and node of this update's first key_nodes new
+                      //   cells, behind them the slots of the others
   uint8_t* data;
   unsigned long long data_bytes;
   int4* staging;
@@ -634,6 +634,12 @@ __device__ __forceinline__ LaneRun lane_run(bool on, T v) {
   return r;
 }
 
+// The slot of backlog entry e (the arena may leave no room for all entries' nodes).
+__device__ __forceinline__ uint32_t* key_slot(const Ctx& c, uint32_t e) {
+  return e < c.key_nodes ? &c.keys[e].x
+                         : reinterpret_cast<uint32_t*>(c.keys + c.key_nodes) + (e - c.key_nodes);
+}
+
 // Per-warp staging of the table slots of new cells (shared memory), flushed
 // to the backlog with one atomic per flush.
 struct WarpBuf {
@@ -660,8 +666,8 @@ __device__ __forceinline__ void warp_flush(const Ctx& c, WarpBuf& wb) {
   for (uint32_t k = lane_id(); k < wb.n; k += 32) {
     const uint32_t e = e0 + k;
     const uint2 at = wb.buf[k];  // slot, node
-    if (e < c.key_nodes) c.key_node[e] = at.y;
-    if (e < c.backlog_cap) c.keys[e] = at.x;
+    if (e < c.key_nodes) c.keys[e] = at;
+    else if (e < c.backlog_cap) *key_slot(c, e) = at.x;
     else set_error(c, E_BACKLOG);
   }
   wb.n = 0;
@@ -1884,15 +1890,15 @@ __device__ void phase_store_voxels(const Ctx& c, uint32_t* smem, uint32_t n_task
       [&](uint32_t w) -> uint32_t {
         const uint32_t e = w * 32u + lane;
         if (e >= n_keys) return NONE;
-        // (where the arena leaves no room for the list of nodes, from the slot)
-        const uint32_t node = e < c.key_nodes ? c.key_node[e]
-                                              : (uint32_t)(c.hash[c.keys[e]].key >> (3u * G));
+        const uint32_t node = e < c.key_nodes
+                                  ? c.keys[e].y
+                                  : (uint32_t)(c.hash[*key_slot(c, e)].key >> (3u * G));
         if (node < c.max_nodes) return node;
         set_error(c, E_INTERNAL);
         return NONE;
       },
       [&](uint32_t w, StoreItem& it) {
-        it.slot = c.keys[w * 32u + lane];
+        it.slot = *key_slot(c, w * 32u + lane);
         it.gref = c.gridref[it.node];
         const ulonglong2 kv = *reinterpret_cast<const ulonglong2*>(c.hash + it.slot);
         // the node's min corner and level

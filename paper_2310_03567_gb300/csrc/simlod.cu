@@ -514,7 +514,7 @@ static const char* const kKernelNames[SIMLOD_N_KERNELS] = {
 
 struct Layout {
   size_t ctl, fctl, batches, child, gridref, cnt, num, meta, pool, pending, alloc_refs, splits,
-      tasks, sp_cur, b_cur, hist, scratch, scur, hash, keys, key_node, staging, data, end;
+      tasks, sp_cur, b_cur, hist, scratch, scur, hash, keys, staging, data, end;
   uint64_t hash_slots, hist_words, key_nodes, max_chunks, max_splits, data_bytes;
 };
 
@@ -671,8 +671,7 @@ bool plan_layout(const simlod_config* c, size_t arena_bytes, Layout* L) {
     L->scratch = take(scratch_bytes(c, hist_words));
     L->scur = take(4 * N);
     L->hash = take(sizeof(HSlot) * L->hash_slots);
-    L->keys = take(4 * c->backlog_capacity);
-    L->key_node = take(4 * key_nodes);
+    L->keys = take(4 * c->backlog_capacity + 4 * key_nodes);
     L->staging = take(16 * B);
     return align_up(o, 256);
   };
@@ -727,8 +726,7 @@ void make_ctx(simlod_t* h) {
   c.hist_words = L.hist_words;
   c.scur = reinterpret_cast<uint32_t*>(a + L.scur);
   c.hash = reinterpret_cast<HSlot*>(a + L.hash);
-  c.keys = reinterpret_cast<uint32_t*>(a + L.keys);
-  c.key_node = reinterpret_cast<uint32_t*>(a + L.key_node);
+  c.keys = reinterpret_cast<uint2*>(a + L.keys);
   c.key_nodes = (uint32_t)L.key_nodes;
   c.staging = reinterpret_cast<int4*>(a + L.staging);
   c.data = a + L.data;
