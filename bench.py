@@ -59,9 +59,9 @@ def update_alg_bytes(B, S, V, K, grid_bytes):
 KERNEL_SOURCES = ("paper_2310_03567_gb300/csrc/device.cuh", "paper_2310_03567_gb300/csrc/fused.cuh",
                   "include/simlod.h", "paper_2310_03567_gb300/_build.py")
 TRAFFIC_PER_LAUNCH = {
-    # clustered-300M, one launch over its 54 batches: 31.76 GB read + 14.19 GB
-    # written in 29.72 ms (profiles/k_fused_clustered300m_dram.md)
-    ("677a18cd436eca1a", "clustered-300000000"): 45.95e9,
+    # clustered-300M, one launch over its 54 batches: 31.56 GB read + 14.19 GB
+    # written in 29.71 ms (profiles/k_fused_clustered300m_dram.md)
+    ("c2d9cf460ef7e612", "clustered-300000000"): 45.75e9,
 }
 
 
